@@ -335,16 +335,19 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __rest
         first = false;
     }
     if (!aborted && !first) {
-        // warp w reads TMEM lanes 32w .. 32w+31 of every M-tile: A rows m*128 + 32w + lane
+        // a warp can read only the TMEM lane quarter 32 (w % 4) .. + 31: warps
+        // 0-3 take the even M-tiles and warps 4-7 the odd ones, A rows
+        // m*128 + 32 (w % 4) + lane
         tc_fence_after();
         float* part = partial + (size_t)blockIdx.x * (9 * CIN * COUT + COUT);
+        const int q4 = warp & 3;
 #pragma unroll 1
-        for (int m = 0; m < S::MT; ++m) {
-            const int r = m * kM + 32 * warp + lane;
+        for (int m = warp >> 2; m < S::MT; m += kWgThreads / 128) {
+            const int r = m * kM + 32 * q4 + lane;
 #pragma unroll
             for (int cb = 0; cb < S::N; cb += 16) {
                 float v[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(m * S::N + cb), v);
+                tmem_ld16(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(m * S::N + cb), v);
                 if (r < S::MR) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i)

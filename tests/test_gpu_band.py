@@ -367,6 +367,46 @@ def test_backward_layers_match_elementwise(fbs, oracle_mod):
         assert err <= GRAD_TOL, (l, err)
 
 
+def test_weight_gradients_repeat_and_match_on_a_training_crop(fbs, oracle_mod):
+    """A crop of the size the network is trained on (several chunks of pixels per
+    CTA of the weight-gradient kernel): every gradient repeats bit for bit, and
+    every layer's weight and bias gradient lies within the FP32 accumulation
+    bound of the FP64 sum over the kernels' own operands."""
+    from tests import _band_ref as br
+    H, W, D, h = 640, 1280, 64, 8
+    L, R = _rand_pair(31, H, W, 3, shift=20)
+    rng = np.random.default_rng(32)
+    li = rng.integers(0, D, (H, W)).astype(np.int32)
+    li[:, : W // 2] = 20
+    ls = (li + rng.uniform(-0.5, 0.5, (H, W))).astype(np.float32)
+    Hq, Wq, _ = oracle_mod.quarter_shape(H, W, D)
+    na, ng = _trace_sizes(Hq, Wq)
+    acts = torch.empty(na, dtype=torch.float32, device="cuda")
+    grads = torch.empty(ng, dtype=torch.float32, device="cuda")
+    runs = []
+    with fbs.Context(0) as ctx:
+        fbs.fbs_band_net_set_params(ctx.ctx, _params(2))
+        dl, dr, dli, dls = _dev(L), _dev(R), _dev(li), _dev(ls)
+        for _ in range(4):
+            grad = np.zeros(bn.param_count(), np.float32)
+            fbs.fbs_band_net_train_step(ctx.ctx, dl, dr, H, W, 3, D, dli, dls, h, 0.0, None, grad)
+            runs.append(grad)
+        fbs.fbs_band_net_trace(ctx.ctx, acts, grads)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(ctx.ctx)
+    assert all(np.array_equal(runs[0], g) for g in runs[1:])
+    (x0, ys, _), (gs, go) = br.split_trace(acts.cpu().numpy(), grads.cpu().numpy(), Hq, Wq)
+    inputs, outs = [x0[..., :6]] + ys, gs + [go[..., :2]]
+    o = 0
+    for l, (ci, co) in enumerate(zip(bn.CIN, bn.COUT)):
+        dW, db, dWa, dba = br.weight_grad_with_scale(inputs[l], outs[l])
+        g = runs[0][o: o + 9 * ci * co + co].astype(np.float64)
+        o += 9 * ci * co + co
+        N = Hq * Wq
+        assert np.all(np.abs(g[: 9 * ci * co].reshape(dW.shape) - dW) <= br.gamma(N) * dWa + 2.0 ** -24 * np.abs(dW)), l + 1
+        assert np.all(np.abs(g[9 * ci * co:] - db) <= br.gamma(N) * dba + 2.0 ** -24 * np.abs(db)), l + 1
+
+
 def test_training_steps_reduce_the_loss(fbs, oracle_mod):
     """Labels 4 e* + 3 (a constant correction of the coarse winner that the
     network can represent through its biases): 100 Adam steps on one pair
