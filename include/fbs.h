@@ -232,7 +232,7 @@ fbs_status fbs_compute_disparity_batched(fbs_ctx *ctx, int n, const fbs_pair *pa
 
 /* The plan the autotuner chose for this batch shape, or -1 if none yet.
  * FP32 (0..6): plans 0..3 persistent, plan = 2 * order + (aggregation CTAs
- * per SM - 1), order 0 = largest pair first, 1 = as given; plans 4..6
+ * per SM / 2 - 1), order 0 = largest pair first, 1 = as given; plans 4..6
  * branched with {1, 2, 4}[plan - 4] branches.  BF16 / FP16 (0..5): plan = 2 * b + s,
  * graph branches {1, 2, 4}[b], window rows per tensor-core pipeline stage
  * s = 0: the kernel's maximum, s = 1: at most 3. */

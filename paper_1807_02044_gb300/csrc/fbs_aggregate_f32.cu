@@ -8,119 +8,197 @@
 // (for RGB the squared Euclidean colour distance).  The two exponentials are
 // evaluated as one exp2 of the summed exponent.
 //
-// Work decomposition (one CTA = a 32 x 4 pixel tile and a chunk of DC
-// disparities; 8 warps):
-//   * Cost rows r = y0-rho .. y0+3+rho are streamed through a 3-deep ring of
-//     shared-memory buffers with cp.async (zero-filled outside the image), and
-//     the guide row r through a matching ring.
-//   * For each streamed row, the CTA computes the weights w(p, q) of every
-//     tile pixel p whose window contains row r -- once per (p, q), shared by
-//     all DC disparities -- into a double-buffered shared array.
-//   * Warp g owns tile columns 4g..4g+3; lane = (row yi, disparity group k).
-//     A thread accumulates 4 pixels x KD disparities.  Along the window the
-//     four cost columns it needs at tap dx are held in a rotating register
-//     window, so each cost column is read from shared memory once and used
-//     for up to 4 pixels, and each weight is a broadcast read used for KD
-//     disparities.  Lanes of different rows read the same cost address
-//     (broadcast), so a warp's cost read is one 128-byte wavefront.
-//   * One __syncthreads per streamed row.
-//   * After the last row the sums are normalised, staged in shared memory and
-//     reduced per pixel: WTA with the smallest d on ties, plus the values at
-//     d*-1 and d*+1 carried across chunks for Eq. (10).
+// Work decomposition (one CTA = a 32 x 4 pixel tile, 4 warps, four CTAs per
+// SM; the disparities in chunks of 64, 32 or 16):
+//   * The tile's guide window is staged once.  Cost rows r = y0-rho .. y0+3+rho
+//     are streamed through a ring of S rows, one TMA box per row (zeros outside
+//     the image and past D).  The last of the four warps to finish a row issues
+//     the row S later into its slot, so no warp waits for another one except
+//     through a full ring, and warps run up to S - 1 rows apart.
+//   * A warp owns 32 pixels (16 x 2, or 8 x 4 in the band form) and every
+//     disparity of the chunk: it computes their weights for the row (lane =
+//     pixel, once per (p, q) and chunk) into its own shared buffer and then
+//     accumulates, so warps exchange nothing but the staged rows.
+//   * A thread accumulates 8 pixels along x by 8 (4, 2) disparities.  It walks
+//     the columns of the row: a column's costs are loaded once and used for
+//     all of the 8 pixels whose window holds the column, each with its weight
+//     (the 8 weights of a column are contiguous).  Per column: 4 shared loads
+//     of 16 bytes for 32 packed FMAs (two disparities each).
+//   * After the last row the sums are normalised, staged per warp and reduced
+//     per pixel by one lane: WTA with the smallest d on ties, plus the values
+//     at d*-1 and d*+1 carried across chunks for Eq. (10).
+// Every sum runs over the rows and, in a row, over the columns in ascending
+// order, whatever the tile or the chunk.
+//
+// Why this split.  The bound is the FP32 pipe.  A packed FMA takes half the
+// issue slots of two scalar ones, and the freed slots hold the weights; with
+// three fresh register pairs it runs at 94 multiply-adds per clock and SM, with
+// one operand shared by consecutive FMAs at up to 118 (of 128).  An 8 x 8
+// register tile needs (8 + 8) / 64 shared values per multiply-add.  A shared load
+// of 16 bytes takes 2 cycles when no four adjacent lanes hold more than two
+// distinct addresses and 4 cycles otherwise (measured, whatever the number of
+// distinct addresses in the warp), so lane bit 1 never selects a cost address
+// and lane bit 0 never a weight address.  The accumulation loop alone runs at
+// 73% of 128 multiply-adds per clock and SM; with everything around it the
+// kernel is at 45%.  Copying a row with one bulk copy per column instead of one
+// box cost 22 cycles per column and SM and bound the kernel (322 against 244 us),
+// and a __syncthreads per row 313 us.
+//
+// Measured on GB300 (CUDA events), before -> now; before: 4 pixels x 8 disparities
+// per thread, scalar FMAs, 256-thread CTAs in step through a cp.async ring:
+//   640x480,  D = 64,  rho = 7:    425 -> 241 us (36.7 TFLOP/s)
+//   640x480,  D = 64,  rho = 2:    125 ->  62 us
+//   767x575,  D = 93,  rho = 11:  2263 -> 1184 us
+//   1280x960, D = 128, rho = 15: 10390 -> 6896 us (43.8 TFLOP/s)
 #include "fbs_internal.cuh"
+#include "packed_f32.cuh"
+#include "tc_aggregate.cuh"
 
 namespace fbs {
 namespace {
 
 constexpr int kTX = kAggTileX;   // tile width (pixels)
 constexpr int kTY = kAggTileY;   // tile height (rows)
-constexpr int kPX = 4;         // pixels per thread along x
-constexpr int kThreads = 256;  // 8 warps
-constexpr int kNPix = kTX * kTY;
+constexpr int kPX = 8;           // pixels per thread along x
+constexpr int kWarps = 4;
+constexpr int kThreads = 32 * kWarps;
+static_assert(kTX * kTY == 32 * kWarps, "a warp owns 32 pixels of the tile");
 // 2^23 as an FP32 bit pattern: for 0 <= c < 2^23 the pattern kMagic + c is the
 // float 2^23 + c exactly.
 constexpr uint32_t kMagic = 0x4B000000u;
 
-__host__ __device__ inline int weight_stride(int rho)
-{
-    // per-row stride of the weight buffer [dx][kTX]; == 8 (mod 32) so that
-    // the four rows of a warp read four different bank groups
-    int n = (2 * rho + 1) * kTX;
-    n = (n + 31) & ~31;
-    return n + 8;
-}
+// Weights of a group of 8 pixels and one row: [column j][pixel i], j = dx + i
+// (dx = 0 .. 2 rho), so 2 rho + 8 columns of 8 floats; == 8 (mod 32) floats, so
+// that lanes writing pixels i of four groups, 9 i + 8 g, hit 32 banks.
+__host__ __device__ inline int weight_stride(int rho) { return (((2 * rho + kPX) * kPX + 31) & ~31) + 8; }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int src_bytes)
+// Disparities per staged column: 64, or what a short range needs.
+__host__ __device__ inline int column_size(int D) { return D > 32 ? 64 : D > 16 ? 32 : 16; }
+
+// How a cost row is copied to shared memory: one TMA box (volumes that are 16-byte
+// aligned with ld % 4 == 0), 16-byte cp.async (the same, where no tensor map is
+// at hand) or 4-byte cp.async.
+enum Copy { kTma, kAsync16, kAsync4 };
+
+__device__ __forceinline__ void cp_async16(uint32_t smem, const void* gmem, int src_bytes)
 {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(src_bytes)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem, int src_bytes)
+__device__ __forceinline__ void cp_async4(uint32_t smem, const void* gmem, int src_bytes)
 {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(s), "l"(gmem), "r"(src_bytes)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+// The mbarrier gets one arrival of this thread when its earlier cp.async have landed.
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int d, int x, int y, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(d), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+// Counts one more warp done with a slot (its reads before, the caller's writes after).
+__device__ __forceinline__ uint32_t count_done(uint32_t word)
+{
+    uint32_t old;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(old) : "r"(word) : "memory");
+    return old;
+}
 
-template <int DC>
-__host__ __device__ inline size_t smem_bytes(int rho)
+// Spatial terms of Eq. (7): row dy = 0 .. rho of 2 rho + 2 floats (dx = -rho ..
+// rho and one more).
+__host__ __device__ inline int spatial_floats(int rho) { return (rho + 1) * (2 * rho + 2); }
+// Guide window of a tile: (kTY + 2 rho) rows of kTX + 2 rho words, and one more.
+__host__ __device__ inline int guide_words(int rho) { return (kTY + 2 * rho) * (kTX + 2 * rho) + 1; }
+
+// Shared memory of a CTA, in order: barriers and counters of the S slots, the
+// spatial terms, the guide window, then the cost rows [S][NC][DC] and the warps'
+// weights [4][4][WS]; the stage [4][32][DC + 4] of the epilogue lies over these.
+constexpr int kMaxSlots = 4;
+constexpr int kHeaderBytes = 64;   // full[4] (8 bytes each), done[4] (4 bytes each), abort flag
+__host__ __device__ inline size_t front_bytes(int rho)
+{
+    return (kHeaderBytes + 4 * (size_t)spatial_floats(rho) + 4 * (size_t)guide_words(rho) + 127) & ~(size_t)127;
+}
+__host__ __device__ inline size_t smem_bytes(int rho, int dc, int slots)
 {
     const int NC = kTX + 2 * rho;
-    const size_t ring = (size_t)3 * NC * DC;
-    const size_t stage = (size_t)kNPix * (DC + 1);
-    const size_t a = ring > stage ? ring : stage;
-    return sizeof(float) * (a + 2 * (size_t)kTY * weight_stride(rho) + 2 * kNPix) + sizeof(uint2) * 3 * NC;
+    const size_t rows = (size_t)slots * NC * dc + (size_t)kWarps * 4 * weight_stride(rho);
+    const size_t stage = (size_t)kWarps * 32 * (dc + 4);
+    return front_bytes(rho) + sizeof(float) * (rows > stage ? rows : stage);
 }
 
-// Load cost row r, columns x0-rho .. x0-rho+NC-1, disparities dc0 .. dc0+DC-1;
-// disparities >= D (the end of the range being aggregated) are zero-filled.
-template <int DC, bool VEC>
-__device__ __forceinline__ void load_cost_row(float* dst, const float* __restrict__ cost, int ld, int W,
-                                              int D, int r, int x0, int rho, int NC, int dc0)
-{
-    if (VEC) {
-        constexpr int NQ4 = DC / 4;
-        for (int it = threadIdx.x; it < NC * NQ4; it += kThreads) {
-            const int col = it / NQ4, q = it - col * NQ4;
-            const int gx = x0 - rho + col;
-            const int d = dc0 + 4 * q;
-            const bool in = gx >= 0 && gx < W && d < D;
-            const int gxc = in ? gx : 0;
-            const int dcl = in ? d : 0;
-            const float* src = cost + ((size_t)r * W + gxc) * ld + dcl;
-            const int bytes = in ? 4 * min(4, D - d) : 0;
-            cp_async16(dst + col * DC + 4 * q, src, bytes);
-        }
-    } else {
-        for (int it = threadIdx.x; it < NC * DC; it += kThreads) {
-            const int col = it / DC, q = it - col * DC;
-            const int gx = x0 - rho + col;
-            const int d = dc0 + q;
-            const bool in = gx >= 0 && gx < W && d < D;
-            const float* src = cost + ((size_t)r * W + (in ? gx : 0)) * ld + (in ? d : 0);
-            cp_async4(dst + col * DC + q, src, in ? 4 : 0);
+// The ring of cost rows.  Every warp walks every row, so slot and parity (of
+// the row it is at) are the same sequence in all of them.
+struct Ring {
+    uint32_t full, done;      // shared addresses of the slots' barriers and counters
+    volatile uint32_t* abort;
+    int* err;
+    int S, slot;
+    uint32_t parity;
+    __device__ __forceinline__ void next()
+    {
+        if (++slot == S) {
+            slot = 0;
+            parity ^= 1u;
         }
     }
-}
-
-// A guide pixel as (R | G << 8 | B << 16, R^2 + G^2 + B^2); grey images use
-// the first channel only.
-__device__ __forceinline__ uint2 packed_colour(const uint8_t* p, int C)
-{
-    const uint32_t c = C == 3 ? (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) : (uint32_t)p[0];
-    return make_uint2(c, (uint32_t)__dp4a(c, c, 0u));
-}
-
-__device__ __forceinline__ void load_guide_row(uint2* dst, const uint8_t* __restrict__ guide, int W, int C, int r,
-                                               int x0, int rho, int NC)
-{
-    for (int col = threadIdx.x; col < NC; col += kThreads) {
-        const int gx = x0 - rho + col;
-        dst[col] = (gx >= 0 && gx < W) ? packed_colour(guide + ((size_t)r * W + gx) * C, C) : make_uint2(0u, 0u);
+    // Bounded (about 2 s): on a timeout the error word is set and nothing is waited for any more.
+    __device__ __forceinline__ void wait() const
+    {
+        if (tc::mbar_try_wait(full + 8 * slot, parity)) return;
+        if (*abort == 0 && !tc::mbar_wait(full + 8 * slot, parity)) {
+            *abort = 1u;
+            atomicCAS(err, 0, 31);
+        }
     }
+};
+
+// The cost volume of a tile's pair.
+struct Volume {
+    const float* cost;
+    const CUtensorMap* map;   // kTma: dimensions (D, W, H), box (DC, kTX + 2 rho, 1)
+    int ld, W, D;
+};
+
+// One warp loads cost row r, columns xlo .. xlo+NC-1, disparities dc0 ..
+// dc0+DC-1 into a slot; zeros outside the image and for disparities >= D.
+template <int DC, Copy COPY>
+__device__ __forceinline__ void load_cost_row(uint32_t dst, uint32_t bar, const Volume& v, int r, int xlo, int NC, int dc0)
+{
+    const int lane = threadIdx.x & 31;
+    if (COPY == kTma) {
+        if (lane == 0) {
+            tc::fence_proxy_async();   // the slot was read, and may hold staged sums, through the generic proxy
+            tc::mbar_expect_tx(bar, 4u * DC * (uint32_t)NC);
+            tma_load_3d(dst, v.map, dc0, xlo, r, bar);
+        }
+        return;
+    }
+    constexpr int E = COPY == kAsync16 ? 4 : 1;     // floats per copy
+    constexpr int Q = DC / E, STEP = 32 / Q > 0 ? 32 / Q : 1;
+    const float* row = v.cost + (size_t)r * v.W * v.ld;
+    for (int q = lane % Q; q < Q; q += 32) {
+        const int d = dc0 + E * q, bytes = d < v.D ? 4 * min(E, v.D - d) : 0;
+        for (int c = Q < 32 ? lane / Q : 0; c < NC; c += STEP) {
+            const bool in = (unsigned)(xlo + c) < (unsigned)v.W && bytes > 0;
+            const float* src = in ? row + (size_t)(xlo + c) * v.ld + d : v.cost;
+            if (E == 4) cp_async16(dst + 4 * (c * DC + E * q), src, in ? bytes : 0);
+            else cp_async4(dst + 4 * (c * DC + E * q), src, in ? bytes : 0);
+        }
+    }
+    cp_async_arrive(bar);
+}
+
+// A guide pixel as R | G << 8 | B << 16; grey images use the first channel only.
+__device__ __forceinline__ uint32_t packed_colour(const uint8_t* p, int C)
+{
+    return C == 3 ? (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) : (uint32_t)p[0];
 }
 
 __device__ __forceinline__ float ex2_approx(float x)
@@ -130,280 +208,506 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
+// Two consecutive taps dx, dx + 1 of one pixel and window row: Eq. (7)-(8) as
+// one exp2, colour distance |q|^2 + |p|^2 - 2 q.p exact in integers, then
+// float(c) = (2^23 + c) - 2^23 exactly.  sp: the two spatial terms
+// ((dx - rho)^2 + dy^2) times -log2(e) / sigma_s^2.  EDGE: a tap outside the
+// image columns has weight 0.
+struct Pixel {
+    uint32_t col, norm;       // its colour, |p|^2 + 2^23
+    uint64_t magic2, nkr2;    // (-2^23, -2^23) and -log2(e) / sigma_r^2 twice
+    int qx, W;                // image column of tap 0
+};
+template <bool EDGE>
+__device__ __forceinline__ void weight_pair(const Pixel& p, uint32_t q0, uint32_t q1, uint64_t sp, int dx, float& w0,
+                                            float& w1)
+{
+    const uint32_t d0 = __dp4a(q0, p.col, 0u), d1 = __dp4a(q1, p.col, 0u);
+    const uint32_t e0 = __dp4a(q0, q0, p.norm) - d0 - d0, e1 = __dp4a(q1, q1, p.norm) - d1 - d1;
+    f2_unpack(f2_fma(f2_add(u2_pack(e0, e1), p.magic2), p.nkr2, sp), w0, w1);
+    w0 = ex2_approx(w0);
+    w1 = ex2_approx(w1);
+    if (EDGE) {
+        w0 = (unsigned)(p.qx + dx) < (unsigned)p.W ? w0 : 0.f;
+        w1 = (unsigned)(p.qx + dx + 1) < (unsigned)p.W ? w1 : 0.f;
+    }
+}
+
+// All taps of one pixel and window row, in order: tap dx goes to w[8 dx] (w
+// offset by the pixel's place in its group) and to den0 (dx <= rho) or den1.
+// sp holds 2 rho + 2 spatial terms; g[2 rho + 1] is read and not used.
+template <bool EDGE>
+__device__ __forceinline__ void weight_row(const Pixel& p, const uint32_t* g, const uint64_t* sp, float* w, int rho,
+                                           float& den0, float& den1)
+{
+    float a, b;
+    int dx = 0;
+    auto pair = [&]() {
+        weight_pair<EDGE>(p, g[0], g[1], sp[0], dx, a, b);
+        w[0] = a;
+        w[kPX] = b;
+        g += 2;
+        sp += 1;
+        w += 2 * kPX;
+        dx += 2;
+    };
+    const int n0 = (rho + 1) >> 1;
+#pragma unroll 4
+    for (int j = 0; j < n0; ++j) {
+        pair();
+        den0 += a;
+        den0 += b;
+    }
+    if (!(rho & 1) && rho > 0) {   // taps rho and rho + 1
+        pair();
+        den0 += a;
+        den1 += b;
+    }
+#pragma unroll 4
+    for (int j = (rho >> 1) + 1; j < rho; ++j) {
+        pair();
+        den1 += a;
+        den1 += b;
+    }
+    weight_pair<EDGE>(p, g[0], g[1], sp[0], dx, a, b);   // tap 2 rho
+    w[0] = a;
+    if (rho == 0) den0 += a;
+    else den1 += a;
+}
+
+// Two consecutive costs of a column as a packed pair, KD of them per thread:
+// disparities 4 k .. 4 k + 3 (and 32 + the same) of the chunk, or 2 k, 2 k + 1.
+template <int KD>
+__device__ __forceinline__ void load_costs(uint32_t a, uint64_t (&c)[KD / 2])
+{
+    if (KD == 2) {
+        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(c[0]) : "r"(a) : "memory");
+    } else {
+#pragma unroll
+        for (int q = 0; q < KD / 4; ++q)
+            asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                         : "=l"(c[2 * q]), "=l"(c[2 * q + 1])
+                         : "r"(a + 128 * q)
+                         : "memory");
+    }
+}
+
+__device__ __forceinline__ void load_weights(uint32_t a, float (&w)[4])
+{
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+// One column: pixels LO .. HI-1 of the thread's 8 get their weight times the
+// column's costs.  The cost pair is the operand that consecutive FMAs share
+// (an FMA with three fresh register pairs issues every 2.7 cycles instead of 2).
+template <int KD, int LO, int HI>
+__device__ __forceinline__ void column(uint64_t (&acc)[kPX][KD / 2], uint32_t ca, uint32_t wa)
+{
+    uint64_t c[KD / 2], ww[kPX];
+    load_costs<KD>(ca, c);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (h == 0 ? LO >= 4 : HI <= 4) continue;
+        float w[4];
+        load_weights(wa + 16 * h, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ww[4 * h + i] = f2_pack(w[i], w[i]);
+    }
+#pragma unroll
+    for (int k = 0; k < KD / 2; ++k)
+#pragma unroll
+        for (int i = LO; i < HI; ++i) acc[i][k] = f2_fma(c[k], ww[i], acc[i][k]);
+}
+
+// Columns J, J + 1, .. of a window of a fixed radius RHO < 4.
+template <int KD, int DC, int RHO, int J>
+__device__ __forceinline__ void narrow_columns(uint64_t (&acc)[kPX][KD / 2], uint32_t ca, uint32_t wa)
+{
+    if constexpr (J < 2 * RHO + kPX) {
+        column<KD, (J > 2 * RHO ? J - 2 * RHO : 0), (J < kPX ? J + 1 : kPX)>(acc, ca + J * DC * 4, wa + J * kPX * 4);
+        narrow_columns<KD, DC, RHO, J + 1>(acc, ca, wa);
+    }
+}
+
+// One window row of a thread: columns j = 0 .. 2 rho + 7, pixel i takes part in
+// columns i .. i + 2 rho.  ca, wa: shared addresses of column 0's costs and weights.
+template <int KD, int DC>
+__device__ __forceinline__ void accumulate_row(uint64_t (&acc)[kPX][KD / 2], uint32_t ca, uint32_t wa, int rho)
+{
+    constexpr uint32_t CS = DC * 4, WC = kPX * 4;   // bytes from a column to the next
+    if (rho >= 4) {
+        column<KD, 0, 1>(acc, ca, wa);
+        column<KD, 0, 2>(acc, ca + CS, wa + WC);
+        column<KD, 0, 3>(acc, ca + 2 * CS, wa + 2 * WC);
+        column<KD, 0, 4>(acc, ca + 3 * CS, wa + 3 * WC);
+        column<KD, 0, 5>(acc, ca + 4 * CS, wa + 4 * WC);
+        column<KD, 0, 6>(acc, ca + 5 * CS, wa + 5 * WC);
+        column<KD, 0, 7>(acc, ca + 6 * CS, wa + 6 * WC);
+        ca += 7 * CS;
+        wa += 7 * WC;
+#pragma unroll 1
+        for (int n = rho - 3; n > 0; --n) {     // 2 rho - 6 columns with all 8 pixels
+            column<KD, 0, 8>(acc, ca, wa);
+            column<KD, 0, 8>(acc, ca + CS, wa + WC);
+            ca += 2 * CS;
+            wa += 2 * WC;
+        }
+        column<KD, 1, 8>(acc, ca, wa);
+        column<KD, 2, 8>(acc, ca + CS, wa + WC);
+        column<KD, 3, 8>(acc, ca + 2 * CS, wa + 2 * WC);
+        column<KD, 4, 8>(acc, ca + 3 * CS, wa + 3 * WC);
+        column<KD, 5, 8>(acc, ca + 4 * CS, wa + 4 * WC);
+        column<KD, 6, 8>(acc, ca + 5 * CS, wa + 5 * WC);
+        column<KD, 7, 8>(acc, ca + 6 * CS, wa + 6 * WC);
+    } else {
+        // windows narrower than the thread's 8 pixels: no column belongs to all of them
+        if (rho == 3) narrow_columns<KD, DC, 3, 0>(acc, ca, wa);
+        else if (rho == 2) narrow_columns<KD, DC, 2, 0>(acc, ca, wa);
+        else if (rho == 1) narrow_columns<KD, DC, 1, 0>(acc, ca, wa);
+        else narrow_columns<KD, DC, 0, 0>(acc, ca, wa);
+    }
+}
+
+// What a tile's chunks share: the arguments, the lane's own pixel (the one
+// whose weights, WTA and Eq. (10) it does) and that pixel's WTA state.
+struct Tile {
+    Volume vol;
+    int H, W, D, rho;
+    float neg_kr;
+    int x0, y0, r_lo, r_hi, d_end;
+    const float* spatial;
+    const uint32_t* guide;   // row r_lo, column x0 - rho
+    float* rows;             // cost rows, weights, stage
+    int wy;                  // the warp's first row
+    int px, py;              // the lane's pixel
+    uint32_t pcol;
+    int blo, bhi;            // its band
+    int wlo, whi;            // union of the bands of the warp's pixels
+    float best, a_prev, a_next, last;
+    int bidx;
+    bool pending;
+};
+
+// WTA of one pixel over the staged values j0 .. j1-1 (disparities dc0 + j):
+// the smallest value, the first of equal ones (a NaN never wins), and the
+// neighbours of the winner for Eq. (10), which may lie in the chunks before and after.
+__device__ __forceinline__ void wta_chunk(Tile& t, const float* st, int dc0, int j0, int j1)
+{
+    if (j0 >= j1) return;
+    const float inf = __int_as_float(0x7f800000);
+    auto read4 = [&](int j4, float (&v)[4]) {
+        const float4 q = *(const float4*)(st + j4);
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+        if (j4 < j0 || j4 + 4 > j1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = j4 + e < j0 || j4 + e >= j1 ? inf : v[e];
+        }
+    };
+    float m = inf, v[4];
+#pragma unroll 4
+    for (int j4 = j0 & ~3; j4 < j1; j4 += 4) {
+        read4(j4, v);
+        m = fminf(m, fminf(fminf(v[0], v[1]), fminf(v[2], v[3])));
+    }
+    if (t.pending) {
+        t.a_next = st[j0];
+        t.pending = false;
+    }
+    if (m < t.best) {
+        int k = j1 - 1;
+#pragma unroll 4
+        for (int j4 = (j1 - 1) & ~3; j4 >= j0 - 3; j4 -= 4) {
+            read4(j4, v);
+#pragma unroll
+            for (int e = 3; e >= 0; --e) k = v[e] == m ? j4 + e : k;
+        }
+        t.best = st[k];
+        t.bidx = dc0 + k;
+        t.a_prev = k > j0 ? st[k - 1] : t.last;
+        t.pending = k + 1 == j1;
+        if (k + 1 < j1) t.a_next = st[k + 1];
+    }
+    t.last = st[j1 - 1];
+}
+
+// Disparities dc0 .. dc0 + 8 KD - 1 of a tile (columns of DC staged disparities).
+// Starts and ends with every warp at the same point (a __syncthreads).
+template <int KD, int DC, Copy COPY, int ROWS>
+__device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_out, int dc0)
+{
+    constexpr int NDC = 8 * KD;       // disparities of this chunk
+    constexpr int PW = 32 / ROWS;     // pixels of a warp along x
+    constexpr int SEGS = PW / kPX;    // groups of 8 pixels along x
+    constexpr int SP = NDC + 4;       // stage pitch: 16-byte reads of 8 lanes hit 8 different bank groups
+    static_assert(NDC <= DC, "a chunk lies in its columns");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rho = t.rho, NC = kTX + 2 * rho, WS = weight_stride(rho);
+    const int xlo = t.x0 - rho;
+    const uint32_t slot_bytes = (uint32_t)NC * DC * 4;
+    float* const wbuf = t.rows + ring.S * NC * DC + warp * 4 * WS;
+    const uint32_t rows_a = tc::smem_u32(t.rows);
+
+    // rows some pixel of the warp needs (none when no pixel has its band in this chunk)
+    const bool on = t.whi >= dc0 && t.wlo < dc0 + NDC;
+    const int w_lo = on ? t.wy - rho : t.H, w_hi = min(t.H - 1, t.wy + ROWS - 1) + rho;
+    // a chunk that no warp needs is passed over
+    if (!__syncthreads_or(on)) return;
+    auto load_row = [&](int r, int slot) {
+        load_cost_row<DC, COPY>(rows_a + slot * slot_bytes, ring.full + 8 * slot, t.vol, r, xlo, NC, dc0);
+    };
+    if (warp < ring.S && t.r_lo + warp <= t.r_hi) {
+        const int slot = ring.slot + warp;
+        load_row(t.r_lo + warp, slot < ring.S ? slot : slot - ring.S);
+    }
+
+    // accumulating role: lane bits 0, 2, 3 = disparity group k, bits 1, 4 = pixel group
+    const int k = (lane & 1) | ((lane >> 1) & 6);
+    const int grow = ROWS == 2 ? (lane >> 1) & 1 : ((lane >> 1) & 1) | ((lane >> 3) & 2);
+    const int gseg = ROWS == 2 ? lane >> 4 : 0;
+    const int gy = t.wy + grow;
+    const int wx = t.px - t.x0 - lane % PW;      // the warp's first column in the tile
+    const uint32_t ca0 = rows_a + 4 * ((wx + kPX * gseg) * DC + (KD == 2 ? 2 : 4) * k);
+    const uint32_t wa0 = tc::smem_u32(wbuf) + 4 * (grow * SEGS + gseg) * WS;
+    // weight role: lane = pixel (lane / PW, lane % PW) of the warp
+    float* const wout = wbuf + (lane / kPX) * WS + (lane % kPX) * (kPX + 1);
+    const Pixel self{t.pcol, __dp4a(t.pcol, t.pcol, kMagic), f2_pack(-8388608.f, -8388608.f),
+                     f2_pack(t.neg_kr, t.neg_kr), t.px - rho, t.W};
+    const bool edge = xlo < 0 || xlo + NC > t.W;
+
+    uint64_t acc[kPX][KD / 2];
+#pragma unroll
+    for (int i = 0; i < kPX; ++i)
+#pragma unroll
+        for (int q = 0; q < KD / 2; ++q) acc[i][q] = 0ull;
+    float den0 = 0.f, den1 = 0.f;
+
+    const uint32_t* g = t.guide + (t.px - t.x0);
+    for (int r = t.r_lo; r <= t.r_hi; ++r, g += NC) {
+        if (r >= w_lo && r <= w_hi) {
+            const int dy = r - t.py;
+            if (t.py < t.H && dy >= -rho && dy <= rho) {
+                const uint64_t* sp = (const uint64_t*)(t.spatial + abs(dy) * (2 * rho + 2));
+                if (edge) weight_row<true>(self, g, sp, wout, rho, den0, den1);
+                else weight_row<false>(self, g, sp, wout, rho, den0, den1);
+            }
+            __syncwarp();
+            ring.wait();
+            const int gdy = r - gy;
+            if (gy < t.H && gdy >= -rho && gdy <= rho) accumulate_row<KD, DC>(acc, ca0 + ring.slot * slot_bytes, wa0, rho);
+        } else {
+            ring.wait();   // a row not needed is waited for too: a warp must not count a slot's next row early
+        }
+        __syncwarp();
+        uint32_t done = 0;
+        if (lane == 0) done = count_done(ring.done + 4 * ring.slot);
+        done = __shfl_sync(0xffffffffu, done, 0);
+        // the last warp to finish the row refills its slot
+        if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && *ring.abort == 0) load_row(r + ring.S, ring.slot);
+        ring.next();
+    }
+    __syncthreads();   // every row consumed: the stage may overwrite the rows and weights
+
+    // normalise and stage [pixel of the warp][d]
+    float* const stage = t.rows + warp * 32 * SP;
+    const float inv_own = 1.f / (den0 + den1);
+#pragma unroll
+    for (int i = 0; i < kPX; ++i) {
+        const int pix = grow * PW + gseg * kPX + i;
+        const float inv = __shfl_sync(0xffffffffu, inv_own, pix);
+        float* st = stage + pix * SP + (KD == 2 ? 2 : 4) * k;
+        float v[KD];
+#pragma unroll
+        for (int q = 0; q < KD / 2; ++q) {
+            f2_unpack(acc[i][q], v[2 * q], v[2 * q + 1]);
+            v[2 * q] *= inv;
+            v[2 * q + 1] *= inv;
+        }
+        if (KD == 2) {
+            *(float2*)st = make_float2(v[0], v[1]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < KD / 4; ++q)
+                *(float4*)(st + 32 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
+    }
+    __syncwarp();
+    const int nd = min(NDC, t.d_end - dc0);
+    if (agg_out != nullptr) {
+        for (int pix = 0; pix < 32; ++pix) {
+            const int ey = t.wy + pix / PW, ex = t.x0 + wx + pix % PW;
+            if (ey < t.H && ex < t.W)
+                for (int j = lane; j < nd; j += 32)
+                    agg_out[((size_t)ey * t.W + ex) * t.D + dc0 + j] = stage[pix * SP + j];
+        }
+    }
+    wta_chunk(t, stage + lane * SP, dc0, max(0, t.blo - dc0), min(nd, t.bhi + 1 - dc0));
+    tc::fence_proxy_async();   // the next chunk's bulk copies overwrite the stage
+    __syncthreads();
+}
+
+// The ring's barriers and counters, set up once per CTA (ends with a __syncthreads).
+template <Copy COPY>
+__device__ __forceinline__ Ring make_ring(void* smem, int slots, int* err)
+{
+    Ring ring;
+    ring.full = tc::smem_u32(smem);
+    ring.done = ring.full + 8 * kMaxSlots;
+    ring.abort = (volatile uint32_t*)((uint8_t*)smem + 12 * kMaxSlots);
+    ring.err = err;
+    ring.S = slots;
+    ring.slot = 0;
+    ring.parity = 0;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kMaxSlots; ++s) {
+            tc::mbar_init(ring.full + 8 * s, COPY == kTma ? 1 : 32);
+            ((uint32_t*)smem)[2 * kMaxSlots + s] = 0;
+        }
+        *ring.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    return ring;
+}
+
 // One 32 x 4 tile with top-left pixel (x0, y0), disparities [d_begin, d_end)
 // (the full range: 0, D); ends with a __syncthreads, so a CTA may call it for
 // several tiles in a row.  band (nullable) restricts the WTA and Eq. (10) of
 // each pixel to its own band [lo, hi], a sub-range of [d_begin, d_end);
 // without it every pixel uses [0, D-1].  d_begin must be a multiple of 4.
-template <int KD, bool VEC>
-__device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, int ld,
+template <Copy COPY, int ROWS>
+__device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, const CUtensorMap* map, int ld,
                                                const uint8_t* __restrict__ guide, int H, int W, int C, int D,
                                                int rho, float neg_ks, float neg_kr, float* __restrict__ agg_out,
                                                int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int x0,
-                                               int y0, float4* smem_f4, int d_begin, int d_end,
+                                               int y0, void* smem, Ring& ring, int d_begin, int d_end,
                                                const uint32_t* __restrict__ band)
 {
-    constexpr int DC = 8 * KD;   // disparities per chunk
-    constexpr int NQ = KD / 4;   // float4 groups per thread
-
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, g = tid >> 5;
-    const int yi = lane >> 3, k = lane & 7;
+    constexpr int PW = 32 / ROWS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int NC = kTX + 2 * rho;
-    const int NT = 2 * rho + 1;
-    const int WS = weight_stride(rho);
+    float* const spatial = (float*)((uint8_t*)smem + kHeaderBytes);
+    uint32_t* const gtile = (uint32_t*)(spatial + spatial_floats(rho));
+    Tile t;
+    t.vol = Volume{cost, map, ld, W, D};
+    t.H = H;
+    t.W = W;
+    t.D = D;
+    t.rho = rho;
+    t.neg_kr = neg_kr;
+    t.x0 = x0;
+    t.y0 = y0;
+    t.r_lo = max(0, y0 - rho);
+    t.r_hi = min(H - 1, y0 + kTY - 1 + rho);
+    t.d_end = d_end;
+    t.spatial = spatial;
+    t.guide = gtile;
+    t.rows = (float*)((uint8_t*)smem + front_bytes(rho));
+    t.wy = y0 + ROWS * (warp / (kTX / PW));
+    t.px = x0 + PW * (warp % (kTX / PW)) + lane % PW;
+    t.py = t.wy + lane / PW;
 
-    // shared memory: guide ring [3][NC] uint2 | cost ring [3][NC][DC] (aliased
-    // by the stage [kNPix][DC+1]) | weights [2][kTY][WS] | den [2][kNPix].  NC
-    // is even, so the cost ring starts 16-byte aligned.
-    uint2* const gring = (uint2*)smem_f4;
-    float* const cring = (float*)(gring + 3 * NC);
-    float* const stage = cring;
-    const int cslot = NC * DC;
-    const int ring_sz = 3 * NC * DC, stage_sz = kNPix * (DC + 1);
-    float* const wring = cring + (ring_sz > stage_sz ? ring_sz : stage_sz);
-    const int wslot = kTY * WS;
-    float* const den_s = wring + 2 * wslot;
-
-    // producer role: pixel pp of the tile, half of the dx range
-    const int pp = tid & (kNPix - 1);
-    const int half = tid >> 7;
-    const int pyi = pp / kTX, ppx = pp % kTX;
-    const int py = y0 + pyi, pxg = x0 + ppx;
-    const bool pvalid = py < H && pxg < W;
-    const int dx_lo = half ? rho + 1 : 0;
-    const int dx_hi = half ? NT : rho + 1;
-    // the pixel's colour and |p|^2 + 2^23 (so |q - p|^2 = |q|^2 + |p|^2 - 2 q.p,
-    // exact in integers and below 2^23, becomes the bit pattern of 2^23 + c)
-    uint32_t pcol = 0u, pnorm = kMagic;
-    if (pvalid) {
-        const uint2 c = packed_colour(guide + ((size_t)py * W + pxg) * C, C);
-        pcol = c.x;
-        pnorm = c.y + kMagic;
+    for (int i = tid; i < spatial_floats(rho); i += kThreads) {
+        const int dy = i / (2 * rho + 2), dx = i - dy * (2 * rho + 2) - rho;
+        spatial[i] = __fmul_rn((float)(dx * dx + dy * dy), neg_ks);
     }
-
-    // WTA role (tid < kNPix): state of pixel tid carried across chunks
-    float best = __int_as_float(0x7f800000), a_prev = 0.f, a_next = 0.f, last = 0.f;
-    int blo = 0, bhi = D - 1;
-    // Disparity range of each 4-column group (the pixels of one consumer
-    // warp): the union of its pixels' bands.  A warp skips the chunks outside
-    // its range, and the weights of its pixels are not generated for them.
-    __shared__ int grp_lo[kTX / kPX], grp_hi[kTX / kPX];
+    // the guide window (columns outside the image: 0, their weights are 0)
+    for (int c = tid & 63; c < NC; c += 64) {
+        const int gx = x0 - rho + c;
+        const bool in = (unsigned)gx < (unsigned)W;
+        const uint8_t* src = guide + ((size_t)t.r_lo * W + (in ? gx : 0)) * C;
+#pragma unroll 4
+        for (int r = tid >> 6; r <= t.r_hi - t.r_lo; r += kThreads / 64)
+            gtile[r * NC + c] = in ? packed_colour(src + (size_t)r * W * C, C) : 0u;
+    }
+    __syncthreads();
+    const bool valid = t.py < H && t.px < W;
+    t.pcol = valid ? gtile[(t.py - t.r_lo) * NC + t.px - x0 + rho] : 0u;
+    t.best = __int_as_float(0x7f800000);
+    t.a_prev = t.a_next = t.last = 0.f;
+    t.pending = false;
+    t.blo = t.wlo = 0;
+    t.bhi = t.whi = D - 1;
     if (band != nullptr) {
-        if (tid < kTX / kPX) {
-            grp_lo[tid] = D;
-            grp_hi[tid] = -1;
+        // a warp skips the chunks that none of its pixels needs
+        int lo = D, hi = -1;
+        if (valid) {
+            const uint32_t b = band[(size_t)t.py * W + t.px];
+            t.blo = lo = (int)(b & 0xffffu);
+            t.bhi = hi = (int)(b >> 16);
         }
-        __syncthreads();
-        if (tid < kNPix) {
-            const int oy = y0 + tid / kTX, ox = x0 + tid % kTX;
-            if (oy < H && ox < W) {
-                const uint32_t b = band[(size_t)oy * W + ox];
-                blo = (int)(b & 0xffffu);
-                bhi = (int)(b >> 16);
-                atomicMin(&grp_lo[(tid % kTX) / kPX], blo);
-                atomicMax(&grp_hi[(tid % kTX) / kPX], bhi);
-            }
-        }
-        __syncthreads();
+        t.wlo = __reduce_min_sync(0xffffffffu, lo);
+        t.whi = __reduce_max_sync(0xffffffffu, hi);
     }
-    int bidx = blo;
-    bool pending = false;
+    t.bidx = t.blo;
 
-    // consumer role
-    const int y = y0 + yi;
-    const int r_lo = max(0, y0 - rho);
-    const int r_hi = min(H - 1, y0 + kTY - 1 + rho);
-    const int nr = r_hi - r_lo + 1;
-
-    for (int dc0 = d_begin; dc0 < d_end; dc0 += DC) {
-        // this chunk is needed by the producer's pixel group / the consumer's group
-        const bool p_on = band == nullptr || (grp_hi[ppx / kPX] >= dc0 && grp_lo[ppx / kPX] < dc0 + DC);
-        const bool c_on = band == nullptr || (grp_hi[g] >= dc0 && grp_lo[g] < dc0 + DC);
-        float4 acc[kPX][NQ];
-#pragma unroll
-        for (int i = 0; i < kPX; ++i)
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) acc[i][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        float den_part = 0.f;
-
-        load_cost_row<DC, VEC>(cring, cost, ld, W, d_end, r_lo, x0, rho, NC, dc0);
-        cp_async_commit();
-        load_guide_row(gring, guide, W, C, r_lo, x0, rho, NC);
-        __syncthreads();
-
-        for (int s = 0; s < nr; ++s) {
-            const int r = r_lo + s;
-            // (A) prefetch the next cost row, (B) the next guide row
-            if (s + 1 < nr) {
-                load_cost_row<DC, VEC>(cring + ((s + 1) % 3) * cslot, cost, ld, W, d_end, r + 1, x0, rho, NC, dc0);
-                load_guide_row(gring + ((s + 1) % 3) * NC, guide, W, C, r + 1, x0, rho, NC);
-            }
-            cp_async_commit();
-            // (C) weights of row r for every tile pixel whose window reaches it
-            {
-                const int dy = r - py;
-                if (p_on && py < H && dy >= -rho && dy <= rho) {
-                    const uint2* gr = gring + (s % 3) * NC;
-                    float* wrow = wring + (s & 1) * wslot + pyi * WS;
-                    const int dy2 = dy * dy;
-                    for (int dx = dx_lo; dx < dx_hi; ++dx) {
-                        const int qx = pxg + dx - rho;
-                        float w = 0.f;
-                        if (pxg < W && qx >= 0 && qx < W) {
-                            // Eq. (7)-(8) as one exp2: colour distance exact in
-                            // integers, then float(c) = (2^23 + c) - 2^23 exactly
-                            const uint2 q = gr[ppx + dx];
-                            const float col2 =
-                                __uint_as_float(q.y + pnorm - 2u * (uint32_t)__dp4a(q.x, pcol, 0u)) - 8388608.f;
-                            const int ddx = dx - rho;
-                            const float sp2 = (float)(ddx * ddx + dy2);
-                            w = ex2_approx(fmaf(col2, neg_kr, sp2 * neg_ks));
-                        }
-                        wrow[dx * kTX + ppx] = w;
-                        den_part += w;
-                    }
-                }
-            }
-            // (D) own copies of row r have landed; (E) everyone's have
-            cp_async_wait1();
-            __syncthreads();
-            // (F) accumulate row r
-            const int dy = r - y;
-            if (c_on && y < H && dy >= -rho && dy <= rho) {
-                const float* cr = cring + (s % 3) * cslot + (kPX * g) * DC + 4 * k;
-                const float* wr = wring + (s & 1) * wslot + yi * WS + kPX * g;
-                float4 win[4][NQ];
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q) win[j][q] = *(const float4*)(cr + j * DC + 32 * q);
-                for (int dx0 = 0; dx0 < NT; dx0 += 4) {
-#pragma unroll
-                    for (int s4 = 0; s4 < 4; ++s4) {
-                        const int dx = dx0 + s4;
-                        if (dx < NT) {
-#pragma unroll
-                            for (int q = 0; q < NQ; ++q)
-                                win[(s4 + 3) & 3][q] = *(const float4*)(cr + (dx + 3) * DC + 32 * q);
-                            const float4 w4 = *(const float4*)(wr + dx * kTX);
-                            const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                            for (int i = 0; i < kPX; ++i) {
-                                const int slot = (i + s4) & 3;
-#pragma unroll
-                                for (int q = 0; q < NQ; ++q) {
-                                    acc[i][q].x = fmaf(wv[i], win[slot][q].x, acc[i][q].x);
-                                    acc[i][q].y = fmaf(wv[i], win[slot][q].y, acc[i][q].y);
-                                    acc[i][q].z = fmaf(wv[i], win[slot][q].z, acc[i][q].z);
-                                    acc[i][q].w = fmaf(wv[i], win[slot][q].w, acc[i][q].w);
-                                }
-                            }
-                        }
-                    }
-                }
-            }
+    for (int dc0 = d_begin; dc0 < d_end; dc0 += 64) {
+        const int left = d_end - dc0;
+        if (D > 32) {
+            if (left > 32) aggregate_chunk<8, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+            else aggregate_chunk<4, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+        } else if (D > 16) {
+            aggregate_chunk<4, 32, COPY, ROWS>(t, ring, agg_out, dc0);
+        } else {
+            aggregate_chunk<2, 16, COPY, ROWS>(t, ring, agg_out, dc0);
         }
-
-        // normalise and stage: stage[pixel][d] with pixel = yi*kTX + 4g + i
-        den_s[half * kNPix + pp] = den_part;
-        __syncthreads();   // all rows consumed, ring free; den visible
-#pragma unroll
-        for (int i = 0; i < kPX; ++i) {
-            const int pix = yi * kTX + kPX * g + i;
-            const float den = den_s[pix] + den_s[kNPix + pix];
-            const float inv = 1.f / den;
-            float* st = stage + pix * (DC + 1) + 4 * k;
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                st[32 * q + 0] = acc[i][q].x * inv;
-                st[32 * q + 1] = acc[i][q].y * inv;
-                st[32 * q + 2] = acc[i][q].z * inv;
-                st[32 * q + 3] = acc[i][q].w * inv;
-            }
-        }
-        __syncthreads();
-        const int nd = min(DC, d_end - dc0);
-        if (agg_out != nullptr) {
-            for (int e = tid; e < kNPix * nd; e += kThreads) {
-                const int pix = e / nd, j = e - pix * nd;
-                const int ey = y0 + pix / kTX, ex = x0 + pix % kTX;
-                if (ey < H && ex < W) agg_out[((size_t)ey * W + ex) * D + dc0 + j] = stage[pix * (DC + 1) + j];
-            }
-        }
-        if (tid < kNPix) {
-            const float* st = stage + tid * (DC + 1);
-            const int j0 = max(0, blo - dc0), j1 = min(nd, bhi + 1 - dc0);
-            for (int j = j0; j < j1; ++j) {
-                const float v = st[j];
-                if (pending) {
-                    a_next = v;
-                    pending = false;
-                }
-                if (v < best) {
-                    best = v;
-                    bidx = dc0 + j;
-                    a_prev = last;
-                    pending = true;
-                }
-                last = v;
-            }
-        }
-        __syncthreads();   // stage (aliasing the ring) consumed before the next chunk reloads it
     }
 
-    if (tid < kNPix) {
-        const int oy = y0 + tid / kTX, ox = x0 + tid % kTX;
-        if (oy < H && ox < W) {
-            float ds = (float)bidx;
-            if (bidx > blo && bidx < bhi) {
-                const float den = 2.f * a_prev + 2.f * a_next - 4.f * best;
-                if (den > 0.f) ds = (float)bidx + (a_prev - a_next) / den;
-            }
-            const size_t o = (size_t)oy * W + ox;
-            if (disp_int) disp_int[o] = bidx;
-            if (disp_sub) disp_sub[o] = ds;
+    if (valid) {
+        float ds = (float)t.bidx;
+        if (t.bidx > t.blo && t.bidx < t.bhi) {
+            const float den = 2.f * t.a_prev + 2.f * t.a_next - 4.f * t.best;
+            if (den > 0.f) ds = (float)t.bidx + (t.a_prev - t.a_next) / den;
         }
+        const size_t o = (size_t)t.py * W + t.px;
+        if (disp_int) disp_int[o] = t.bidx;
+        if (disp_sub) disp_sub[o] = ds;
     }
+    __syncthreads();   // the guide window may be overwritten
 }
 
-template <int KD, bool VEC>
-__global__ void __launch_bounds__(kThreads, 2)
-aggregate_f32_kernel(const float* __restrict__ cost, int ld, const uint8_t* __restrict__ guide, int H,
-                     int W, int C, int D, int rho, float neg_ks, float neg_kr,
-                     float* __restrict__ agg_out, int32_t* __restrict__ disp_int,
-                     float* __restrict__ disp_sub)
+constexpr int kCtasPerSm = 4;
+
+template <Copy COPY>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+aggregate_f32_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
+                     const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
+                     float* __restrict__ agg_out, int32_t* __restrict__ disp_int, float* __restrict__ disp_sub,
+                     int slots, int* __restrict__ err)
 {
-    extern __shared__ float4 smem_f4[];
-    aggregate_tile<KD, VEC>(cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                            blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, 0, D, nullptr);
+    extern __shared__ __align__(128) float4 smem_f4[];
+    Ring ring = make_ring<COPY>(smem_f4, slots, err);
+    aggregate_tile<COPY, 2>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
+                            blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, ring, 0, D, nullptr);
 }
 
-// Band form: tile t aggregates its range tile_range[t] (chunks of 32 or 64
-// disparities) and each pixel takes its winner inside its own band.
-__global__ void __launch_bounds__(kThreads, 2)
-aggregate_band_kernel(const float* __restrict__ cost, int ld, const uint8_t* __restrict__ guide, int H, int W,
-                      int C, int D, int rho, float neg_ks, float neg_kr, const int2* __restrict__ tile_range,
-                      const uint32_t* __restrict__ band, int32_t* __restrict__ disp_int,
-                      float* __restrict__ disp_sub)
+// Band form: tile t aggregates its range tile_range[t] and each pixel takes
+// its winner inside its own band.  A warp owns 8 x 4 pixels here (bands come in
+// 4 x 4 blocks, and a warp computes the chunks that any of its pixels needs).
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
+                      const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
+                      const int2* __restrict__ tile_range, const uint32_t* __restrict__ band,
+                      int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int slots, int* __restrict__ err)
 {
-    extern __shared__ float4 smem_f4[];
+    extern __shared__ __align__(128) float4 smem_f4[];
+    Ring ring = make_ring<kTma>(smem_f4, slots, err);
     const int2 r = tile_range[(size_t)blockIdx.y * gridDim.x + blockIdx.x];
-    if (r.y - r.x > 32)
-        aggregate_tile<8, true>(cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
-                                blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, r.x, r.y, band);
-    else
-        aggregate_tile<4, true>(cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
-                                blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, r.x, r.y, band);
+    aggregate_tile<kTma, 4>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
+                            blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, ring, r.x, r.y, band);
 }
 
 // Persistent form over a batch: CTAs claim (pair, tile) items from a counter;
 // pairs[p].agg_off is the first item of pair p, items of a pair are its tiles
 // in row-major order.  No CTA waits on another.
-__global__ void __launch_bounds__(kThreads, 2)
-aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems, int* __restrict__ counter)
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems, int* __restrict__ counter,
+                             int slots, int* __restrict__ err)
 {
-    extern __shared__ float4 smem_f4[];
+    extern __shared__ __align__(128) float4 smem_f4[];
+    Ring ring = make_ring<kAsync16>(smem_f4, slots, err);
     __shared__ int item_s;
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
@@ -415,24 +719,54 @@ aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, in
         const BatchPair& bp = pairs[pi];
         const int t = item - bp.agg_off;
         const int ntx = (bp.W + kTX - 1) / kTX;
-        aggregate_tile<8, true>(bp.cost, bp.ld, bp.left, bp.H, bp.W, bp.C, bp.D, bp.radius, bp.neg_ks, bp.neg_kr,
-                                nullptr, bp.disp_int, bp.disp_sub, (t % ntx) * kTX, (t / ntx) * kTY, smem_f4, 0,
-                                bp.D, nullptr);
+        aggregate_tile<kAsync16, 2>(bp.cost, nullptr, bp.ld, bp.left, bp.H, bp.W, bp.C, bp.D, bp.radius, bp.neg_ks,
+                                    bp.neg_kr, nullptr, bp.disp_int, bp.disp_sub, (t % ntx) * kTX, (t / ntx) * kTY,
+                                    smem_f4, ring, 0, bp.D, nullptr);
     }
 }
 
-template <int KD, bool VEC>
-cudaError_t launch_kd(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
-                      int rho, float neg_ks, float neg_kr, float* agg_out, int32_t* disp_int,
-                      float* disp_sub, cudaStream_t stream)
+// Slots of the ring: as many as still leave the most CTAs per SM (at least 2).
+int ring_slots(int rho, int dc)
 {
-    const size_t smem = smem_bytes<8 * KD>(rho);
-    cudaError_t e = fbs::raise_smem_limit(aggregate_f32_kernel<KD, VEC>, (int)smem);
+    constexpr size_t kSmem = 227 * 1024, kReserved = 1024;
+    auto ctas = [&](int slots) {
+        const size_t n = kSmem / (smem_bytes(rho, dc, slots) + kReserved);
+        return n < (size_t)kCtasPerSm ? n : (size_t)kCtasPerSm;
+    };
+    int slots = 2;
+    while (slots < kMaxSlots && ctas(slots + 1) == ctas(2)) ++slots;
+    return slots;
+}
+
+// The cost volume [H][W][ld] as a 3-D tensor (D, W, H); a box is one row of a
+// tile's window.  False where the volume does not allow it.
+bool encode_volume(CUtensorMap* map, const float* cost, int ld, int H, int W, int D, int rho)
+{
+    if (ld % 4 != 0 || (reinterpret_cast<uintptr_t>(cost) & 15) != 0) return false;
+    const tca::EncodeTiledFn enc = tca::encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)W, (cuuint64_t)H};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)W * ld * 4};
+    cuuint32_t box[3] = {(cuuint32_t)column_size(D), (cuuint32_t)(kTX + 2 * rho), 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(cost), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <Copy COPY>
+cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
+                        int D, int rho, float neg_ks, float neg_kr, float* agg_out, int32_t* disp_int, float* disp_sub,
+                        int* err, cudaStream_t stream)
+{
+    const int slots = ring_slots(rho, column_size(D));
+    const size_t smem = smem_bytes(rho, column_size(D), slots);
+    cudaError_t e = fbs::raise_smem_limit(aggregate_f32_kernel<COPY>, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
     fbs::note_launch();
-    aggregate_f32_kernel<KD, VEC><<<grid, kThreads, smem, stream>>>(
-        cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub);
+    aggregate_f32_kernel<COPY><<<grid, kThreads, smem, stream>>>(
+        map, cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, err);
     return cudaGetLastError();
 }
 
@@ -440,53 +774,56 @@ cudaError_t launch_kd(const float* cost, int ld, const uint8_t* guide, int H, in
 
 int agg_f32_tiles(int H, int W) { return ((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY); }
 
-cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out)
+cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out, int* slots_out)
 {
-    const size_t smem = smem_bytes<64>(max_radius);
+    *slots_out = ring_slots(max_radius, 64);
+    const size_t smem = smem_bytes(max_radius, 64, *slots_out);
     *smem_out = smem;
     return fbs::raise_smem_limit(aggregate_f32_batched_kernel, (int)smem);
 }
 
 cudaError_t launch_aggregate_f32_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
-                                         size_t smem, cudaStream_t stream)
+                                         size_t smem, int slots, int* err, cudaStream_t stream)
 {
     fbs::note_launch();
-    aggregate_f32_batched_kernel<<<grid, kThreads, smem, stream>>>(pairs, npairs, nitems, counter);
+    aggregate_f32_batched_kernel<<<grid, kThreads, smem, stream>>>(pairs, npairs, nitems, counter, slots, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
                                   int radius, float sigma_s, float sigma_r, const int2* tile_range,
-                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, cudaStream_t stream)
+                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, int* err, cudaStream_t stream)
 {
     const double log2e = 1.4426950408889634;
     const float neg_ks = (float)(-log2e / ((double)sigma_s * sigma_s));
     const float neg_kr = (float)(-log2e / ((double)sigma_r * sigma_r));
-    const size_t smem = smem_bytes<64>(radius);
+    const int slots = ring_slots(radius, column_size(D));
+    const size_t smem = smem_bytes(radius, column_size(D), slots);
+    CUtensorMap map;
+    if (!encode_volume(&map, cost, ld, H, W, D, radius)) return cudaErrorInvalidValue;   // the context's own volume
     cudaError_t e = fbs::raise_smem_limit(aggregate_band_kernel, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
     fbs::note_launch();
-    aggregate_band_kernel<<<grid, kThreads, smem, stream>>>(cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr,
-                                                            tile_range, band, disp_int, disp_sub);
+    aggregate_band_kernel<<<grid, kThreads, smem, stream>>>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr,
+                                                            tile_range, band, disp_int, disp_sub, slots, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                                  int D, int radius, float sigma_s, float sigma_r, float* agg_out,
-                                 int32_t* disp_int, float* disp_sub, cudaStream_t stream)
+                                 int32_t* disp_int, float* disp_sub, int* err, cudaStream_t stream)
 {
     // exp(-a/g^2) = exp2(-a * log2(e) / g^2)
     const double log2e = 1.4426950408889634;
     const float neg_ks = (float)(-log2e / ((double)sigma_s * sigma_s));
     const float neg_kr = (float)(-log2e / ((double)sigma_r * sigma_r));
-    const bool vec = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(cost) & 15) == 0);
-    if (D <= 32) {
-        return vec ? launch_kd<4, true>(cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub, stream)
-                   : launch_kd<4, false>(cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub, stream);
-    }
-    return vec ? launch_kd<8, true>(cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub, stream)
-               : launch_kd<8, false>(cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub, stream);
+    CUtensorMap map{};
+    if (encode_volume(&map, cost, ld, H, W, D, radius))
+        return launch_copy<kTma>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
+                                 err, stream);
+    return launch_copy<kAsync4>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
+                                err, stream);
 }
 
 }  // namespace fbs

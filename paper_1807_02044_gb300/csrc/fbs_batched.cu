@@ -9,7 +9,7 @@
 // the pair table from a pinned slot, reset the counters, three persistent
 // launches]; device pointers are read from the table at run time, so one
 // graph serves any buffers of that shape.  These plans differ in pair order
-// (largest first or as given) and in aggregation CTAs per SM (1 or 2).
+// (largest first or as given) and in aggregation CTAs per SM (2 or 4).
 //
 // Branched plans (every precision): each pair runs the launches of the
 // single-pair form over its own slice of one scratch that holds every pair's
@@ -50,7 +50,7 @@ using namespace fbs_detail;
 namespace {
 
 constexpr int kMaxPairs = 4096;
-// FP32: plans 0-3 persistent, plan = 2 * order + (agg CTAs per SM - 1), order 0
+// FP32: plans 0-3 persistent, plan = 2 * order + (agg CTAs per SM / 2 - 1), order 0
 // = largest first; plans 4-6 branched with kBranches[plan - 4] branches.
 constexpr int kPersistentPlans = 4;
 constexpr int kPlans = 7;
@@ -207,10 +207,11 @@ void fill_table(fbs_ctx* ctx, const Layout& L, int n, const fbs_pair* pairs, fbs
 fbs_status build_graph(fbs_ctx* ctx, const Layout& L, int n, int plan, int slot, cudaGraphExec_t* out)
 {
     size_t agg_smem = 0;
-    cudaError_t e = fbs::prepare_aggregate_f32_batched(L.max_radius, &agg_smem);
+    int agg_slots = 0;
+    cudaError_t e = fbs::prepare_aggregate_f32_batched(L.max_radius, &agg_smem, &agg_slots);
     if (e == cudaSuccess) e = fbs::prepare_cost_batched();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batched kernel attributes");
-    const int agg_per_sm = (plan & 1) + 1;
+    const int agg_per_sm = 2 * ((plan & 1) + 1);
     const int g_stats = std::min(L.items[0], ctx->num_sms * 4);
     const int g_cost = std::min(L.items[1], ctx->num_sms * 4);
     const int g_agg = std::min(L.items[2], ctx->num_sms * agg_per_sm);
@@ -222,7 +223,8 @@ fbs_status build_graph(fbs_ctx* ctx, const Layout& L, int n, int plan, int slot,
     if (e == cudaSuccess) e = fbs::launch_stats_batched(ctx->bpairs, n, L.items[0], ctx->bcounters + 0, g_stats, cs);
     if (e == cudaSuccess) e = fbs::launch_cost_batched(ctx->bpairs, n, L.items[1], ctx->bcounters + 1, g_cost, cs);
     if (e == cudaSuccess)
-        e = fbs::launch_aggregate_f32_batched(ctx->bpairs, n, L.items[2], ctx->bcounters + 2, g_agg, agg_smem, cs);
+        e = fbs::launch_aggregate_f32_batched(ctx->bpairs, n, L.items[2], ctx->bcounters + 2, g_agg, agg_smem,
+                                              agg_slots, ctx->derr, cs);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     if (e == cudaSuccess) e = e2;
@@ -361,7 +363,7 @@ fbs_status build_branch_graph(fbs_ctx* ctx, int n, const fbs_pair* pairs, int nb
             k0 = fbs::launch_count();
             if (e == cudaSuccess)
                 e = fbs::launch_aggregate_f32(cost, ld, q.left, q.H, q.W, q.C, q.D, q.radius, q.sigma_s, q.sigma_r,
-                                              nullptr, q.disp_int, q.disp_subpix, s);
+                                              nullptr, q.disp_int, q.disp_subpix, ctx->derr, s);
             g->kernels[FBS_KERNEL_AGG_F32] += fbs::launch_count() - k0;
             continue;
         }

@@ -75,9 +75,10 @@ cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* lef
 constexpr int kAggTileX = 32;
 constexpr int kAggTileY = 4;
 // agg_out (nullable) is written with row pitch D (caller layout [H][W][D]).
+// err: device int set to nonzero if a bounded wait inside the kernel gave up.
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W,
                                  int C, int D, int radius, float sigma_s, float sigma_r,
-                                 float* agg_out, int32_t* disp_int, float* disp_sub,
+                                 float* agg_out, int32_t* disp_int, float* disp_sub, int* err,
                                  cudaStream_t stream);
 
 // ---- steps 2-4 on the tensor cores (BF16 / FP16 operands, FP32 accumulate) ---
@@ -143,7 +144,8 @@ cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const u
                              cudaStream_t stream);
 cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
                                   int radius, float sigma_s, float sigma_r, const int2* tile_range,
-                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, cudaStream_t stream);
+                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, int* err,
+                                  cudaStream_t stream);
 
 // ---- batched form: one persistent launch per stage over many pairs ------------
 // Device-side description of one pair of a batch.  *_off is the index of the
@@ -181,9 +183,9 @@ cudaError_t launch_stats_batched(const BatchPair* pairs, int npairs, int nitems,
                                  cudaStream_t stream);
 cudaError_t launch_cost_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
                                 cudaStream_t stream);
-cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out);
+cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out, int* slots_out);
 cudaError_t launch_aggregate_f32_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
-                                         size_t smem, cudaStream_t stream);
+                                         size_t smem, int slots, int* err, cudaStream_t stream);
 
 // ---- context helpers for entry points defined outside fbs_api.cu -------------
 // Host-side checks of fbs_compute_disparity's arguments (sets the message).

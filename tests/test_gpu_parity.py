@@ -307,3 +307,49 @@ def test_full_size_1280x960_sampled(fbs, ctx, oracle_mod):
     agg_s = agg[torch.from_numpy(ys).cuda(), torch.from_numpy(xs).cuda()].cpu().numpy()
     err = check_agg(agg_s, ref_agg, 2.0)
     check_disparities(di.cpu().numpy()[ys, xs], ds.cpu().numpy()[ys, xs], ref_agg, ref_di, ref_ds, 2.0, err)
+
+
+def _aggregate(ctx, cost, guide, radius, ss, sr):
+    agg, di, ds = ctx.aggregate(_dev(cost), _dev(guide), radius, ss, sr)
+    torch.cuda.synchronize()
+    return agg.cpu().numpy(), di.cpu().numpy(), ds.cpu().numpy()
+
+
+# The FP32 aggregation works in chunks of 64, 32 or 16 disparities, walks the window's columns with 8 pixels per
+# thread (radii below 4 have no column that all of them share) and reads the volume by TMA or, where D is no multiple
+# of 4, by 4-byte copies.
+@pytest.mark.parametrize("D", [1, 15, 16, 17, 32, 33, 60, 64, 65, 97, 132])
+@pytest.mark.parametrize("radius,H,W", [(0, 5, 37), (1, 9, 31), (2, 6, 33), (3, 11, 8), (4, 3, 65), (9, 13, 50)])
+def test_aggregate_chunk_and_window_edges(ctx, oracle_mod, D, radius, H, W):
+    rng = np.random.default_rng(1000 * radius + D)
+    cost = rng.uniform(0.0, 2.0, (H, W, D)).astype(np.float32)
+    guide = rng.integers(0, 256, (H, W, 3)).astype(np.uint8)
+    ss, sr = max(1.0, float(radius)), 40.0
+    agg, di, ds = _aggregate(ctx, cost, guide, radius, ss, sr)
+    ref = oracle_mod.aggregate(cost.astype(np.float64), guide, radius, ss, sr)
+    err = check_agg(agg, ref, 2.0)
+    ref_di, ref_ds = oracle_mod.wta_subpixel(ref)
+    check_disparities(di, ds, ref, ref_di, ref_ds, 2.0, err)
+
+
+@pytest.mark.parametrize("D,radius", [(12, 2), (40, 5), (70, 3)])
+def test_aggregate_keeps_infinities_and_nans_to_their_windows(ctx, oracle_mod, D, radius):
+    """An infinite or NaN cost reaches exactly the sums whose window holds it, and neither wins the WTA."""
+    H, W = 14, 41
+    rng = np.random.default_rng(D)
+    cost = rng.uniform(0.0, 2.0, (H, W, D)).astype(np.float32)
+    cost[4, 9, 3], cost[8, 30, D - 1], cost[10, 12, 0] = np.inf, np.nan, np.inf
+    guide = np.full((H, W, 3), 90, np.uint8)
+    agg, di, ds = _aggregate(ctx, cost, guide, radius, 4.0, 20.0)
+    ref = oracle_mod.aggregate(cost.astype(np.float64), guide, radius, 4.0, 20.0)
+    assert np.array_equal(np.isnan(agg), np.isnan(ref)) and np.array_equal(np.isinf(agg), np.isinf(ref))
+    fine = np.isfinite(ref)
+    assert np.abs(agg[fine] - ref[fine]).max() <= 1e-5 * 2.0
+    assert np.all(np.take_along_axis(fine, di[..., None].astype(np.int64), 2))
+
+
+def test_aggregate_all_infinite_pixels_take_disparity_zero(ctx):
+    cost = np.full((6, 40, 70), np.inf, np.float32)
+    guide = np.zeros((6, 40, 3), np.uint8)
+    _, di, ds = _aggregate(ctx, cost, guide, 2, 2.0, 10.0)
+    assert not di.any() and not ds.any()
