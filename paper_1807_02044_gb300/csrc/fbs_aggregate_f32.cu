@@ -76,19 +76,19 @@ __host__ __device__ inline int weight_stride(int rho) { return (((2 * rho + kPX)
 __host__ __device__ inline int column_size(int D) { return D > 32 ? 64 : D > 16 ? 32 : 16; }
 
 // How a cost row is copied to shared memory: one TMA box (volumes that are 16-byte
-// aligned with ld % 4 == 0), 16-byte cp.async (the same, where no tensor map is
-// at hand) or 4-byte cp.async.
-enum Copy { kTma, kAsync16, kAsync4 };
+// aligned with ld % 4 == 0), or cp.async of so many bytes by every thread: 16
+// (the same volumes, where no tensor map is at hand) or 4 (any volume: 640x480,
+// D = 63, rho = 7: 318 us against 236 us at D = 64 by TMA; 470 us before).
+enum Copy { kTma = 0, kAsync16 = 16, kAsync4 = 4 };
 
-__device__ __forceinline__ void cp_async16(uint32_t smem, const void* gmem, int src_bytes)
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t smem, const void* gmem, int src_bytes)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t smem, const void* gmem, int src_bytes)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes)
-                 : "memory");
+    if (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;\n" ::"r"(smem), "l"(gmem), "r"(src_bytes), "n"(BYTES)
+                     : "memory");
 }
 // The mbarrier gets one arrival of this thread when its earlier cp.async have landed.
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar)
@@ -116,11 +116,11 @@ __host__ __device__ inline int spatial_floats(int rho) { return (rho + 1) * (2 *
 // Guide window of a tile: (kTY + 2 rho) rows of kTX + 2 rho words, and one more.
 __host__ __device__ inline int guide_words(int rho) { return (kTY + 2 * rho) * (kTX + 2 * rho) + 1; }
 
-// Shared memory of a CTA, in order: barriers and counters of the S slots, the
+// Shared memory of a CTA, in order: the barriers of the S slots, the
 // spatial terms, the guide window, then the cost rows [S][NC][DC] and the warps'
 // weights [4][4][WS]; the stage [4][32][DC + 4] of the epilogue lies over these.
 constexpr int kMaxSlots = 4;
-constexpr int kHeaderBytes = 64;   // full[4] (8 bytes each), done[4] (4 bytes each), abort flag
+constexpr int kHeaderBytes = 80;   // full[4], done[4] (8 bytes each), abort flag
 __host__ __device__ inline size_t front_bytes(int rho)
 {
     return (kHeaderBytes + 4 * (size_t)spatial_floats(rho) + 4 * (size_t)guide_words(rho) + 127) & ~(size_t)127;
@@ -135,8 +135,13 @@ __host__ __device__ inline size_t smem_bytes(int rho, int dc, int slots)
 
 // The ring of cost rows.  Every warp walks every row, so slot and parity (of
 // the row it is at) are the same sequence in all of them.
+//   kTma: done[slot] counts the warps that have finished the slot's row; the
+//   last one issues the box of the row S later.
+//   cp.async: every warp loads a quarter of each row, once all of them have
+//   arrived at the barrier done[slot]; a warp waits for that when it starts
+//   the next row.
 struct Ring {
-    uint32_t full, done;      // shared addresses of the slots' barriers and counters
+    uint32_t full, done;      // shared addresses, 8 bytes per slot
     volatile uint32_t* abort;
     int* err;
     int S, slot;
@@ -149,10 +154,10 @@ struct Ring {
         }
     }
     // Bounded (about 2 s): on a timeout the error word is set and nothing is waited for any more.
-    __device__ __forceinline__ void wait() const
+    __device__ __forceinline__ void wait(uint32_t bar, uint32_t par) const
     {
-        if (tc::mbar_try_wait(full + 8 * slot, parity)) return;
-        if (*abort == 0 && !tc::mbar_wait(full + 8 * slot, parity)) {
+        if (tc::mbar_try_wait(bar, par)) return;
+        if (*abort == 0 && !tc::mbar_wait(bar, par)) {
             *abort = 1u;
             atomicCAS(err, 0, 31);
         }
@@ -166,33 +171,38 @@ struct Volume {
     int ld, W, D;
 };
 
-// One warp loads cost row r, columns xlo .. xlo+NC-1, disparities dc0 ..
-// dc0+DC-1 into a slot; zeros outside the image and for disparities >= D.
+// Load cost row r, columns xlo .. xlo+NC-1, disparities dc0 .. dc0+DC-1 into a
+// slot; zeros outside the image and for disparities >= D.  kTma: one warp;
+// otherwise all of them, a thread its share.
 template <int DC, Copy COPY>
 __device__ __forceinline__ void load_cost_row(uint32_t dst, uint32_t bar, const Volume& v, int r, int xlo, int NC, int dc0)
 {
-    const int lane = threadIdx.x & 31;
-    if (COPY == kTma) {
-        if (lane == 0) {
+    if constexpr (COPY == kTma) {
+        if ((threadIdx.x & 31) == 0) {
             tc::fence_proxy_async();   // the slot was read, and may hold staged sums, through the generic proxy
             tc::mbar_expect_tx(bar, 4u * DC * (uint32_t)NC);
             tma_load_3d(dst, v.map, dc0, xlo, r, bar);
         }
-        return;
-    }
-    constexpr int E = COPY == kAsync16 ? 4 : 1;     // floats per copy
-    constexpr int Q = DC / E, STEP = 32 / Q > 0 ? 32 / Q : 1;
-    const float* row = v.cost + (size_t)r * v.W * v.ld;
-    for (int q = lane % Q; q < Q; q += 32) {
-        const int d = dc0 + E * q, bytes = d < v.D ? 4 * min(E, v.D - d) : 0;
-        for (int c = Q < 32 ? lane / Q : 0; c < NC; c += STEP) {
-            const bool in = (unsigned)(xlo + c) < (unsigned)v.W && bytes > 0;
-            const float* src = in ? row + (size_t)(xlo + c) * v.ld + d : v.cost;
-            if (E == 4) cp_async16(dst + 4 * (c * DC + E * q), src, in ? bytes : 0);
-            else cp_async4(dst + 4 * (c * DC + E * q), src, in ? bytes : 0);
+    } else {
+        constexpr int E = COPY / 4;                     // floats per copy
+        constexpr int Q = DC / E, STEP = kThreads / Q;  // copies per column, columns per pass
+        static_assert(STEP >= 1, "a pass covers whole columns");
+        const int q = threadIdx.x % Q, c0 = threadIdx.x / Q, d = dc0 + E * q, bytes = d < v.D ? 4 * min(E, v.D - d) : 0;
+        const float* src = v.cost + ((ptrdiff_t)r * v.W + xlo + c0) * v.ld + d;
+        const ptrdiff_t step = (ptrdiff_t)STEP * v.ld;
+        uint32_t to = dst + 4 * (c0 * DC + E * q);
+        if (xlo >= 0 && xlo + NC <= v.W && dc0 + DC <= v.D) {
+#pragma unroll 4
+            for (int c = c0; c < NC; c += STEP, to += 4 * STEP * DC, src += step) cp_async<COPY>(to, src, COPY);
+        } else {
+#pragma unroll 2
+            for (int c = c0; c < NC; c += STEP, to += 4 * STEP * DC, src += step) {
+                const bool in = (unsigned)(xlo + c) < (unsigned)v.W && bytes > 0;
+                cp_async<COPY>(to, in ? src : v.cost, in ? bytes : 0);
+            }
         }
+        cp_async_arrive(bar);
     }
-    cp_async_arrive(bar);
 }
 
 // A guide pixel as R | G << 8 | B << 16; grey images use the first channel only.
@@ -458,9 +468,10 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
     auto load_row = [&](int r, int slot) {
         load_cost_row<DC, COPY>(rows_a + slot * slot_bytes, ring.full + 8 * slot, t.vol, r, xlo, NC, dc0);
     };
-    if (warp < ring.S && t.r_lo + warp <= t.r_hi) {
-        const int slot = ring.slot + warp;
-        load_row(t.r_lo + warp, slot < ring.S ? slot : slot - ring.S);
+    // the first S rows
+    for (int i = COPY == kTma ? warp : 0; i < ring.S && t.r_lo + i <= t.r_hi; i += COPY == kTma ? kWarps : 1) {
+        const int slot = ring.slot + i;
+        load_row(t.r_lo + i, slot < ring.S ? slot : slot - ring.S);
     }
 
     // accumulating role: lane bits 0, 2, 3 = disparity group k, bits 1, 4 = pixel group
@@ -486,6 +497,14 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
 
     const uint32_t* g = t.guide + (t.px - t.x0);
     for (int r = t.r_lo; r <= t.r_hi; ++r, g += NC) {
+        if constexpr (COPY != kTma) {
+            // refill the slot of the row before
+            if (r > t.r_lo && r - 1 + ring.S <= t.r_hi) {
+                const int slot = ring.slot == 0 ? ring.S - 1 : ring.slot - 1;
+                ring.wait(ring.done + 8 * slot, ring.slot == 0 ? ring.parity ^ 1u : ring.parity);
+                load_row(r - 1 + ring.S, slot);
+            }
+        }
         if (r >= w_lo && r <= w_hi) {
             const int dy = r - t.py;
             if (t.py < t.H && dy >= -rho && dy <= rho) {
@@ -494,18 +513,23 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
                 else weight_row<false>(self, g, sp, wout, rho, den0, den1);
             }
             __syncwarp();
-            ring.wait();
+            ring.wait(ring.full + 8 * ring.slot, ring.parity);
             const int gdy = r - gy;
             if (gy < t.H && gdy >= -rho && gdy <= rho) accumulate_row<KD, DC>(acc, ca0 + ring.slot * slot_bytes, wa0, rho);
         } else {
-            ring.wait();   // a row not needed is waited for too: a warp must not count a slot's next row early
+            ring.wait(ring.full + 8 * ring.slot, ring.parity);   // a row not needed is waited for too: a warp must not count a slot's next row early
         }
         __syncwarp();
-        uint32_t done = 0;
-        if (lane == 0) done = count_done(ring.done + 4 * ring.slot);
-        done = __shfl_sync(0xffffffffu, done, 0);
-        // the last warp to finish the row refills its slot
-        if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && *ring.abort == 0) load_row(r + ring.S, ring.slot);
+        if constexpr (COPY == kTma) {
+            uint32_t done = 0;
+            if (lane == 0) done = count_done(ring.done + 8 * ring.slot);
+            done = __shfl_sync(0xffffffffu, done, 0);
+            // the last warp to finish the row refills its slot
+            if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && *ring.abort == 0)
+                load_row(r + ring.S, ring.slot);
+        } else {
+            if (lane == 0) tc::mbar_arrive(ring.done + 8 * ring.slot);
+        }
         ring.next();
     }
     __syncthreads();   // every row consumed: the stage may overwrite the rows and weights
@@ -536,11 +560,16 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
     __syncwarp();
     const int nd = min(NDC, t.d_end - dc0);
     if (agg_out != nullptr) {
-        for (int pix = 0; pix < 32; ++pix) {
-            const int ey = t.wy + pix / PW, ex = t.x0 + wx + pix % PW;
-            if (ey < t.H && ex < t.W)
-                for (int j = lane; j < nd; j += 32)
-                    agg_out[((size_t)ey * t.W + ex) * t.D + dc0 + j] = stage[pix * SP + j];
+        for (int row = 0; row < ROWS && t.wy + row < t.H; ++row) {
+            const int npx = min(PW, t.W - t.x0 - wx);
+            float* o = agg_out + ((size_t)(t.wy + row) * t.W + t.x0 + wx) * t.D + dc0 + lane;
+            const float* st = stage + row * PW * SP + lane;
+#pragma unroll 4
+            for (int pix = 0; pix < npx; ++pix, o += t.D, st += SP) {
+#pragma unroll
+                for (int j = 0; j < NDC; j += 32)
+                    if (lane + j < nd) o[j] = st[j];
+            }
         }
     }
     wta_chunk(t, stage + lane * SP, dc0, max(0, t.blo - dc0), min(nd, t.bhi + 1 - dc0));
@@ -555,15 +584,16 @@ __device__ __forceinline__ Ring make_ring(void* smem, int slots, int* err)
     Ring ring;
     ring.full = tc::smem_u32(smem);
     ring.done = ring.full + 8 * kMaxSlots;
-    ring.abort = (volatile uint32_t*)((uint8_t*)smem + 12 * kMaxSlots);
+    ring.abort = (volatile uint32_t*)((uint8_t*)smem + 16 * kMaxSlots);
     ring.err = err;
     ring.S = slots;
     ring.slot = 0;
     ring.parity = 0;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxSlots; ++s) {
-            tc::mbar_init(ring.full + 8 * s, COPY == kTma ? 1 : 32);
-            ((uint32_t*)smem)[2 * kMaxSlots + s] = 0;
+            tc::mbar_init(ring.full + 8 * s, COPY == kTma ? 1 : kThreads);
+            if (COPY == kTma) ((uint32_t*)smem)[2 * (kMaxSlots + s)] = 0;
+            else tc::mbar_init(ring.done + 8 * s, kWarps);
         }
         *ring.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
