@@ -490,9 +490,9 @@ def run_ours(args):
     ld = (p.D + 3) // 4 * 4
     vol = 4 * p.H * p.W * ld if args.prec == "f32" else 2 * p.H * p.D * ((p.W + 7) // 8 * 8)
     cost_bytes = 2 * p.H * p.W * p.C + vol
-    cost_kernel = "cost_kernel" if args.prec == "f32" else "cost_xb_kernel"
+    cost_kernel = "cost_kernel" if args.prec == "f32" else "cost_xb_ncc_kernel"
     roofline_cost = {"kernel": "cost_kernel (+ grey_stats_kernel)" if args.prec == "f32" else
-                     "cost_xb_kernel (statistics, costs, pad rows and guide in one launch)", "bound": "hbm",
+                     "cost_xb_ncc_kernel (statistics, costs, pad rows and guide in one launch)", "bound": "hbm",
                      "achieved": cost_bytes / (cost_launch_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "avg_launch_ms": cost_launch_ms, "launches": cost_n,
                      "algorithmic": "read both images once, write the cost volume once",

@@ -20,14 +20,13 @@
 //     products per output column summed by a sliding 3-column window);
 //     results are staged in shared memory as [d][x] and written out with D
 //     innermost.
-//   * cost_xb_kernel, 16-bit x-blocked [H][ceil(W/8)][Dp][8] (the tensor-core
+//   * cost_xb_ncc_kernel, 16-bit x-blocked [H][ceil(W/8)][Dp][8] (the tensor-core
 //     aggregation): for a row y and a block of 8 columns, the Dp x 8 block is
 //     contiguous, so the tensor-core kernel's TMA reads contiguous blocks that
 //     land as K-major core matrices; columns x >= W of the last block are 0.
-//     One launch computes the statistics of the rows it stages (a CTA covers
-//     up to 4 output rows and stages their grey rows once), the costs (8
-//     pixels x 8 disparities per thread), the pad rows D .. Dp-1 and the left
-//     image's packed guide.
+//     One launch computes the statistics of the rows it stages, the costs, the
+//     pad rows D .. Dp-1 and the left image's packed guide (its comment says how);
+//     cost_xb_tad_kernel does the same for TAD.
 // Both round the normalisation the same way (ncc_cost), so the 16-bit volume
 // equals the FP32 volume rounded to 16 bits.
 //
@@ -40,6 +39,7 @@
 
 #include "fbs_internal.cuh"
 #include "packed_f32.cuh"
+#include "tc_aggregate.cuh"
 
 namespace fbs {
 namespace {
@@ -439,20 +439,17 @@ __global__ void right_edge_fill_kernel(int H, int W, int D, int ld, float maxc, 
     }
 }
 
-// ---- 16-bit x-blocked volume: one thread per (block of 8 columns, 8 disparities)
+// ---- TAD, 16-bit x-blocked volume: one thread per (block of 8 columns, 8 disparities)
 //
 // The layout [H][ceil(W/8)][Dp][8] keeps the 8 columns of a block contiguous
 // for each d, so a thread that owns one block and 8 consecutive disparities
 // computes the 8 x 8 costs in registers, one 16-byte row per d.  Lanes own
 // consecutive disparity groups of a block; the warp passes its 256 rows
 // through a private shared-memory buffer so that each store instruction
-// writes 32 consecutive rows (512 contiguous bytes within a block).  The left 3x10 grey window and the left
-// statistics stay in registers; the right window (3x10 values and 8 block
-// statistics) slides one column per disparity, 5 new shared-memory values.
-// Per (p, d): three multiply-adds per column product shared by three pixels,
-// the sliding 3-column sum, the numerator and ncc_cost -- about 10
-// instructions.  Staged rows use a skewed index c + c/8, so lanes reading
-// columns 8 apart hit different banks.
+// writes 32 consecutive rows (512 contiguous bytes within a block).  The left
+// pixels stay in registers, the right ones slide one column per disparity.
+// Staged rows use a skewed index c + c/8, so lanes reading columns 8 apart hit
+// different banks.
 constexpr int kXbThreads = 256;
 
 __device__ __forceinline__ int skew(int c) { return c + (c >> 3); }
@@ -472,25 +469,20 @@ __host__ __device__ inline int xb_blocks_per_cta(int D)
 // both when lanes write their 8 rows and when the warp reads 32 consecutive rows).
 constexpr int kXbWarpRows = 256 + 32;
 
-// Output rows per CTA (1, 2 or 4, chosen at launch): the CTA stages grey rows
-// y0-1 .. y0+rows once for all of them (rows + 2 rows of each image instead of
-// 3 per output row).
+// Output rows per CTA (1, 2 or 4, chosen at launch).
 constexpr int kXbMaxRows = 4;
 
-__host__ __device__ inline size_t cost_xb_stage_ints(int mode, int D, int rows)
+__host__ __device__ inline size_t cost_xb_stage_ints(int D, int rows)
 {
     const int npx = 8 * xb_blocks_per_cta(D);
-    const int Ll = skew_len(npx + 2), Lr = skew_len(npx + D + 9), Lp = skew_len(npx);
-    // NCC: grey rows of both images, then per output row the left and right
-    // block statistics; TAD: per output row the packed pixels of both images
-    const size_t n = mode == 0 ? (size_t)((rows + 2) * (Ll + Lr) + rows * (2 * Lp + 2 * Lr))
-                               : (size_t)rows * (Lp + Lr);
-    return (n + 3) & ~(size_t)3;   // the output buffers that follow are 16-byte aligned
+    const int Lr = skew_len(npx + D + 9), Lp = skew_len(npx);
+    // per output row the packed pixels of both images
+    return ((size_t)rows * (Lp + Lr) + 3) & ~(size_t)3;   // the output buffers that follow are 16-byte aligned
 }
 
-template <int MODE, typename T>
+template <typename T>
 __global__ void __launch_bounds__(kXbThreads, 2)
-cost_xb_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C, int D, float tau,
+cost_xb_tad_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C, int D, float tau,
                T* __restrict__ out, uint2* __restrict__ rgbx, int rows)
 {
     extern __shared__ int sm_xb[];
@@ -507,93 +499,31 @@ cost_xb_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int
     const int nrows = min(rows, H - y0);
     const int x0 = xb0 * 8;
     const int npx = xbc * 8;
-    const int nl = npx + 2;            // left grey columns x0-1 .. x0+npx
     // right columns x0-D-8 .. x0+npx (origin rb): the 8 extra columns keep every
     // index of a thread's 8 disparities >= 0 also past D (those rows are not stored)
     const int nr = npx + D + 9;
     const int rb = x0 - D - 8;
-    const int Ll = skew_len(nl), Lr = skew_len(nr), Lp = skew_len(npx);
+    const int Lr = skew_len(nr), Lp = skew_len(npx);
 
-    int* gl = sm_xb;                             // [rows + 2][Ll]: grey rows y0-1 ..
-    int* gr = gl + (rows + 2) * Ll;              // [rows + 2][Lr]
-    int* sl = gr + (rows + 2) * Lr;              // [rows][Lp]
-    float* rl = (float*)(sl + rows * Lp);        // [rows][Lp]
-    int* sr = (int*)(rl + rows * Lp);            // [rows][Lr]
-    float* rr = (float*)(sr + rows * Lr);        // [rows][Lr]
-    uint32_t* pl = (uint32_t*)sm_xb;             // TAD: left pixels [rows][Lp]
-    uint32_t* pr = pl + rows * Lp;               // TAD: right pixels [rows][Lr], origin rb
+    uint32_t* pl = (uint32_t*)sm_xb;             // left pixels [rows][Lp]
+    uint32_t* pr = pl + rows * Lp;               // right pixels [rows][Lr], origin rb
 
-    // staging: grey values (channel sums) of rows y0-1 .. y0+nrows at clamped
-    // columns, then for each output row the statistics S, 1/sqrt(9Q - S^2) of
-    // every staged block centre exactly as grey_stats_kernel computes them, and
-    // the left pixels' packed guide
-    auto grey = [&](const uint8_t* img, int yy, int x) -> int {
-        const uint8_t* q = img + ((size_t)yy * W + x) * C;
-        return C == 3 ? (int)q[0] + (int)q[1] + (int)q[2] : (int)q[0];
-    };
+    // staging: the pixels of the output rows at clamped columns, and the left
+    // image's packed guide
     auto colour = [&](const uint8_t* img, int yy, int x) -> uint32_t {
         const uint8_t* q = img + ((size_t)yy * W + clampi(x, 0, W - 1)) * C;
         return C == 3 ? (uint32_t)q[0] | ((uint32_t)q[1] << 8) | ((uint32_t)q[2] << 16) : (uint32_t)q[0];
     };
-    if (MODE == 0) {
-        for (int c = tid; c < nl; c += nthr) {
-            const int x = clampi(x0 - 1 + c, 0, W - 1);
-            for (int j = 0; j < nrows + 2; ++j) gl[j * Ll + skew(c)] = grey(L, clampi(y0 - 1 + j, 0, H - 1), x);
-        }
-        for (int c = tid; c < nr; c += nthr) {
-            const int x = clampi(rb + c, 0, W - 1);
-            for (int j = 0; j < nrows + 2; ++j) gr[j * Lr + skew(c)] = grey(R, clampi(y0 - 1 + j, 0, H - 1), x);
-        }
-        __syncthreads();
-        for (int e = tid; e < nrows * npx; e += nthr) {
-            // left centre x0 + i of output row k sits at staged column i + 1 of rows k .. k+2
-            const int k = e / npx, i = e - k * npx;
-            const int* g = gl + k * Ll;
-            int sum = 0, sq = 0;
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    const int v = g[j * Ll + skew(i + m)];
-                    sum += v;
-                    sq += v * v;
-                }
-            const int var = 9 * sq - sum * sum;
-            sl[k * Lp + skew(i)] = sum;
-            rl[k * Lp + skew(i)] = var > 0 ? rsqrtf((float)var) : 0.f;
-            if (x0 + i < W) {
-                const uint32_t col = colour(L, y0 + k, x0 + i);
-                rgbx[(size_t)(y0 + k) * rgbx_pitch(W) + x0 + i] = make_uint2(col, (uint32_t)__dp4a(col, col, 0u));
-            }
-        }
-        for (int e = tid; e < nrows * (nr - 2); e += nthr) {
-            const int k = e / (nr - 2), c = 1 + e - k * (nr - 2);
-            const int* g = gr + k * Lr;
-            int sum = 0, sq = 0;
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                for (int m = -1; m <= 1; ++m) {
-                    const int v = g[j * Lr + skew(c + m)];
-                    sum += v;
-                    sq += v * v;
-                }
-            const int var = 9 * sq - sum * sum;
-            sr[k * Lr + skew(c)] = sum;
-            rr[k * Lr + skew(c)] = var > 0 ? rsqrtf((float)var) : 0.f;
-        }
-    } else {
-        for (int e = tid; e < nrows * npx; e += nthr) {
-            const int k = e / npx, c = e - k * npx;
-            const uint32_t col = colour(L, y0 + k, x0 + c);
-            pl[k * Lp + skew(c)] = col;
-            if (x0 + c < W)
-                rgbx[(size_t)(y0 + k) * rgbx_pitch(W) + x0 + c] = make_uint2(col, (uint32_t)__dp4a(col, col, 0u));
-        }
-        for (int e = tid; e < nrows * nr; e += nthr) {
-            const int k = e / nr, c = e - k * nr;
-            pr[k * Lr + skew(c)] = colour(R, y0 + k, rb + c);
-        }
+    for (int e = tid; e < nrows * npx; e += nthr) {
+        const int k = e / npx, c = e - k * npx;
+        const uint32_t col = colour(L, y0 + k, x0 + c);
+        pl[k * Lp + skew(c)] = col;
+        if (x0 + c < W)
+            rgbx[(size_t)(y0 + k) * rgbx_pitch(W) + x0 + c] = make_uint2(col, (uint32_t)__dp4a(col, col, 0u));
+    }
+    for (int e = tid; e < nrows * nr; e += nthr) {
+        const int k = e / nr, c = e - k * nr;
+        pr[k * Lr + skew(c)] = colour(R, y0 + k, rb + c);
     }
     __syncthreads();
 
@@ -606,106 +536,14 @@ cost_xb_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int
     const int xl = 8 * xbl;            // the block's first pixel, relative to x0
     const int xbase = x0 + xl;
     const int lane = tid & 31;
-    constexpr bool kBf16 = std::is_same<T, __nv_bfloat16>::value;
-    uint4* wbuf = (uint4*)(sm_xb + cost_xb_stage_ints(MODE, D, rows)) + (size_t)(tid >> 5) * kXbWarpRows;
+    uint4* wbuf = (uint4*)(sm_xb + cost_xb_stage_ints(D, rows)) + (size_t)(tid >> 5) * kXbWarpRows;
     uint4* mine = wbuf + 9 * lane;     // rows 8*lane + s at 9*lane + s
 
     for (int k = 0; k < nrows; ++k) {
         const int y = y0 + k;
-        // this output row's staged rows (grey rows k .. k+2 are y-1 .. y+1) and statistics
-        const int* glk = gl + k * Ll;
-        const int* grk = gr + k * Lr;
-        const int* slk = sl + k * Lp;
-        const float* rlk = rl + k * Lp;
-        const int* srk = sr + k * Lr;
-        const float* rrk = rr + k * Lr;
         const uint32_t* plk = pl + k * Lp;
         const uint32_t* prk = pr + k * Lr;
-        (void)glk, (void)grk, (void)slk, (void)rlk, (void)srk, (void)rrk, (void)plk, (void)prk;
-        if (!active) {
-        } else if (MODE == 0) {
-            int glw[3][10], grw[3][10], sli[8], srw[8];
-            float rli[8], rrw[8];
-    #pragma unroll
-            for (int j = 0; j < 3; ++j)
-    #pragma unroll
-                for (int c = 0; c < 10; ++c) glw[j][c] = glk[j * Ll + skew(xl + c)];
-    #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                sli[i] = slk[skew(xl + i)];
-                rli[i] = rlk[skew(xl + i)];
-            }
-            // right block of (x, d) spans columns x-d-1 .. x-d+1: index (x - d - 1 + k) - rb
-            int base = xl - d0 - 1 + D + 8;
-    #pragma unroll
-            for (int j = 0; j < 3; ++j)
-    #pragma unroll
-                for (int c = 0; c < 10; ++c) grw[j][c] = grk[j * Lr + skew(base + c)];
-    #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                srw[i] = srk[skew(base + 1 + i)];
-                rrw[i] = rrk[skew(base + 1 + i)];
-            }
-            // the normalisation of a pixel pair is one packed multiply and one packed
-            // FMA (per lane exactly ncc_cost); threads whose 8 pixels are inside the
-            // image and match inside it for all 8 disparities skip the two masks
-            const uint64_t ones2 = f2_pack(1.f, 1.f);
-            auto sweep = [&](auto masked) {
-    #pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const int d = d0 + s;
-                    if (s > 0) {
-                        // d grew by one: the window slides one column to the left
-                        --base;
-    #pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-    #pragma unroll
-                            for (int c = 9; c > 0; --c) grw[j][c] = grw[j][c - 1];
-                            grw[j][0] = grk[j * Lr + skew(base)];
-                        }
-    #pragma unroll
-                        for (int i = 7; i > 0; --i) {
-                            srw[i] = srw[i - 1];
-                            rrw[i] = rrw[i - 1];
-                        }
-                        srw[0] = srk[skew(base + 1)];
-                        rrw[0] = rrk[skew(base + 1)];
-                    }
-                    int cp[10];
-    #pragma unroll
-                    for (int c = 0; c < 10; ++c)
-                        cp[c] = glw[0][c] * grw[0][c] + glw[1][c] * grw[1][c] + glw[2][c] * grw[2][c];
-                    int P = cp[0] + cp[1] + cp[2];
-                    int num[8];
-    #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        if (i > 0) P += cp[i + 2] - cp[i - 1];
-                        num[i] = 9 * P - sli[i] * srw[i];
-                    }
-                    uint32_t w[4];
-    #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint64_t t = f2_mul(f2_pack(rli[2 * q], rli[2 * q + 1]), f2_pack(rrw[2 * q], rrw[2 * q + 1]));
-                        const uint64_t nn = f2_pack(-__int2float_rn(num[2 * q]), -__int2float_rn(num[2 * q + 1]));
-                        float c0, c1;
-                        f2_unpack(f2_fma(nn, t, ones2), c0, c1);
-                        if (decltype(masked)::value) {
-                            const int x = xbase + 2 * q;
-                            c0 = x - d < 0 ? 2.f : c0;
-                            c1 = x + 1 - d < 0 ? 2.f : c1;
-                            c0 = x < W ? c0 : 0.f;
-                            c1 = x + 1 < W ? c1 : 0.f;
-                        }
-                        w[q] = pack_16x2<kBf16>(c0, c1);
-                    }
-                    mine[s] = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            };
-            if (xbase + 7 < W && xbase >= d0 + 7)
-                sweep(std::integral_constant<bool, false>{});
-            else
-                sweep(std::integral_constant<bool, true>{});
-        } else {
+        if (active) {
             const float inv_c = 1.f / (float)C;
             uint32_t pli[8], prw[8];
     #pragma unroll
@@ -768,14 +606,305 @@ cost_xb_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int
     }
 }
 
-size_t cost_xb_smem_bytes(int mode, int D, int rows)
+// ---- NCC, 16-bit x-blocked volume ----------------------------------------------
+// A CTA covers 64 pixels x 4 rows and every disparity.  All of Eq. (1) runs in
+// FP32 on exact integers: with the grey values moved by a constant a
+// (which changes neither 9 P - S_l S_r nor the variances) |g - a| <= 383, so
+// every product, block sum, 9 P' and S_l' S_r' is an integer below 2^24, and
+// 9 P' - S_l' S_r' comes out of one FMA rounded once -- the integer converted to
+// float.  A thread computes two output rows y, y + 1 at once: with p_j the
+// products of grey rows y-1 .. y+2, the column sums are p_0 + t and t + p_3,
+// t = p_1 + p_2 (4 FMAs for two sums), and everything after them is packed, one
+// row per half.
+//   * Staging: per column and pair of output rows a float4 of the four grey rows
+//     y-1 .. y+2, then per block centre a float4 (S(y), S(y+1), 1/sqrt V(y),
+//     1/sqrt V(y+1)).  Index c + c/4: lanes 4 columns apart read 16 bytes each
+//     without conflicts.
+//   * A lane owns 4 pixels x 2 rows (lanes 0-15: the 64 pixels of rows y0, y0+1;
+//     16-31: of the next two) and 16 disparities of its warp: the left window
+//     (6 columns x 4 rows) stays in registers, the right one slides one column
+//     (2 shared loads) per disparity.  Per pair of costs: 6 FMAs and 1.75 packed
+//     additions for the block sum P', 3 packed operations for the normalisation.
+//   * Lanes 2i, 2i + 1 hold the two halves of a block of 8 pixels: they exchange
+//     a row each, so that a lane has 16 bytes (8 pixels) of its row per
+//     disparity, and stage them in the warp's buffer; one TMA store per pair of
+//     rows writes 8 blocks x 16 disparities.  (Direct stores of 32 bytes per
+//     lane, each in a line of its own, kept the load/store pipe 76% busy:
+//     123 us at 1280x960, D = 128.)
+// Bound: instruction issue of the sweep (11.5 instructions per cost with the
+// staging; the integer form it replaces took 30), then the volume's writes to HBM.
+// CTAs of 4 warps (four per SM) overlap one another's staging best: 1920x1080,
+// D = 256: 316 us against 334 us with 8 warps, 345 us with 8 warps and 8 rows
+// (before the column sums went from packed to scalar FMAs).
+// Measured on GB300 (CUDA events), BF16, before -> now: 640x480, D = 64: 35.5 ->
+// 19.8 us; 1280x960, D = 128: 188 -> 89.5 us; 1920x1080, D = 256: 557 -> 274 us
+// (1.13 GB written: 4.1 TB/s).
+constexpr int kNccPx = 64;
+constexpr int kNccWarps = 4;
+constexpr int kNccRows = 4;      // two pairs
+
+__host__ __device__ inline int skew4(int c) { return c + (c >> 2); }
+__host__ __device__ inline int ncc_groups(int D) { return (D + 15) / 16; }          // of 16 disparities
+__host__ __device__ inline int ncc_right_cols(int D) { return 16 * ncc_groups(D) + kNccPx + 1; }
+// float4 entries of the four staged arrays, per pair of rows
+__host__ __device__ inline int ncc_left_len() { return skew4(kNccPx + 2); }
+__host__ __device__ inline int ncc_right_len(int D) { return skew4(ncc_right_cols(D)) + 1; }
+// Store buffer of a warp: two pairs of rows, each [d / 8][block][row][8 d x 8
+// pixels] (128-byte lines, TMA's 128-byte swizzle) of 16 disparities and 8 blocks.
+constexpr int kNccPairBytes = 2 * 8 * 2 * 128, kNccWarpBytes = 2 * kNccPairBytes;
+__host__ __device__ inline size_t ncc_smem_bytes(int D)
 {
-    const int nwarps = (xb_blocks_per_cta(D) * ((D + 7) / 8) + 31) / 32;
-    return sizeof(int) * cost_xb_stage_ints(mode, D, rows) + (size_t)nwarps * kXbWarpRows * 16;
+    return 1024 + (size_t)kNccWarps * kNccWarpBytes + (size_t)2 * 16 * 2 * (ncc_left_len() + ncc_right_len(D));
 }
 
-template <int MODE, typename T>
-cudaError_t launch_cost_xb(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W, int C,
+template <bool BF16>
+__global__ void __launch_bounds__(32 * kNccWarps, 4)
+cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* __restrict__ L,
+                   const uint8_t* __restrict__ R, int H, int W, int C, int D, uint2* __restrict__ rgbx)
+{
+    extern __shared__ uint8_t sm_ncc[];
+    // let a programmatically launched successor (the tensor-core aggregation)
+    // start its set-up once every CTA of this grid has started; it waits for
+    // this grid's completion before it reads anything this kernel writes
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int ROWS = kNccRows, PAIRS = ROWS / 2, nthr = 32 * kNccWarps;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int x0 = blockIdx.x * kNccPx, y0 = blockIdx.y * ROWS;
+    const int ng = ncc_groups(D), nr = ncc_right_cols(D);
+    const int rb = x0 - 16 * ng;             // image column of right column 0
+    const int LL = ncc_left_len(), RL = ncc_right_len(D);
+    uint8_t* const buffers = sm_ncc + ((1024u - (tc::smem_u32(sm_ncc) & 1023u)) & 1023u);
+    float4* const gl = (float4*)(buffers + kNccWarps * kNccWarpBytes);   // [PAIRS][LL]: columns x0 - 1 ..
+    float4* const sl = gl + PAIRS * LL;      // [PAIRS][LL]: centres x0 ..
+    float4* const gr = sl + PAIRS * LL;      // [PAIRS][RL]: columns rb ..
+    float4* const sr = gr + PAIRS * RL;      // [PAIRS][RL]: centres rb ..
+
+    // ---- grey rows y0-1 .. y0+ROWS of both images at clamped columns, and the
+    // left image's packed guide
+    const int shift = C == 3 ? 382 : 128;
+    for (int e = tid; e < kNccPx + 2 + nr; e += nthr) {
+        const bool left = e < kNccPx + 2;
+        const int c = left ? e : e - (kNccPx + 2);
+        const int xs = left ? x0 - 1 + c : rb + c;
+        const uint8_t* img = (left ? L : R) + (size_t)clampi(xs, 0, W - 1) * C;
+        uint32_t col[ROWS + 2];
+#pragma unroll
+        for (int j = 0; j < ROWS + 2; ++j) {
+            const uint8_t* q = img + (uint32_t)(clampi(y0 - 1 + j, 0, H - 1) * W) * (uint32_t)C;
+            col[j] = C == 3 ? (uint32_t)q[0] | ((uint32_t)q[1] << 8) | ((uint32_t)q[2] << 16) : (uint32_t)q[0];
+        }
+        float4* dst = (left ? gl : gr) + skew4(c);
+        float g[ROWS + 2];
+#pragma unroll
+        for (int j = 0; j < ROWS + 2; ++j) g[j] = (float)((int)__dp4a(col[j], 0x01010101u, 0u) - shift);
+#pragma unroll
+        for (int k = 0; k < PAIRS; ++k)
+            dst[k * (left ? LL : RL)] = make_float4(g[2 * k], g[2 * k + 1], g[2 * k + 2], g[2 * k + 3]);
+        if (left && c >= 1 && c <= kNccPx && xs < W) {
+            uint2* o = rgbx + (size_t)y0 * rgbx_pitch(W) + xs;
+#pragma unroll
+            for (int j = 1; j <= ROWS; ++j)
+                if (y0 + j - 1 < H)
+                    o[(size_t)(j - 1) * rgbx_pitch(W)] = make_uint2(col[j], (uint32_t)__dp4a(col[j], col[j], 0u));
+        }
+    }
+    __syncthreads();
+    // ---- block statistics of every centre (all exact up to the reciprocal square root)
+    const int ncl = kNccPx, ncr = nr - 2;    // right centres rb + 1 .. rb + nr - 2
+    for (int q = tid; q < ncl + ncr; q += nthr) {
+        const bool left = q < ncl;
+        const int cc = left ? q + 1 : q - ncl + 1;   // the centre's column in the grey array
+        const float4* g = (left ? gl : gr);
+        const int i0 = skew4(cc - 1), i1 = skew4(cc), i2 = skew4(cc + 1), len = left ? LL : RL;
+        float4* dst = left ? sl + skew4(q) : sr + i1;
+#pragma unroll
+        for (int k = 0; k < PAIRS; ++k, g += len, dst += len) {
+            const float4 v3[3] = {g[i0], g[i1], g[i2]};
+            float s0 = 0.f, s1 = 0.f, q0 = 0.f, q1 = 0.f;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float4 v = v3[j];
+                const float m = v.y + v.z, mq = fmaf(v.y, v.y, v.z * v.z);
+                s0 += m + v.x;
+                s1 += m + v.w;
+                q0 += fmaf(v.x, v.x, mq);
+                q1 += fmaf(v.w, v.w, mq);
+            }
+            const float a0 = fmaf(9.f, q0, -(s0 * s0)), a1 = fmaf(9.f, q1, -(s1 * s1));
+            *dst = make_float4(s0, s1, a0 > 0.f ? rsqrtf(a0) : 0.f, a1 > 0.f ? rsqrtf(a1) : 0.f);
+        }
+    }
+    __syncthreads();
+
+    const int p = lane & 15, odd = lane & 1;
+    const int xl = 4 * p, xbase = x0 + xl;
+    // the lane's line of its pair's buffer, (block, row) = (p / 2, odd): chunk s of
+    // 8 disparities sits at chunk s ^ (line % 8)
+    const int line = 2 * (p >> 1) + odd;
+    const uint32_t buf = tc::smem_u32(buffers) + (tid >> 5) * kNccWarpBytes;
+    const uint32_t chunk0 = buf + (lane >> 4) * kNccPairBytes + line * 128 + (line & 7) * 16;
+    auto put = [&](int s, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"((chunk0 ^ ((s & 7) * 16)) + (s >> 3) * (8 * 2 * 128)),
+                     "r"(a), "r"(b), "r"(c), "r"(d)
+                     : "memory");
+    };
+
+    const int rp = lane >> 4;
+    for (int grp = tid >> 5; grp <= ng; grp += kNccWarps) {
+        // the warp's previous stores have read its buffer
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
+        auto store = [&]() {
+            tc::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (y0 + 2 * h < H)
+                        asm volatile(
+                            "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                                (uint64_t)&out_map),
+                            "r"(0), "r"(y0 + 2 * h), "r"(x0 >> 3), "r"(2 * grp), "r"(buf + h * kNccPairBytes)
+                            : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+        };
+        if (grp == ng) {
+            // the 16 rows after the costs: one of ones (the normaliser), then zeros
+            const uint32_t one = BF16 ? 0x3F803F80u : 0x3C003C00u;
+#pragma unroll
+            for (int s = 0; s < 16; ++s) put(s, s == 0 ? one : 0u, s == 0 ? one : 0u, s == 0 ? one : 0u, s == 0 ? one : 0u);
+            store();
+            continue;
+        }
+
+        // left window and statistics
+        const float4* glw = gl + rp * LL + skew4(xl);
+        const float4* slw = sl + rp * LL + skew4(xl);
+        float4 lw[6];
+        uint64_t sli[4], rli[4];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            // -9 g: the block sums come out as -9 P' (the products stay below 2^24 / 9)
+            const float4 v = glw[j + (j >> 2)];
+            lw[j] = make_float4(-9.f * v.x, -9.f * v.y, -9.f * v.z, -9.f * v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = slw[i];
+            sli[i] = f2_pack(v.x, v.y);
+            rli[i] = f2_pack(v.z, v.w);
+        }
+        const uint64_t one2 = f2_pack(1.f, 1.f);
+
+        const int d0 = 16 * grp;
+        // right column of (x, d), window offset k: x - d + k - rb = base + (i + k - s)
+        const int base = xl + 16 * ng - d0;
+        const float4* grw = gr + rp * RL + skew4(base);
+        const float4* srw = sr + rp * RL + skew4(base);
+        auto at = [](int m) { return m + (m >> 2); };   // offset of column base + m (base is a multiple of 4)
+        float4 rw[6];
+        uint64_t sri[4], rri[4];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) rw[j] = grw[at(j - 1)];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = srw[at(i)];
+            sri[i] = f2_pack(v.x, v.y);
+            rri[i] = f2_pack(v.z, v.w);
+        }
+        // lanes whose 4 pixels are inside the image and match inside it for all 16
+        // disparities of the range skip the masks
+        auto sweep = [&](auto masked) {
+#pragma unroll
+            for (int s = 0; s < 16; ++s) {
+                const int d = d0 + s;
+                if (s > 0) {
+                    // d grew by one: the window slides one column to the left
+#pragma unroll
+                    for (int j = 5; j > 0; --j) rw[j] = rw[j - 1];
+                    rw[0] = grw[at(-1 - s)];
+#pragma unroll
+                    for (int i = 3; i > 0; --i) {
+                        sri[i] = sri[i - 1];
+                        rri[i] = rri[i - 1];
+                    }
+                    const float4 v = srw[at(-s)];
+                    sri[0] = f2_pack(v.x, v.y);
+                    rri[0] = f2_pack(v.z, v.w);
+                }
+                uint64_t cs[6];
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    const float t = fmaf(lw[j].y, rw[j].y, lw[j].z * rw[j].z);
+                    cs[j] = f2_pack(fmaf(lw[j].x, rw[j].x, t), fmaf(lw[j].w, rw[j].w, t));
+                }
+                const uint64_t a0 = f2_add(cs[0], cs[1]), a1 = f2_add(cs[2], cs[3]), a2 = f2_add(cs[4], cs[5]);
+                const uint64_t P[4] = {f2_add(a0, cs[2]), f2_add(cs[1], a1), f2_add(a1, cs[4]), f2_add(cs[3], a2)};
+                float c0[4], c1[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    // S_l' S_r' - 9 P' rounded once, times the rounded product of the normalisers, plus 1
+                    const uint64_t nn = f2_fma(sli[i], sri[i], P[i]);
+                    f2_unpack(f2_fma(nn, f2_mul(rli[i], rri[i]), one2), c0[i], c1[i]);
+                    if (decltype(masked)::value) {
+                        const int x = xbase + i;
+                        if (x - d < 0) c0[i] = c1[i] = 2.f;
+                        if (x >= W || d >= D) c0[i] = c1[i] = 0.f;
+                    }
+                }
+                const uint32_t w0 = pack_16x2<BF16>(c0[0], c0[1]), w1 = pack_16x2<BF16>(c0[2], c0[3]);
+                const uint32_t v0 = pack_16x2<BF16>(c1[0], c1[1]), v1 = pack_16x2<BF16>(c1[2], c1[3]);
+                const uint32_t e0 = __shfl_xor_sync(0xffffffffu, odd ? w0 : v0, 1);
+                const uint32_t e1 = __shfl_xor_sync(0xffffffffu, odd ? w1 : v1, 1);
+                const uint32_t o0 = odd ? e0 : w0, o1 = odd ? e1 : w1, o2 = odd ? v0 : e0, o3 = odd ? v1 : e1;
+                put(s, o0, o1, o2, o3);
+            }
+        };
+        const bool inside = xbase + 3 < W && xbase >= d0 + 15 && d0 + 16 <= D;
+        if (__all_sync(0xffffffffu, inside))
+            sweep(std::integral_constant<bool, false>{});
+        else
+            sweep(std::integral_constant<bool, true>{});
+        store();
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+
+template <bool BF16>
+cudaError_t launch_cost_xb_ncc(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W, int C,
+                               int D, void* out, cudaStream_t stream)
+{
+    // the volume as (8 disparities x 8 columns = 128 contiguous bytes, image row, block, d / 8)
+    const tca::EncodeTiledFn enc = tca::encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const int nxb = (W + 7) / 8, Dp = tc_block_rows(D);
+    cuuint64_t dims[4] = {64, (cuuint64_t)H, (cuuint64_t)nxb, (cuuint64_t)(Dp / 8)};
+    cuuint64_t strides[3] = {(cuuint64_t)nxb * Dp * 16, (cuuint64_t)Dp * 16, 128};
+    cuuint32_t box[4] = {64, 2, kNccPx / 8, 2};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUtensorMap map;
+    if (enc(&map, BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, out, dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    const size_t smem = ncc_smem_bytes(D);
+    cudaError_t e = fbs::raise_smem_limit(cost_xb_ncc_kernel<BF16>, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((W + kNccPx - 1) / kNccPx, (H + kNccRows - 1) / kNccRows);
+    fbs::note_launch();
+    cost_xb_ncc_kernel<BF16><<<grid, 32 * kNccWarps, smem, stream>>>(map, left, right, H, W, C, D, sc.rgbx);
+    return cudaGetLastError();
+}
+
+size_t cost_xb_tad_smem_bytes(int D, int rows)
+{
+    const int nwarps = (xb_blocks_per_cta(D) * ((D + 7) / 8) + 31) / 32;
+    return sizeof(int) * cost_xb_stage_ints(D, rows) + (size_t)nwarps * kXbWarpRows * 16;
+}
+
+template <typename T>
+cudaError_t launch_cost_xb_tad(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W, int C,
                            int D, float tau, T* out, cudaStream_t stream)
 {
     const int ndg = (D + 7) / 8;
@@ -790,13 +919,13 @@ cudaError_t launch_cost_xb(const CostScratch& sc, const uint8_t* left, const uin
     if (e != cudaSuccess) return e;
     int rows = kXbMaxRows;
     while (rows > 1 && (long long)gx * ((H + rows - 1) / rows) < 4LL * sms) rows /= 2;
-    const size_t smem = cost_xb_smem_bytes(MODE, D, rows);
-    e = fbs::raise_smem_limit(cost_xb_kernel<MODE, T>, (int)smem);
+    const size_t smem = cost_xb_tad_smem_bytes(D, rows);
+    e = fbs::raise_smem_limit(cost_xb_tad_kernel<T>, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid(gx, (H + rows - 1) / rows);
     fbs::note_launch();
     const int nthr = (xbc * ndg + 31) / 32 * 32;   // whole warps (the write-out shuffles need all lanes)
-    cost_xb_kernel<MODE, T><<<grid, nthr, smem, stream>>>(left, right, H, W, C, D, tau, out, sc.rgbx, rows);
+    cost_xb_tad_kernel<T><<<grid, nthr, smem, stream>>>(left, right, H, W, C, D, tau, out, sc.rgbx, rows);
     return cudaGetLastError();
 }
 
@@ -959,10 +1088,10 @@ cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* lef
     // one launch: statistics, costs, pad rows and the packed guide (sc.rgbx)
     if (D > 256 || !sc.rgbx) return cudaErrorInvalidValue;   // serves the tensor-core form only
     if (mode == 0)
-        return bf16 ? launch_cost_xb<0>(sc, left, right, H, W, C, D, tau, (__nv_bfloat16*)cost, stream)
-                    : launch_cost_xb<0>(sc, left, right, H, W, C, D, tau, (__half*)cost, stream);
-    return bf16 ? launch_cost_xb<1>(sc, left, right, H, W, C, D, tau, (__nv_bfloat16*)cost, stream)
-                : launch_cost_xb<1>(sc, left, right, H, W, C, D, tau, (__half*)cost, stream);
+        return bf16 ? launch_cost_xb_ncc<true>(sc, left, right, H, W, C, D, cost, stream)
+                    : launch_cost_xb_ncc<false>(sc, left, right, H, W, C, D, cost, stream);
+    return bf16 ? launch_cost_xb_tad(sc, left, right, H, W, C, D, tau, (__nv_bfloat16*)cost, stream)
+                : launch_cost_xb_tad(sc, left, right, H, W, C, D, tau, (__half*)cost, stream);
 }
 
 }  // namespace fbs

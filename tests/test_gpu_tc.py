@@ -186,3 +186,33 @@ def test_kernel_accounting_counts_every_launch(fbs, prec, expect):
         fbs.fbs_sync(ctx.ctx)
     assert got == {k: 3 * v for k, v in expect.items()}
 
+
+
+# The 16-bit cost kernel covers 64 pixels x 4 rows per CTA, 16 disparities per warp.
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("H,W,C,D", [(1, 1, 1, 1), (3, 7, 3, 15), (4, 64, 1, 16), (5, 65, 3, 17), (9, 129, 3, 40),
+                                     (6, 200, 1, 64), (2, 61, 3, 130), (7, 300, 3, 256)])
+def test_radius_zero_maps_are_those_of_the_rounded_fp32_costs(fbs, prec, H, W, C, D):
+    """With radius 0 the aggregated value is the 16-bit cost itself, so the maps are
+    exactly those of the FP32 volume (another kernel) rounded to 16 bits."""
+    rng = np.random.default_rng(H + W + D)
+    L = rng.integers(0, 256, (H, W, C)).astype(np.uint8)
+    R = np.roll(L, -min(5, W - 1), axis=1)
+    R = np.clip(R.astype(np.int32) + rng.integers(-40, 41, R.shape), 0, 255).astype(np.uint8)
+    L[:, : W // 3] //= 64                    # flat blocks and exact ties
+    dl, dr = torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()
+    with fbs.Context(0, prec=fbs.FBS_PREC_BF16 if prec == "bf16" else fbs.FBS_PREC_F16) as ctx:
+        di, ds = ctx.compute_disparity(dl, dr, D, 0, 1.0, 10.0)
+        cost = ctx.cost_volume(dl, dr, D)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(ctx.ctx)
+    A = cost.to(torch.bfloat16 if prec == "bf16" else torch.float16).float().cpu().numpy()
+    best = A.argmin(2)
+    i = np.clip(best, 1, max(1, D - 2))[..., None]
+    take = lambda k: np.take_along_axis(A, np.clip(i + k, 0, D - 1), 2)[..., 0]  # noqa: E731
+    a, b, c = take(-1), take(0), take(1)
+    den = np.float32(2) * a + np.float32(2) * c - np.float32(4) * b
+    ok = (best > 0) & (best < D - 1) & (den > 0)
+    sub = best + np.where(ok, (a - c) / np.where(ok, den, np.float32(1)), np.float32(0)).astype(np.float32)
+    assert np.array_equal(di.cpu().numpy(), best)
+    np.testing.assert_allclose(ds.cpu().numpy(), sub, rtol=0, atol=2.0 ** -22 * max(1, D))
