@@ -652,6 +652,9 @@ __device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, c
         for (int r = tid >> 6; r <= t.r_hi - t.r_lo; r += kThreads / 64)
             gtile[r * NC + c] = in ? packed_colour(src + (size_t)r * W * C, C) : 0u;
     }
+    // what precedes needs only the caller's image; the cost volume is written by the
+    // kernel before this one (a no-op for an ordinary launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     const bool valid = t.py < H && t.px < W;
     t.pcol = valid ? gtile[(t.py - t.r_lo) * NC + t.px - x0 + rho] : 0u;
@@ -724,6 +727,7 @@ aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __re
 {
     extern __shared__ __align__(128) float4 smem_f4[];
     Ring ring = make_ring<kTma>(smem_f4, slots, err);
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the ranges and bands come from earlier kernels
     const int2 r = tile_range[(size_t)blockIdx.y * gridDim.x + blockIdx.x];
     aggregate_tile<kTma, 4>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
                             blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, ring, r.x, r.y, band);
@@ -787,13 +791,16 @@ bool encode_volume(CUtensorMap* map, const float* cost, int ld, int H, int W, in
 template <Copy COPY>
 cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                         int D, int rho, float neg_ks, float neg_kr, float* agg_out, int32_t* disp_int, float* disp_sub,
-                        int* err, cudaStream_t stream)
+                        int* err, bool after_cost, cudaStream_t stream)
 {
     const int slots = ring_slots(rho, column_size(D));
     const size_t smem = smem_bytes(rho, column_size(D), slots);
     cudaError_t e = fbs::raise_smem_limit(aggregate_f32_kernel<COPY>, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
+    if (after_cost)
+        return fbs::launch_after(aggregate_f32_kernel<COPY>, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D,
+                                 rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, err);
     fbs::note_launch();
     aggregate_f32_kernel<COPY><<<grid, kThreads, smem, stream>>>(
         map, cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, err);
@@ -834,15 +841,13 @@ cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guid
     cudaError_t e = fbs::raise_smem_limit(aggregate_band_kernel, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
-    fbs::note_launch();
-    aggregate_band_kernel<<<grid, kThreads, smem, stream>>>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr,
-                                                            tile_range, band, disp_int, disp_sub, slots, err);
-    return cudaGetLastError();
+    return fbs::launch_after(aggregate_band_kernel, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D, radius,
+                             neg_ks, neg_kr, tile_range, band, disp_int, disp_sub, slots, err);
 }
 
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                                  int D, int radius, float sigma_s, float sigma_r, float* agg_out,
-                                 int32_t* disp_int, float* disp_sub, int* err, cudaStream_t stream)
+                                 int32_t* disp_int, float* disp_sub, int* err, bool after_cost, cudaStream_t stream)
 {
     // exp(-a/g^2) = exp2(-a * log2(e) / g^2)
     const double log2e = 1.4426950408889634;
@@ -851,9 +856,9 @@ cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide
     CUtensorMap map{};
     if (encode_volume(&map, cost, ld, H, W, D, radius))
         return launch_copy<kTma>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                 err, stream);
+                                 err, after_cost, stream);
     return launch_copy<kAsync4>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                err, stream);
+                                err, after_cost, stream);
 }
 
 }  // namespace fbs

@@ -363,7 +363,7 @@ fbs_status build_branch_graph(fbs_ctx* ctx, int n, const fbs_pair* pairs, int nb
             k0 = fbs::launch_count();
             if (e == cudaSuccess)
                 e = fbs::launch_aggregate_f32(cost, ld, q.left, q.H, q.W, q.C, q.D, q.radius, q.sigma_s, q.sigma_r,
-                                              nullptr, q.disp_int, q.disp_subpix, ctx->derr, s);
+                                              nullptr, q.disp_int, q.disp_subpix, ctx->derr, true, s);
             g->kernels[FBS_KERNEL_AGG_F32] += fbs::launch_count() - k0;
             continue;
         }

@@ -4,7 +4,7 @@
 // channel sum, n = 9 and the block sums S = sum g, Q = sum g^2 and
 // P = sum g_l g_r, Eq. (1) multiplied through by n^2 reads
 //     c = (n P - S_l S_r) / sqrt((n Q_l - S_l^2) (n Q_r - S_r^2)).
-// Every sum and both numerator terms are exact in int32 (g <= 765), so only the
+// Every sum and both numerator terms are exact integers (grey_shift), so only the
 // final normalisation is rounded.  Stored cost: C = 1 - c.  Boundary rules:
 // blocks clamp to the image; u - d < 0 gives the maximum cost 2; a block of
 // zero variance gives c = 0.
@@ -13,13 +13,8 @@
 // computed once per pixel, so the per-(p, d) work is the dot product P.  Two
 // kernels write the two layouts:
 //   * cost_kernel, [H][W][ld] float32 (D innermost; the FP32 aggregation),
-//     padding d in [D, ld) written as 0.  A pre-pass (grey_stats_kernel: g, S,
-//     1/sqrt(nQ - S^2)) fills statistics planes; a thread owns a run of 4
-//     pixels and 8 consecutive disparities (left 3x6 grey window in
-//     registers, right window sliding one column per disparity, three column
-//     products per output column summed by a sliding 3-column window);
-//     results are staged in shared memory as [d][x] and written out with D
-//     innermost.
+//     padding d in [D, ld) written as 0.  A pre-pass (grey_stats_kernel) fills
+//     planes of the shifted grey value, its block sum and 1/sqrt(nQ - S^2).
 //   * cost_xb_ncc_kernel, 16-bit x-blocked [H][ceil(W/8)][Dp][8] (the tensor-core
 //     aggregation): for a row y and a block of 8 columns, the Dp x 8 block is
 //     contiguous, so the tensor-core kernel's TMA reads contiguous blocks that
@@ -27,7 +22,7 @@
 //     One launch computes the statistics of the rows it stages, the costs, the
 //     pad rows D .. Dp-1 and the left image's packed guide (its comment says how);
 //     cost_xb_tad_kernel does the same for TAD.
-// Both round the normalisation the same way (ncc_cost), so the 16-bit volume
+// Both round the normalisation the same way (ncc_cost2), so the 16-bit volume
 // equals the FP32 volume rounded to 16 bits.
 //
 // TAD (not in the paper): C = min(mean_c |I_l(u,v) - I_r(u-d,v)|, tau), tau
@@ -44,80 +39,69 @@
 namespace fbs {
 namespace {
 
-constexpr int kXS = 128;          // pixels per CTA along x
-constexpr int kDC = 64;           // disparities per pass
-constexpr int kThreads = 256;     // 32 runs of 4 pixels x 8 groups of 8 disparities
-constexpr int kStage = kXS + 1;   // staged row pitch (odd: conflict-free transposed reads)
-constexpr int kNRG = kXS + kDC + 2;        // right grey columns per pass
-constexpr int kQR = (kNRG + 3) / 4;        // de-interleaved quarter length of a right row
-constexpr int kQS = (kXS + kDC) / 4;       // same for the right block statistics
-
-// Lanes of a warp own pixel runs 4*run .. 4*run+3 and read or write column
-// 4*run + k together; storing column c at (c & 3) * quarter + (c >> 2) puts
-// those 32 accesses in 32 different banks.
-__device__ __forceinline__ int stage_pos(int x) { return (x & 3) * 32 + (x >> 2); }
-__device__ __forceinline__ int rpos(int c) { return (c & 3) * kQR + (c >> 2); }
-__device__ __forceinline__ int spos(int c) { return (c & 3) * kQS + (c >> 2); }
-
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-// C = 1 - c with c = num * (rv_l * rv_r): one rounded product of the two
-// normalisers, then one fused multiply-add (every cost kernel uses this, so the
-// FP32 and the 16-bit volumes hold the same values before the 16-bit rounding).
-__device__ __forceinline__ float ncc_cost(int num, float rv_l, float rv_r)
-{
-    return __fmaf_rn(-__int2float_rn(num), __fmul_rn(rv_l, rv_r), 1.f);
-}
+// Grey values are moved by this constant: 9 P - S_l S_r and the variances do not
+// change, and with |g - a| <= 383 every product, block sum, 9 P' and S_l' S_r'
+// is an integer below 2^24, exact in FP32.
+__host__ __device__ inline int grey_shift(int C) { return C == 3 ? 382 : 128; }
 
-// Per-pixel statistics of one image: g = channel sum, S = 3x3 box sum of g
-// (clamped), rv = 1/sqrt(9 Q - S^2) or 0 for a flat block.
-__device__ __forceinline__ void stats_pixel(const uint8_t* __restrict__ src, int img, int H, int W, int C, int x,
-                                            int y, int16_t* __restrict__ g_out, int* __restrict__ s_out,
-                                            float* __restrict__ rv_out, uint2* __restrict__ rgbx)
+// ---- statistics pre-pass of the FP32 layout (Sec. II-A, Sec. III) ----------------
+// Per pixel and image: g' = channel sum - shift, S' = 3x3 sum of g' (clamped),
+// rv = 1 / sqrt(9 Q - S^2) or 0 for a flat block.  A CTA stages the grey values of
+// 128 x 8 pixels and their border once; a thread owns a column and carries the
+// row sums of three rows.
+constexpr int kStatX = 128, kStatY = 8;
+
+__device__ __forceinline__ void stats_tile(const uint8_t* __restrict__ src, int H, int W, int C, int x0, int y0,
+                                           int16_t* __restrict__ g_out, float* __restrict__ s_out,
+                                           float* __restrict__ rv_out, float (*g)[kStatX + 2])
 {
-    const size_t plane = (size_t)H * W;
-    int s = 0, q = 0;
+    const int shift = grey_shift(C);
+    for (int c = threadIdx.x; c < kStatX + 2; c += kStatX) {
+        const uint8_t* p = src + (size_t)clampi(x0 - 1 + c, 0, W - 1) * C;
 #pragma unroll
-    for (int j = -1; j <= 1; ++j) {
-        const int yy = clampi(y + j, 0, H - 1);
-#pragma unroll
-        for (int k = -1; k <= 1; ++k) {
-            const uint8_t* p = src + ((size_t)yy * W + clampi(x + k, 0, W - 1)) * C;
-            int g = p[0];
-            if (C == 3) g += p[1] + p[2];
-            s += g;
-            q += g * g;
+        for (int j = 0; j < kStatY + 2; ++j) {
+            const uint8_t* q = p + (size_t)clampi(y0 - 1 + j, 0, H - 1) * W * C;
+            g[j][c] = (float)((C == 3 ? (int)q[0] + (int)q[1] + (int)q[2] : (int)q[0]) - shift);
         }
     }
-    const uint8_t* p = src + ((size_t)y * W + x) * C;
-    int g = p[0];
-    if (C == 3) g += p[1] + p[2];
-    if (rgbx != nullptr && img == 0) {
-        const uint32_t c = C == 3 ? (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) : (uint32_t)p[0];
-        rgbx[(size_t)y * rgbx_pitch(W) + x] = make_uint2(c, (uint32_t)__dp4a(c, c, 0u));
+    __syncthreads();
+    const int c = threadIdx.x, x = x0 + c;
+    if (x < W) {
+        float h0 = 0.f, h1 = 0.f, q0 = 0.f, q1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < kStatY + 2; ++j) {
+            const float a = g[j][c], b = g[j][c + 1], d = g[j][c + 2];
+            const float h = a + b + d, q = fmaf(a, a, fmaf(b, b, d * d));
+            const int y = y0 + j - 2;
+            if (j >= 2 && y < H) {
+                const float s = h0 + h1 + h, v = fmaf(9.f, q0 + q1 + q, -(s * s));
+                const size_t o = (size_t)y * W + x;
+                g_out[o] = (int16_t)g[j - 1][c + 1];
+                s_out[o] = s;
+                rv_out[o] = v > 0.f ? rsqrtf(v) : 0.f;
+            }
+            h0 = h1, h1 = h;
+            q0 = q1, q1 = q;
+        }
     }
-    const int v = 9 * q - s * s;
-    const size_t o = img * plane + (size_t)y * W + x;
-    g_out[o] = (int16_t)g;
-    s_out[o] = s;
-    rv_out[o] = v > 0 ? rsqrtf((float)v) : 0.f;
 }
 
-__global__ void __launch_bounds__(256)
-grey_stats_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C,
-                  int16_t* __restrict__ g_out, int* __restrict__ s_out, float* __restrict__ rv_out,
-                  uint2* __restrict__ rgbx)
+__global__ void __launch_bounds__(kStatX)
+grey_stats_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C, CostScratch sc)
 {
-    const int img = blockIdx.z;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= W) return;
-    stats_pixel(img == 0 ? L : R, img, H, W, C, x, blockIdx.y, g_out, s_out, rv_out, rgbx);
+    __shared__ float g[kStatY + 2][kStatX + 2];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const size_t o = blockIdx.z * (size_t)H * W;
+    stats_tile(blockIdx.z == 0 ? L : R, H, W, C, blockIdx.x * kStatX, blockIdx.y * kStatY, sc.g + o, sc.s + o, sc.rv + o, g);
 }
 
-// Batched statistics: an item is one row of one pair (both images).
-__global__ void __launch_bounds__(256)
+// Batched statistics: an item is one 128 x 8 tile of one pair (both images).
+__global__ void __launch_bounds__(kStatX)
 grey_stats_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems, int* __restrict__ counter)
 {
+    __shared__ float g[kStatY + 2][kStatX + 2];
     __shared__ int item_s;
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
@@ -126,19 +110,19 @@ grey_stats_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int n
         __syncthreads();
         if (item >= nitems) break;
         const BatchPair& bp = pairs[find_pair(pairs, npairs, item, &BatchPair::stat_off)];
-        const int y = item - bp.stat_off;
         if (bp.mode != 0) continue;   // TAD needs no statistics
-        for (int x = threadIdx.x; x < bp.W; x += blockDim.x)
-            for (int img = 0; img < 2; ++img)
-                stats_pixel(img == 0 ? bp.left : bp.right, img, bp.H, bp.W, bp.C, x, y, bp.sc.g, bp.sc.s, bp.sc.rv,
-                            bp.sc.rgbx);
+        const int t = item - bp.stat_off, nx = (bp.W + kStatX - 1) / kStatX;
+        for (int img = 0; img < 2; ++img) {
+            const size_t o = img * (size_t)bp.H * bp.W;
+            stats_tile(img == 0 ? bp.left : bp.right, bp.H, bp.W, bp.C, (t % nx) * kStatX, (t / nx) * kStatY, bp.sc.g + o,
+                       bp.sc.s + o, bp.sc.rv + o, g);
+            __syncthreads();
+        }
     }
 }
 
 template <typename T>
 __device__ __forceinline__ T to_out(float v);
-template <>
-__device__ __forceinline__ float to_out<float>(float v) { return v; }
 template <>
 __device__ __forceinline__ __nv_bfloat16 to_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <>
@@ -156,202 +140,311 @@ __device__ __forceinline__ uint4 pack8(const T (&v)[8])
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// MODE 0: NCC from the statistics planes; MODE 1: TAD from the raw images.
-// out is [H][W][ld] (T = float).
-// One row y and 128 pixels from x0, disparities [d_begin, d_end) (all: 0, D);
-// ends with a __syncthreads.  out_r (nullable, FP32 layout only): the right
-// view's volume, which holds the same costs at (x - d, y, d) (Sec. II-A, Sec. III).
-template <int MODE, typename T>
-__device__ __forceinline__ void cost_tile(const int16_t* __restrict__ gplane, const int* __restrict__ splane,
-                                          const float* __restrict__ rvplane, const uint8_t* __restrict__ L,
-                                          const uint8_t* __restrict__ R, int H, int W, int C, int D, int ld, float tau,
-                                          T* __restrict__ out, int x0, int y, int* smem_i, int d_begin, int d_end,
-                                          float* __restrict__ out_r = nullptr)
+// Index of column c in a staged row of 16-byte entries: lanes 4 columns apart
+// read 16 bytes each without conflicts.
+__host__ __device__ inline int skew4(int c) { return c + (c >> 2); }
+
+// The block sums of two output rows y, y + 1 for 4 pixels: lw, rw are 6 columns of
+// the two windows, each the grey rows y-1 .. y+2.  With p_j the products of a
+// column's rows, its sums are p_0 + t and t + p_3, t = p_1 + p_2.
+__device__ __forceinline__ void block_sums(const float4 (&lw)[6], const float4 (&rw)[6], uint64_t (&P)[4])
 {
-    const int tid = threadIdx.x;
-    const int nxs = min(kXS, W - x0);
+    uint64_t cs[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const float t = fmaf(lw[j].y, rw[j].y, lw[j].z * rw[j].z);
+        cs[j] = f2_pack(fmaf(lw[j].x, rw[j].x, t), fmaf(lw[j].w, rw[j].w, t));
+    }
+    const uint64_t a0 = f2_add(cs[0], cs[1]), a1 = f2_add(cs[2], cs[3]), a2 = f2_add(cs[4], cs[5]);
+    P[0] = f2_add(a0, cs[2]);
+    P[1] = f2_add(cs[1], a1);
+    P[2] = f2_add(a1, cs[4]);
+    P[3] = f2_add(cs[3], a2);
+}
+
+// The costs C = 1 - c of two rows from -9 P' (minus9p), S' and rv of both blocks:
+// S_l' S_r' - 9 P' rounded once, times the rounded product of the normalisers,
+// plus 1 (every cost kernel uses this, so the FP32 and the 16-bit volumes hold
+// the same values before the 16-bit rounding).
+__device__ __forceinline__ uint64_t ncc_cost2(uint64_t minus9p, uint64_t sl, uint64_t sr, uint64_t rl, uint64_t rr,
+                                              uint64_t one2)
+{
+    return f2_fma(f2_fma(sl, sr, minus9p), f2_mul(rl, rr), one2);
+}
+
+// ---- FP32 volume [H][W][ld], D innermost ------------------------------------------
+// A CTA (4 warps) covers 64 pixels x 4 rows of one view and disparities
+// [d_begin, d_end), up to 128 at a time; a warp takes 16 of them, a lane 4
+// pixels x 2 rows (lanes 0-15: rows y0, y0+1; 16-31: the next two).  The window of
+// the view's own image (6 columns x 4 grey rows) stays in registers, the other
+// image's slides one column (2 shared loads) per disparity; NCC as above, TAD from
+// the packed pixels.  Costs are transposed through the warp's buffer ([row][pixel]
+// [8 d], entry XOR pixel / 4, conflict-free) and leave as 32-byte runs per pixel.
+// MIRROR computes the right view: its own image is the right one, and the other
+// window slides the other way (Sec. II-A, Sec. III); the two products and sums
+// commute, so cost_r(x, y, d) = cost(x + d, y, d) bit for bit.
+// VW: floats per store -- 4 (ld % 4 == 0, 16-byte aligned), 2 (ld even, 8-byte
+// aligned) or 1.
+// Bound: the load/store pipe (88% busy at 1280x960, D = 128: half of it shared-
+// memory traffic of the windows and the transposition, half the scattered
+// 32-byte runs).  Measured on GB300 with the pre-pass, before -> now (before:
+// integer products, one row x 128 pixels per CTA, stores after a block-wide
+// transposition): 640x480, D = 64: 50 -> 34 us; 1280x960, D = 128: 293 -> 177 us;
+// 1920x1080, D = 256: 906 -> 554 us; NCC 767x575, D = 93: 108 -> 61 us.
+constexpr int kCostPx = 64, kCostRows = 4, kCostWarps = 4, kCostThreads = 32 * kCostWarps;
+constexpr int kCostPass = 128;                               // disparities per pass
+constexpr int kCostLeft = 82;                                // >= skew4(66)
+constexpr int kCostRight = (kCostPass + 68) * 5 / 4 + 2;     // >= skew4(16 ng + 68)
+constexpr int kCostBuf = kCostRows * kCostPx * 8 * 4;        // bytes of a warp's buffer
+constexpr size_t kCostSmem = (size_t)kCostWarps * kCostBuf + (size_t)4 * 16 * (kCostLeft + kCostRight);
+
+struct CostArgs {
+    CostScratch sc;                 // NCC: statistics of both images
+    const uint8_t *left, *right;    // TAD
+    int H, W, C, D, ld;
+    float tau;
+    float* out;
+};
+
+template <int MODE, bool MIRROR, int VW>
+__device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int d_begin, int d_end, void* smem)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int H = a.H, W = a.W, D = a.D;
+    uint8_t* const buf = (uint8_t*)smem + warp * kCostBuf;
+    float4* const gl = (float4*)((uint8_t*)smem + kCostWarps * kCostBuf);   // [2][kCostLeft]: columns x0 - 1 ..
+    float4* const sl = gl + 2 * kCostLeft;    // [2][kCostLeft]: centres x0 ..
+    float4* const gr = sl + 2 * kCostLeft;    // [2][kCostRight]: columns rb ..
+    float4* const sr = gr + 2 * kCostRight;   // [2][kCostRight]: centres rb ..
     const size_t plane = (size_t)H * W;
-    // layout: stage [kDC][kStage] float | left grey [3][kXS+2] | right grey [3][kXS+kDC+2] |
-    //         S_l, rv_l [kXS] | S_r, rv_r [kXS+kDC]
-    float* stage = (float*)smem_i;
-    int* gl = (int*)(stage + kDC * kStage);
-    int* gr = gl + 3 * (kXS + 2);      // [3][4 * kQR], column c at rpos(c)
-    int* sl = gr + 3 * 4 * kQR;
-    float* rl = (float*)(sl + kXS);
-    int* sr = (int*)(rl + kXS);
-    float* rr = (float*)(sr + kXS + kDC);
-    uchar4* pl = (uchar4*)gl;          // TAD: raw left row [kXS]
-    uchar4* pr = pl + kXS;             // TAD: raw right row [kXS + kDC]
+    const size_t own = MIRROR ? plane : 0, other = MIRROR ? 0 : plane;
+    const uint8_t* const own_img = MIRROR ? a.right : a.left;
+    const uint8_t* const other_img = MIRROR ? a.left : a.right;
 
-    const int run = tid & 31;          // pixels 4*run .. 4*run+3 of the CTA
-    const int dg = tid >> 5;           // disparities dc + 8*dg .. +7
-    const int xl0 = 4 * run;
-
-    if (MODE == 0) {
-        // left grey window rows y-1..y+1, virtual columns x0-1 .. x0+kXS
-        for (int i = tid; i < 3 * (kXS + 2); i += kThreads) {
-            const int j = i / (kXS + 2), c = i - j * (kXS + 2);
-            gl[i] = gplane[(size_t)clampi(y - 1 + j, 0, H - 1) * W + clampi(x0 - 1 + c, 0, W - 1)];
+    // one column of an image: grey rows y0-1 .. y0+4 and the statistics of rows
+    // y0 .. y0+3 (NCC), or the packed pixels of rows y0 .. y0+3 (TAD, in gl / gr)
+    auto stage = [&](size_t img, const uint8_t* src, int x, float4* g0, float4* g1, float4* s0, float4* s1) {
+        x = clampi(x, 0, W - 1);
+        if (MODE == 0) {
+            float g[6], s[4], v[4];
+#pragma unroll
+            for (int j = 0; j < 6; ++j) g[j] = (float)a.sc.g[img + (uint32_t)(clampi(y0 - 1 + j, 0, H - 1) * W + x)];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const size_t o = img + (uint32_t)(min(y0 + j, H - 1) * W + x);
+                s[j] = a.sc.s[o];
+                v[j] = a.sc.rv[o];
+            }
+            *g0 = make_float4(g[0], g[1], g[2], g[3]);
+            *g1 = make_float4(g[2], g[3], g[4], g[5]);
+            if (s0) {
+                *s0 = make_float4(s[0], s[1], v[0], v[1]);
+                *s1 = make_float4(s[2], s[3], v[2], v[3]);
+            }
+        } else {
+            uint32_t c[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint8_t* q = src + ((size_t)min(y0 + j, H - 1) * W + x) * a.C;
+                c[j] = a.C == 3 ? (uint32_t)q[0] | ((uint32_t)q[1] << 8) | ((uint32_t)q[2] << 16) : (uint32_t)q[0];
+            }
+            *g0 = make_float4(__uint_as_float(c[0]), __uint_as_float(c[1]), 0.f, 0.f);
+            *g1 = make_float4(__uint_as_float(c[2]), __uint_as_float(c[3]), 0.f, 0.f);
         }
-        for (int i = tid; i < kXS; i += kThreads) {
-            const int x = clampi(x0 + i, 0, W - 1);
-            sl[i] = splane[(size_t)y * W + x];
-            rl[i] = rvplane[(size_t)y * W + x];
-        }
-    } else {
-        for (int i = tid; i < kXS; i += kThreads) {
-            const uint8_t* p = L + ((size_t)y * W + clampi(x0 + i, 0, W - 1)) * C;
-            pl[i] = C == 3 ? make_uchar4(p[0], p[1], p[2], 0) : make_uchar4(p[0], 0, 0, 0);
-        }
+    };
+    for (int c = tid; c < kCostPx + 2; c += kCostThreads) {
+        // centre x0 + c - 1 sits at column c of gl and entry c - 1 of sl
+        const bool centre = c >= 1 && c <= kCostPx;
+        float4* s0 = sl + skew4(centre ? c - 1 : 0);
+        stage(own, own_img, x0 - 1 + c, gl + skew4(c), gl + kCostLeft + skew4(c), centre ? s0 : nullptr, s0 + kCostLeft);
     }
 
-    for (int dc = d_begin; dc < d_end; dc += kDC) {
-        // right columns for this pass: virtual columns rb .. rb + NRG - 1 with
-        // rb = x0 - dc - kDC - 1; the right block of (x, d) spans x-d-1 .. x-d+1
-        const int rb = x0 - dc - kDC - 1;
-        if (MODE == 0) {
-            for (int i = tid; i < 3 * kNRG; i += kThreads) {
-                const int j = i / kNRG, c = i - j * kNRG;
-                gr[j * 4 * kQR + rpos(c)] =
-                    gplane[plane + (size_t)clampi(y - 1 + j, 0, H - 1) * W + clampi(rb + c, 0, W - 1)];
-            }
-            // right block centres rb+1 .. rb+kXS+kDC
-            for (int i = tid; i < kXS + kDC; i += kThreads) {
-                const int x = clampi(rb + 1 + i, 0, W - 1);
-                sr[spos(i)] = splane[plane + (size_t)y * W + x];
-                rr[spos(i)] = rvplane[plane + (size_t)y * W + x];
-            }
-        } else {
-            for (int i = tid; i < kXS + kDC; i += kThreads) {
-                const uint8_t* p = R + ((size_t)y * W + clampi(rb + 1 + i, 0, W - 1)) * C;
-                pr[i] = C == 3 ? make_uchar4(p[0], p[1], p[2], 0) : make_uchar4(p[0], 0, 0, 0);
-            }
-        }
-        __syncthreads();
+    const int p = lane & 15, rp = lane >> 4;
+    const int xl = 4 * p, xbase = x0 + xl;
+    const float inv_c = 1.f / (float)a.C;
+    const uint64_t one2 = f2_pack(1.f, 1.f);
+    auto at = [](int m) { return m + (m >> 2); };   // offset of column base + m (base a multiple of 4)
+    // entry (i, e) of 8 bytes: pixel 4 p + i, disparities 2 e, 2 e + 1 of 8, at 8 * ((4 i + e) ^ p)
+    const uint32_t put0 = tc::smem_u32(buf) + 2 * rp * (kCostPx * 32) + 128 * p + 8 * p;
 
-        const int d_first = dc + 8 * dg;
-        if (MODE == 0) {
-            int glw[3][6];
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-#pragma unroll
-                for (int c = 0; c < 6; ++c) glw[j][c] = gl[j * (kXS + 2) + xl0 + c];
-            int sli[4];
-            float rli[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                sli[i] = sl[xl0 + i];
-                rli[i] = rl[xl0 + i];
-            }
-            // right window for d_first: virtual columns x0+xl0-d-1 .. +4, index (col - rb)
-            int grw[3][6];
-            int srw[4];
-            float rrw[4];
-            {
-                const int base = x0 + xl0 - d_first - 1 - rb;
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) grw[j][c] = gr[j * 4 * kQR + rpos(base + c)];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    srw[i] = sr[spos(base + i)];
-                    rrw[i] = rr[spos(base + i)];
-                }
-            }
-#pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                const int d = d_first + s;
-                if (s > 0) {
-                    // slide one column to the left: d grew by one
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-#pragma unroll
-                        for (int c = 5; c > 0; --c) grw[j][c] = grw[j][c - 1];
-                    }
-                    const int base = x0 + xl0 - d - 1 - rb;
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) grw[j][0] = gr[j * 4 * kQR + rpos(base)];
-#pragma unroll
-                    for (int i = 3; i > 0; --i) {
-                        srw[i] = srw[i - 1];
-                        rrw[i] = rrw[i - 1];
-                    }
-                    srw[0] = sr[spos(base)];
-                    rrw[0] = rr[spos(base)];
-                }
-                int cp[6];
-#pragma unroll
-                for (int c = 0; c < 6; ++c) cp[c] = glw[0][c] * grw[0][c] + glw[1][c] * grw[1][c] + glw[2][c] * grw[2][c];
-                float* st = stage + (d - dc) * kStage + run;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int x = x0 + xl0 + i;
-                    const int num = 9 * (cp[i] + cp[i + 1] + cp[i + 2]) - sli[i] * srw[i];
-                    st[32 * i] = x - d < 0 ? 2.f : ncc_cost(num, rli[i], rrw[i]);
-                }
-            }
-        } else {
-            const float inv_c = 1.f / (float)C;
-#pragma unroll 2
-            for (int s = 0; s < 8; ++s) {
-                const int d = d_first + s;
-                float* st = stage + (d - dc) * kStage + run;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int x = x0 + xl0 + i;
-                    float cst = tau;
-                    if (x - d >= 0) {
-                        const uchar4 a = pl[xl0 + i];
-                        const uchar4 b = pr[x - d - (rb + 1)];
-                        const int sad = abs((int)a.x - (int)b.x) + abs((int)a.y - (int)b.y) + abs((int)a.z - (int)b.z);
-                        cst = fminf((float)sad * inv_c, tau);
-                    }
-                    st[32 * i] = cst;
-                }
-            }
-        }
+    for (int dp = d_begin; dp < d_end; dp += kCostPass) {
+        const int ng = min(kCostPass / 16, (d_end - dp + 15) / 16);
+        // other image's columns of this pass, from rb on; column x -+ d + k of
+        // disparity dp + 16 g + s is base + m with base = xl + (MIRROR ? 4 + 16 g : 16 (ng - g)),
+        // m = i + k -+ s
+        const int rb = MIRROR ? x0 + dp - 4 : x0 - dp - 16 * ng;
+        const int nr = 16 * ng + (MIRROR ? 68 : 65);
+        for (int c = tid; c < nr; c += kCostThreads)
+            stage(other, other_img, rb + c, gr + skew4(c), gr + kCostRight + skew4(c), sr + skew4(c),
+                  sr + kCostRight + skew4(c));
         __syncthreads();
+        for (int grp = warp; grp < ng; grp += kCostWarps) {
+            const int d0 = dp + 16 * grp;
+            const int base = xl + (MIRROR ? 4 + 16 * grp : 16 * (ng - grp));
+            const float4* glw = gl + rp * kCostLeft + skew4(xl);
+            const float4* slw = sl + rp * kCostLeft + skew4(xl);
+            const float4* grw = gr + rp * kCostRight + skew4(base);
+            const float4* srw = sr + rp * kCostRight + skew4(base);
+            constexpr int ST = MIRROR ? 1 : -1;     // columns the window moves per disparity
+            constexpr int IN = MIRROR ? 5 : 0;      // where the new column comes in
 
-        const int nd = min(kDC, d_end - dc);
-        // out[(y*W + x)*ld + d]; padding d in [D, ld) of the last pass written as 0
-        const int ndw = (dc + kDC >= d_end) ? (d_end == D ? ld - dc : d_end - dc) : kDC;
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int x = warp; x < nxs; x += kThreads / 32) {
-            T* o = out + ((size_t)y * W + x0 + x) * ld + dc;
-            const int px = stage_pos(x);
-            for (int dd = lane; dd < ndw; dd += 32) o[dd] = to_out<T>(dd < nd ? stage[dd * kStage + px] : 0.f);
-        }
-        if (out_r != nullptr) {
-            // right pixel xr = x - d receives the contiguous disparities
-            // max(dc, x0 - xr) .. min(dc + nd - 1, x0 + nxs - 1 - xr) of this pass
-            const int xr_lo = max(0, x0 - dc - nd + 1), xr_hi = x0 + nxs - 1 - dc;
-            for (int xr = xr_lo + warp; xr <= xr_hi; xr += kThreads / 32) {
-                const int dlo = max(dc, x0 - xr), dhi = min(dc + nd - 1, x0 + nxs - 1 - xr);
-                float* o = out_r + ((size_t)y * W + xr) * ld;
-                for (int d = dlo + lane; d <= dhi; d += 32) o[d] = stage[(d - dc) * kStage + stage_pos(xr + d - x0)];
+            // writes 8 disparities from d8 on out of the warp's buffer
+            auto flush = [&](int d8) {
+                __syncwarp();
+                constexpr int L = 8 / VW, PXI = 32 / L;      // lanes per pixel, pixels per store
+                const int e = lane % L, d = d8 + VW * e;
+                const bool din = VW == 4 ? d < a.ld && d < ((d_end + 3) & ~3) : d < min(D, d_end);
+#pragma unroll
+                for (int r = 0; r < kCostRows; ++r) {
+                    if (y0 + r >= H) break;
+                    float* o = a.out + ((size_t)(y0 + r) * W + x0 + lane / L) * a.ld + d;
+#pragma unroll 4
+                    for (int j = 0; j < kCostPx / PXI; ++j, o += (size_t)PXI * a.ld) {
+                        const int px = PXI * j + lane / L, pp = px >> 2, c = 4 * (px & 3) + e * VW / 2;
+                        const uint8_t* q = buf + r * (kCostPx * 32) + 128 * pp;
+                        if (x0 + px >= W || !din) continue;
+                        if (VW == 4) {
+                            const float4 v = *(const float4*)(q + 8 * ((c ^ pp) & ~1));
+                            *(float4*)o = pp & 1 ? make_float4(v.z, v.w, v.x, v.y) : v;
+                        } else if (VW == 2) {
+                            *(float2*)o = *(const float2*)(q + 8 * (c ^ pp));
+                        } else {
+                            *o = *(const float*)(q + 8 * (c ^ pp) + 4 * (e & 1));
+                        }
+                    }
+                }
+                __syncwarp();
+            };
+            auto put = [&](int s, const float (&c)[4][2][2]) {   // c[pixel][row][s even, odd]
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"((put0 ^ (8 * (4 * i + ((s >> 1) & 3)))) +
+                                                                              h * (kCostPx * 32)),
+                                     "f"(c[i][h][0]), "f"(c[i][h][1])
+                                     : "memory");
+            };
+            // outside the image or no match there: the maximum; d >= D: 0
+            auto mask = [&](float v, int i, int d, float most) {
+                const int x = xbase + i;
+                return d >= D ? 0.f : (MIRROR ? x + d >= W : x - d < 0) ? most : v;
+            };
+
+            if (MODE == 0) {
+                float4 lw[6], rw[6];
+                uint64_t sli[4], rli[4], sri[4], rri[4];
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    // -9 g': the block sums come out as -9 P' (exact: products below 2^24 / 9)
+                    const float4 v = glw[at(j)];
+                    lw[j] = make_float4(-9.f * v.x, -9.f * v.y, -9.f * v.z, -9.f * v.w);
+                    rw[j] = grw[at(j - 1)];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = slw[i], w = srw[at(i)];
+                    sli[i] = f2_pack(v.x, v.y);
+                    rli[i] = f2_pack(v.z, v.w);
+                    sri[i] = f2_pack(w.x, w.y);
+                    rri[i] = f2_pack(w.z, w.w);
+                }
+                auto sweep = [&](auto masked) {
+                    float c[4][2][2];
+#pragma unroll
+                    for (int s = 0; s < 16; ++s) {
+                        if (s > 0) {
+#pragma unroll
+                            for (int j = 0; j < 5; ++j) {
+                                if (MIRROR) rw[j] = rw[j + 1];
+                                else rw[5 - j] = rw[4 - j];
+                            }
+                            rw[IN] = grw[at(MIRROR ? 4 + s : -1 - s)];
+#pragma unroll
+                            for (int i = 0; i < 3; ++i) {
+                                if (MIRROR) sri[i] = sri[i + 1], rri[i] = rri[i + 1];
+                                else sri[3 - i] = sri[2 - i], rri[3 - i] = rri[2 - i];
+                            }
+                            const float4 v = srw[at(MIRROR ? 3 + s : -s)];
+                            sri[MIRROR ? 3 : 0] = f2_pack(v.x, v.y);
+                            rri[MIRROR ? 3 : 0] = f2_pack(v.z, v.w);
+                        }
+                        uint64_t P[4];
+                        block_sums(lw, rw, P);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float v0, v1;
+                            f2_unpack(ncc_cost2(P[i], sli[i], sri[i], rli[i], rri[i], one2), v0, v1);
+                            c[i][0][s & 1] = decltype(masked)::value ? mask(v0, i, d0 + s, 2.f) : v0;
+                            c[i][1][s & 1] = decltype(masked)::value ? mask(v1, i, d0 + s, 2.f) : v1;
+                        }
+                        if (s & 1) put(s, c);
+                        if ((s & 7) == 7) flush(d0 + s - 7);
+                    }
+                };
+                const bool inside = d0 + 16 <= D && (MIRROR ? xbase + 3 + d0 + 15 < W : xbase >= d0 + 15);
+                if (__all_sync(0xffffffffu, inside)) sweep(std::integral_constant<bool, false>{});
+                else sweep(std::integral_constant<bool, true>{});
+            } else {
+                uint32_t pl[4][2], pr[4][2];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = glw[at(i + 1)], w = grw[at(i)];
+                    pl[i][0] = __float_as_uint(v.x), pl[i][1] = __float_as_uint(v.y);
+                    pr[i][0] = __float_as_uint(w.x), pr[i][1] = __float_as_uint(w.y);
+                }
+                float c[4][2][2];
+#pragma unroll
+                for (int s = 0; s < 16; ++s) {
+                    if (s > 0) {
+#pragma unroll
+                        for (int i = 0; i < 3; ++i)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                if (MIRROR) pr[i][h] = pr[i + 1][h];
+                                else pr[3 - i][h] = pr[2 - i][h];
+                            }
+                        const float4 w = grw[at(MIRROR ? 3 + s : -s)];
+                        pr[MIRROR ? 3 : 0][0] = __float_as_uint(w.x);
+                        pr[MIRROR ? 3 : 0][1] = __float_as_uint(w.y);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int sad = (int)__dp4a(__vabsdiffu4(pl[i][h], pr[i][h]), 0x01010101u, 0u);
+                            c[i][h][s & 1] = mask(fminf((float)sad * inv_c, a.tau), i, d0 + s, a.tau);
+                        }
+                    if (s & 1) put(s, c);
+                    if ((s & 7) == 7) flush(d0 + s - 7);
+                }
             }
+            (void)ST;
         }
-        __syncthreads();
+        __syncthreads();   // the staged columns may be overwritten
     }
 }
 
-template <int MODE, typename T>
-__global__ void __launch_bounds__(kThreads)
-cost_kernel(const int16_t* __restrict__ gplane, const int* __restrict__ splane, const float* __restrict__ rvplane,
-            const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C, int D, int ld,
-            float tau, T* __restrict__ out)
+template <int MODE, bool MIRROR, int VW>
+__global__ void __launch_bounds__(kCostThreads, 4) cost_kernel(const CostArgs a)
 {
-    extern __shared__ int smem_i[];
-    cost_tile<MODE, T>(gplane, splane, rvplane, L, R, H, W, C, D, ld, tau, out, blockIdx.x * kXS, blockIdx.y,
-                               smem_i, 0, D);
+    extern __shared__ __align__(128) float4 sm_cost[];
+    // the aggregation's set-up may start; the statistics must have been written
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    cost_tile<MODE, MIRROR, VW>(a, blockIdx.x * kCostPx, blockIdx.y * kCostRows, 0, a.D, sm_cost);
 }
 
-// Batched FP32 cost volumes [H][W][ld]: an item is (row, 128-pixel segment) of a pair.
-__global__ void __launch_bounds__(kThreads)
+__device__ __forceinline__ CostArgs pair_args(const BatchPair& bp)
+{
+    return CostArgs{bp.sc, bp.left, bp.right, bp.H, bp.W, bp.C, bp.D, bp.ld, bp.tau, bp.cost};
+}
+
+// Batched FP32 cost volumes [H][W][ld]: an item is one 64 x 4 tile of a pair.
+__global__ void __launch_bounds__(kCostThreads, 4)
 cost_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems, int* __restrict__ counter)
 {
-    extern __shared__ int smem_i[];
+    extern __shared__ __align__(128) float4 sm_cost[];
     __shared__ int item_s;
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
@@ -361,42 +454,39 @@ cost_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems,
         if (item >= nitems) break;
         const BatchPair& bp = pairs[find_pair(pairs, npairs, item, &BatchPair::cost_off)];
         const int t = item - bp.cost_off;
-        const int nseg = (bp.W + kXS - 1) / kXS;
-        const int x0 = (t % nseg) * kXS, y = t / nseg;
-        if (bp.mode == 0)
-            cost_tile<0, float>(bp.sc.g, bp.sc.s, bp.sc.rv, bp.left, bp.right, bp.H, bp.W, bp.C, bp.D, bp.ld,
-                                       bp.tau, bp.cost, x0, y, smem_i, 0, bp.D);
-        else
-            cost_tile<1, float>(bp.sc.g, bp.sc.s, bp.sc.rv, bp.left, bp.right, bp.H, bp.W, bp.C, bp.D, bp.ld,
-                                       bp.tau, bp.cost, x0, y, smem_i, 0, bp.D);
+        const int nseg = (bp.W + kCostPx - 1) / kCostPx;
+        const CostArgs a = pair_args(bp);
+        const int x0 = (t % nseg) * kCostPx, y0 = (t / nseg) * kCostRows;
+        if (bp.mode == 0) cost_tile<0, false, 4>(a, x0, y0, 0, bp.D, sm_cost);
+        else cost_tile<1, false, 4>(a, x0, y0, 0, bp.D, sm_cost);
     }
 }
 
-// Band form: NCC costs of row y, pixels x0 .. x0+127, for the disparities
-// that some aggregation tile reading this segment needs: the hull of the
-// ranges [d_begin, d_end) of every tile whose window halo (the tile grown by
-// rho) overlaps the segment.  Entries outside that hull are not written.
-__global__ void __launch_bounds__(kThreads)
-cost_band_kernel(const int16_t* __restrict__ gplane, const int* __restrict__ splane,
-                 const float* __restrict__ rvplane, int H, int W, int D, int ld, int rho,
-                 const int2* __restrict__ tile_range, int ntx, int nty, float* __restrict__ out)
+// Band form: NCC costs of a 64 x 4 tile for the disparities that some aggregation
+// tile reading it needs: the hull of the ranges [d_begin, d_end) of every
+// aggregation tile whose window halo (the tile grown by rho) overlaps it.
+// Entries outside that hull are not written (but for the rest of a run of 4).
+__global__ void __launch_bounds__(kCostThreads, 4)
+cost_band_kernel(const CostArgs a, int rho, const int2* __restrict__ tile_range, int ntx, int nty)
 {
-    extern __shared__ int smem_i[];
+    extern __shared__ __align__(128) float4 sm_cost[];
     __shared__ int lo_s, hi_s;
-    const int x0 = blockIdx.x * kXS, y = blockIdx.y;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int x0 = blockIdx.x * kCostPx, y0 = blockIdx.y * kCostRows;
     if (threadIdx.x == 0) {
-        lo_s = D;
+        lo_s = a.D;
         hi_s = 0;
     }
     __syncthreads();
-    // tiles ty with 4ty - rho <= y <= 4ty + 3 + rho, tx with halo columns meeting [x0, x0 + 127]
-    const int ty0 = max(0, (y - rho + kAggTileY * 64) / kAggTileY - 64);
-    const int ty1 = min(nty - 1, (y + rho) / kAggTileY);
+    // aggregation tiles ty with 4 ty - rho <= y0 + 3 and y0 <= 4 ty + 3 + rho, tx likewise
+    const int ty0 = max(0, (y0 - rho + kAggTileY * 64) / kAggTileY - 64);
+    const int ty1 = min(nty - 1, (y0 + kCostRows - 1 + rho) / kAggTileY);
     const int tx0 = max(0, (x0 - rho + kAggTileX * 64) / kAggTileX - 64);
-    const int tx1 = min(ntx - 1, (x0 + kXS - 1 + rho) / kAggTileX);
+    const int tx1 = min(ntx - 1, (x0 + kCostPx - 1 + rho) / kAggTileX);
     const int nx = tx1 - tx0 + 1;
-    int lo = D, hi = 0;
-    for (int i = threadIdx.x; i < (ty1 - ty0 + 1) * nx; i += kThreads) {
+    int lo = a.D, hi = 0;
+    for (int i = threadIdx.x; i < (ty1 - ty0 + 1) * nx; i += kCostThreads) {
         const int2 r = tile_range[(size_t)(ty0 + i / nx) * ntx + tx0 + i % nx];
         lo = min(lo, r.x);
         hi = max(hi, r.y);
@@ -408,35 +498,7 @@ cost_band_kernel(const int16_t* __restrict__ gplane, const int* __restrict__ spl
     __syncthreads();
     const int d_begin = lo_s, d_end = hi_s;
     if (d_begin >= d_end) return;
-    cost_tile<0, float>(gplane, splane, rvplane, nullptr, nullptr, H, W, 1, D, ld, 0.f, out, x0, y, smem_i,
-                               d_begin, d_end);
-}
-
-// Both views at once (FP32 layouts): the left volume as cost_kernel writes it
-// and the right volume from the same staged costs.
-template <int MODE>
-__global__ void __launch_bounds__(kThreads)
-cost_lr_kernel(const int16_t* __restrict__ gplane, const int* __restrict__ splane, const float* __restrict__ rvplane,
-               const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W, int C, int D, int ld,
-               float tau, float* __restrict__ out, float* __restrict__ out_r)
-{
-    extern __shared__ int smem_i[];
-    cost_tile<MODE, float>(gplane, splane, rvplane, L, R, H, W, C, D, ld, tau, out, blockIdx.x * kXS, blockIdx.y,
-                                  smem_i, 0, D, out_r);
-}
-
-// Right volume entries with no left pixel (xr + d >= W): the maximum cost;
-// d in [D, ld) padding: 0.
-__global__ void right_edge_fill_kernel(int H, int W, int D, int ld, float maxc, float* __restrict__ out_r)
-{
-    const int y = blockIdx.x;
-    const int x_first = max(0, W - D);
-    const int n = (W - x_first) * ld;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int xr = x_first + i / ld, d = i % ld;
-        if (d >= D) out_r[((size_t)y * W + xr) * ld + d] = 0.f;
-        else if (xr + d >= W) out_r[((size_t)y * W + xr) * ld + d] = maxc;
-    }
+    cost_tile<0, false, 4>(a, x0, y0, d_begin, d_end, sm_cost);
 }
 
 // ---- TAD, 16-bit x-blocked volume: one thread per (block of 8 columns, 8 disparities)
@@ -608,14 +670,10 @@ cost_xb_tad_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R,
 
 // ---- NCC, 16-bit x-blocked volume ----------------------------------------------
 // A CTA covers 64 pixels x 4 rows and every disparity.  All of Eq. (1) runs in
-// FP32 on exact integers: with the grey values moved by a constant a
-// (which changes neither 9 P - S_l S_r nor the variances) |g - a| <= 383, so
-// every product, block sum, 9 P' and S_l' S_r' is an integer below 2^24, and
-// 9 P' - S_l' S_r' comes out of one FMA rounded once -- the integer converted to
-// float.  A thread computes two output rows y, y + 1 at once: with p_j the
-// products of grey rows y-1 .. y+2, the column sums are p_0 + t and t + p_3,
-// t = p_1 + p_2 (4 FMAs for two sums), and everything after them is packed, one
-// row per half.
+// FP32 on exact integers (grey_shift), and 9 P' - S_l' S_r' comes out of one FMA
+// rounded once -- the integer converted to float.  A thread computes two output
+// rows at once (block_sums: 4 FMAs for a column's two sums), and everything
+// after them is packed, one row per half.
 //   * Staging: per column and pair of output rows a float4 of the four grey rows
 //     y-1 .. y+2, then per block centre a float4 (S(y), S(y+1), 1/sqrt V(y),
 //     1/sqrt V(y+1)).  Index c + c/4: lanes 4 columns apart read 16 bytes each
@@ -643,7 +701,6 @@ constexpr int kNccPx = 64;
 constexpr int kNccWarps = 4;
 constexpr int kNccRows = 4;      // two pairs
 
-__host__ __device__ inline int skew4(int c) { return c + (c >> 2); }
 __host__ __device__ inline int ncc_groups(int D) { return (D + 15) / 16; }          // of 16 disparities
 __host__ __device__ inline int ncc_right_cols(int D) { return 16 * ncc_groups(D) + kNccPx + 1; }
 // float4 entries of the four staged arrays, per pair of rows
@@ -681,7 +738,7 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
 
     // ---- grey rows y0-1 .. y0+ROWS of both images at clamped columns, and the
     // left image's packed guide
-    const int shift = C == 3 ? 382 : 128;
+    const int shift = grey_shift(C);
     for (int e = tid; e < kNccPx + 2 + nr; e += nthr) {
         const bool left = e < kNccPx + 2;
         const int c = left ? e : e - (kNccPx + 2);
@@ -833,20 +890,12 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
                     sri[0] = f2_pack(v.x, v.y);
                     rri[0] = f2_pack(v.z, v.w);
                 }
-                uint64_t cs[6];
-#pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    const float t = fmaf(lw[j].y, rw[j].y, lw[j].z * rw[j].z);
-                    cs[j] = f2_pack(fmaf(lw[j].x, rw[j].x, t), fmaf(lw[j].w, rw[j].w, t));
-                }
-                const uint64_t a0 = f2_add(cs[0], cs[1]), a1 = f2_add(cs[2], cs[3]), a2 = f2_add(cs[4], cs[5]);
-                const uint64_t P[4] = {f2_add(a0, cs[2]), f2_add(cs[1], a1), f2_add(a1, cs[4]), f2_add(cs[3], a2)};
+                uint64_t P[4];
+                block_sums(lw, rw, P);
                 float c0[4], c1[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    // S_l' S_r' - 9 P' rounded once, times the rounded product of the normalisers, plus 1
-                    const uint64_t nn = f2_fma(sli[i], sri[i], P[i]);
-                    f2_unpack(f2_fma(nn, f2_mul(rli[i], rri[i]), one2), c0[i], c1[i]);
+                    f2_unpack(ncc_cost2(P[i], sli[i], sri[i], rli[i], rri[i], one2), c0[i], c1[i]);
                     if (decltype(masked)::value) {
                         const int x = xbase + i;
                         if (x - d < 0) c0[i] = c1[i] = 2.f;
@@ -929,51 +978,54 @@ cudaError_t launch_cost_xb_tad(const CostScratch& sc, const uint8_t* left, const
     return cudaGetLastError();
 }
 
-size_t cost_smem_bytes()
+template <int MODE, bool MIRROR, int VW>
+cudaError_t launch_cost_vw(const CostArgs& a, cudaStream_t stream)
 {
-    return sizeof(float) * (size_t)kDC * kStage +
-           sizeof(int) * (size_t)(3 * (kXS + 2) + 3 * 4 * kQR + 2 * kXS + 2 * (kXS + kDC));
+    cudaError_t e = fbs::raise_smem_limit(cost_kernel<MODE, MIRROR, VW>, (int)kCostSmem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((a.W + kCostPx - 1) / kCostPx, (a.H + kCostRows - 1) / kCostRows);
+    if (MODE == 0 || MIRROR)   // behind the statistics or the other view
+        return fbs::launch_after(cost_kernel<MODE, MIRROR, VW>, grid, kCostThreads, kCostSmem, stream, a);
+    fbs::note_launch();
+    cost_kernel<MODE, MIRROR, VW><<<grid, kCostThreads, kCostSmem, stream>>>(a);
+    return cudaGetLastError();
 }
 
-template <int MODE, typename T>
-cudaError_t launch_cost_kernel(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                               int C, int D, int ld, float tau, T* out, cudaStream_t stream)
+// One view of the FP32 volume (mode 0: after the statistics).
+cudaError_t launch_cost_view(const CostArgs& a, int mode, bool mirror, cudaStream_t stream)
 {
-    const size_t smem = cost_smem_bytes();
-    cudaError_t e = fbs::raise_smem_limit(cost_kernel<MODE, T>, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((W + kXS - 1) / kXS, H);
-    fbs::note_launch();
-    cost_kernel<MODE, T><<<grid, kThreads, smem, stream>>>(sc.g, sc.s, sc.rv, left, right, H, W, C, D, ld,
-                                                                   tau, out);
-    return cudaGetLastError();
+    const uintptr_t o = reinterpret_cast<uintptr_t>(a.out);
+    if (a.ld % 4 == 0 && (o & 15) == 0) {
+        if (mirror) return mode == 0 ? launch_cost_vw<0, true, 4>(a, stream) : launch_cost_vw<1, true, 4>(a, stream);
+        return mode == 0 ? launch_cost_vw<0, false, 4>(a, stream) : launch_cost_vw<1, false, 4>(a, stream);
+    }
+    if (mirror) return cudaErrorInvalidValue;   // the context's own volume
+    if (a.ld % 2 == 0 && (o & 7) == 0)
+        return mode == 0 ? launch_cost_vw<0, false, 2>(a, stream) : launch_cost_vw<1, false, 2>(a, stream);
+    return mode == 0 ? launch_cost_vw<0, false, 1>(a, stream) : launch_cost_vw<1, false, 1>(a, stream);
 }
 
 cudaError_t launch_stats(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W, int C,
                          cudaStream_t stream)
 {
-    dim3 grid((W + 255) / 256, H, 2);
     fbs::note_launch();
-    grey_stats_kernel<<<grid, 256, 0, stream>>>(left, right, H, W, C, sc.g, sc.s, sc.rv, sc.rgbx);
+    grey_stats_kernel<<<dim3((W + kStatX - 1) / kStatX, (H + kStatY - 1) / kStatY, 2), kStatX, 0, stream>>>(left, right, H, W,
+                                                                                                        C, sc);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-int stats_items(int H, int W) { return H; }
-int cost_items(int H, int W) { return H * ((W + kXS - 1) / kXS); }
-size_t cost_kernel_smem() { return cost_smem_bytes(); }
+int stats_items(int H, int W) { return ((H + kStatY - 1) / kStatY) * ((W + kStatX - 1) / kStatX); }
+int cost_items(int H, int W) { return ((H + kCostRows - 1) / kCostRows) * ((W + kCostPx - 1) / kCostPx); }
 
-cudaError_t prepare_cost_batched()
-{
-    return fbs::raise_smem_limit(cost_batched_kernel, (int)cost_smem_bytes());
-}
+cudaError_t prepare_cost_batched() { return fbs::raise_smem_limit(cost_batched_kernel, (int)kCostSmem); }
 
 cudaError_t launch_stats_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
                                  cudaStream_t stream)
 {
     fbs::note_launch();
-    grey_stats_batched_kernel<<<grid, 256, 0, stream>>>(pairs, npairs, nitems, counter);
+    grey_stats_batched_kernel<<<grid, kStatX, 0, stream>>>(pairs, npairs, nitems, counter);
     return cudaGetLastError();
 }
 
@@ -981,7 +1033,7 @@ cudaError_t launch_cost_batched(const BatchPair* pairs, int npairs, int nitems, 
                                 cudaStream_t stream)
 {
     fbs::note_launch();
-    cost_batched_kernel<<<grid, kThreads, cost_smem_bytes(), stream>>>(pairs, npairs, nitems, counter);
+    cost_batched_kernel<<<grid, kCostThreads, kCostSmem, stream>>>(pairs, npairs, nitems, counter);
     return cudaGetLastError();
 }
 
@@ -1019,7 +1071,7 @@ CostScratch carve_cost_scratch(void* base, int H, int W)
     uint8_t* p = (uint8_t*)base;
     sc.g = (int16_t*)p;
     p += (n * sizeof(int16_t) + 255) & ~(size_t)255;
-    sc.s = (int*)p;
+    sc.s = (float*)p;
     p += (n * sizeof(int) + 255) & ~(size_t)255;
     sc.rv = (float*)p;
     return sc;
@@ -1028,57 +1080,30 @@ CostScratch carve_cost_scratch(void* base, int H, int W)
 cudaError_t launch_cost_build(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                               int C, int D, int ld, int mode, float tau, float* cost, cudaStream_t stream)
 {
-    if (mode == 0) {
-        cudaError_t e = launch_stats(sc, left, right, H, W, C, stream);
-        if (e != cudaSuccess) return e;
-        return launch_cost_kernel<0, float>(sc, left, right, H, W, C, D, ld, tau, cost, stream);
-    }
-    return launch_cost_kernel<1, float>(sc, left, right, H, W, C, D, ld, tau, cost, stream);
+    cudaError_t e = mode == 0 ? launch_stats(sc, left, right, H, W, C, stream) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost}, mode, false, stream);
 }
 
 cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                              int C, int D, int ld, int radius, const int2* tile_range, float* cost, cudaStream_t stream)
 {
     cudaError_t e = launch_stats(sc, left, right, H, W, C, stream);
-    if (e != cudaSuccess) return e;
-    const size_t smem = cost_smem_bytes();
-    e = fbs::raise_smem_limit(cost_band_kernel, (int)smem);
+    if (e == cudaSuccess) e = fbs::raise_smem_limit(cost_band_kernel, (int)kCostSmem);
     if (e != cudaSuccess) return e;
     const int ntx = (W + kAggTileX - 1) / kAggTileX, nty = (H + kAggTileY - 1) / kAggTileY;
-    dim3 grid((W + kXS - 1) / kXS, H);
-    fbs::note_launch();
-    cost_band_kernel<<<grid, kThreads, smem, stream>>>(sc.g, sc.s, sc.rv, H, W, D, ld, radius, tile_range, ntx, nty,
-                                                       cost);
-    return cudaGetLastError();
+    return fbs::launch_after(cost_band_kernel, dim3((W + kCostPx - 1) / kCostPx, (H + kCostRows - 1) / kCostRows), kCostThreads,
+                             kCostSmem, stream, CostArgs{sc, left, right, H, W, C, D, ld, 0.f, cost}, radius, tile_range, ntx,
+                             nty);
 }
 
 cudaError_t launch_cost_build_lr(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                                  int C, int D, int ld, int mode, float tau, float* cost, float* cost_r,
                                  cudaStream_t stream)
 {
-    cudaError_t e = cudaSuccess;
-    if (mode == 0) e = launch_stats(sc, left, right, H, W, C, stream);
+    cudaError_t e = launch_cost_build(sc, left, right, H, W, C, D, ld, mode, tau, cost, stream);
     if (e != cudaSuccess) return e;
-    const size_t smem = cost_smem_bytes();
-    dim3 grid((W + kXS - 1) / kXS, H);
-    if (mode == 0) {
-        e = fbs::raise_smem_limit(cost_lr_kernel<0>, (int)smem);
-        fbs::note_launch();
-        if (e == cudaSuccess)
-            cost_lr_kernel<0><<<grid, kThreads, smem, stream>>>(sc.g, sc.s, sc.rv, left, right, H, W, C, D, ld, tau,
-                                                                cost, cost_r);
-    } else {
-        e = fbs::raise_smem_limit(cost_lr_kernel<1>, (int)smem);
-        fbs::note_launch();
-        if (e == cudaSuccess)
-            cost_lr_kernel<1><<<grid, kThreads, smem, stream>>>(sc.g, sc.s, sc.rv, left, right, H, W, C, D, ld, tau,
-                                                                cost, cost_r);
-    }
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    fbs::note_launch();
-    right_edge_fill_kernel<<<H, 256, 0, stream>>>(H, W, D, ld, mode == 0 ? 2.f : tau, cost_r);
-    return cudaGetLastError();
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost_r}, mode, true, stream);
 }
 
 cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H,

@@ -24,18 +24,41 @@ inline cudaError_t raise_smem_limit(K* kernel, size_t bytes)
     return raise_smem_limit((const void*)kernel, bytes);
 }
 
+// A kernel launched programmatically behind the previous kernel of the stream: its
+// CTAs may start once every CTA of that one has started and signalled, and it
+// waits (griddepcontrol.wait) before it touches anything an earlier kernel writes.
+// Only for kernels whose predecessor in the stream is the library's own.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
+                                const Args&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launch();
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 // Cost volume rows are padded to a multiple of 4 floats so that one pixel's
 // disparity vector starts on a 16-byte boundary (vector loads, TMA, cp.async).
 inline int padded_ld(int D) { return (D + 3) & ~3; }
 
 // ---- step 1: matching cost, Eq. (1)-(3) or TAD -------------------------------
-// Per-pixel statistics of both images (grey value, 3x3 block sum, 1/sqrt of
-// the block variance times n^2), computed by a pre-pass and read by the FP32
+// Per-pixel statistics of both images (shifted grey value, its 3x3 block sum,
+// 1/sqrt of the block variance times n^2), computed by a pre-pass and read by the FP32
 // layout's cost kernels (the 16-bit x-blocked cost kernel computes them in
 // shared memory and uses only rgbx).  Both images: 2*H*W entries each.
 struct CostScratch {
     int16_t* g;
-    int* s;
+    float* s;
     float* rv;
     uint2* rgbx;      // optional: left image as (R | G << 8 | B << 16, R^2 + G^2 + B^2), pitch rgbx_pitch(W)
 };
@@ -76,10 +99,12 @@ constexpr int kAggTileX = 32;
 constexpr int kAggTileY = 4;
 // agg_out (nullable) is written with row pitch D (caller layout [H][W][D]).
 // err: device int set to nonzero if a bounded wait inside the kernel gave up.
+// after_cost: the previous kernel of the stream is one of this library's (the cost
+// build), so the launch may be programmatic.
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W,
                                  int C, int D, int radius, float sigma_s, float sigma_r,
                                  float* agg_out, int32_t* disp_int, float* disp_sub, int* err,
-                                 cudaStream_t stream);
+                                 bool after_cost, cudaStream_t stream);
 
 // ---- steps 2-4 on the tensor cores (BF16 / FP16 operands, FP32 accumulate) ---
 // cost: 16-bit x-blocked volume (see launch_cost_build_xblock16), 16-byte
@@ -177,7 +202,6 @@ __device__ __forceinline__ int find_pair(const BatchPair* pairs, int n, int item
 int stats_items(int H, int W);
 int cost_items(int H, int W);
 int agg_f32_tiles(int H, int W);
-size_t cost_kernel_smem();
 cudaError_t prepare_cost_batched();
 cudaError_t launch_stats_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
                                  cudaStream_t stream);

@@ -353,3 +353,35 @@ def test_aggregate_all_infinite_pixels_take_disparity_zero(ctx):
     guide = np.zeros((6, 40, 3), np.uint8)
     _, di, ds = _aggregate(ctx, cost, guide, 2, 2.0, 10.0)
     assert not di.any() and not ds.any()
+
+
+# The FP32 cost kernel covers 64 pixels x 4 rows per CTA, 16 disparities per warp, 128 per pass, and stores 4, 2 or 1
+# floats at a time (D a multiple of 4, even, odd).
+@pytest.mark.parametrize("mode,tau", [(0, 0.0), (1, 25.0)])
+@pytest.mark.parametrize("H,W,C,D", [(1, 1, 1, 1), (2, 63, 3, 2), (5, 64, 1, 3), (4, 65, 3, 16), (3, 40, 1, 17),
+                                     (6, 131, 3, 33), (5, 200, 3, 128), (3, 170, 1, 129), (4, 300, 3, 258)])
+def test_cost_volume_tile_edges(fbs, oracle_mod, mode, tau, H, W, C, D):
+    rng = np.random.default_rng(7 * D + W)
+    L = rng.integers(0, 256, (H, W, C)).astype(np.uint8)
+    R = np.roll(L, -min(4, W - 1), axis=1)
+    R = np.clip(R.astype(np.int32) + rng.integers(-30, 31, R.shape), 0, 255).astype(np.uint8)
+    L[:, : W // 4] = 77                      # flat blocks
+    with fbs.Context(0, cost=mode) as c:
+        cost = c.cost_volume(_dev(L), _dev(R), D, tau)
+        torch.cuda.synchronize()
+    check_agg(cost.cpu().numpy(), oracle_mod.cost_volume(L, R, D, mode, tau), tau if mode else 2.0)
+
+
+@pytest.mark.parametrize("H,W,D", [(6, 70, 20), (5, 150, 140), (7, 66, 64)])
+def test_right_view_tile_edges(fbs, oracle_mod, H, W, D):
+    """The right view's volume (the other window slides the other way) over tile and pass edges."""
+    rng = np.random.default_rng(D)
+    L = rng.integers(0, 256, (H, W, 3)).astype(np.uint8)
+    R = np.clip(np.roll(L, -6, axis=1).astype(np.int32) + rng.integers(-20, 21, L.shape), 0, 255).astype(np.uint8)
+    out = [torch.empty((H, W), dtype=t, device="cuda") for t in (torch.int32, torch.float32) * 2]
+    with fbs.Context(0) as c:
+        fbs.fbs_compute_disparity_lr(c.ctx, _dev(L), _dev(R), H, W, 3, D, 3, 3.0, 30.0, 0.0, *out, False)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(c.ctx)
+    ri, rs, ragg = oracle_mod.fbs_right(L, R, D, 3, 3.0, 30.0, want_agg=True)
+    check_disparities(out[2].cpu().numpy(), out[3].cpu().numpy(), ragg, ri, rs, 2.0)
