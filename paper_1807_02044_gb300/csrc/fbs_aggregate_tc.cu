@@ -20,7 +20,9 @@
 //     ones row makes the same product also sum the rounded weights, so the
 //     numerator and the normaliser use the same weights.
 // A ring of S stages of R rows each (S >= 2) lets the threads produce the
-// next stage while the tensor core works on the current one; TMA runs ahead.  After the last row,
+// next stage while the tensor core works on the current one; TMA runs ahead.
+// Where fewer than four rows fit twice, two groups of the threads take the
+// stages in turn (tc_plan).  After the last row,
 // four warps read the accumulator rows (one pixel per TMEM lane), normalise
 // in FP32, and do WTA (smallest d on ties) and Eq. (10) in registers.
 //
@@ -57,6 +59,7 @@ struct TcParams {
     int rho, rho8, KW, NH, ntx, ntiles;
     int R;          // window rows per pipeline stage
     int S;          // pipeline stages (weights and cost rows share the stage index)
+    int NG;         // groups of producer warps that take the stages in turn (the kernel's template argument)
     int nacc;       // accumulator buffers in TMEM (2 = epilogue overlaps the next tile)
     uint32_t acc_stride, den_col, tmem_cols;
     float neg_ks, neg_kr;
@@ -119,14 +122,14 @@ struct TileWalk {
 // Pipeline: a stage holds R consecutive window rows of one tile (the last
 // stage of a tile may hold fewer).  For stage g in slot s = g % S:
 //   producers  wait empty[s] (stage g - S consumed), write R rows of weights,
-//              arrive full_a[s] (one arrival per warp);
+//              arrive full_a[s] (one arrival per warp that writes the stage);
 //   TMA        waits empty[s], loads R cost rows, full_b[s] completes on bytes;
 //   MMA        waits full_a[s] and full_b[s], issues R * KW/16 MMAs, commits
 //              to empty[s]; after a tile's last stage commits acc_full[ab];
 //   epilogue   waits acc_full[ab], reads the accumulator, arrives acc_empty[ab].
 // One wait/commit pair per R rows keeps the single-thread control path
 // (which shares its scheduler with busy warps) off the critical path.
-template <bool BF16, int NPT, int PM>
+template <bool BF16, int NPT, int PM, int NG>
 __global__ void __launch_bounds__(kThreads, 1)
 aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap gmap, TcParams p,
                     float* __restrict__ agg_out, int32_t* __restrict__ disp_int, float* __restrict__ disp_sub,
@@ -157,7 +160,7 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
     // ---- set-up --------------------------------------------------------------
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(full_a0 + 8 * s, kProducerWarps);   // one elected arrival per producer warp
+            mbar_init(full_a0 + 8 * s, kProducerWarps / NG);   // one arrival per warp of the stage's group
             mbar_init(full_b0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, 1);
         }
@@ -196,7 +199,9 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
     if (warp < kProducerWarps) {
         // ================= weight producers =================================
         // Warp w covers the pixel rows ty = 2 (w >> 2) and ty + 1 of the tile
-        // and, within every stage, the window rows r with r % 4 == w % 4; lane
+        // and, within every stage, the window rows r with r % 4 == w % 4 (of two
+        // groups, warps with w % 4 >= 2 write stages 0, 2, .. and the others
+        // stages 1, 3, .., each window row r == w % 2); lane
         // -> pixel column xm = lane & 15 and pair phase h = lane >> 4.  Pixel
         // (xm, y) needs window columns kcen - rho .. kcen + rho (kcen = xm +
         // rho8), covered by rho + 1 pairs of adjacent columns (k, k + 1)
@@ -234,6 +239,7 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
         const uint64_t nkr2 = f2_pack(p.neg_kr, p.neg_kr);
         const unsigned two_rho = (unsigned)(2 * p.rho);
         uint32_t gs = 0, gu = 0, t = 0;   // stage slot and use count of the next stage
+        [[maybe_unused]] bool mine = rq < 2;   // two groups: did this warp's write the last stage?
         bool stop = false;
         for (TileWalk tw(p.ntx); tw.tile < p.ntiles && !stop; tw.next(), ++t) {
             const int tx0 = tw.tx * kTW, ty0 = tw.ty * kTH;
@@ -273,6 +279,16 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
             for (int h0 = hr_lo; h0 < hr_hi; h0 += R) {
                 const int nr = min(R, hr_hi - h0);
                 const uint32_t s = gs, use = gu;   // g % S, g / S, carried below
+                if constexpr (NG == 2) {
+                    mine = !mine;
+                    if (!mine) {   // the other group's stage
+                        if (++gs == (uint32_t)S) {
+                            gs = 0;
+                            ++gu;
+                        }
+                        continue;
+                    }
+                }
                 // one lane waits for the MMAs that last read stage s; the warp follows
                 bool ok = true;
                 if (lane == 0 && use > 0) ok = mbar_wait_or_abort(empty0 + 8 * s, (use - 1) & 1, abort_flag, p.wait_cycles);
@@ -283,7 +299,7 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
                 }
                 uint8_t* ast = a_base + s * a_stage;
 #pragma unroll
-                for (int r = rq; r < kMaxR; r += 4) {
+                for (int r = NG == 1 ? rq : rq & 1; r < (NG == 1 ? kMaxR : 2); r += 4) {
                     if (r >= nr) break;
                     const int hr = h0 + r;
                     const int dy = hr - ty;   // row offset + rho of the upper pixel
@@ -549,11 +565,11 @@ cudaError_t launch_hwd_to_xblock16(const float* in, int H, int W, int D, bool bf
 
 namespace {
 
-template <bool BF16, int NPT, int PM>
+template <bool BF16, int NPT, int PM, int NG>
 cudaError_t run_tc(const CUtensorMap& map, const CUtensorMap& gmap, const TcParams& p, const TcSmem& L, int grid,
                    float* agg_out, int32_t* disp_int, float* disp_sub, int* err, cudaStream_t stream)
 {
-    cudaError_t e = fbs::raise_smem_limit(aggregate_tc_kernel<BF16, NPT, PM>, (int)L.total);
+    cudaError_t e = fbs::raise_smem_limit(aggregate_tc_kernel<BF16, NPT, PM, NG>, (int)L.total);
     if (e != cudaSuccess) return e;
     // programmatic stream serialization: the kernel may start while the
     // previous kernel of the stream (the cost build, which signals early) ends
@@ -568,7 +584,7 @@ cudaError_t run_tc(const CUtensorMap& map, const CUtensorMap& gmap, const TcPara
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     fbs::note_launch();
-    e = cudaLaunchKernelEx(&cfg, aggregate_tc_kernel<BF16, NPT, PM>, map, gmap, p, agg_out, disp_int, disp_sub, err);
+    e = cudaLaunchKernelEx(&cfg, aggregate_tc_kernel<BF16, NPT, PM, NG>, map, gmap, p, agg_out, disp_int, disp_sub, err);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -607,12 +623,43 @@ bool tc_plan(int H, int W, int C, int D, int radius, float sigma_s, float sigma_
     // 2 stages in 227 KB, then as many stages (<= 6) as fit.  Fewer, larger
     // stages per tile measured faster than deeper pipelines of small stages:
     // each stage costs the producers a wait, a proxy fence and an arrival
-    for (p.R = max_rows < 1 || max_rows > kMaxR ? kMaxR : max_rows; p.R >= 1; --p.R) {
-        for (p.S = 6; p.S >= 2; --p.S) {
-            L = tc_smem_layout(p.KW, p.Nb, p.NH, p.R, p.S);
-            if (L.total <= 227 * 1024) return true;
-        }
+    auto fits = [&](int R, int S) {
+        L = tc_smem_layout(p.KW, p.Nb, p.NH, R, S);
+        p.R = R;
+        p.S = S;
+        return L.total <= 227 * 1024;
+    };
+    const int cap = max_rows < 1 || max_rows > kMaxR ? kMaxR : max_rows;
+    // Where four rows do not fit twice, one group of 16 producer warps (four
+    // warps for each of four rows) leaves warps without a row.  Two groups of
+    // eight, each writing every other stage of two rows, keep all of them
+    // busy, and one group's fence and wait run beside the other's arithmetic.
+    // Aggregation, one group -> two: 1280 x 960, D = 128, radius 15 773 -> 693 us;
+    // 1920 x 1080, D = 256, radius 9 1343 -> 1280 us; 1280 x 720, D = 128,
+    // radius 10 390 -> 371 us, radius 12 472 -> 427 us.  At radius 9 three rows
+    // carry too little work for the extra stages (D = 128: 337 -> 341 us), and
+    // from four rows up one group wins (640 x 480, D = 64, radius 7: 57 us at
+    // 8 rows x 2 stages, 72 us in two groups of 4 x 4).
+    p.NG = 1;
+    if (radius > 15) {
+        // these column-pair counts spill registers, and what shared memory
+        // leaves of the 256 KB is the L1 cache that holds the spills: the
+        // smallest two-group ring is the fastest (1280 x 720, D = 64, radius 20:
+        // one group 3.48 ms, 2 x 3 2.70 ms, 2 x 2 1.81 ms; D = 256, radius 24:
+        // one group 8.9 ms, 1 x 3 6.5 ms, 1 x 2 4.4 ms)
+        p.NG = 2;
+        return (cap >= 2 && fits(2, 2)) || fits(1, 2);
     }
+    if (!fits(4, 2) && (radius > 9 || !fits(3, 2))) {
+        p.NG = 2;
+        for (int R = min(cap, 2); R >= 1; --R)
+            for (int S = 6; S >= 2; --S)
+                if (fits(R, S)) return true;
+        return false;
+    }
+    for (int R = cap; R >= 1; --R)
+        for (int S = 6; S >= 2; --S)
+            if (fits(R, S)) return true;
     return false;
 }
 
@@ -699,28 +746,31 @@ cudaError_t launch_aggregate_tc(const void* cost, const uint2* rgbx, int H, int 
     // rounded up and the surplus pairs are switched off per pair.
     const int npt = (radius + 2) / 2;
     const int pm = (radius & 1) ? 0 : 1;
-#define FBS_TC_CASE(n)                                                                                         \
-    if (npt == n)                                                                                             \
-        return pm == 0 ? (bf16 ? run_tc<true, n, 0>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream)  \
-                               : run_tc<false, n, 0>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream)) \
-                       : (bf16 ? run_tc<true, n, 1>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream)  \
-                               : run_tc<false, n, 1>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream));
-    FBS_TC_CASE(1)
-    FBS_TC_CASE(2)
-    FBS_TC_CASE(3)
-    FBS_TC_CASE(4)
-    FBS_TC_CASE(5)
-    FBS_TC_CASE(6)
-    FBS_TC_CASE(7)
-    FBS_TC_CASE(8)
+    // Two groups of producer warps (tc_plan) need a radius of 9 or more.
+#define FBS_TC_RUN(n, pm, ng)                                                                               \
+    return bf16 ? run_tc<true, n, pm, ng>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream)  \
+                : run_tc<false, n, pm, ng>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream)
+#define FBS_TC_CASE(n, ng)                \
+    if (npt == n && p.NG == ng) {         \
+        if (pm == 0) FBS_TC_RUN(n, 0, ng); \
+        FBS_TC_RUN(n, 1, ng);             \
+    }
+    FBS_TC_CASE(1, 1)
+    FBS_TC_CASE(2, 1)
+    FBS_TC_CASE(3, 1)
+    FBS_TC_CASE(4, 1)
+    FBS_TC_CASE(5, 1)
+    FBS_TC_CASE(6, 1)
+    FBS_TC_CASE(7, 1)
+    FBS_TC_CASE(8, 1)
+    if (npt == 5 && pm == 0 && p.NG == 2) FBS_TC_RUN(5, 0, 2);
+    FBS_TC_CASE(6, 2)
+    FBS_TC_CASE(7, 2)
+    FBS_TC_CASE(8, 2)
+    if (npt > 8 && npt <= 10) FBS_TC_RUN(10, 2, 2);
+    if (npt > 10 && npt <= 13) FBS_TC_RUN(13, 2, 2);
 #undef FBS_TC_CASE
-#define FBS_TC_CASE(n)                                                                                     \
-    if (npt <= n)                                                                                         \
-        return bf16 ? run_tc<true, n, 2>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream) \
-                    : run_tc<false, n, 2>(map, gmap, p, L, grid, agg_out, disp_int, disp_sub, err, stream);
-    FBS_TC_CASE(10)
-    FBS_TC_CASE(13)
-#undef FBS_TC_CASE
+#undef FBS_TC_RUN
     return cudaErrorInvalidValue;
 }
 

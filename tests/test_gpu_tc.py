@@ -88,6 +88,20 @@ def test_tc_aggregation_within_rounding_bound(fbs, oracle_mod, prec, H, W, C, D,
 
 
 @pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("H,W,C,D,r", [
+    (26, 40, 3, 256, 24),   # one row a stage, two stages
+    (21, 45, 1, 32, 16),    # the smallest radius that always takes two groups
+    (20, 50, 3, 256, 9),    # two rows, two stages
+    (33, 37, 1, 128, 15),   # two rows, three stages; odd counts of window rows in the border tiles
+    (1, 5000, 1, 256, 12),  # one stage a tile, several tiles a block: the groups take whole tiles in turn
+])
+def test_tc_two_producer_groups(fbs, oracle_mod, prec, H, W, C, D, r):
+    """Shapes whose stages two groups of producer warps write in turn: the same
+    bound as for every other shape."""
+    test_tc_aggregation_within_rounding_bound(fbs, oracle_mod, prec, H, W, C, D, r)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
 def test_tc_full_size_bench_workload_bad_pixels(fbs, oracle_mod, prec):
     """640x480 RGB, D=64, radius 7 (the benchmark workload): aggregated costs
     of 400 sampled pixels within the 16-bit rounding bound of the FP64 oracle
