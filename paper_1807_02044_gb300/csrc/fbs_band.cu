@@ -32,165 +32,265 @@ __global__ void bf16_to_f32_kernel(const __nv_bfloat16* __restrict__ src, float*
 
 // ---- features (readings B1-B3) ---------------------------------------------------
 // Quarter-resolution intensity of both images: integer sum of the channel
-// sums over the 4x4 block, pixels clamped to the image.
-__global__ void band_downsample_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W,
-                                       int C, int32_t* __restrict__ gq)
+// sums over the 4x4 block, pixels clamped to the image; and, for the coarse
+// costs, the sum of a pixel's 3x3 block of them (coordinates clamped to the
+// quarter image) and nine times the sum of its squares less the squared sum, as
+// a float (0 only for a constant block): 9 x 12240^2 < 2^31, the rest is exact
+// in 64 bits.  A CTA sums its tile of 30 x 8 and the border once, one sum per
+// thread, in shared memory.
+constexpr int kQuarterX = 32;   // with the border
+constexpr int kQuarterY = 10;
+
+struct BlockStat {
+    int sum;
+    float var;
+};
+
+// Channel sum of the 4 x 4 pixels from column 4 X, row 4 Y on, clamped.
+template <int C>
+__device__ __forceinline__ int block_sum(const uint8_t* __restrict__ src, int X, int Y, int H, int W)
 {
-    const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
-    const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y, img = blockIdx.z;
-    if (X >= Wq) return;
-    const uint8_t* src = img == 0 ? L : R;
     int s = 0;
-    for (int j = 0; j < 4; ++j) {
-        const int y = min(4 * Y + j, H - 1);
+    if ((reinterpret_cast<uintptr_t>(src) & 3) == 0 && (W * C) % 4 == 0 && 4 * X + 3 < W) {
+        uint32_t w[4][C];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                w[j][c] = reinterpret_cast<const uint32_t*>(src + ((size_t)min(4 * Y + j, H - 1) * W + 4 * X) * C)[c];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int c = 0; c < C; ++c) s = (int)__dp4a(w[j][c], 0x01010101u, (uint32_t)s);
+        return s;
+    }
+    for (int j = 0; j < 4; ++j)
         for (int i = 0; i < 4; ++i) {
-            const uint8_t* p = src + ((size_t)y * W + min(4 * X + i, W - 1)) * C;
-            s += p[0];
-            if (C == 3) s += p[1] + p[2];
+            const uint8_t* p = src + ((size_t)min(4 * Y + j, H - 1) * W + min(4 * X + i, W - 1)) * C;
+#pragma unroll
+            for (int c = 0; c < C; ++c) s += p[c];
         }
-    }
-    gq[(size_t)img * Hq * Wq + (size_t)Y * Wq + X] = s;
+    return s;
 }
 
-// Coarse cost from exact integer sums; the normalisation uses correctly
-// rounded FP32 operations in the order of the definition, so every
-// evaluation of the same (X, Y, e) gives the same bits.
-__device__ __forceinline__ float coarse_from_sums(long long P9, long long Sl, long long Sr, long long Vl,
-                                                  long long Vr)
+template <int C>
+__global__ void __launch_bounds__(kQuarterX * kQuarterY)
+band_quarter_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R, int H, int W,
+                    int32_t* __restrict__ gq, BlockStat* __restrict__ stat)
 {
-    if (Vl == 0 || Vr == 0) return 1.f;
-    const long long num = P9 - Sl * Sr;
-    const float vv = __fmul_rn(__ll2float_rn(Vl), __ll2float_rn(Vr));
-    const float c = __fdiv_rn(__ll2float_rn(num), __fsqrt_rn(vv));
-    return __fsub_rn(1.f, c);
+    __shared__ int g[kQuarterY][kQuarterX];
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
+    const int tx = threadIdx.x % kQuarterX, ty = threadIdx.x / kQuarterX;
+    const int X = blockIdx.x * (kQuarterX - 2) + tx - 1, Y = blockIdx.y * (kQuarterY - 2) + ty - 1;
+    g[ty][tx] = block_sum<C>(blockIdx.z == 0 ? L : R, clampi(X, 0, Wq - 1), clampi(Y, 0, Hq - 1), H, W);
+    __syncthreads();
+    if (tx == 0 || tx == kQuarterX - 1 || ty == 0 || ty == kQuarterY - 1 || X >= Wq || Y >= Hq) return;
+    int S = 0, Q = 0;
+#pragma unroll
+    for (int j = -1; j < 2; ++j)
+#pragma unroll
+        for (int i = -1; i < 2; ++i) {
+            const int v = g[ty + j][tx + i];
+            S += v;
+            Q += v * v;
+        }
+    const size_t o = ((size_t)blockIdx.z * Hq + Y) * Wq + X;
+    gq[o] = g[ty][tx];
+    stat[o] = BlockStat{S, __ll2float_rn(9 * (long long)Q - (long long)S * S)};
 }
 
-// Coarse cost volume K [Hq][Wq][Dq] (FP32).  A CTA covers 64 consecutive
-// quarter pixels of one row; each thread slides its right block one column
-// per e (three new values), and the costs of 32 consecutive e are staged in
-// shared memory so that every warp stores 128 contiguous bytes.
-constexpr int kCoarseX = 64;
-constexpr int kCoarseE = 32;
-
-__global__ void __launch_bounds__(kCoarseX)
-band_coarse_cost_kernel(const int32_t* __restrict__ gq, int Hq, int Wq, int Dq, float* __restrict__ K)
-{
-    __shared__ float tile[kCoarseX][kCoarseE + 1];
-    const int X0 = blockIdx.x * kCoarseX, Y = blockIdx.y;
-    const int X = X0 + threadIdx.x;
-    const bool valid = X < Wq;
-    const int32_t* gl = gq;
-    const int32_t* gr = gq + (size_t)Hq * Wq;
-    const int Xc = valid ? X : Wq - 1;
-    int yr[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) yr[j] = clampi(Y - 1 + j, 0, Hq - 1) * Wq;
-    long long Sl = 0, Ql = 0;
-    int lw[3][3], rw[3][3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            lw[j][i] = gl[yr[j] + clampi(Xc - 1 + i, 0, Wq - 1)];
-            Sl += lw[j][i];
-            Ql += (long long)lw[j][i] * lw[j][i];
-            rw[j][i] = gr[yr[j] + clampi(Xc - 1 + i, 0, Wq - 1)];
-        }
-    const long long Vl = 9 * Ql - Sl * Sl;
-    const int nx = min(kCoarseX, Wq - X0);
-    for (int e0 = 0; e0 < Dq; e0 += kCoarseE) {
-        const int ne = min(kCoarseE, Dq - e0);
-        for (int k = 0; k < ne; ++k) {
-            const int e = e0 + k;
-            if (e > 0) {
-                const int xc = clampi(Xc - e - 1, 0, Wq - 1);
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    rw[j][2] = rw[j][1];
-                    rw[j][1] = rw[j][0];
-                    rw[j][0] = gr[yr[j] + xc];
-                }
-            }
-            float c = 2.f;
-            if (Xc - e >= 0) {
-                long long Sr = 0, Qr = 0, P = 0;
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        Sr += rw[j][i];
-                        Qr += (long long)rw[j][i] * rw[j][i];
-                        P += lw[j][i] * rw[j][i];   // <= 12240^2, exact in int32
-                    }
-                c = coarse_from_sums(9 * P, Sl, Sr, Vl, 9 * Qr - Sr * Sr);
-            }
-            tile[threadIdx.x][k] = c;
-        }
-        __syncthreads();
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int x = warp; x < nx; x += kCoarseX / 32)
-            if (lane < ne) K[((size_t)Y * Wq + X0 + x) * Dq + e0 + lane] = tile[x][lane];
-        __syncthreads();
-    }
-}
-
-// Reading B3: row sums over the clipped 5-column window (X' ascending) ...
+// Row sums Kh [Hq][Wq][Dq] of the coarse cost volume over the clipped
+// 5-column window (X' ascending; reading B3).  A thread takes one e and walks
+// kRowX columns of a row (and two on either side, recomputed by the
+// neighbours): the block product of a column is three new integer products and
+// the two columns before it, the cost a handful of correctly rounded FP32
+// operations more (every evaluation of the same (X, Y, e) gives the same bits),
+// and the last five costs are in registers.  Lanes are consecutive e: the left
+// pixels are broadcast from shared memory, the right ones adjacent there, and
+// the sums stored 128 bytes at a time.  Bound by issue (the division and the
+// square root are half of it).  The costs with nine products each, by way of a
+// volume in memory and a kernel of row sums, took 30 + 22 us at 320 x 160
+// quarter pixels, Dq = 64, now 15 (each alone, cold caches); the whole of
+// fbs_band_features 120.4 us then, 31.1 now.
 constexpr int kAggR = 2;
+constexpr int kRowX = 16;
+constexpr int kRowChunks = 4;                       // kRowX columns each, per CTA
+constexpr int kRowSpan = kRowX * kRowChunks;
+constexpr int kRowThreads = 256;
 
-__global__ void band_row_sum_kernel(const float* __restrict__ K, int Hq, int Wq, int Dq, float* __restrict__ Kh)
+// One column of three rows, and the statistics of its middle pixel.
+struct __align__(16) RowColumn {
+    int g[3];
+    int sum;
+};
+
+inline size_t row_sum_smem(int Dq) { return (size_t)(2 * (kRowSpan + 2 * kAggR + 2) + Dq) * (sizeof(RowColumn) + 4); }
+
+__global__ void __launch_bounds__(kRowThreads)
+band_row_sum_kernel(const int32_t* __restrict__ gq, const BlockStat* __restrict__ stat, int Hq, int Wq, int Dq,
+                    float* __restrict__ Kh)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)Hq * Wq * Dq) return;
-    const int e = (int)(i % Dq);
-    const size_t q = i / Dq;
-    const int X = (int)(q % Wq), Y = (int)(q / Wq);
-    float s = 0.f;
-    for (int x = max(0, X - kAggR); x <= min(Wq - 1, X + kAggR); ++x) s = __fadd_rn(s, K[((size_t)Y * Wq + x) * Dq + e]);
-    Kh[i] = s;
+    extern __shared__ __align__(16) uint8_t row_smem[];
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // left columns xl0 .. , right columns xl0 - Dq ..: every column a window of
+    // this CTA reads, coordinates clamped to the image
+    constexpr int kLeft = kRowSpan + 2 * kAggR + 2;
+    const int Y = blockIdx.y, xc = blockIdx.x * kRowSpan, xl0 = xc - kAggR - 1;
+    const int nright = kLeft + Dq;
+    RowColumn* lc = reinterpret_cast<RowColumn*>(row_smem);
+    RowColumn* rc = lc + kLeft;
+    float* lv = reinterpret_cast<float*>(rc + nright);
+    float* rv = lv + kLeft;
+    const size_t P = (size_t)Hq * Wq;
+    for (int i = threadIdx.x; i < kLeft + nright; i += kRowThreads) {
+        const bool right = i >= kLeft;
+        const int x = clampi(right ? xl0 - Dq + i - kLeft : xl0 + i, 0, Wq - 1);
+        const size_t o = right ? P : 0;
+        RowColumn c;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) c.g[j] = gq[o + (size_t)clampi(Y - 1 + j, 0, Hq - 1) * Wq + x];
+        const BlockStat s = stat[o + (size_t)Y * Wq + x];
+        c.sum = right ? s.sum : -s.sum;
+        lc[i] = c;
+        lv[i] = s.var;
+    }
+    __syncthreads();
+    for (int item = threadIdx.x; item < kRowChunks * Dq; item += kRowThreads) {
+        const int e = item % Dq, X0 = xc + item / Dq * kRowX;
+        if (X0 >= Wq) break;
+        // entry i: column X0 - kAggR - 1 + i, and that column less e
+        const RowColumn *l = lc + (X0 - xc), *r = rc + (X0 - xc) + Dq - e;
+        const float *vl = lv + (X0 - xc), *vr = rv + (X0 - xc) + Dq - e;
+        auto product = [&](const RowColumn& a, const RowColumn& b) {
+            return a.g[0] * b.g[0] + a.g[1] * b.g[1] + a.g[2] * b.g[2];
+        };
+        float* out = Kh + ((size_t)Y * Wq + X0) * Dq + e;
+        float k[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // costs of the last five columns
+        RowColumn a1 = l[1], b1 = r[1];
+        int p0 = product(l[0], r[0]), p1 = product(a1, b1);
+        const int nx = Wq - X0;
+#pragma unroll
+        for (int i = 0; i < kRowX + 2 * kAggR; ++i) {
+            const int dx = i - kAggR;   // column X0 + dx
+            const RowColumn a2 = l[i + 2], b2 = r[i + 2];
+            const int p2 = product(a2, b2);
+            float c = 0.f;              // outside the image: adds nothing
+            if (X0 + dx >= 0 && dx < nx) {
+                const float va = vl[i + 1], vb = vr[i + 1];
+                const long long num = 9ll * (p0 + p1 + p2) + (long long)a1.sum * b1.sum;
+                c = va != 0.f && vb != 0.f
+                        ? __fsub_rn(1.f, __fdiv_rn(__ll2float_rn(num), __fsqrt_rn(__fmul_rn(va, vb)))) : 1.f;
+                if (X0 + dx < e) c = 2.f;
+            }
+            k[i % 5] = c;
+            if (i >= 2 * kAggR && dx - kAggR < nx) {
+                out[(size_t)(i - 2 * kAggR) * Dq] =
+                    __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(k[(i + 1) % 5], k[(i + 2) % 5]), k[(i + 3) % 5]),
+                                        k[(i + 4) % 5]), c);
+            }
+            p0 = p1;
+            p1 = p2;
+            a1 = a2;
+            b1 = b2;
+        }
+    }
 }
 
-// ... then the sum of the row sums (Y' ascending) divided by the tap count.
-__global__ void band_col_mean_kernel(const float* __restrict__ Kh, int Hq, int Wq, int Dq, float* __restrict__ Kb)
+// The minimum over a warp of finite floats.
+__device__ __forceinline__ float warp_min(float v)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)Hq * Wq * Dq) return;
-    const int e = (int)(i % Dq);
-    const size_t q = i / Dq;
-    const int X = (int)(q % Wq), Y = (int)(q / Wq);
-    const int y0 = max(0, Y - kAggR), y1 = min(Hq - 1, Y + kAggR);
-    const int x0 = max(0, X - kAggR), x1 = min(Wq - 1, X + kAggR);
-    float s = 0.f;
-    for (int y = y0; y <= y1; ++y) s = __fadd_rn(s, Kh[((size_t)y * Wq + X) * Dq + e]);
-    Kb[i] = __fdiv_rn(s, (float)((y1 - y0 + 1) * (x1 - x0 + 1)));
+    // order-preserving: negative floats with their other bits inverted
+    const int b = __float_as_int(v), k = b ^ ((b >> 31) & 0x7fffffff);
+    const int m = __reduce_min_sync(0xffffffffu, k);
+    return __int_as_float(m ^ ((m >> 31) & 0x7fffffff));
 }
 
-// One thread per quarter pixel: winner of Kbar (smallest e on ties), the best
-// non-adjacent cost and the winner's neighbours give the six features; x0
-// receives them as BF16 [P][8] (two zero channels), feat (nullable) as FP32
-// [P][6], estar the winner.
-__global__ void __launch_bounds__(128)
-band_features_kernel(const int32_t* __restrict__ gq, const float* __restrict__ Kb, int H, int W, int C, int D,
+// The 5x5 means Kbar of a quarter pixel's coarse costs (sum of the row sums,
+// Y' ascending, divided by the tap count), their winner (smallest e on ties),
+// the best non-adjacent cost and the winner's neighbours give the six
+// features; x0 receives them as BF16 [P][8] (two zero channels), feat
+// (nullable) as FP32 [P][6], estar the winner.  A warp takes eight pixels of a
+// column, lanes over e: the twelve row sums that their windows cover are read
+// once each, and the eight pixels' features are finished together, one lane
+// each.  Bound by issue.  The division by the tap count is a multiplication by
+// its reciprocal and one residual step (Markstein's theorem; checked for every
+// significand and all tap counts to be the correctly rounded quotient).  A
+// kernel that stored the means and one thread per pixel that read them twice
+// took 23.5 + 35 us at 320 x 160, Dq = 64; now 14.6 (alone, cold caches).
+constexpr int kFeatWarps = 4;
+constexpr int kFeatRows = 8;
+
+__global__ void __launch_bounds__(32 * kFeatWarps)
+band_features_kernel(const int32_t* __restrict__ gq, const float* __restrict__ Kh, int H, int W, int C, int D,
                      __nv_bfloat16* __restrict__ x0, float* __restrict__ feat, int32_t* __restrict__ estar)
 {
+    extern __shared__ float means[];
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int Hq = (H + 3) / 4, Wq = (W + 3) / 4, Dq = (D + 3) / 4;
-    const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int X = blockIdx.x * kFeatWarps + warp, Y0 = blockIdx.y * kFeatRows;
     if (X >= Wq) return;
-    const size_t i = (size_t)Y * Wq + X;
-    const float* k = Kb + i * Dq;
-    int best = 0;
-    float k1 = k[0];
-    for (int e = 1; e < Dq; ++e) {
-        const float v = k[e];
-        if (v < k1) {
-            k1 = v;
-            best = e;
+    float* mean = means + warp * kFeatRows * Dq;
+    const int yl = Y0 + lane;   // lane q's pixel, q < kFeatRows
+    const float taps_l = (float)((min(Hq - 1, yl + kAggR) - max(0, yl - kAggR) + 1) *
+                                 (min(Wq - 1, X + kAggR) - max(0, X - kAggR) + 1));
+    const float rtaps_l = __frcp_rn(taps_l);
+    const size_t row = (size_t)Wq * Dq;
+    const float* k = Kh + (ptrdiff_t)(Y0 - kAggR) * (ptrdiff_t)row + (size_t)X * Dq;
+    float v1[kFeatRows];
+    int b1[kFeatRows];
+#pragma unroll
+    for (int q = 0; q < kFeatRows; ++q) {
+        v1[q] = __int_as_float(0x7f800000);
+        b1[q] = 1 << 30;
+    }
+    for (int e0 = 0; e0 < Dq; e0 += 32) {
+        const int e = e0 + lane;
+        const bool ok = e < Dq;
+        float t[kFeatRows + 2 * kAggR];   // rows outside the image add nothing
+#pragma unroll
+        for (int j = 0; j < kFeatRows + 2 * kAggR; ++j)
+            t[j] = ok && (unsigned)(Y0 - kAggR + j) < (unsigned)Hq ? k[(ptrdiff_t)j * (ptrdiff_t)row + e] : 0.f;
+#pragma unroll
+        for (int q = 0; q < kFeatRows; ++q) {
+            const float taps = __shfl_sync(0xffffffffu, taps_l, q), rtaps = __shfl_sync(0xffffffffu, rtaps_l, q);
+            const float s = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(t[q], t[q + 1]), t[q + 2]), t[q + 3]), t[q + 4]);
+            const float d = __fmul_rn(s, rtaps);
+            const float v = __fmaf_rn(__fmaf_rn(-d, taps, s), rtaps, d);
+            if (ok) {
+                mean[q * Dq + e] = v;
+                if (v < v1[q]) {
+                    v1[q] = v;
+                    b1[q] = e;
+                }
+            }
         }
     }
-    float k2 = 2.f;
-    for (int e = 0; e < Dq; ++e)
-        if (abs(e - best) >= 2 && k[e] < k2) k2 = k[e];
-    const float km = best > 0 ? k[best - 1] : 2.f;
-    const float kp = best < Dq - 1 ? k[best + 1] : 2.f;
+    __syncwarp();
+    float k1 = 0.f, k2 = 0.f;
+    int best = 0;
+#pragma unroll
+    for (int q = 0; q < kFeatRows; ++q) {
+        const float m1 = warp_min(v1[q]);
+        const int b = __reduce_min_sync(0xffffffffu, v1[q] == m1 ? b1[q] : 1 << 30);
+        float m2 = 2.f;
+        for (int e = lane; e < Dq; e += 32)
+            if ((unsigned)(e - b + 1) > 2u) m2 = fminf(m2, mean[q * Dq + e]);
+        m2 = warp_min(m2);
+        if (lane == q) {
+            k1 = m1;
+            k2 = m2;
+            best = b;
+        }
+    }
+    if (lane >= kFeatRows || yl >= Hq) return;
+    mean += lane * Dq;
+    const size_t i = (size_t)yl * Wq + X;
+    const float km = best > 0 ? mean[best - 1] : 2.f;
+    const float kp = best < Dq - 1 ? mean[best + 1] : 2.f;
     float f[6];
     f[0] = __fsub_rn(__fdiv_rn((float)gq[i], (float)(16 * 255 * C)), 0.5f);
     f[1] = __fdiv_rn((float)best, (float)Dq);
@@ -285,19 +385,6 @@ band_tiles_kernel(const float* __restrict__ centre, const float* __restrict__ co
     if (threadIdx.x == 0) tile_range[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = make_int2(lo_s & ~3, hi_s + 1);
 }
 
-// ---- network head: full-resolution centre and confidence -------------------------
-__global__ void band_head_kernel(const float* __restrict__ out, const int32_t* __restrict__ estar, int H, int W,
-                                 float* __restrict__ centre, float* __restrict__ conf)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-    if (x >= W) return;
-    const int Wq = (W + 3) / 4;
-    const size_t i = (size_t)(y >> 2) * Wq + (x >> 2);
-    const size_t p = (size_t)y * W + x;
-    if (centre) centre[p] = __fmul_rn(4.f, __fadd_rn((float)estar[i], out[2 * i]));
-    if (conf) conf[p] = 1.f / (1.f + expf(-out[2 * i + 1]));
-}
-
 }  // namespace
 
 cudaError_t launch_band_tiles(const float* centre, const float* conf, int H, int W, int D, int half_band,
@@ -337,8 +424,8 @@ size_t al256(size_t n) { return (n + 255) & ~(size_t)255; }
 // Scratch of one quarter-resolution problem, carved from ctx->band_ws.
 struct NetScratch {
     int32_t* gq;                 // [2][P]
-    float* kq;                   // coarse costs [P][Dq], then their 5x5 means
-    float* kh;                   // row sums [P][Dq]
+    fbs::BlockStat* stat;        // [2][P]; lies in y[0], which the features' readers write
+    float* kh;                   // row sums of the coarse costs [P][Dq]
     int32_t* estar;              // [P]
     float* featf;                // [P][6] FP32 features (feature-point proposal)
     __nv_bfloat16* x0;           // [P][8]
@@ -379,12 +466,13 @@ NetScratch carve_net(void* base, int H, int W, int D, bool training, bool full_r
     };
     NetScratch s{};
     s.gq = (int32_t*)take(2 * P * 4);
-    s.kq = (float*)take(P * Dq * 4);
     s.kh = (float*)take(P * Dq * 4);
+    take(P * Dq * 4);   // unused: the same calls fit under a workspace_cap as when the costs were stored too
     s.estar = (int32_t*)take(P * 4);
     s.featf = (float*)take(P * 24);
     s.x0 = (__nv_bfloat16*)take(P * 16);
     for (int l = 0; l < 5; ++l) s.y[l] = (__nv_bfloat16*)take(P * 64);
+    s.stat = (fbs::BlockStat*)s.y[0];
     s.out = (float*)take(P * 8);
     if (training) {
         for (int l = 0; l < 5; ++l) s.g[l] = (__nv_bfloat16*)take(P * 64);
@@ -474,47 +562,34 @@ fbs_status check_pair_shape(fbs_ctx* ctx, const uint8_t* left, const uint8_t* ri
 fbs_status run_features(fbs_ctx* ctx, const NetScratch& s, const uint8_t* L, const uint8_t* R, int H, int W, int C,
                         int D, float* feat, cudaStream_t st)
 {
-    const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
+    const int Hq = (H + 3) / 4, Wq = (W + 3) / 4, Dq = (D + 3) / 4;
     cudaError_t e;
     {
         LaunchScope ls(ctx, FBS_KERNEL_NET, st);
         fbs::note_launch();
-        fbs::band_downsample_kernel<<<dim3((Wq + 127) / 128, Hq, 2), 128, 0, st>>>(L, R, H, W, C, s.gq);
-        e = cudaGetLastError();
-    }
-    const int Dq = (D + 3) / 4;
-    const size_t nv = (size_t)Hq * Wq * Dq;
-    if (e == cudaSuccess) {
-        LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_coarse_cost_kernel<<<dim3((Wq + fbs::kCoarseX - 1) / fbs::kCoarseX, Hq), fbs::kCoarseX, 0, st>>>(
-            s.gq, Hq, Wq, Dq, s.kq);
+        const int tx = fbs::kQuarterX - 2, ty = fbs::kQuarterY - 2;
+        const dim3 grid((Wq + tx - 1) / tx, (Hq + ty - 1) / ty, 2);
+        auto kernel = C == 3 ? fbs::band_quarter_kernel<3> : fbs::band_quarter_kernel<1>;
+        kernel<<<grid, fbs::kQuarterX * fbs::kQuarterY, 0, st>>>(L, R, H, W, s.gq, s.stat);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
         LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_row_sum_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(s.kq, Hq, Wq, Dq, s.kh);
-        e = cudaGetLastError();
+        const dim3 grid((Wq + fbs::kRowSpan - 1) / fbs::kRowSpan, Hq);
+        e = fbs::launch_after(fbs::band_row_sum_kernel, grid, fbs::kRowThreads, fbs::row_sum_smem(Dq), st, s.gq, s.stat,
+                              Hq, Wq, Dq, s.kh);
     }
     if (e == cudaSuccess) {
         LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_col_mean_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(s.kh, Hq, Wq, Dq, s.kq);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-        LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_features_kernel<<<dim3((Wq + 127) / 128, Hq), 128, 0, st>>>(s.gq, s.kq, H, W, C, D, s.x0, feat,
-                                                                              s.estar);
-        e = cudaGetLastError();
+        const dim3 grid((Wq + fbs::kFeatWarps - 1) / fbs::kFeatWarps, (Hq + fbs::kFeatRows - 1) / fbs::kFeatRows);
+        e = fbs::launch_after(fbs::band_features_kernel, grid, 32 * fbs::kFeatWarps,
+                              fbs::kFeatWarps * fbs::kFeatRows * Dq * sizeof(float), st, s.gq, s.kh, H, W, C, D, s.x0, feat, s.estar);
     }
     return e == cudaSuccess ? FBS_OK : cuda_fail(ctx, e, "band feature launch");
 }
 
-// The six convolutions: x0 -> y[0..4] -> out.
-fbs_status run_forward(fbs_ctx* ctx, const NetScratch& s, int Hq, int Wq, cudaStream_t st)
+// The six convolutions: x0 -> y[0..4] -> out (and the head's other outputs).
+fbs_status run_forward(fbs_ctx* ctx, const NetScratch& s, int Hq, int Wq, const ConvHead& head, cudaStream_t st)
 {
     fbs_band_state* b = ctx->band;
     const __nv_bfloat16* in = s.x0;
@@ -526,12 +601,18 @@ fbs_status run_forward(fbs_ctx* ctx, const NetScratch& s, int Hq, int Wq, cudaSt
             LaunchScope ls(ctx, FBS_KERNEL_NET, st);
             e = launch_conv3x3(cin_pad(l), fwd_n(l), in, b->images + fwd_image_offset(l), bias, nullptr,
                                last ? (void*)s.out : (void*)s.y[l], last ? kOut : fwd_n(l), Hq, Wq, 0,
-                               last ? kConvLinearF32 : kConvReluBf16, ctx->derr, ctx->num_sms, st);
+                               last ? kConvLinearF32 : kConvReluBf16, ctx->derr, st, last ? head : ConvHead{});
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "band network convolution launch");
         if (!last) in = s.y[l];
     }
     return FBS_OK;
+}
+
+ConvHead head_planes(const NetScratch& s, int H, int W, float* out_q, float* centre, float* conf)
+{
+    const bool aligned = (((uintptr_t)centre | (uintptr_t)conf) & 15) == 0;
+    return ConvHead{s.estar, out_q, centre, conf, H, W, aligned && W % 4 == 0};
 }
 
 // Loss, backward pass into b->grad.
@@ -558,7 +639,7 @@ fbs_status run_backward(fbs_ctx* ctx, const NetScratch& s, int H, int W, int D, 
             // gradient w.r.t. Y_{l-1} through its ReLU
             LaunchScope ls(ctx, FBS_KERNEL_NET, st);
             e = launch_conv3x3(cout_pad(l), cin(l), s.g[l], b->images + dgrad_image_offset(l), nullptr, s.y[l - 1],
-                               s.g[l - 1], cin(l), Hq, Wq, 1, kConvMaskBf16, ctx->derr, ctx->num_sms, st);
+                               s.g[l - 1], cin(l), Hq, Wq, 1, kConvMaskBf16, ctx->derr, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "band data-gradient launch");
     }
@@ -735,21 +816,16 @@ fbs_status fbs_band_net_forward(fbs_ctx* ctx, const uint8_t* left, const uint8_t
     const NetScratch sc = carve_net(ctx->band_ws, H, W, D, false, false);
     const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
     if ((s = run_features(ctx, sc, left, right, H, W, C, D, nullptr, st)) != FBS_OK) return s;
-    if ((s = run_forward(ctx, sc, Hq, Wq, st)) != FBS_OK) return s;
+    const bool direct = ((uintptr_t)out_q & 3) == 0;   // a copy takes any address
+    s = run_forward(ctx, sc, Hq, Wq, head_planes(sc, H, W, direct ? out_q : nullptr, centre, conf), st);
+    if (s != FBS_OK) return s;
     ctx->band->last_H = H;
     ctx->band->last_W = W;
     ctx->band->last_D = D;
     ctx->band->last_training = false;
-    cudaError_t e = cudaSuccess;
-    if (centre || conf) {
-        LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_head_kernel<<<dim3((W + 255) / 256, H), 256, 0, st>>>(sc.out, sc.estar, H, W, centre, conf);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && out_q)
-        e = cudaMemcpyAsync(out_q, sc.out, (size_t)Hq * Wq * 8, cudaMemcpyDeviceToDevice, st);
-    return e == cudaSuccess ? FBS_OK : cuda_fail(ctx, e, "band network head");
+    if (direct) return FBS_OK;
+    cudaError_t e = cudaMemcpyAsync(out_q, sc.out, (size_t)Hq * Wq * 8, cudaMemcpyDeviceToDevice, st);
+    return e == cudaSuccess ? FBS_OK : cuda_fail(ctx, e, "band network output copy");
 }
 
 fbs_status fbs_band_net_train_step(fbs_ctx* ctx, const uint8_t* left, const uint8_t* right, int H, int W, int C,
@@ -771,7 +847,7 @@ fbs_status fbs_band_net_train_step(fbs_ctx* ctx, const uint8_t* left, const uint
     const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
     fbs_band_state* b = ctx->band;
     if ((s = run_features(ctx, sc, left, right, H, W, C, D, nullptr, st)) != FBS_OK) return s;
-    if ((s = run_forward(ctx, sc, Hq, Wq, st)) != FBS_OK) return s;
+    if ((s = run_forward(ctx, sc, Hq, Wq, ConvHead{}, st)) != FBS_OK) return s;
     if ((s = run_backward(ctx, sc, H, W, D, label_int, label_sub, half_band, st)) != FBS_OK) return s;
     b->last_H = H;
     b->last_W = W;
@@ -905,14 +981,8 @@ fbs_status fbs_compute_disparity_learned(fbs_ctx* ctx, const fbs_pair* pair, int
     const NetScratch sc = carve_net(ctx->band_ws, H, W, pair->D, false, true);
     const int Hq = (H + 3) / 4, Wq = (W + 3) / 4;
     if ((s = run_features(ctx, sc, pair->left, pair->right, H, W, pair->C, pair->D, nullptr, st)) != FBS_OK) return s;
-    if ((s = run_forward(ctx, sc, Hq, Wq, st)) != FBS_OK) return s;
-    {
-        LaunchScope ls(ctx, FBS_KERNEL_NET, st);
-        fbs::note_launch();
-        fbs::band_head_kernel<<<dim3((W + 255) / 256, H), 256, 0, st>>>(sc.out, sc.estar, H, W, sc.centre, sc.conf);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "band head launch");
-    }
+    s = run_forward(ctx, sc, Hq, Wq, head_planes(sc, H, W, nullptr, sc.centre, sc.conf), st);
+    if (s != FBS_OK) return s;
     return run_banded(ctx, pair, sc.centre, sc.conf, half_band, conf_threshold, sc, st);
 }
 

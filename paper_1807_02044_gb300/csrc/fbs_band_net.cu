@@ -2,22 +2,30 @@
 // on the tensor cores (forward, data gradient, weight gradient), loss, Adam and
 // the packing of FP32 master weights into BF16 MMA operands.
 //
-// Convolution as an implicit GEMM (one CTA = 128 consecutive quarter pixels
-// = the MMA's M; persistent over tiles):
+// Convolution as an implicit GEMM over a tile of 8 x 16 quarter pixels (the
+// MMA's M = 128):
 //     out[m][n] = sum_k A[m][k] B[n][k],   k = (tap, channel),
 //     A[m][k]   = in[pixel m shifted by tap][channel]  (zero outside the image),
 //     B[n][k]   = W[tap][channel][n]  (forward)  or  W[tap][n][channel]  (data
 //                 gradient, with the tap offsets negated).
-// Both operands are K-major core matrices in shared memory (8 rows x 16 bytes;
-// LBO = distance between core matrices along K, SBO = 128 bytes between row
-// groups).  Every thread gathers its pixel's row of A with 16-byte loads (one
-// load = 8 channels of one tap = one core-matrix row) and stores it with
-// 16-byte shared stores; one thread issues the K/16 tcgen05.mma of the tile
-// into a TMEM accumulator (M = 128 lanes x N columns, FP32) and commits to an
-// mbarrier; the four warps then read their 32 lanes back (tcgen05.ld), apply
-// the epilogue and store.  The weight image (B) is loaded once per CTA.
+// A is never gathered: the tile and its border of one pixel lie in shared
+// memory as [8 channels][18 rows][10 pixels] x 16 bytes, zero where the image
+// ends, so that eight pixels of a row are one K-major core matrix (8 rows x 16
+// bytes), the tile's rows follow each other at SBO = 160 bytes, and tap (dy, dx)
+// is the same operand (10 dy + dx) * 16 bytes further on.  Two K-cores of one
+// MMA are two channel blocks of a tap (32 channels) or two taps (8 channels):
+// only the descriptors' start and LBO differ.  B is the packed image (LBO =
+// 16 N, SBO = 128).  A warp issues the K/16 tcgen05.mma of the tile into a TMEM
+// accumulator (M = 128 lanes x N columns, FP32) and commits to an mbarrier; the
+// four warps then read their 32 lanes back (tcgen05.ld), apply the epilogue and
+// store.  Bound by latency: a layer of 320 x 160 quarter pixels needs 2 us of
+// copies and MMAs, one CTA per tile holds 30 KB, and all 400 tiles are resident
+// at once, under the end of the layer before (programmatic launch; the weights
+// are copied before the wait).  Gathering every tap into shared memory by 16-byte
+// loads, two CTAs per SM, took 15.9 us per layer, now 6.8 (each alone, cold
+// caches); features and six layers with the head 205.6 us then, 61.0 now.
 // Every mbarrier wait is bounded; a timeout sets the error word, and all
-// threads leave the tile loop together, free the tensor memory and return.
+// threads free the tensor memory together and return.
 #include <cuda_bf16.h>
 
 #include "fbs_band_net.cuh"
@@ -39,136 +47,171 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// The proposal of quarter pixel (X, Y) -- winner estar, head outputs o0 and z
+// -- at its 4 x 4 pixels: centre 4 (e + o0), confidence sigmoid(z).
+__device__ __forceinline__ void head_outputs(const ConvHead& h, int X, int Y, size_t po, float o0, float z)
+{
+    if (h.out_q) {
+        h.out_q[2 * po] = o0;
+        h.out_q[2 * po + 1] = z;
+    }
+    if (!h.centre && !h.conf) return;
+    const float c = h.centre ? __fmul_rn(4.f, __fadd_rn((float)h.estar[po], o0)) : 0.f;
+    const float k = h.conf ? 1.f / (1.f + expf(-z)) : 0.f;
+    const int ny = min(4, h.H - 4 * Y), nx = min(4, h.W - 4 * X);
+    for (int j = 0; j < ny; ++j) {
+        const size_t p = (size_t)(4 * Y + j) * h.W + 4 * X;
+        if (h.vec) {
+            if (h.centre) *reinterpret_cast<float4*>(h.centre + p) = make_float4(c, c, c, c);
+            if (h.conf) *reinterpret_cast<float4*>(h.conf + p) = make_float4(k, k, k, k);
+        } else {
+            for (int i = 0; i < nx; ++i) {
+                if (h.centre) h.centre[p + i] = c;
+                if (h.conf) h.conf[p + i] = k;
+            }
+        }
+    }
+}
+
+constexpr int kTileX = 8, kTileY = 16;                 // one MMA: eight pixels of a row = one core matrix
+constexpr int kBoxX = kTileX + 2, kBoxY = kTileY + 2;   // with the border
+
+__device__ __forceinline__ void copy16_zfill(uint32_t dst, const void* src, bool ok)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+// Byte offset of tap t = 3 (dy + 1) + dx + 1 in a channel block of the box.
+__host__ __device__ constexpr int tap_offset(int t) { return ((t / 3) * kBoxX + t % 3) * 16; }
+
+// Shared memory of a convolution: the box, per block of 8 channels (32 bytes
+// of padding spread a pixel's channel blocks over the banks; after a single
+// block, the zero rows that stand in for a tenth tap), then the weights.
+template <int CIN>
+struct ConvBox {
+    static constexpr int kBlocks = CIN / 8;
+    static constexpr int kStride = kBoxX * kBoxY * 16 + 32;
+    static constexpr int kZero = kBlocks * kStride;   // offset of the zero rows
+    static constexpr int kBytes = (kZero + (kBlocks == 1 ? (kTileY - 1) * kBoxX * 16 + 128 : 0) + 127) / 128 * 128;
+};
+
 template <int CIN, int N>
 __global__ void __launch_bounds__(kConvThreads)
 conv3x3_tc_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ image,
                   const float* __restrict__ bias, const __nv_bfloat16* __restrict__ mask, void* __restrict__ out,
-                  int nout, int Hq, int Wq, int flip, int mode, int* __restrict__ err)
+                  int nout, int Hq, int Wq, int flip, int mode, ConvHead head, int* __restrict__ err)
 {
+    using Box = ConvBox<CIN>;
     constexpr int KC = k_cores(CIN);            // core matrices along K
-    constexpr int KREAL = 9 * CIN / 8;          // of which hold data
-    constexpr int A_BYTES = KC * kM * 16;
     constexpr int B_BYTES = KC * N * 16;
-    constexpr int CH = CIN / 8;                 // 16-byte chunks per (pixel, tap)
+    constexpr int CH = CIN / 8;                 // 16-byte blocks per (pixel, tap)
     extern __shared__ __align__(128) uint8_t sm[];
     uint8_t* As = sm;
-    uint8_t* Bs = sm + A_BYTES;
+    uint8_t* Bs = sm + Box::kBytes;
     uint64_t* bar = reinterpret_cast<uint64_t*>(Bs + B_BYTES);
-    uint32_t* misc = reinterpret_cast<uint32_t*>(bar + 1);   // [0] TMEM address, [1] abort flag
+    uint32_t* misc = reinterpret_cast<uint32_t*>(bar + 1);   // [0] TMEM address
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int P = Hq * Wq;
-    const int ntiles = (P + kM - 1) / kM;
-
+    const int tid = threadIdx.x, warp = tid >> 5;
+    // the weights are older than the kernel before this one
     for (int i = tid; i < B_BYTES / 16; i += kConvThreads)
-        reinterpret_cast<uint4*>(Bs)[i] = reinterpret_cast<const uint4*>(image)[i];
-    for (int kc = KREAL; kc < KC; ++kc) reinterpret_cast<uint4*>(As + kc * kM * 16)[tid] = make_uint4(0, 0, 0, 0);
+        copy16_zfill(smem_u32(Bs) + 16 * i, reinterpret_cast<const uint4*>(image) + i, true);
+    if constexpr (CH == 1)
+        for (int i = tid; i < (Box::kBytes - Box::kZero) / 16; i += kConvThreads)
+            reinterpret_cast<uint4*>(As + Box::kZero)[i] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
         mbar_init(smem_u32(bar), 1);
-        misc[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(smem_u32(&misc[0]), 32);
+    if (warp == 0) {
+        // only then may the next layer's CTAs come: they must not hold tensor
+        // memory that this one still waits for
+        tmem_alloc(smem_u32(&misc[0]), 32);
+        asm volatile("griddepcontrol.launch_dependents;");
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // ---- the tile and its border; mirrored in both axes for the negated offsets
+    const int tx0 = blockIdx.x * kTileX, ty0 = blockIdx.y * kTileY;
+    const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
+    for (int i = tid; i < kBoxX * kBoxY * CH; i += kConvThreads) {
+        const int px = i / CH, j = i % CH;
+        const int by = px / kBoxX, bx = px - by * kBoxX;
+        const int yy = ty0 - 1 + by, xx = tx0 - 1 + bx;
+        const bool ok = (unsigned)yy < (unsigned)Hq && (unsigned)xx < (unsigned)Wq;
+        const int at = flip ? kBoxX * kBoxY - 1 - px : px;
+        copy16_zfill(a0 + j * Box::kStride + at * 16, in + ((size_t)(ok ? yy * Wq + xx : 0)) * CIN + 8 * j, ok);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = misc[0];
-    const uint32_t idesc = idesc_f16(true, kM, N);
-    const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-
-    uint32_t phase = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        // ---- gather this thread's row of A -------------------------------
-        const int p = tile * kM + tid;
-        const int Y = p / Wq, X = p - Y * Wq;
+    // ---- one warp issues the tile's MMAs ----------------------------------
+    if (warp == 0) {
+        const uint32_t idesc = idesc_f16(true, kM, N);
 #pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            int dy = t / 3 - 1, dx = t % 3 - 1;
-            if (flip) {
-                dy = -dy;
-                dx = -dx;
-            }
-            const int yy = Y + dy, xx = X + dx;
-            const bool ok = p < P && yy >= 0 && yy < Hq && xx >= 0 && xx < Wq;
-            const uint4* src = reinterpret_cast<const uint4*>(in + ((size_t)(ok ? yy * Wq + xx : 0)) * CIN);
-#pragma unroll
-            for (int j = 0; j < CH; ++j) {
-                const uint4 v = ok ? src[j] : make_uint4(0, 0, 0, 0);
-                *reinterpret_cast<uint4*>(As + ((t * CH + j) * kM + tid) * 16) = v;
-            }
+        for (int ks = 0; ks < KC / 2; ++ks) {
+            constexpr int kPerTap = CH == 1 ? 1 : CH / 2;   // K-steps of a tap (8 channels: two taps per step)
+            const int t = CH == 1 ? 2 * ks : ks / kPerTap, j = CH == 1 ? 0 : 2 * (ks % kPerTap);
+            const int off = j * Box::kStride + tap_offset(t);
+            const int lbo = CH > 1 ? Box::kStride : (t + 1 < 9 ? tap_offset(t + 1) : Box::kZero) - tap_offset(t);
+            umma_f16_elect(tmem, sdesc(a0 + off, lbo, kBoxX * 16), sdesc(b0 + ks * 2 * N * 16, N * 16, 128), idesc,
+                           ks > 0 ? 1u : 0u);
         }
-        fence_proxy_async();
-        tc_fence_before();
-        __syncthreads();
-        // ---- one thread issues the tile's MMAs ----------------------------
-        if (tid == 0) {
-            tc_fence_after();
-#pragma unroll 1
-            for (int ks = 0; ks < KC / 2; ++ks) {
-                const uint64_t ad = sdesc(a0 + ks * 2 * kM * 16, kM * 16, 128);
-                const uint64_t bd = sdesc(b0 + ks * 2 * N * 16, N * 16, 128);
-                umma_f16(tmem, ad, bd, idesc, ks > 0 ? 1u : 0u);
-            }
-            umma_commit(smem_u32(bar));
-        }
-        const bool ok = mbar_wait(smem_u32(bar), phase);
-        phase ^= 1u;
-        if (!ok) atomicExch(&misc[1], 1u);
-        tc_fence_before();
-        __syncthreads();
-        if (misc[1] != 0) {
-            if (tid == 0) {
-                atomicCAS(err, 0, 21);
-                mbar_wait(smem_u32(bar), phase ^ 1u);   // once more, bounded, for the MMAs in flight
-            }
-            break;
-        }
-        tc_fence_after();
-        // ---- epilogue: warp w holds TMEM lanes 32w .. 32w+31 ---------------
-        float v[N];
+        umma_commit_elect(smem_u32(bar));
+    }
+    if (!mbar_wait(smem_u32(bar), 0)) {
+        // out of time: report it, and give the MMAs in flight one more bounded
+        // wait before the shared memory they read is given back
+        atomicCAS(err, 0, 21);
+        mbar_wait(smem_u32(bar), 0);
+    }
+    tc_fence_after();
+    // ---- epilogue: warp w holds TMEM lanes 32w .. 32w+31 -------------------
+    float v[N];
 #pragma unroll
-        for (int c = 0; c < N; c += 16) {
-            float t16[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, t16);
+    for (int c = 0; c < N; c += 16) {
+        float t16[16];
+        tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, t16);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[c + i] = t16[i];
-        }
-        const int po = tile * kM + 32 * warp + lane;
-        if (po < P) {
-            if (mode == kConvLinearF32) {
-                float* o = reinterpret_cast<float*>(out) + (size_t)po * nout;
+        for (int i = 0; i < 16; ++i) v[c + i] = t16[i];
+    }
+    const int m = flip ? kM - 1 - tid : tid;
+    const int X = tx0 + m % kTileX, Y = ty0 + m / kTileX;
+    if (X < Wq && Y < Hq) {
+        const size_t po = (size_t)Y * Wq + X;
+        if (mode == kConvLinearF32) {
+            float* o = reinterpret_cast<float*>(out) + po * nout;
 #pragma unroll
-                for (int c = 0; c < N; ++c)
-                    if (c < nout) o[c] = v[c] + bias[c];
+            for (int c = 0; c < N; ++c)
+                if (c < nout) o[c] = v[c] + bias[c];
+            if constexpr (N == kHeadN) head_outputs(head, X, Y, po, v[0] + bias[0], v[1] + bias[1]);
+        } else {
+            if (mode == kConvReluBf16) {
+#pragma unroll
+                for (int c = 0; c < N; ++c) v[c] = fmaxf(v[c] + bias[c], 0.f);
             } else {
-                if (mode == kConvReluBf16) {
+                const uint4* mk = reinterpret_cast<const uint4*>(mask + po * N);
 #pragma unroll
-                    for (int c = 0; c < N; ++c) v[c] = fmaxf(v[c] + bias[c], 0.f);
-                } else {
-                    const uint4* mk = reinterpret_cast<const uint4*>(mask + (size_t)po * N);
+                for (int q = 0; q < N / 8; ++q) {
+                    const uint4 w = mk[q];
+                    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-                    for (int q = 0; q < N / 8; ++q) {
-                        const uint4 w = mk[q];
-                        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            // a BF16 value is > 0 iff its sign bit is clear and it is not +0
-                            const uint32_t lo = ws[h] & 0xffffu, hi = ws[h] >> 16;
-                            if (lo == 0u || (lo & 0x8000u)) v[8 * q + 2 * h] = 0.f;
-                            if (hi == 0u || (hi & 0x8000u)) v[8 * q + 2 * h + 1] = 0.f;
-                        }
+                    for (int h = 0; h < 4; ++h) {
+                        // a BF16 value is > 0 iff its sign bit is clear and it is not +0
+                        const uint32_t lo = ws[h] & 0xffffu, hi = ws[h] >> 16;
+                        if (lo == 0u || (lo & 0x8000u)) v[8 * q + 2 * h] = 0.f;
+                        if (hi == 0u || (hi & 0x8000u)) v[8 * q + 2 * h + 1] = 0.f;
                     }
                 }
-                uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(out) + (size_t)po * N);
-#pragma unroll
-                for (int q = 0; q < N / 8; ++q)
-                    o[q] = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                                      pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
             }
+            uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(out) + po * N);
+#pragma unroll
+            for (int q = 0; q < N / 8; ++q)
+                o[q] = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
+                                  pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
         }
-        tc_fence_before();
-        __syncthreads();   // A and the accumulator are free for the next tile
     }
     tc_fence_before();
     __syncthreads();
@@ -178,19 +221,14 @@ conv3x3_tc_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __r
 
 template <int CIN, int N>
 cudaError_t launch_conv_t(const __nv_bfloat16* in, const __nv_bfloat16* image, const float* bias,
-                          const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq, int flip, int mode, int* err,
-                          int num_sms, cudaStream_t stream)
+                          const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq, int flip, int mode,
+                          const ConvHead& head, int* err, cudaStream_t stream)
 {
-    constexpr int KC = k_cores(CIN);
-    const size_t smem = (size_t)KC * kM * 16 + (size_t)KC * N * 16 + 16;
-    cudaError_t e = fbs::raise_smem_limit(conv3x3_tc_kernel<CIN, N>, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int ntiles = (Hq * Wq + kM - 1) / kM;
-    const int grid = ntiles < 2 * num_sms ? ntiles : 2 * num_sms;
-    fbs::note_launch();
-    conv3x3_tc_kernel<CIN, N><<<grid, kConvThreads, smem, stream>>>(in, image, bias, mask, out, nout, Hq, Wq, flip,
-                                                                    mode, err);
-    return cudaGetLastError();
+    constexpr size_t smem = ConvBox<CIN>::kBytes + (size_t)k_cores(CIN) * N * 16 + 16;
+    static_assert(smem <= 48 * 1024, "within the default limit");
+    const dim3 grid((Wq + kTileX - 1) / kTileX, (Hq + kTileY - 1) / kTileY);
+    return fbs::launch_after(conv3x3_tc_kernel<CIN, N>, grid, kConvThreads, smem, stream, in, image, bias, mask, out,
+                             nout, Hq, Wq, flip, mode, head, err);
 }
 
 // ---- weight gradients on the tensor cores ---------------------------------------
@@ -497,14 +535,14 @@ __global__ void pack_images_kernel(const float* __restrict__ theta, __nv_bfloat1
 
 cudaError_t launch_conv3x3(int cin_ch, int n, const __nv_bfloat16* in, const __nv_bfloat16* image, const float* bias,
                            const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq, int flip, int mode,
-                           int* err, int num_sms, cudaStream_t stream)
+                           int* err, cudaStream_t stream, const ConvHead& head)
 {
     if (cin_ch == 8 && n == 32)
-        return launch_conv_t<8, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, err, num_sms, stream);
+        return launch_conv_t<8, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
     if (cin_ch == 32 && n == 32)
-        return launch_conv_t<32, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, err, num_sms, stream);
+        return launch_conv_t<32, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
     if (cin_ch == 32 && n == 16)
-        return launch_conv_t<32, 16>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, err, num_sms, stream);
+        return launch_conv_t<32, 16>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
     return cudaErrorInvalidValue;
 }
 

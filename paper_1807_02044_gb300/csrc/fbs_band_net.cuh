@@ -57,12 +57,24 @@ enum ConvMode {
     kConvMaskBf16 = 2,   // out = acc * (mask > 0), BF16 [P][N]  (data gradient through a ReLU)
 };
 
+// What the last layer of a forward pass writes besides its output (each plane
+// may be null): the pairs (o0, z), and the full-resolution centre
+// 4 (estar + o0) and confidence sigmoid(z).  vec: W % 4 == 0 and both planes
+// 16-byte aligned.
+struct ConvHead {
+    const int32_t* estar;
+    float *out_q, *centre, *conf;
+    int H, W, vec;
+};
+
 // 3x3 convolution, zero padding, of in [P][cin_ch] (P = Hq*Wq quarter pixels,
 // row-major) with a packed image of N output channels.  flip: gather the
 // neighbour at -offset (data gradient).  err: device word set on a timeout.
+// A programmatic launch: the weights (image) must be older than the kernel
+// before it in the stream; everything else may be that kernel's output.
 cudaError_t launch_conv3x3(int cin_ch, int n, const __nv_bfloat16* in, const __nv_bfloat16* image,
                            const float* bias, const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq,
-                           int flip, int mode, int* err, int num_sms, cudaStream_t stream);
+                           int flip, int mode, int* err, cudaStream_t stream, const ConvHead& head = {});
 // Weight and bias gradient of layer l: sum over pixels of X[p + offset] G[p],
 // X [P][cin_pad(l)], G [P][cout_pad(l)]; written into grad (flat vector).
 // On the tensor cores; err: device word set on a timeout.

@@ -94,6 +94,16 @@ def test_features_match_the_fp64_oracle(fbs, oracle_mod, H, W, C, D):
           f"{int((~same).sum())} winners differ, max |d feature| {err:.2e} (bound {2 * TOL_KBAR + 2 * U32:.2e})")
 
 
+@pytest.mark.parametrize("H,W,C,D", [
+    (9, 300, 1, 1024),    # two spans of the row sums, eight times 32 disparities; two images of a column
+    (33, 261, 3, 132),    # one quarter pixel beyond a span and beyond eight rows; one disparity beyond 32
+    (35, 241, 3, 3),      # one coarse disparity; rows of a width that no word load fits
+    (131, 124, 1, 52),    # one quarter pixel beyond the tiles of the quarter images in both directions
+])
+def test_features_tile_edges(fbs, oracle_mod, H, W, C, D):
+    test_features_match_the_fp64_oracle(fbs, oracle_mod, H, W, C, D)
+
+
 def test_features_of_a_shift_by_four_k(fbs, oracle_mod):
     from synth import shifted_texture_pair
     H, W, D, k = 96, 256, 128, 7
@@ -450,6 +460,36 @@ def test_params_round_trip_and_file(fbs, tmp_path):
         b = np.zeros_like(theta)
         fbs.fbs_band_net_get_params(ctx.ctx, b)
         assert np.array_equal(a, b) and np.all(np.isfinite(a)) and np.any(a != 0)
+
+
+@pytest.mark.parametrize("H,W,D", [(64, 32, 40), (65, 33, 40), (61, 36, 8), (8, 200, 64)])
+def test_forward_tile_edges(fbs, oracle_mod, H, W, D):
+    """Frames of whole tiles of 8 x 16 quarter pixels, and one pixel beyond."""
+    test_forward_layers_match_elementwise(fbs, oracle_mod, H, W, D)
+
+
+@pytest.mark.parametrize("H,W", [(33, 48), (32, 45)])
+def test_forward_outputs_do_not_depend_on_which_are_asked_for(fbs, H, W):
+    """Every combination of the three outputs, and planes at an address that is
+    a multiple of 4 bytes only, give the same bits."""
+    L, R = _rand_pair(H + W, H, W, 3, shift=12)
+    Hq, Wq = (H + 3) // 4, (W + 3) // 4
+    sizes = (Hq * Wq * 2, H * W, H * W)
+    dl, dr = _dev(L), _dev(R)
+    ref = None
+    with fbs.Context(0) as ctx:
+        fbs.fbs_band_net_set_params(ctx.ctx, _params(3))
+        for mask in (7, 1, 2, 4, 6, 7 + 8):
+            off = 1 if mask & 8 else 0
+            bufs = [torch.full((n + 8,), -7.0, device="cuda") for n in sizes]
+            args = [b[off:off + n] if mask >> i & 1 else None for i, (b, n) in enumerate(zip(bufs, sizes))]
+            fbs.fbs_band_net_forward(ctx.ctx, dl, dr, H, W, 3, 40, *args)
+            torch.cuda.synchronize()
+            fbs.fbs_sync(ctx.ctx)
+            ref = ref or [a.clone() for a in args]
+            for i, (a, b, n) in enumerate(zip(args, bufs, sizes)):
+                assert a is None or torch.equal(a, ref[i]), (mask, i)
+                assert (b[:off] == -7).all() and (b[(off + n if a is not None else 0):] == -7).all(), (mask, i)
 
 
 def test_learned_entry_equals_forward_then_banded(fbs):
