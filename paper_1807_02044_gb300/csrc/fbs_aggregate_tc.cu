@@ -213,12 +213,7 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
         // computed only for the pixel rows whose window it lies in (zeros for
         // the other).  PM says which pairs exist: all NPT (odd radius), all
         // but the last one of phase 1 (even radius), or per-pair flags.
-        // Colour distance: |q - p|^2 = |q|^2 + |p|^2 - 2 q.p, exact in integers
-        // (|q|^2 comes with the guide tile, q.p is one dp4a).  It is below 2^23,
-        // so carrying kMagic in |p|^2 turns the integer into the bits of
-        // 2^23 + c and one packed subtraction gives both columns' c as exact
-        // floats; the exponent argument c*neg_kr + (sx + sy) of a column pair is
-        // one packed add and one packed FMA (the same roundings as scalar code).
+        // (the weights of a pair: tc_weights.)
         const int ty = 2 * (warp >> 2), rq = warp & 3;
         const int xm = lane & 15, h = lane >> 4;
         const int m0 = 16 * ty + xm;   // A row of the upper pixel; the lower one is m0 + 16
@@ -235,7 +230,6 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
         const uint32_t gcol = (uint32_t)(c0 + 2 * h) * 8;   // byte offset of pair 0 in a guide row
         const uint32_t g_row = (uint32_t)KW * 8;            // bytes of one guide row
         const float ninf = __int_as_float(0xff800000);
-        const uint64_t magic2 = f2_pack(-8388608.f, -8388608.f);
         const uint64_t nkr2 = f2_pack(p.neg_kr, p.neg_kr);
         const unsigned two_rho = (unsigned)(2 * p.rho);
         uint32_t gs = 0, gu = 0, t = 0;   // stage slot and use count of the next stage
@@ -255,7 +249,8 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
             // the image only feed their own accumulator rows, never stored)
             const uint2 pc0 = *(const uint2*)(gt + (ty + p.rho) * g_row + kcen * 8);
             const uint2 pc1 = *(const uint2*)(gt + (ty + 1 + p.rho) * g_row + kcen * 8);
-            const uint32_t pcol0 = pc0.x, pp0 = pc0.y + kMagic, pcol1 = pc1.x, pp1 = pc1.y + kMagic;
+            const uint32_t pcol0 = pc0.x, pcol1 = pc1.x;
+            const uint64_t norm0 = tc_norm(pc0.y), norm1 = tc_norm(pc1.y);
             uint64_t sxp[NPT];
 #pragma unroll
             for (int j = 0; j < NPT; ++j) {
@@ -271,8 +266,7 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
             const uint8_t* gth = gt + gcol;
             auto row_pairs = [&](uint8_t* arow, const uint8_t* grow, uint64_t sy0, uint64_t sy1, int which)
                                  __attribute__((always_inline)) {
-                tc_row_pairs<BF16, NPT>(arow, grow, po, on, sxp, sy0, sy1, which, pcol0, pp0, pcol1, pp1, magic2,
-                                        nkr2);
+                tc_row_pairs<BF16, NPT>(arow, grow, po, on, sxp, sy0, sy1, which, pcol0, norm0, pcol1, norm1, nkr2);
             };
             const int hr_lo = max(0, p.rho - ty0);
             const int hr_hi = min(p.NH, p.H - ty0 + p.rho);

@@ -215,7 +215,6 @@ __device__ __forceinline__ ProducerState produce_run(const TcBatchPair* __restri
     const uint32_t g_row = (uint32_t)KW * 8;
     const uint32_t a_row = (uint32_t)(KW / 8) * kALbo;
     const float ninf = __int_as_float(0xff800000);
-    const uint64_t magic2 = f2_pack(-8388608.f, -8388608.f);
     const uint64_t nkr2 = f2_pack(P.neg_kr, P.neg_kr);
     const unsigned two_rho = (unsigned)(2 * rho);
     // spatial y-term of row offset i - rho, (ks dy^2, ks dy^2): the one-pair
@@ -240,7 +239,8 @@ __device__ __forceinline__ ProducerState produce_run(const TcBatchPair* __restri
         const uint8_t* gt = g_base + tb * g_slot;
         const uint2 pc0 = *(const uint2*)(gt + (ty + rho) * g_row + kcen * 8);
         const uint2 pc1 = *(const uint2*)(gt + (ty + 1 + rho) * g_row + kcen * 8);
-        const uint32_t pcol0 = pc0.x, pp0 = pc0.y + kMagic, pcol1 = pc1.x, pp1 = pc1.y + kMagic;
+        const uint32_t pcol0 = pc0.x, pcol1 = pc1.x;
+        const uint64_t norm0 = tc_norm(pc0.y), norm1 = tc_norm(pc1.y);
         uint64_t sxp[NPT];
 #pragma unroll
         for (int j = 0; j < NPT; ++j) {
@@ -255,7 +255,7 @@ __device__ __forceinline__ ProducerState produce_run(const TcBatchPair* __restri
         const uint8_t* gth = gt + gcol;
         auto row_pairs = [&](uint8_t* arow, const uint8_t* grow, uint64_t sy0, uint64_t sy1, int which)
                              __attribute__((always_inline)) {
-            tc_row_pairs<BF16, NPT>(arow, grow, po, on, sxp, sy0, sy1, which, pcol0, pp0, pcol1, pp1, magic2, nkr2);
+            tc_row_pairs<BF16, NPT>(arow, grow, po, on, sxp, sy0, sy1, which, pcol0, norm0, pcol1, norm1, nkr2);
         };
         const int hr_lo = max(0, rho - ty0);
         const int hr_hi = min(NH, H - ty0 + rho);

@@ -36,9 +36,13 @@ constexpr int kMaxR = 8;          // window rows per stage, at most
 // shared-memory banks.
 constexpr uint32_t kALbo = 2048 + 64;
 constexpr int kMaxRho2 = 2 * 24 + 1;   // row offsets -rho .. rho of the largest radius
-// 2^23 as an FP32 bit pattern: for 0 <= c < 2^23 the pattern kMagic + c is the
-// float 2^23 + c exactly, so subtracting 2^23 gives float(c) exactly.
+// A guide entry q has |q|^2 - 2 q.p = -|p|^2 .. 255^2 * 3 for a pixel p; kBias more
+// is in 0 .. 2^23 - 1, and for such a c the FP32 bit pattern kMagic + c is the
+// float 2^23 + c exactly.  kMagicDot is the addend of q.p that puts kMagic +
+// kBias into |q|^2 - 2 (q.p + kMagicDot), modulo 2^32.
 constexpr uint32_t kMagic = 0x4B000000u;
+constexpr uint32_t kBias = 1u << 18;
+constexpr uint32_t kMagicDot = 0u - (kMagic + kBias) / 2;
 
 inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
@@ -105,20 +109,28 @@ __device__ __forceinline__ void raise_abort(volatile uint32_t* abort_flag, int* 
 
 // The two 16-bit weights of one column pair of one pixel, Eq. (7)-(8).
 // Colour distance: |q - p|^2 = |q|^2 + |p|^2 - 2 q.p, exact in integers (|q|^2
-// comes with the guide entry, q.p is one dp4a).  It is below 2^23, so carrying
-// kMagic in pp = |p|^2 + kMagic turns the integer into the bits of 2^23 + c and
-// one packed subtraction (magic2 = -2^23 twice) gives both columns' c as exact
-// floats; the exponent argument c * neg_kr + (sx + sy) is one packed FMA.
+// comes with the guide entry, q.p is one dp4a).  Two instructions per column
+// give the bits of the float 2^23 + kBias + |q|^2 - 2 q.p, and one packed
+// addition of norm = |p|^2 - 2^23 - kBias (tc_norm) both columns' exact c; the
+// exponent argument c * neg_kr + (sx + sy) is one packed FMA.  (The producers are
+// bound by issue; |p|^2 added as an integer is one instruction more per weight:
+// 1280 x 960, D = 128, radius 15 694 us against 669, 767 x 575, D = 93, radius 11
+// 163 against 157.)
 template <bool BF16>
-__device__ __forceinline__ uint32_t tc_weights(const uint4 q, uint32_t pcol, uint32_t pp, uint64_t sxy,
-                                               uint64_t magic2, uint64_t nkr2)
+__device__ __forceinline__ uint32_t tc_weights(const uint4 q, uint32_t pcol, uint64_t norm, uint64_t sxy,
+                                               uint64_t nkr2)
 {
-    const uint32_t e0 = q.y + pp - 2u * __dp4a(q.x, pcol, 0u);
-    const uint32_t e1 = q.w + pp - 2u * __dp4a(q.z, pcol, 0u);
-    const uint64_t c = f2_add(u2_pack(e0, e1), magic2);
+    const uint32_t e0 = q.y - 2u * __dp4a(q.x, pcol, kMagicDot);
+    const uint32_t e1 = q.w - 2u * __dp4a(q.z, pcol, kMagicDot);
+    const uint64_t c = f2_add(u2_pack(e0, e1), norm);
     float a0, a1;
     f2_unpack(f2_fma(c, nkr2, sxy), a0, a1);
     return pack_16x2<BF16>(ex2_approx(a0), ex2_approx(a1));
+}
+__device__ __forceinline__ uint64_t tc_norm(uint32_t sq)
+{
+    const float v = (float)((int)sq - (1 << 23) - (int)kBias);   // exact
+    return f2_pack(v, v);
 }
 
 // Byte offsets of a producer thread's column pairs in a window row of the A
@@ -144,8 +156,8 @@ __device__ __forceinline__ TcPairOffsets tc_pair_offsets(int u, int m0)
 template <bool BF16, int NPT>
 __device__ __forceinline__ void tc_row_pairs(uint8_t* arow, const uint8_t* grow, const TcPairOffsets po,
                                              const bool (&on)[NPT], const uint64_t (&sxp)[NPT], uint64_t sy0,
-                                             uint64_t sy1, int which, uint32_t pcol0, uint32_t pp0, uint32_t pcol1,
-                                             uint32_t pp1, uint64_t magic2, uint64_t nkr2)
+                                             uint64_t sy1, int which, uint32_t pcol0, uint64_t norm0, uint32_t pcol1,
+                                             uint64_t norm1, uint64_t nkr2)
 {
     // at most 5 pairs at a time: their loads first
 #pragma unroll
@@ -161,9 +173,9 @@ __device__ __forceinline__ void tc_row_pairs(uint8_t* arow, const uint8_t* grow,
             const int j = j0 + i;
             if (!on[j]) continue;
             uint8_t* a = arow + ((j & 1) ? po.odd : po.even) + (j >> 1) * kALbo;
-            *(uint32_t*)a = (which & 1) ? tc_weights<BF16>(q[i], pcol0, pp0, f2_add(sxp[j], sy0), magic2, nkr2) : 0u;
+            *(uint32_t*)a = (which & 1) ? tc_weights<BF16>(q[i], pcol0, norm0, f2_add(sxp[j], sy0), nkr2) : 0u;
             *(uint32_t*)(a + 256) =
-                (which & 2) ? tc_weights<BF16>(q[i], pcol1, pp1, f2_add(sxp[j], sy1), magic2, nkr2) : 0u;
+                (which & 2) ? tc_weights<BF16>(q[i], pcol1, norm1, f2_add(sxp[j], sy1), nkr2) : 0u;
         }
     }
 }
@@ -173,6 +185,15 @@ __device__ __forceinline__ void tc_row_pairs(uint8_t* arow, const uint8_t* grow,
 // den_col, the N disparity columns from 0.  Writes the D values to arow when
 // it is not null, and returns the WTA winner (smallest d on ties) with its
 // two neighbours for Eq. (10).
+//
+// First the smallest value of every 16 (rounding is monotonic, so the smallest
+// normalised value is the smallest sum normalised), and the first 16 that attain
+// the minimum; then those 16 again, once per different answer in the warp (few:
+// the lanes are neighbouring pixels), for the first place and its
+// neighbours.  About 2 instructions per value instead of 7 in one
+// pass, while the next tile waits for the accumulator if it is the only one
+// (D > 240: 1920 x 1080, D = 256, radius 9 1279 -> 1182 us; with two, D = 128,
+// radius 7 395 -> 385 us).
 struct TcWta {
     int bidx;
     float best, a_prev, a_next;
@@ -183,12 +204,8 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
     tmem_ld16(tbase + den_col, dv);
     const float inv = 1.f / dv[0];
     const float finf = __int_as_float(0x7f800000);
-    float best = finf, a_prev = 0.f, a_next = 0.f, last = 0.f;
-    int bidx = 0;
-    bool pend = false;   // the best is the previous chunk's last value: its successor comes next
-    const uint64_t inv2 = f2_pack(inv, inv);
-    // WTA over chunks of 16 values, keeping the neighbours of the running
-    // best; two chunks per accumulator read
+    TcWta r{0, finf, 0.f, 0.f};
+    int chunk = -1;
     for (int c0 = 0; c0 < N; c0 += 32) {
         float v[2][16];
         if (c0 + 16 < N)
@@ -200,12 +217,10 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
             const int cb = c0 + 16 * hc;
             if (cb >= N) break;
             float* w = v[hc];
-#pragma unroll
-            for (int i = 0; i < 16; i += 2) f2_unpack(f2_mul(f2_pack(w[i], w[i + 1]), inv2), w[i], w[i + 1]);
             if (arow) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    if (cb + i < D) arow[cb + i] = w[i];
+                    if (cb + i < D) arow[cb + i] = w[i] * inv;
             }
             if (cb + 16 > D) {
                 // disparities past D (zero cost rows) never win
@@ -213,22 +228,34 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
                 for (int i = 0; i < 16; ++i)
                     if (cb + i >= D) w[i] = finf;
             }
-            a_next = pend ? w[0] : a_next;
+            float m[4];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const bool lt = w[i] < best;
-                best = lt ? w[i] : best;
-                bidx = lt ? cb + i : bidx;
-                a_prev = lt ? (i > 0 ? w[i - 1] : last) : a_prev;
-                if (i < 15)
-                    a_next = lt ? w[i + 1] : a_next;
-                else
-                    pend = lt;
-            }
-            last = w[15];
+            for (int i = 0; i < 4; ++i) m[i] = fminf(fminf(w[i], w[4 + i]), fminf(w[8 + i], w[12 + i]));
+            const float low = fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) * inv;
+            const bool lt = low < r.best;
+            r.best = lt ? low : r.best;
+            chunk = lt ? cb : chunk;
         }
     }
-    return TcWta{bidx, best, a_prev, a_next};
+    unsigned todo = __ballot_sync(0xffffffffu, chunk >= 0);
+    while (todo) {
+        const int cb = __shfl_sync(0xffffffffu, chunk, __ffs(todo) - 1);
+        float v[18];   // columns cb - 1 .. cb + 16 (at the ends of the range any other)
+        tmem_ld18(tbase + (uint32_t)cb, tbase + (uint32_t)(cb > 0 ? cb - 1 : cb), tbase + (uint32_t)(cb + 16), v);
+        if (chunk == cb) {
+#pragma unroll
+            for (int i = 0; i < 18; ++i) v[i] = cb + i - 1 < D ? v[i] * inv : finf;
+#pragma unroll
+            for (int i = 16; i >= 1; --i) {
+                const bool eq = v[i] == r.best;
+                r.bidx = eq ? cb + i - 1 : r.bidx;
+                r.a_prev = eq ? v[i - 1] : r.a_prev;
+                r.a_next = eq ? v[i + 1] : r.a_next;
+            }
+        }
+        todo &= ~__ballot_sync(0xffffffffu, chunk == cb);
+    }
+    return r;
 }
 
 // Eq. (10): the vertex of the parabola through the winner and its

@@ -102,6 +102,33 @@ def test_tc_two_producer_groups(fbs, oracle_mod, prec, H, W, C, D, r):
 
 
 @pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("D", [1, 2, 15, 16, 17, 31, 32, 33, 48, 100, 240, 241, 256])
+def test_tc_winner_takes_the_first_of_equal_costs(fbs, prec, D):
+    """With radius 0 the aggregated value is the cost itself.  Costs of four
+    values only: every pixel has ties within and across the blocks of 16 that the
+    epilogue reads, and winners at their edges; maps exactly the first minimum and
+    its parabola in FP32."""
+    H, W = 19, 37
+    rng = np.random.default_rng(D)
+    cost = (rng.integers(0, 4, size=(H, W, D)) / 8 + 0.25).astype(np.float32)
+    cost[:8] += 0.25                             # upper rows: a single smallest value
+    np.put_along_axis(cost[:8], rng.integers(0, D, size=(8, W, 1)), np.float32(0.125), axis=2)
+    guide = rng.integers(0, 256, size=(H, W, 3)).astype(np.uint8)
+    with fbs.Context(0, prec=_prec(fbs, prec)) as ctx:
+        _, di, ds = ctx.aggregate(_dev(cost), _dev(guide), 0, 1.0, 12.0)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(ctx.ctx)
+    k = cost.argmin(axis=2)
+    np.testing.assert_array_equal(di.cpu().numpy(), k)
+    pad = np.pad(cost, ((0, 0), (0, 0), (1, 1)))
+    at = [np.take_along_axis(pad, (k + i)[..., None], axis=2)[..., 0] for i in (0, 1, 2)]
+    dd = 2 * at[0] + 2 * at[2] - 4 * at[1]
+    inner = (k > 0) & (k < D - 1) & (dd > 0)
+    ref = np.where(inner, k + (at[0] - at[2]) / np.where(inner, dd, 1), k).astype(np.float32)
+    np.testing.assert_array_equal(ds.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
 def test_tc_full_size_bench_workload_bad_pixels(fbs, oracle_mod, prec):
     """640x480 RGB, D=64, radius 7 (the benchmark workload): aggregated costs
     of 400 sampled pixels within the 16-bit rounding bound of the FP64 oracle
