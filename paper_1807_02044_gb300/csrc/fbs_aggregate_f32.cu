@@ -46,7 +46,7 @@
 //
 // Measured on GB300 (CUDA events), before -> now; before: 4 pixels x 8 disparities
 // per thread, scalar FMAs, 256-thread CTAs in step through a cp.async ring:
-//   640x480,  D = 64,  rho = 7:    425 -> 241 us (36.7 TFLOP/s)
+//   640x480,  D = 64,  rho = 7:    425 -> 232 us (38.1 TFLOP/s)
 //   640x480,  D = 64,  rho = 2:    125 ->  62 us
 //   767x575,  D = 93,  rho = 11:  2263 -> 1184 us
 //   1280x960, D = 128, rho = 15: 10390 -> 6896 us (43.8 TFLOP/s)
@@ -219,12 +219,13 @@ __device__ __forceinline__ float ex2_approx(float x)
 }
 
 // Two consecutive taps dx, dx + 1 of one pixel and window row: Eq. (7)-(8) as
-// one exp2, colour distance |q|^2 + |p|^2 - 2 q.p exact in integers, then
-// float(c) = (2^23 + c) - 2^23 exactly.  sp: the two spatial terms
+// one exp2, colour distance exact in integers (bytewise differences, their
+// squares: one instruction less per weight than |q|^2 + |p|^2 - 2 q.p, 1203 ->
+// 1136 us at 767x575, D = 93, rho = 11), then float(c) = (2^23 + c) - 2^23 exactly.  sp: the two spatial terms
 // ((dx - rho)^2 + dy^2) times -log2(e) / sigma_s^2.  EDGE: a tap outside the
 // image columns has weight 0.
 struct Pixel {
-    uint32_t col, norm;       // its colour, |p|^2 + 2^23
+    uint32_t col;             // its colour
     uint64_t magic2, nkr2;    // (-2^23, -2^23) and -log2(e) / sigma_r^2 twice
     int qx, W;                // image column of tap 0
 };
@@ -232,8 +233,8 @@ template <bool EDGE>
 __device__ __forceinline__ void weight_pair(const Pixel& p, uint32_t q0, uint32_t q1, uint64_t sp, int dx, float& w0,
                                             float& w1)
 {
-    const uint32_t d0 = __dp4a(q0, p.col, 0u), d1 = __dp4a(q1, p.col, 0u);
-    const uint32_t e0 = __dp4a(q0, q0, p.norm) - d0 - d0, e1 = __dp4a(q1, q1, p.norm) - d1 - d1;
+    const uint32_t d0 = __vabsdiffu4(q0, p.col), d1 = __vabsdiffu4(q1, p.col);
+    const uint32_t e0 = __dp4a(d0, d0, kMagic), e1 = __dp4a(d1, d1, kMagic);
     f2_unpack(f2_fma(f2_add(u2_pack(e0, e1), p.magic2), p.nkr2, sp), w0, w1);
     w0 = ex2_approx(w0);
     w1 = ex2_approx(w1);
@@ -484,7 +485,7 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
     const uint32_t wa0 = tc::smem_u32(wbuf) + 4 * (grow * SEGS + gseg) * WS;
     // weight role: lane = pixel (lane / PW, lane % PW) of the warp
     float* const wout = wbuf + (lane / kPX) * WS + (lane % kPX) * (kPX + 1);
-    const Pixel self{t.pcol, __dp4a(t.pcol, t.pcol, kMagic), f2_pack(-8388608.f, -8388608.f),
+    const Pixel self{t.pcol, f2_pack(-8388608.f, -8388608.f),
                      f2_pack(t.neg_kr, t.neg_kr), t.px - rho, t.W};
     const bool edge = xlo < 0 || xlo + NC > t.W;
 
