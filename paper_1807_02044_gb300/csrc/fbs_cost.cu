@@ -174,29 +174,33 @@ __device__ __forceinline__ uint64_t ncc_cost2(uint64_t minus9p, uint64_t sl, uin
 
 // ---- FP32 volume [H][W][ld], D innermost ------------------------------------------
 // A CTA (4 warps) covers 64 pixels x 4 rows of one view and disparities
-// [d_begin, d_end), up to 128 at a time; a warp takes 16 of them, a lane 4
-// pixels x 2 rows (lanes 0-15: rows y0, y0+1; 16-31: the next two).  The window of
-// the view's own image (6 columns x 4 grey rows) stays in registers, the other
-// image's slides one column (2 shared loads) per disparity; NCC as above, TAD from
-// the packed pixels.  Costs are transposed through the warp's buffer ([row][pixel]
-// [8 d], entry XOR pixel / 4, conflict-free) and leave as 32-byte runs per pixel.
+// [d_begin, d_end), up to 128 per staging of the other image and 32 per step; a
+// warp takes 8 of them, a lane 4 pixels x 2 rows (lanes 0-15: rows y0, y0+1;
+// 16-31: the next two).  The window of the view's own image (6 columns x 4 grey
+// rows) stays in registers, the other image's slides one column (2 shared loads)
+// per disparity; NCC as above, TAD from the packed pixels.  Costs are transposed
+// through a buffer of the CTA ([row][pixel][32 d], entry XOR pixel / 4,
+// conflict-free) and leave as runs of up to 128 bytes per pixel, a row per warp.
 // MIRROR computes the right view: its own image is the right one, and the other
 // window slides the other way (Sec. II-A, Sec. III); the two products and sums
 // commute, so cost_r(x, y, d) = cost(x + d, y, d) bit for bit.
 // VW: floats per store -- 4 (ld % 4 == 0, 16-byte aligned), 2 (ld even, 8-byte
 // aligned) or 1.
-// Bound: the load/store pipe (88% busy at 1280x960, D = 128: half of it shared-
-// memory traffic of the windows and the transposition, half the scattered
-// 32-byte runs).  Measured on GB300 with the pre-pass, before -> now (before:
-// integer products, one row x 128 pixels per CTA, stores after a block-wide
-// transposition): 640x480, D = 64: 50 -> 34 us; 1280x960, D = 128: 293 -> 177 us;
-// 1920x1080, D = 256: 906 -> 554 us; NCC 767x575, D = 93: 108 -> 61 us.
+// Bound: the load/store pipe.  A store instruction costs it a cycle per line of
+// 128 bytes that it touches, so a warp that wrote its own 8 disparities of 16
+// pixels (runs of 32 bytes) spent two thirds of its cycles there.  Measured on
+// GB300 with the pre-pass, integer products, one row x 128 pixels per CTA and
+// stores after a block-wide transposition -> runs of 32 bytes per warp -> now:
+// 640x480, D = 64: 50 -> 33.5 -> 26.4 us; 1280x960, D = 128: 293 -> 177 -> 138 us;
+// 1920x1080, D = 256: 906 -> 554 -> 414 us; 767x575, D = 93: 108 -> 61 -> 46 us;
+// TAD 641x479, D = 71 (4-byte stores): 54 us in runs of 32 bytes, now 30.
 constexpr int kCostPx = 64, kCostRows = 4, kCostWarps = 4, kCostThreads = 32 * kCostWarps;
 constexpr int kCostPass = 128;                               // disparities per pass
 constexpr int kCostLeft = 82;                                // >= skew4(66)
 constexpr int kCostRight = (kCostPass + 68) * 5 / 4 + 2;     // >= skew4(16 ng + 68)
-constexpr int kCostBuf = kCostRows * kCostPx * 8 * 4;        // bytes of a warp's buffer
-constexpr size_t kCostSmem = (size_t)kCostWarps * kCostBuf + (size_t)4 * 16 * (kCostLeft + kCostRight);
+constexpr int kCostStep = 8 * kCostWarps;                    // disparities per step, 8 per warp
+constexpr int kCostBuf = kCostRows * kCostPx * kCostStep * 4;   // bytes of the buffer
+constexpr size_t kCostSmem = (size_t)kCostBuf + (size_t)4 * 16 * (kCostLeft + kCostRight);
 
 struct CostArgs {
     CostScratch sc;                 // NCC: statistics of both images
@@ -211,8 +215,8 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = a.H, W = a.W, D = a.D;
-    uint8_t* const buf = (uint8_t*)smem + warp * kCostBuf;
-    float4* const gl = (float4*)((uint8_t*)smem + kCostWarps * kCostBuf);   // [2][kCostLeft]: columns x0 - 1 ..
+    uint8_t* const buf = (uint8_t*)smem;
+    float4* const gl = (float4*)((uint8_t*)smem + kCostBuf);   // [2][kCostLeft]: columns x0 - 1 ..
     float4* const sl = gl + 2 * kCostLeft;    // [2][kCostLeft]: centres x0 ..
     float4* const gr = sl + 2 * kCostLeft;    // [2][kCostRight]: columns rb ..
     float4* const sr = gr + 2 * kCostRight;   // [2][kCostRight]: centres rb ..
@@ -264,8 +268,11 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
     const float inv_c = 1.f / (float)a.C;
     const uint64_t one2 = f2_pack(1.f, 1.f);
     auto at = [](int m) { return m + (m >> 2); };   // offset of column base + m (base a multiple of 4)
-    // entry (i, e) of 8 bytes: pixel 4 p + i, disparities 2 e, 2 e + 1 of 8, at 8 * ((4 i + e) ^ p)
-    const uint32_t put0 = tc::smem_u32(buf) + 2 * rp * (kCostPx * 32) + 128 * p + 8 * p;
+    // buffer [row][pixel][step's disparities]; entry e of 8 bytes (disparities 2 e,
+    // 2 e + 1) of pixel 4 p + i at 8 * (e ^ p)
+    constexpr int PB = kCostStep * 4, RB = kCostPx * PB;   // bytes of a pixel, of a row
+    static_assert(PB == 128, "16 entries per pixel, XORed with 16 pixel groups");
+    const uint32_t put0 = tc::smem_u32(buf) + 2 * rp * RB + 4 * p * PB + 8 * (p ^ (4 * warp));
 
     for (int dp = d_begin; dp < d_end; dp += kCostPass) {
         const int ng = min(kCostPass / 16, (d_end - dp + 15) / 16);
@@ -278,9 +285,9 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
             stage(other, other_img, rb + c, gr + skew4(c), gr + kCostRight + skew4(c), sr + skew4(c),
                   sr + kCostRight + skew4(c));
         __syncthreads();
-        for (int grp = warp; grp < ng; grp += kCostWarps) {
-            const int d0 = dp + 16 * grp;
-            const int base = xl + (MIRROR ? 4 + 16 * grp : 16 * (ng - grp));
+        for (int dq = dp; dq < min(dp + kCostPass, d_end); dq += kCostStep) {
+            const int d0 = dq + 8 * warp;
+            const int base = xl + (MIRROR ? 4 + d0 - dp : 16 * ng - (d0 - dp));
             const float4* glw = gl + rp * kCostLeft + skew4(xl);
             const float4* slw = sl + rp * kCostLeft + skew4(xl);
             const float4* grw = gr + rp * kCostRight + skew4(base);
@@ -288,40 +295,12 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
             constexpr int ST = MIRROR ? 1 : -1;     // columns the window moves per disparity
             constexpr int IN = MIRROR ? 5 : 0;      // where the new column comes in
 
-            // writes 8 disparities from d8 on out of the warp's buffer
-            auto flush = [&](int d8) {
-                __syncwarp();
-                constexpr int L = 8 / VW, PXI = 32 / L;      // lanes per pixel, pixels per store
-                const int e = lane % L, d = d8 + VW * e;
-                const bool din = VW == 4 ? d < a.ld && d < ((d_end + 3) & ~3) : d < min(D, d_end);
-#pragma unroll
-                for (int r = 0; r < kCostRows; ++r) {
-                    if (y0 + r >= H) break;
-                    float* o = a.out + ((size_t)(y0 + r) * W + x0 + lane / L) * a.ld + d;
-#pragma unroll 4
-                    for (int j = 0; j < kCostPx / PXI; ++j, o += (size_t)PXI * a.ld) {
-                        const int px = PXI * j + lane / L, pp = px >> 2, c = 4 * (px & 3) + e * VW / 2;
-                        const uint8_t* q = buf + r * (kCostPx * 32) + 128 * pp;
-                        if (x0 + px >= W || !din) continue;
-                        if (VW == 4) {
-                            const float4 v = *(const float4*)(q + 8 * ((c ^ pp) & ~1));
-                            *(float4*)o = pp & 1 ? make_float4(v.z, v.w, v.x, v.y) : v;
-                        } else if (VW == 2) {
-                            *(float2*)o = *(const float2*)(q + 8 * (c ^ pp));
-                        } else {
-                            *o = *(const float*)(q + 8 * (c ^ pp) + 4 * (e & 1));
-                        }
-                    }
-                }
-                __syncwarp();
-            };
             auto put = [&](int s, const float (&c)[4][2][2]) {   // c[pixel][row][s even, odd]
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
-                        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"((put0 ^ (8 * (4 * i + ((s >> 1) & 3)))) +
-                                                                              h * (kCostPx * 32)),
+                        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"((put0 ^ (8 * (s >> 1))) + i * PB + h * RB),
                                      "f"(c[i][h][0]), "f"(c[i][h][1])
                                      : "memory");
             };
@@ -331,7 +310,8 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                 return d >= D ? 0.f : (MIRROR ? x + d >= W : x - d < 0) ? most : v;
             };
 
-            if (MODE == 0) {
+            if (d0 >= d_end) {
+            } else if (MODE == 0) {
                 float4 lw[6], rw[6];
                 uint64_t sli[4], rli[4], sri[4], rri[4];
 #pragma unroll
@@ -352,7 +332,7 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                 auto sweep = [&](auto masked) {
                     float c[4][2][2];
 #pragma unroll
-                    for (int s = 0; s < 16; ++s) {
+                    for (int s = 0; s < 8; ++s) {
                         if (s > 0) {
 #pragma unroll
                             for (int j = 0; j < 5; ++j) {
@@ -379,10 +359,9 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                             c[i][1][s & 1] = decltype(masked)::value ? mask(v1, i, d0 + s, 2.f) : v1;
                         }
                         if (s & 1) put(s, c);
-                        if ((s & 7) == 7) flush(d0 + s - 7);
                     }
                 };
-                const bool inside = d0 + 16 <= D && (MIRROR ? xbase + 3 + d0 + 15 < W : xbase >= d0 + 15);
+                const bool inside = d0 + 8 <= D && (MIRROR ? xbase + 3 + d0 + 7 < W : xbase >= d0 + 7);
                 if (__all_sync(0xffffffffu, inside)) sweep(std::integral_constant<bool, false>{});
                 else sweep(std::integral_constant<bool, true>{});
             } else {
@@ -395,7 +374,7 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                 }
                 float c[4][2][2];
 #pragma unroll
-                for (int s = 0; s < 16; ++s) {
+                for (int s = 0; s < 8; ++s) {
                     if (s > 0) {
 #pragma unroll
                         for (int i = 0; i < 3; ++i)
@@ -416,12 +395,33 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                             c[i][h][s & 1] = mask(fminf((float)sad * inv_c, a.tau), i, d0 + s, a.tau);
                         }
                     if (s & 1) put(s, c);
-                    if ((s & 7) == 7) flush(d0 + s - 7);
                 }
             }
             (void)ST;
+            __syncthreads();
+            // a warp writes one row: up to 128 contiguous bytes per pixel
+            if (y0 + warp < H) {
+                constexpr int L = kCostStep / VW, PXI = 32 / L;      // lanes per pixel, pixels per store
+                const int e = lane % L, d = dq + VW * e;
+                const bool din = VW == 4 ? d < a.ld && d < ((d_end + 3) & ~3) : d < min(D, d_end);
+                const int npx = din ? min(kCostPx, W - x0) : 0;
+                float* o = a.out + ((size_t)(y0 + warp) * W + x0 + lane / L) * a.ld + d;
+                const uint8_t* q = buf + warp * RB + (lane / L) * PB;
+#pragma unroll 4
+                for (int px = lane / L; px < npx; px += PXI, o += (size_t)PXI * a.ld, q += PXI * PB) {
+                    const int pp = px >> 2, c = e * VW / 2;
+                    if (VW == 4) {
+                        const float4 v = *(const float4*)(q + 8 * ((c ^ pp) & ~1));
+                        *(float4*)o = pp & 1 ? make_float4(v.z, v.w, v.x, v.y) : v;
+                    } else if (VW == 2) {
+                        *(float2*)o = *(const float2*)(q + 8 * (c ^ pp));
+                    } else {
+                        *o = *(const float*)(q + 8 * (c ^ pp) + 4 * (e & 1));
+                    }
+                }
+            }
+            __syncthreads();   // the buffer, and after the last step the staged columns, may be overwritten
         }
-        __syncthreads();   // the staged columns may be overwritten
     }
 }
 
