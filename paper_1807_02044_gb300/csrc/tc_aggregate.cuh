@@ -186,14 +186,14 @@ __device__ __forceinline__ void tc_row_pairs(uint8_t* arow, const uint8_t* grow,
 // it is not null, and returns the WTA winner (smallest d on ties) with its
 // two neighbours for Eq. (10).
 //
-// First the smallest value of every 16 (rounding is monotonic, so the smallest
-// normalised value is the smallest sum normalised), and the first 16 that attain
-// the minimum; then those 16 again, once per different answer in the warp (few:
-// the lanes are neighbouring pixels), for the first place and its
-// neighbours.  About 2 instructions per value instead of 7 in one
-// pass, while the next tile waits for the accumulator if it is the only one
-// (D > 240: 1920 x 1080, D = 256, radius 9 1279 -> 1182 us; with two, D = 128,
-// radius 7 395 -> 385 us).
+// Of every 16 values only the smallest is compared with the best so far; where
+// it is smaller, the 16 are searched for its first place and its neighbours: two
+// instructions per value, and four more in a search, instead of always six.  With a
+// single accumulator (D > 240) the next tile waits for them (1920 x 1080, D = 256,
+// radius 9 1282 -> 1210 us; 1280 x 720, D = 192, radius 2 152 -> 130 us).  Where the
+// winners of a warp's 32 pixels have nothing in common (two unrelated noise images)
+// nearly every 16 are searched: 1313 and 162 us.  Only noting the 16 and searching
+// them at the end, from tensor memory, is 1182 us at best and 1419 us there.
 struct TcWta {
     int bidx;
     float best, a_prev, a_next;
@@ -205,7 +205,8 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
     const float inv = 1.f / dv[0];
     const float finf = __int_as_float(0x7f800000);
     TcWta r{0, finf, 0.f, 0.f};
-    int chunk = -1;
+    float last = 0.f;
+    const uint64_t inv2 = f2_pack(inv, inv);
     for (int c0 = 0; c0 < N; c0 += 32) {
         float v[2][16];
         if (c0 + 16 < N)
@@ -217,10 +218,12 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
             const int cb = c0 + 16 * hc;
             if (cb >= N) break;
             float* w = v[hc];
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) f2_unpack(f2_mul(f2_pack(w[i], w[i + 1]), inv2), w[i], w[i + 1]);
             if (arow) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    if (cb + i < D) arow[cb + i] = w[i] * inv;
+                    if (cb + i < D) arow[cb + i] = w[i];
             }
             if (cb + 16 > D) {
                 // disparities past D (zero cost rows) never win
@@ -228,32 +231,25 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
                 for (int i = 0; i < 16; ++i)
                     if (cb + i >= D) w[i] = finf;
             }
-            float m[4];
+            float low = w[15];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) m[i] = fminf(fminf(w[i], w[4 + i]), fminf(w[8 + i], w[12 + i]));
-            const float low = fminf(fminf(m[0], m[1]), fminf(m[2], m[3])) * inv;
-            const bool lt = low < r.best;
-            r.best = lt ? low : r.best;
-            chunk = lt ? cb : chunk;
-        }
-    }
-    unsigned todo = __ballot_sync(0xffffffffu, chunk >= 0);
-    while (todo) {
-        const int cb = __shfl_sync(0xffffffffu, chunk, __ffs(todo) - 1);
-        float v[18];   // columns cb - 1 .. cb + 16 (at the ends of the range any other)
-        tmem_ld18(tbase + (uint32_t)cb, tbase + (uint32_t)(cb > 0 ? cb - 1 : cb), tbase + (uint32_t)(cb + 16), v);
-        if (chunk == cb) {
+            for (int i = 0; i < 14; i += 2) low = fminf(fminf(w[i], w[i + 1]), low);
+            low = fminf(low, w[14]);
+            if (r.bidx == cb - 1) r.a_next = w[0];   // the best was the last of the 16 before
+            if (low < r.best) {
+                r.best = low;
+                r.bidx = cb + 15;
+                r.a_prev = w[14];
 #pragma unroll
-            for (int i = 0; i < 18; ++i) v[i] = cb + i - 1 < D ? v[i] * inv : finf;
-#pragma unroll
-            for (int i = 16; i >= 1; --i) {
-                const bool eq = v[i] == r.best;
-                r.bidx = eq ? cb + i - 1 : r.bidx;
-                r.a_prev = eq ? v[i - 1] : r.a_prev;
-                r.a_next = eq ? v[i + 1] : r.a_next;
+                for (int i = 14; i >= 0; --i) {
+                    const bool eq = w[i] == low;
+                    r.bidx = eq ? cb + i : r.bidx;
+                    r.a_prev = eq ? (i > 0 ? w[i - 1] : last) : r.a_prev;
+                    r.a_next = eq ? w[i + 1] : r.a_next;
+                }
             }
+            last = w[15];
         }
-        todo &= ~__ballot_sync(0xffffffffu, chunk == cb);
     }
     return r;
 }

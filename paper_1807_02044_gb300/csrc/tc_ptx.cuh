@@ -128,24 +128,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 16 columns at taddr, in v[1] .. v[16], and one before and one after them, in flight together.
-__device__ __forceinline__ void tmem_ld18(uint32_t taddr, uint32_t before, uint32_t after, float (&v)[18])
-{
-    uint32_t r[18];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%18];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%16}, [%19];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%17}, [%20];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[0]), "=r"(r[17])
-        : "r"(taddr), "r"(before), "r"(after)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 18; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // Two such loads (32 consecutive columns in two halves) in flight together,
 // then one wait; in one asm statement, so no use of the registers can be
 // scheduled before the wait.
