@@ -642,7 +642,10 @@ bool tc_plan(int H, int W, int C, int D, int radius, float sigma_s, float sigma_
         // one group 3.48 ms, 2 x 3 2.70 ms, 2 x 2 1.81 ms; D = 256, radius 24:
         // one group 8.9 ms, 1 x 3 6.5 ms, 1 x 2 4.4 ms)
         p.NG = 2;
-        return (cap >= 2 && fits(2, 2)) || fits(1, 2);
+        if (!(cap >= 2 && fits(2, 2)) && !fits(1, 2)) return false;
+        // more than half of an SM's shared memory: two CTAs on one SM would leave another idle
+        L.total = L.total > 116 * 1024 ? L.total : 116 * 1024;
+        return true;
     }
     if (!fits(4, 2) && (radius > 9 || !fits(3, 2))) {
         p.NG = 2;

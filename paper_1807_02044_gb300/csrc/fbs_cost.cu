@@ -208,6 +208,7 @@ struct CostArgs {
     int H, W, C, D, ld;
     float tau;
     float* out;
+    bool early;                     // see agg_early
 };
 
 template <int MODE, bool MIRROR, int VW>
@@ -429,15 +430,15 @@ template <int MODE, bool MIRROR, int VW>
 __global__ void __launch_bounds__(kCostThreads, 4) cost_kernel(const CostArgs a)
 {
     extern __shared__ __align__(128) float4 sm_cost[];
-    // the aggregation's set-up may start; the statistics must have been written
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the statistics must have been written
     cost_tile<MODE, MIRROR, VW>(a, blockIdx.x * kCostPx, blockIdx.y * kCostRows, 0, a.D, sm_cost);
+    if (!a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 __device__ __forceinline__ CostArgs pair_args(const BatchPair& bp)
 {
-    return CostArgs{bp.sc, bp.left, bp.right, bp.H, bp.W, bp.C, bp.D, bp.ld, bp.tau, bp.cost};
+    return CostArgs{bp.sc, bp.left, bp.right, bp.H, bp.W, bp.C, bp.D, bp.ld, bp.tau, bp.cost, false};
 }
 
 // Batched FP32 cost volumes [H][W][ld]: an item is one 64 x 4 tile of a pair.
@@ -471,7 +472,7 @@ cost_band_kernel(const CostArgs a, int rho, const int2* __restrict__ tile_range,
 {
     extern __shared__ __align__(128) float4 sm_cost[];
     __shared__ int lo_s, hi_s;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int x0 = blockIdx.x * kCostPx, y0 = blockIdx.y * kCostRows;
     if (threadIdx.x == 0) {
@@ -991,6 +992,20 @@ cudaError_t launch_cost_vw(const CostArgs& a, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+// When may the aggregation's CTAs start: with the cost kernel's (they set up
+// while it runs), or as its CTAs end?  An early CTA takes any place that is
+// free, so where the aggregation does not fill the chip (four CTAs per SM) some
+// SMs get several and others none.  Early for a grid that fills it or for tiles
+// of so little work that the set-up is what counts: 160x120, D = 16, rho = 4 26
+// against 28 us late; late otherwise: 82x196, D = 198, rho = 15 356 against 488 us
+// early, 160x120, D = 64, rho = 7 42 against 50 us, 200x200, D = 64, rho = 3 33
+// against 35 us.
+bool agg_early(int H, int W, int D, int radius)
+{
+    const long long tiles = (long long)((W + kAggTileX - 1) / kAggTileX) * ((H + kAggTileY - 1) / kAggTileY);
+    return tiles >= 4 * 152 || (kAggTileY + 2 * radius) * (8 + 2 * radius) * (long long)D < 100 * 64;
+}
+
 // One view of the FP32 volume (mode 0: after the statistics).
 cudaError_t launch_cost_view(const CostArgs& a, int mode, bool mirror, cudaStream_t stream)
 {
@@ -1078,11 +1093,13 @@ CostScratch carve_cost_scratch(void* base, int H, int W)
 }
 
 cudaError_t launch_cost_build(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                              int C, int D, int ld, int mode, float tau, float* cost, cudaStream_t stream)
+                              int C, int D, int ld, int mode, float tau, float* cost, int agg_radius,
+                              cudaStream_t stream)
 {
     cudaError_t e = mode == 0 ? launch_stats(sc, left, right, H, W, C, stream) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost}, mode, false, stream);
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost, agg_early(H, W, D, agg_radius)}, mode, false,
+                            stream);
 }
 
 cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
@@ -1093,17 +1110,18 @@ cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const u
     if (e != cudaSuccess) return e;
     const int ntx = (W + kAggTileX - 1) / kAggTileX, nty = (H + kAggTileY - 1) / kAggTileY;
     return fbs::launch_after(cost_band_kernel, dim3((W + kCostPx - 1) / kCostPx, (H + kCostRows - 1) / kCostRows), kCostThreads,
-                             kCostSmem, stream, CostArgs{sc, left, right, H, W, C, D, ld, 0.f, cost}, radius, tile_range, ntx,
+                             kCostSmem, stream, CostArgs{sc, left, right, H, W, C, D, ld, 0.f, cost, agg_early(H, W, D, radius)}, radius, tile_range, ntx,
                              nty);
 }
 
 cudaError_t launch_cost_build_lr(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                                 int C, int D, int ld, int mode, float tau, float* cost, float* cost_r,
+                                 int C, int D, int ld, int mode, float tau, float* cost, float* cost_r, int agg_radius,
                                  cudaStream_t stream)
 {
-    cudaError_t e = launch_cost_build(sc, left, right, H, W, C, D, ld, mode, tau, cost, stream);
+    cudaError_t e = launch_cost_build(sc, left, right, H, W, C, D, ld, mode, tau, cost, agg_radius, stream);
     if (e != cudaSuccess) return e;
-    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost_r}, mode, true, stream);
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost_r, agg_early(H, W, D, agg_radius)}, mode, true,
+                            stream);
 }
 
 cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H,

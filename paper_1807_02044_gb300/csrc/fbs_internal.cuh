@@ -69,14 +69,17 @@ size_t rgbx_bytes(int H, int W);
 __host__ __device__ inline int rgbx_pitch(int W) { return (W + 1) & ~1; }
 
 // cost[(y*W + x)*ld + d] for d < D; entries D <= d < ld are written as 0.
+// agg_radius: the window radius of the aggregation that follows (0 if none does);
+// it decides when that kernel's CTAs may start, not the results.
 cudaError_t launch_cost_build(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                              int C, int D, int ld, int mode, float tau, float* cost, cudaStream_t stream);
+                              int C, int D, int ld, int mode, float tau, float* cost, int agg_radius,
+                              cudaStream_t stream);
 
 // Both views (Sec. II-A, Sec. III): cost as launch_cost_build, and cost_r
 // [H][W][ld] the right volume, cost_r(x, y, d) = cost(x + d, y, d), the maximum
 // cost where x + d >= W.
 cudaError_t launch_cost_build_lr(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                                 int C, int D, int ld, int mode, float tau, float* cost, float* cost_r,
+                                 int C, int D, int ld, int mode, float tau, float* cost, float* cost_r, int agg_radius,
                                  cudaStream_t stream);
 
 // 16-bit x-blocked volume cost[((y*ceil(W/8) + x/8)*Dp + d)*8 + x%8] with
