@@ -468,8 +468,8 @@ aggregate_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
                     } else {
                         // B rows 0..127 into accumulator columns 0..127, rows
                         // 128..Nb-1 (with the ones row) into columns 128..Nb-1:
-                        // an MMA of N <= 128 costs the same ~88 cycles as one of
-                        // N = 16, so 128 + 144 beats 256 + a separate 16
+                        // 64 + 72 cycles at D = 256, where 256 + a separate 16 take
+                        // 128 + 52
                         const uint32_t b2 = (128 * 16) >> 4;
                         for (int k = 0; k < nk; ++k) {
                             umma_f16(dacc, ahi | alo, bhi | blo, p.idesc, accumulate);
