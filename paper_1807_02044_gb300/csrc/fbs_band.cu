@@ -424,7 +424,7 @@ size_t al256(size_t n) { return (n + 255) & ~(size_t)255; }
 // Scratch of one quarter-resolution problem, carved from ctx->band_ws.
 struct NetScratch {
     int32_t* gq;                 // [2][P]
-    fbs::BlockStat* stat;        // [2][P]; lies in y[0], which the features' readers write
+    fbs::BlockStat* stat;        // [2][P]; lies in featf: read before the features are written
     float* kh;                   // row sums of the coarse costs [P][Dq]
     int32_t* estar;              // [P]
     float* featf;                // [P][6] FP32 features (feature-point proposal)
@@ -472,7 +472,8 @@ NetScratch carve_net(void* base, int H, int W, int D, bool training, bool full_r
     s.featf = (float*)take(P * 24);
     s.x0 = (__nv_bfloat16*)take(P * 16);
     for (int l = 0; l < 5; ++l) s.y[l] = (__nv_bfloat16*)take(P * 64);
-    s.stat = (fbs::BlockStat*)s.y[0];
+    s.stat = (fbs::BlockStat*)s.featf;
+    static_assert(2 * sizeof(fbs::BlockStat) <= 24, "[2][P] statistics in [P][6] floats");
     s.out = (float*)take(P * 8);
     if (training) {
         for (int l = 0; l < 5; ++l) s.g[l] = (__nv_bfloat16*)take(P * 64);

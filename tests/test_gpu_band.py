@@ -492,6 +492,28 @@ def test_forward_outputs_do_not_depend_on_which_are_asked_for(fbs, H, W):
                 assert (b[:off] == -7).all() and (b[(off + n if a is not None else 0):] == -7).all(), (mask, i)
 
 
+def test_features_leave_the_traced_activations(fbs):
+    """A features call between a forward pass and its trace changes the input
+    features only (it shares their buffer), not the layers' outputs."""
+    H, W, D = 53, 77, 40
+    Hq, Wq = (H + 3) // 4, (W + 3) // 4
+    P = Hq * Wq
+    L, R = _rand_pair(5, H, W, 3, shift=12)
+    L2, R2 = _rand_pair(6, H, W, 3, shift=4)
+    out = torch.empty((Hq, Wq, 2), device="cuda")
+    est = torch.empty((Hq, Wq), dtype=torch.int32, device="cuda")
+    with fbs.Context(0) as ctx:
+        fbs.fbs_band_net_set_params(ctx.ctx, _params(1))
+        acts = [torch.empty(_trace_sizes(Hq, Wq)[0], device="cuda") for _ in range(2)]
+        fbs.fbs_band_net_forward(ctx.ctx, _dev(L), _dev(R), H, W, 3, D, out, None, None)
+        fbs.fbs_band_net_trace(ctx.ctx, acts[0], None)
+        fbs.fbs_band_features(ctx.ctx, _dev(L2), _dev(R2), H, W, 3, D, None, est)
+        fbs.fbs_band_net_trace(ctx.ctx, acts[1], None)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(ctx.ctx)
+    assert torch.equal(acts[0][8 * P:], acts[1][8 * P:])
+
+
 def test_learned_entry_equals_forward_then_banded(fbs):
     H, W, D = 120, 200, 64
     L, R = _rand_pair(12, H, W, 3, shift=14)
