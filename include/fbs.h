@@ -90,8 +90,7 @@ fbs_status fbs_sync(fbs_ctx *ctx);
  * land (a fixed ~2 s bound), frees its tensor memory and records an error
  * that the next fbs_sync returns as FBS_ERR_TIMEOUT; the outputs of that call
  * are invalid and the context stays usable.  0 <= seconds <= 60, 0 = the
- * default (about 2 s).  Applies to kernels launched after the call (batch
- * graphs built earlier keep the limit they were built with). */
+ * default (about 2 s).  Applies to kernels launched after the call. */
 fbs_status fbs_set_wait_limit(fbs_ctx *ctx, double seconds);
 
 /* Failure injection (a test hook; not a step of the method): the next
@@ -219,8 +218,9 @@ typedef struct {
  *   otherwise).  Scratch: every pair's 16-bit volume at once (sum of
  *   H*ceil(W/8)*8*Dp*2 bytes, Dp = round_up(D,16) + 16,
  *   plus the packed guide).
- *   A branched graph holds the pairs' addresses: a new set of buffers
- *   captures a new graph (the context keeps up to 32).
+ *   A branched graph holds the pairs' addresses and sigma_s, sigma_r and tau:
+ *   a new set of buffers or values captures a new graph (the context keeps up
+ *   to 32).
  * The first call of a new shape (the list of H, W, C, D, radius, the cost
  * mode and, for the tensor cores, the precision) runs the library's
  * autotuner: it times each schedule plan on the given data and keeps the

@@ -21,8 +21,8 @@
 // aggregation and small pairs fill the SMs a large pair's last wave leaves
 // idle.  Tensor-core plans also differ in the window rows per pipeline stage
 // (the kernel's maximum, or at most 3: smaller stages, more of them).  The
-// kernels' arguments (and the tensor maps) hold the pairs' addresses, so
-// these graphs are keyed by the buffers too.
+// kernels' arguments (and the tensor maps) hold the pairs' addresses, sigma_s,
+// sigma_r and tau and the wait limit, so these graphs are keyed by them too.
 //
 // Plan 6 of the tensor-core form keeps the per-pair cost builds (2 branches)
 // and replaces the per-pair aggregations by persistent launches that walk
@@ -39,6 +39,7 @@
 
 #include <algorithm>
 #include <cstdio>
+#include <cstring>
 #include <fstream>
 #include <numeric>
 #include <sstream>
@@ -405,6 +406,13 @@ fbs_status build_branch_graph(fbs_ctx* ctx, int n, const fbs_pair* pairs, int nb
     return FBS_OK;
 }
 
+uint32_t float_bits(float v)
+{
+    uint32_t u;
+    std::memcpy(&u, &v, sizeof u);
+    return u;
+}
+
 fbs_status run_branch_plan(fbs_ctx* ctx, const std::string& sig, int n, const fbs_pair* pairs, int plan, int nb,
                            int rows, bool persistent, cudaStream_t stream)
 {
@@ -412,12 +420,14 @@ fbs_status run_branch_plan(fbs_ctx* ctx, const std::string& sig, int n, const fb
     for (int i = 0; i < n; ++i) need += pair_bytes(pairs[i], tc_batch(ctx));
     fbs_status st = ensure(ctx, &ctx->ws, &ctx->ws_bytes, need, "batch cost volumes");
     if (st != FBS_OK) return st;
-    // graphs that hold the pairs' addresses are keyed by them ("g|" prefix)
+    // these graphs hold the pairs' addresses and parameters and the wait limit
+    // as kernel arguments, so all of them are in the key ("g|" prefix)
     std::ostringstream key;
-    key << "g|" << sig << "|p" << plan << "|ws" << (uintptr_t)ctx->ws << std::hex;
+    key << "g|" << sig << "|p" << plan << "|ws" << (uintptr_t)ctx->ws << "|w" << ctx->wait_cycles << std::hex;
     for (int i = 0; i < n; ++i)
         key << "|" << (uintptr_t)pairs[i].left << "," << (uintptr_t)pairs[i].right << ","
-            << (uintptr_t)pairs[i].disp_int << "," << (uintptr_t)pairs[i].disp_subpix;
+            << (uintptr_t)pairs[i].disp_int << "," << (uintptr_t)pairs[i].disp_subpix << "," << float_bits(pairs[i].sigma_s)
+            << "," << float_bits(pairs[i].sigma_r) << "," << float_bits(pairs[i].tau);
     auto it = ctx->bgraphs.find(key.str());
     if (it == ctx->bgraphs.end()) {
         size_t held = 0;

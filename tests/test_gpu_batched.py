@@ -264,3 +264,27 @@ def test_persistent_tensor_core_plan_member_matches_oracle(fbs, oracle_mod):
         ref_di, ref_ds, ref_agg = oracle_mod.fbs(L, R, q["D"], q["radius"], q["sigma_s"], q["sigma_r"], want_agg=True)
         check_disparities(q["disp_int"].cpu().numpy(), q["disp_subpix"].cpu().numpy(), ref_agg, ref_di, ref_ds, 2.0,
                           tol=tol)
+
+
+@pytest.mark.parametrize("prec,mode", [("f32", 0), ("f32", 1), ("bf16", 0), ("bf16", 1)])
+def test_batch_follows_changed_parameters_on_the_same_buffers(fbs, prec, mode):
+    """The images and maps stay where they are and sigma_s, sigma_r and tau
+    (TAD) of one pair change: each call returns the maps of its own
+    parameters, under every plan, also back at the first ones."""
+    p = fbs.FBS_PREC_F32 if prec == "f32" else fbs.FBS_PREC_BF16
+    pairs = _batch(51 + mode, n=4)
+    first = [dict(q) for q in pairs]
+    changes = [dict(sigma_s=1.5), dict(sigma_r=40.0)] + ([dict(tau=7.0)] if mode == 1 else [])
+    with fbs.Context(0, cost=mode, prec=p) as ctx:
+        for plan in range(7):
+            for change in [{}] + changes + [{}]:
+                for q, f in zip(pairs, first):
+                    q.update(f)
+                pairs[2].update(radius=4, **change)
+                fbs.fbs_batch_set_plan(ctx.ctx, pairs, plan)
+                ref = _per_pair(ctx, pairs)
+                fbs.fbs_compute_disparity_batched(ctx.ctx, pairs, torch.cuda.current_stream())
+                torch.cuda.synchronize()
+                for i, (q, (di, ds)) in enumerate(zip(pairs, ref)):
+                    assert torch.equal(q["disp_int"], di), (plan, change, i)
+                    assert torch.equal(q["disp_subpix"], ds), (plan, change, i)
