@@ -602,7 +602,7 @@ fbs_status run_forward(fbs_ctx* ctx, const NetScratch& s, int Hq, int Wq, const 
             LaunchScope ls(ctx, FBS_KERNEL_NET, st);
             e = launch_conv3x3(cin_pad(l), fwd_n(l), in, b->images + fwd_image_offset(l), bias, nullptr,
                                last ? (void*)s.out : (void*)s.y[l], last ? kOut : fwd_n(l), Hq, Wq, 0,
-                               last ? kConvLinearF32 : kConvReluBf16, ctx->derr, st, last ? head : ConvHead{});
+                               last ? kConvLinearF32 : kConvReluBf16, ctx->derr, ctx->wait_cycles, st, last ? head : ConvHead{});
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "band network convolution launch");
         if (!last) in = s.y[l];
@@ -640,7 +640,7 @@ fbs_status run_backward(fbs_ctx* ctx, const NetScratch& s, int H, int W, int D, 
             // gradient w.r.t. Y_{l-1} through its ReLU
             LaunchScope ls(ctx, FBS_KERNEL_NET, st);
             e = launch_conv3x3(cout_pad(l), cin(l), s.g[l], b->images + dgrad_image_offset(l), nullptr, s.y[l - 1],
-                               s.g[l - 1], cin(l), Hq, Wq, 1, kConvMaskBf16, ctx->derr, st);
+                               s.g[l - 1], cin(l), Hq, Wq, 1, kConvMaskBf16, ctx->derr, ctx->wait_cycles, st);
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "band data-gradient launch");
     }

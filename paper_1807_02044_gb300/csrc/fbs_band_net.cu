@@ -99,7 +99,8 @@ template <int CIN, int N>
 __global__ void __launch_bounds__(kConvThreads)
 conv3x3_tc_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ image,
                   const float* __restrict__ bias, const __nv_bfloat16* __restrict__ mask, void* __restrict__ out,
-                  int nout, int Hq, int Wq, int flip, int mode, ConvHead head, int* __restrict__ err)
+                  int nout, int Hq, int Wq, int flip, int mode, ConvHead head, long long wait_cycles,
+                  int* __restrict__ err)
 {
     using Box = ConvBox<CIN>;
     constexpr int KC = k_cores(CIN);            // core matrices along K
@@ -161,25 +162,33 @@ conv3x3_tc_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __r
         }
         umma_commit_elect(smem_u32(bar));
     }
-    if (!mbar_wait(smem_u32(bar), 0)) {
+    // the accumulator load is warp-collective: a warp goes on with all its lanes,
+    // or with none
+    const bool done = __all_sync(0xffffffffu, mbar_wait_for(smem_u32(bar), 0, wait_cycles));
+    if (!done) {
         // out of time: report it, and give the MMAs in flight one more bounded
-        // wait before the shared memory they read is given back
-        atomicCAS(err, 0, 21);
-        mbar_wait(smem_u32(bar), 0);
+        // wait before the memory they use is given back; nothing is stored
+        if ((tid & 31) == 0) {
+            atomicCAS(err, 0, 21);
+            mbar_wait(smem_u32(bar), 0);
+        }
+        __syncwarp();
     }
     tc_fence_after();
     // ---- epilogue: warp w holds TMEM lanes 32w .. 32w+31 -------------------
     float v[N];
+    if (done) {
 #pragma unroll
-    for (int c = 0; c < N; c += 16) {
-        float t16[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, t16);
+        for (int c = 0; c < N; c += 16) {
+            float t16[16];
+            tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, t16);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[c + i] = t16[i];
+            for (int i = 0; i < 16; ++i) v[c + i] = t16[i];
+        }
     }
     const int m = flip ? kM - 1 - tid : tid;
     const int X = tx0 + m % kTileX, Y = ty0 + m / kTileX;
-    if (X < Wq && Y < Hq) {
+    if (done && X < Wq && Y < Hq) {
         const size_t po = (size_t)Y * Wq + X;
         if (mode == kConvLinearF32) {
             float* o = reinterpret_cast<float*>(out) + po * nout;
@@ -222,13 +231,13 @@ conv3x3_tc_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __r
 template <int CIN, int N>
 cudaError_t launch_conv_t(const __nv_bfloat16* in, const __nv_bfloat16* image, const float* bias,
                           const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq, int flip, int mode,
-                          const ConvHead& head, int* err, cudaStream_t stream)
+                          const ConvHead& head, long long wait_cycles, int* err, cudaStream_t stream)
 {
     constexpr size_t smem = ConvBox<CIN>::kBytes + (size_t)k_cores(CIN) * N * 16 + 16;
     static_assert(smem <= 48 * 1024, "within the default limit");
     const dim3 grid((Wq + kTileX - 1) / kTileX, (Hq + kTileY - 1) / kTileY);
     return fbs::launch_after(conv3x3_tc_kernel<CIN, N>, grid, kConvThreads, smem, stream, in, image, bias, mask, out,
-                             nout, Hq, Wq, flip, mode, head, err);
+                             nout, Hq, Wq, flip, mode, head, wait_cycles > 0 ? wait_cycles : kWaitCycles, err);
 }
 
 // ---- weight gradients on the tensor cores ---------------------------------------
@@ -548,14 +557,14 @@ __global__ void pack_images_kernel(const float* __restrict__ theta, __nv_bfloat1
 
 cudaError_t launch_conv3x3(int cin_ch, int n, const __nv_bfloat16* in, const __nv_bfloat16* image, const float* bias,
                            const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq, int flip, int mode,
-                           int* err, cudaStream_t stream, const ConvHead& head)
+                           int* err, long long wait_cycles, cudaStream_t stream, const ConvHead& head)
 {
     if (cin_ch == 8 && n == 32)
-        return launch_conv_t<8, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
+        return launch_conv_t<8, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, wait_cycles, err, stream);
     if (cin_ch == 32 && n == 32)
-        return launch_conv_t<32, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
+        return launch_conv_t<32, 32>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, wait_cycles, err, stream);
     if (cin_ch == 32 && n == 16)
-        return launch_conv_t<32, 16>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, err, stream);
+        return launch_conv_t<32, 16>(in, image, bias, mask, out, nout, Hq, Wq, flip, mode, head, wait_cycles, err, stream);
     return cudaErrorInvalidValue;
 }
 

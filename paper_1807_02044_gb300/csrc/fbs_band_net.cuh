@@ -69,12 +69,14 @@ struct ConvHead {
 
 // 3x3 convolution, zero padding, of in [P][cin_ch] (P = Hq*Wq quarter pixels,
 // row-major) with a packed image of N output channels.  flip: gather the
-// neighbour at -offset (data gradient).  err: device word set on a timeout.
+// neighbour at -offset (data gradient).  err: device word set when the wait for
+// the products runs out (wait_cycles SM clock cycles, 0 = about 2 s).
 // A programmatic launch: the weights (image) must be older than the kernel
 // before it in the stream; everything else may be that kernel's output.
 cudaError_t launch_conv3x3(int cin_ch, int n, const __nv_bfloat16* in, const __nv_bfloat16* image,
                            const float* bias, const __nv_bfloat16* mask, void* out, int nout, int Hq, int Wq,
-                           int flip, int mode, int* err, cudaStream_t stream, const ConvHead& head = {});
+                           int flip, int mode, int* err, long long wait_cycles, cudaStream_t stream,
+                           const ConvHead& head = {});
 // Weight and bias gradient of layer l: sum over pixels of X[p + offset] G[p],
 // X [P][cin_pad(l)], G [P][cout_pad(l)]; written into grad (flat vector).
 // On the tensor cores; err: device word set on a timeout.

@@ -16,6 +16,7 @@ namespace tc {
 constexpr long long kWaitCycles = 4000000000LL;   // ~2 s at 2 GHz
 constexpr unsigned kWaitIters = 1u << 30;
 constexpr uint32_t kSuspendNs = 20000;   // a waiting thread sleeps up to this long per try
+constexpr long long kShortWait = 100000;   // clock cycles, more than such a sleep
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -38,6 +39,32 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "r"(bar), "r"(parity), "r"(kSuspendNs)
         : "memory");
     return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Wait for the completion of the phase with the given parity, for at most
+// `limit` SM clock cycles: by tries that sleep, or by polling where the limit is
+// shorter than a sleep may last.
+__device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, long long limit)
+{
+    const bool polls = limit < kShortWait;
+    if (!polls && mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (unsigned i = 0; i < kWaitIters; ++i) {
+        if (polls ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
+        if (clock64() - t0 > limit) break;
+    }
+    return false;
 }
 // Bounded wait for the completion of the phase with the given parity.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)

@@ -57,6 +57,52 @@ def test_wait_limit_runs_out_and_the_context_recovers(fbs, prec):
             fbs.fbs_set_wait_limit(ctx.ctx, -1.0)
 
 
+def test_convolution_wait_runs_out_and_stores_nothing(fbs):
+    """A limit of a clock cycle is over before the MMAs of a tile can have
+    completed.  Whatever a warp whose wait ran out leaves unstored still holds
+    the value of the first call on the same pair, so the activations and the
+    outputs stay bit for bit what they were, while fbs_sync reports
+    FBS_ERR_TIMEOUT; with the default limit the context computes again."""
+    H, W, D = 96, 160, 64
+    (dl, dr), (el, er) = _pair(3), _pair(4)
+    P = (H // 4) * (W // 4)
+    with fbs.Context(0) as ctx:
+        fbs.fbs_band_net_load(ctx.ctx, fbs.default_band_net_path())
+
+        def forward(left, right, out):
+            fbs.fbs_band_net_forward(ctx.ctx, left, right, H, W, 3, D, *out)
+            torch.cuda.synchronize()
+            return [o.clone() for o in out]
+
+        def outputs():
+            out = [torch.full(s, -7.0, device="cuda") for s in ((H // 4, W // 4, 2), (H, W), (H, W))]
+            torch.cuda.synchronize()   # the call runs on the context's own stream
+            return out
+
+        def trace():
+            acts = torch.empty(P * (8 + 5 * 32 + 2), device="cuda")
+            torch.cuda.synchronize()
+            fbs.fbs_band_net_trace(ctx.ctx, acts, None)
+            torch.cuda.synchronize()
+            return acts
+
+        out, other = outputs(), outputs()
+        first, other_first = forward(dl, dr, out), forward(el, er, other)
+        assert all(torch.equal(a, b) for a, b in zip(first, forward(dl, dr, out)))
+        acts = trace()
+        fbs.fbs_sync(ctx.ctx)
+        fbs.fbs_set_wait_limit(ctx.ctx, 1e-9)
+        late = forward(dl, dr, out)
+        with pytest.raises(fbs.FBSError) as ei:
+            fbs.fbs_sync(ctx.ctx)
+        assert ei.value.status == fbs.FBS_ERR_TIMEOUT and "code 21" in fbs.fbs_last_error(ctx.ctx)
+        assert torch.equal(trace(), acts)
+        assert all(torch.equal(a, b) for a, b in zip(first, late))
+        fbs.fbs_set_wait_limit(ctx.ctx, 0.0)
+        assert all(torch.equal(a, b) for a, b in zip(other_first, forward(el, er, outputs())))
+        fbs.fbs_sync(ctx.ctx)
+
+
 @pytest.mark.parametrize("prec", ["f32", "bf16"])
 def test_injected_launch_failure_is_reported_and_clears(fbs, prec):
     """An injected launch error surfaces as FBS_ERR_CUDA (an allocation error
