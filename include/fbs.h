@@ -85,8 +85,9 @@ fbs_status fbs_sync(fbs_ctx *ctx);
 
 /* Failure detection (not a step of the method).  Every wait of the
  * tensor-core aggregation on another part of the same kernel (its pipeline of
- * weight producers, copies, MMAs and epilogue) and the wait of the band
- * network's convolutions for their MMAs are bounded: after `seconds` of
+ * weight producers, copies, MMAs and epilogue), of the FP32 aggregation on its
+ * copies of cost rows and on the warps that share them, and of the band
+ * network's convolutions for their MMAs is bounded: after `seconds` of
  * SM clock time the kernel stops issuing work, lets its own copies and MMAs
  * land (a fixed ~2 s bound), frees its tensor memory and records an error
  * that the next fbs_sync returns as FBS_ERR_TIMEOUT; the outputs of that call

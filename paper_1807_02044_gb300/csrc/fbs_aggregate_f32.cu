@@ -136,14 +136,19 @@ __host__ __device__ inline size_t smem_bytes(int rho, int dc, int slots)
 // The ring of cost rows.  Every warp walks every row, so slot and parity (of
 // the row it is at) are the same sequence in all of them.
 //   kTma: done[slot] counts the warps that have finished the slot's row; the
-//   last one issues the box of the row S later.
+//   last one issues the box of the row S later.  The word after the count is 0,
+//   or 2 + the parity of the phase that the slot's last box completes.
 //   cp.async: every warp loads a quarter of each row, once all of them have
 //   arrived at the barrier done[slot]; a warp waits for that when it starts
 //   the next row.
+// Every wait is bounded.  When one runs out the error word is set, the warps walk
+// the rows that are left without waiting or copying, and the CTA lets the copies
+// in flight land (drain) and leaves its tile without storing anything.
 struct Ring {
     uint32_t full, done;      // shared addresses, 8 bytes per slot
     volatile uint32_t* abort;
     int* err;
+    long long limit;          // SM clock cycles that a wait may take
     int S, slot;
     uint32_t parity;
     __device__ __forceinline__ void next()
@@ -153,14 +158,32 @@ struct Ring {
             parity ^= 1u;
         }
     }
-    // Bounded (about 2 s): on a timeout the error word is set and nothing is waited for any more.
-    __device__ __forceinline__ void wait(uint32_t bar, uint32_t par) const
+    // False when the phase is not complete and nothing is waited for any more.
+    __device__ __forceinline__ bool wait(uint32_t bar, uint32_t par) const
     {
-        if (tc::mbar_try_wait(bar, par)) return;
-        if (*abort == 0 && !tc::mbar_wait(bar, par)) {
-            *abort = 1u;
-            atomicCAS(err, 0, 31);
+        if (limit >= tc::kShortWait && tc::mbar_try_wait(bar, par)) return true;
+        if (*abort != 0) return false;
+        if (tc::mbar_wait_for(bar, par, limit)) return true;
+        *abort = 1u;
+        atomicCAS(err, 0, 31);
+        return false;
+    }
+    // After a wait ran out, between barriers of the CTA: the copies in flight (those
+    // of a slot's last box; the ones before it were waited for) have landed, or had
+    // about 2 s more.
+    template <Copy COPY>
+    __device__ __forceinline__ void drain() const
+    {
+        if constexpr (COPY == kTma) {
+            if ((int)threadIdx.x < S) {
+                uint32_t armed;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(armed) : "r"(done + 8 * threadIdx.x + 4) : "memory");
+                if (armed != 0) tc::mbar_wait(full + 8 * threadIdx.x, armed & 1u);
+            }
+        } else {
+            asm volatile("cp.async.wait_all;" ::: "memory");
         }
+        __syncthreads();
     }
 };
 
@@ -172,13 +195,17 @@ struct Volume {
 };
 
 // Load cost row r, columns xlo .. xlo+NC-1, disparities dc0 .. dc0+DC-1 into a
-// slot; zeros outside the image and for disparities >= D.  kTma: one warp;
-// otherwise all of them, a thread its share.
+// slot; zeros outside the image and for disparities >= D.  kTma: one warp, which
+// notes the phase (parity) that the box completes; otherwise all of them, a thread
+// its share.
 template <int DC, Copy COPY>
-__device__ __forceinline__ void load_cost_row(uint32_t dst, uint32_t bar, const Volume& v, int r, int xlo, int NC, int dc0)
+__device__ __forceinline__ void load_cost_row(const Ring& ring, int slot, uint32_t parity, uint32_t rows_a, const Volume& v,
+                                              int r, int xlo, int NC, int dc0)
 {
+    const uint32_t dst = rows_a + slot * (uint32_t)(NC * DC * 4), bar = ring.full + 8 * slot;
     if constexpr (COPY == kTma) {
         if ((threadIdx.x & 31) == 0) {
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(ring.done + 8 * slot + 4), "r"(2u + parity) : "memory");
             tc::fence_proxy_async();   // the slot was read, and may hold staged sums, through the generic proxy
             tc::mbar_expect_tx(bar, 4u * DC * (uint32_t)NC);
             tma_load_3d(dst, v.map, dc0, xlo, r, bar);
@@ -445,9 +472,10 @@ __device__ __forceinline__ void wta_chunk(Tile& t, const float* st, int dc0, int
 }
 
 // Disparities dc0 .. dc0 + 8 KD - 1 of a tile (columns of DC staged disparities).
-// Starts and ends with every warp at the same point (a __syncthreads).
+// Starts and ends with every warp at the same point (a __syncthreads).  False (in
+// every thread) when a wait ran out: no copy is in flight and the ring is done with.
 template <int KD, int DC, Copy COPY, int ROWS>
-__device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_out, int dc0)
+__device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_out, int dc0)
 {
     constexpr int NDC = 8 * KD;       // disparities of this chunk
     constexpr int PW = 32 / ROWS;     // pixels of a warp along x
@@ -465,14 +493,15 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
     const bool on = t.whi >= dc0 && t.wlo < dc0 + NDC;
     const int w_lo = on ? t.wy - rho : t.H, w_hi = min(t.H - 1, t.wy + ROWS - 1) + rho;
     // a chunk that no warp needs is passed over
-    if (!__syncthreads_or(on)) return;
-    auto load_row = [&](int r, int slot) {
-        load_cost_row<DC, COPY>(rows_a + slot * slot_bytes, ring.full + 8 * slot, t.vol, r, xlo, NC, dc0);
+    if (!__syncthreads_or(on)) return true;
+    auto load_row = [&](int r, int slot, uint32_t parity) {
+        load_cost_row<DC, COPY>(ring, slot, parity, rows_a, t.vol, r, xlo, NC, dc0);
     };
     // the first S rows
     for (int i = COPY == kTma ? warp : 0; i < ring.S && t.r_lo + i <= t.r_hi; i += COPY == kTma ? kWarps : 1) {
         const int slot = ring.slot + i;
-        load_row(t.r_lo + i, slot < ring.S ? slot : slot - ring.S);
+        if (slot < ring.S) load_row(t.r_lo + i, slot, ring.parity);
+        else load_row(t.r_lo + i, slot - ring.S, ring.parity ^ 1u);
     }
 
     // accumulating role: lane bits 0, 2, 3 = disparity group k, bits 1, 4 = pixel group
@@ -502,8 +531,8 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
             // refill the slot of the row before
             if (r > t.r_lo && r - 1 + ring.S <= t.r_hi) {
                 const int slot = ring.slot == 0 ? ring.S - 1 : ring.slot - 1;
-                ring.wait(ring.done + 8 * slot, ring.slot == 0 ? ring.parity ^ 1u : ring.parity);
-                load_row(r - 1 + ring.S, slot);
+                const uint32_t parity = ring.slot == 0 ? ring.parity ^ 1u : ring.parity;
+                if (ring.wait(ring.done + 8 * slot, parity)) load_row(r - 1 + ring.S, slot, parity ^ 1u);
             }
         }
         if (r >= w_lo && r <= w_hi) {
@@ -527,13 +556,17 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
             done = __shfl_sync(0xffffffffu, done, 0);
             // the last warp to finish the row refills its slot
             if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && *ring.abort == 0)
-                load_row(r + ring.S, ring.slot);
+                load_row(r + ring.S, ring.slot, ring.parity ^ 1u);
         } else {
             if (lane == 0) tc::mbar_arrive(ring.done + 8 * ring.slot);
         }
         ring.next();
     }
-    __syncthreads();   // every row consumed: the stage may overwrite the rows and weights
+    // every row consumed: the stage may overwrite the rows and weights
+    if (__syncthreads_or(*ring.abort != 0)) {
+        ring.drain<COPY>();
+        return false;
+    }
 
     // normalise and stage [pixel of the warp][d]
     float* const stage = t.rows + warp * 32 * SP;
@@ -576,24 +609,26 @@ __device__ __forceinline__ void aggregate_chunk(Tile& t, Ring& ring, float* agg_
     wta_chunk(t, stage + lane * SP, dc0, max(0, t.blo - dc0), min(nd, t.bhi + 1 - dc0));
     tc::fence_proxy_async();   // the next chunk's bulk copies overwrite the stage
     __syncthreads();
+    return true;
 }
 
 // The ring's barriers and counters, set up once per CTA (ends with a __syncthreads).
 template <Copy COPY>
-__device__ __forceinline__ Ring make_ring(void* smem, int slots, int* err)
+__device__ __forceinline__ Ring make_ring(void* smem, int slots, long long limit, int* err)
 {
     Ring ring;
     ring.full = tc::smem_u32(smem);
     ring.done = ring.full + 8 * kMaxSlots;
     ring.abort = (volatile uint32_t*)((uint8_t*)smem + 16 * kMaxSlots);
     ring.err = err;
+    ring.limit = limit;
     ring.S = slots;
     ring.slot = 0;
     ring.parity = 0;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxSlots; ++s) {
             tc::mbar_init(ring.full + 8 * s, COPY == kTma ? 1 : kThreads);
-            if (COPY == kTma) ((uint32_t*)smem)[2 * (kMaxSlots + s)] = 0;
+            if (COPY == kTma) ((uint64_t*)smem)[kMaxSlots + s] = 0;
             else tc::mbar_init(ring.done + 8 * s, kWarps);
         }
         *ring.abort = 0;
@@ -608,8 +643,9 @@ __device__ __forceinline__ Ring make_ring(void* smem, int slots, int* err)
 // several tiles in a row.  band (nullable) restricts the WTA and Eq. (10) of
 // each pixel to its own band [lo, hi], a sub-range of [d_begin, d_end);
 // without it every pixel uses [0, D-1].  d_begin must be a multiple of 4.
+// False (in every thread) when a wait ran out: nothing was stored.
 template <Copy COPY, int ROWS>
-__device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, const CUtensorMap* map, int ld,
+__device__ __forceinline__ bool aggregate_tile(const float* __restrict__ cost, const CUtensorMap* map, int ld,
                                                const uint8_t* __restrict__ guide, int H, int W, int C, int D,
                                                int rho, float neg_ks, float neg_kr, float* __restrict__ agg_out,
                                                int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int x0,
@@ -679,14 +715,16 @@ __device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, c
 
     for (int dc0 = d_begin; dc0 < d_end; dc0 += 64) {
         const int left = d_end - dc0;
+        bool ok;
         if (D > 32) {
-            if (left > 32) aggregate_chunk<8, 64, COPY, ROWS>(t, ring, agg_out, dc0);
-            else aggregate_chunk<4, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+            if (left > 32) ok = aggregate_chunk<8, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+            else ok = aggregate_chunk<4, 64, COPY, ROWS>(t, ring, agg_out, dc0);
         } else if (D > 16) {
-            aggregate_chunk<4, 32, COPY, ROWS>(t, ring, agg_out, dc0);
+            ok = aggregate_chunk<4, 32, COPY, ROWS>(t, ring, agg_out, dc0);
         } else {
-            aggregate_chunk<2, 16, COPY, ROWS>(t, ring, agg_out, dc0);
+            ok = aggregate_chunk<2, 16, COPY, ROWS>(t, ring, agg_out, dc0);
         }
+        if (!ok) return false;
     }
 
     if (valid) {
@@ -700,6 +738,7 @@ __device__ __forceinline__ void aggregate_tile(const float* __restrict__ cost, c
         if (disp_sub) disp_sub[o] = ds;
     }
     __syncthreads();   // the guide window may be overwritten
+    return true;
 }
 
 constexpr int kCtasPerSm = 4;
@@ -709,10 +748,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 aggregate_f32_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
                      const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
                      float* __restrict__ agg_out, int32_t* __restrict__ disp_int, float* __restrict__ disp_sub,
-                     int slots, int* __restrict__ err)
+                     int slots, long long wait_cycles, int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<COPY>(smem_f4, slots, err);
+    Ring ring = make_ring<COPY>(smem_f4, slots, wait_cycles, err);
     aggregate_tile<COPY, 2>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
                             blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, ring, 0, D, nullptr);
 }
@@ -724,10 +763,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
                       const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
                       const int2* __restrict__ tile_range, const uint32_t* __restrict__ band,
-                      int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int slots, int* __restrict__ err)
+                      int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int slots, long long wait_cycles,
+                      int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<kTma>(smem_f4, slots, err);
+    Ring ring = make_ring<kTma>(smem_f4, slots, wait_cycles, err);
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the ranges and bands come from earlier kernels
     const int2 r = tile_range[(size_t)blockIdx.y * gridDim.x + blockIdx.x];
     aggregate_tile<kTma, 4>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
@@ -742,7 +782,7 @@ aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, in
                              int slots, int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<kAsync16>(smem_f4, slots, err);
+    Ring ring = make_ring<kAsync16>(smem_f4, slots, 0, err);
     __shared__ int item_s;
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
@@ -754,9 +794,11 @@ aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, in
         const BatchPair& bp = pairs[pi];
         const int t = item - bp.agg_off;
         const int ntx = (bp.W + kTX - 1) / kTX;
-        aggregate_tile<kAsync16, 2>(bp.cost, nullptr, bp.ld, bp.left, bp.H, bp.W, bp.C, bp.D, bp.radius, bp.neg_ks,
-                                    bp.neg_kr, nullptr, bp.disp_int, bp.disp_sub, (t % ntx) * kTX, (t / ntx) * kTY,
-                                    smem_f4, ring, 0, bp.D, nullptr);
+        ring.limit = bp.wait_cycles;
+        if (!aggregate_tile<kAsync16, 2>(bp.cost, nullptr, bp.ld, bp.left, bp.H, bp.W, bp.C, bp.D, bp.radius, bp.neg_ks,
+                                         bp.neg_kr, nullptr, bp.disp_int, bp.disp_sub, (t % ntx) * kTX, (t / ntx) * kTY,
+                                         smem_f4, ring, 0, bp.D, nullptr))
+            break;
     }
 }
 
@@ -792,7 +834,7 @@ bool encode_volume(CUtensorMap* map, const float* cost, int ld, int H, int W, in
 template <Copy COPY>
 cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                         int D, int rho, float neg_ks, float neg_kr, float* agg_out, int32_t* disp_int, float* disp_sub,
-                        int* err, bool after_cost, cudaStream_t stream)
+                        long long wait_cycles, int* err, bool after_cost, cudaStream_t stream)
 {
     const int slots = ring_slots(rho, column_size(D));
     const size_t smem = smem_bytes(rho, column_size(D), slots);
@@ -801,14 +843,16 @@ cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
     if (after_cost)
         return fbs::launch_after(aggregate_f32_kernel<COPY>, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D,
-                                 rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, err);
+                                 rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, wait_cycles, err);
     fbs::note_launch();
     aggregate_f32_kernel<COPY><<<grid, kThreads, smem, stream>>>(
-        map, cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, err);
+        map, cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, wait_cycles, err);
     return cudaGetLastError();
 }
 
 }  // namespace
+
+long long wait_limit(long long wait_cycles) { return wait_cycles > 0 ? wait_cycles : tc::kWaitCycles; }
 
 int agg_f32_tiles(int H, int W) { return ((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY); }
 
@@ -830,7 +874,8 @@ cudaError_t launch_aggregate_f32_batched(const BatchPair* pairs, int npairs, int
 
 cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
                                   int radius, float sigma_s, float sigma_r, const int2* tile_range,
-                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, int* err, cudaStream_t stream)
+                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, long long wait_cycles, int* err,
+                                  cudaStream_t stream)
 {
     const double log2e = 1.4426950408889634;
     const float neg_ks = (float)(-log2e / ((double)sigma_s * sigma_s));
@@ -843,12 +888,13 @@ cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guid
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
     return fbs::launch_after(aggregate_band_kernel, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D, radius,
-                             neg_ks, neg_kr, tile_range, band, disp_int, disp_sub, slots, err);
+                             neg_ks, neg_kr, tile_range, band, disp_int, disp_sub, slots, wait_limit(wait_cycles), err);
 }
 
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                                  int D, int radius, float sigma_s, float sigma_r, float* agg_out,
-                                 int32_t* disp_int, float* disp_sub, int* err, bool after_cost, cudaStream_t stream)
+                                 int32_t* disp_int, float* disp_sub, long long wait_cycles, int* err, bool after_cost,
+                                 cudaStream_t stream)
 {
     // exp(-a/g^2) = exp2(-a * log2(e) / g^2)
     const double log2e = 1.4426950408889634;
@@ -857,9 +903,9 @@ cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide
     CUtensorMap map{};
     if (encode_volume(&map, cost, ld, H, W, D, radius))
         return launch_copy<kTma>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                 err, after_cost, stream);
+                                 wait_limit(wait_cycles), err, after_cost, stream);
     return launch_copy<kAsync4>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                err, after_cost, stream);
+                                wait_limit(wait_cycles), err, after_cost, stream);
 }
 
 }  // namespace fbs

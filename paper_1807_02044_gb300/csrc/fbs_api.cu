@@ -94,7 +94,7 @@ fbs_status run_path(fbs_ctx* ctx, const uint8_t* left, const uint8_t* right, int
     {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_f32(cost, ld, left, H, W, C, D, radius, sigma_s, sigma_r, nullptr, disp_int,
-                                      disp_subpix, ctx->derr, true, st);
+                                      disp_subpix, ctx->wait_cycles, ctx->derr, true, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "aggregation launch");
     return FBS_OK;
@@ -456,7 +456,7 @@ fbs_status fbs_aggregate(fbs_ctx* ctx, const float* cost, const uint8_t* guide, 
     {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_f32(cost, D, guide, H, W, C, D, radius, sigma_s, sigma_r, agg_out, disp_int,
-                                      disp_subpix, ctx->derr, false, st);
+                                      disp_subpix, ctx->wait_cycles, ctx->derr, false, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "aggregation launch");
     return FBS_OK;

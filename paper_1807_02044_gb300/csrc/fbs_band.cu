@@ -672,7 +672,7 @@ fbs_status run_banded(fbs_ctx* ctx, const fbs_pair* p, const float* centre, cons
     {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_band(cost, ld, p->left, H, W, p->C, D, p->radius, p->sigma_s, p->sigma_r,
-                                       s.tile_range, s.band, p->disp_int, p->disp_subpix, ctx->derr, st);
+                                       s.tile_range, s.band, p->disp_int, p->disp_subpix, ctx->wait_cycles, ctx->derr, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "band aggregation launch");
     return FBS_OK;

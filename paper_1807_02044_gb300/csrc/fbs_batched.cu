@@ -190,6 +190,7 @@ void fill_table(fbs_ctx* ctx, const Layout& L, int n, const fbs_pair* pairs, fbs
         b.neg_ks = (float)(-log2e / ((double)q.sigma_s * q.sigma_s));
         b.neg_kr = (float)(-log2e / ((double)q.sigma_r * q.sigma_r));
         b.tau = q.tau;
+        b.wait_cycles = fbs::wait_limit(ctx->wait_cycles);
         uint8_t* base = (uint8_t*)ctx->ws + L.off[k];
         b.sc = fbs::carve_cost_scratch(base, q.H, q.W);
         b.cost = (float*)(base + fbs::cost_scratch_bytes(q.H, q.W));
@@ -364,7 +365,7 @@ fbs_status build_branch_graph(fbs_ctx* ctx, int n, const fbs_pair* pairs, int nb
             k0 = fbs::launch_count();
             if (e == cudaSuccess)
                 e = fbs::launch_aggregate_f32(cost, ld, q.left, q.H, q.W, q.C, q.D, q.radius, q.sigma_s, q.sigma_r,
-                                              nullptr, q.disp_int, q.disp_subpix, ctx->derr, true, s);
+                                              nullptr, q.disp_int, q.disp_subpix, ctx->wait_cycles, ctx->derr, true, s);
             g->kernels[FBS_KERNEL_AGG_F32] += fbs::launch_count() - k0;
             continue;
         }

@@ -101,13 +101,16 @@ cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* lef
 constexpr int kAggTileX = 32;
 constexpr int kAggTileY = 4;
 // agg_out (nullable) is written with row pitch D (caller layout [H][W][D]).
-// err: device int set to nonzero if a bounded wait inside the kernel gave up.
+// wait_cycles (0 = about 2 s) limits each wait of a CTA on its copies and warps;
+// err: device int set to nonzero if one gave up.
 // after_cost: the previous kernel of the stream is one of this library's (the cost
 // build), so the launch may be programmatic.
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W,
                                  int C, int D, int radius, float sigma_s, float sigma_r,
-                                 float* agg_out, int32_t* disp_int, float* disp_sub, int* err,
-                                 bool after_cost, cudaStream_t stream);
+                                 float* agg_out, int32_t* disp_int, float* disp_sub, long long wait_cycles,
+                                 int* err, bool after_cost, cudaStream_t stream);
+// The limit in SM clock cycles that wait_cycles stands for.
+long long wait_limit(long long wait_cycles);
 
 // ---- steps 2-4 on the tensor cores (BF16 / FP16 operands, FP32 accumulate) ---
 // cost: 16-bit x-blocked volume (see launch_cost_build_xblock16), 16-byte
@@ -172,8 +175,8 @@ cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const u
                              cudaStream_t stream);
 cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
                                   int radius, float sigma_s, float sigma_r, const int2* tile_range,
-                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, int* err,
-                                  cudaStream_t stream);
+                                  const uint32_t* band, int32_t* disp_int, float* disp_sub, long long wait_cycles,
+                                  int* err, cudaStream_t stream);
 
 // ---- batched form: one persistent launch per stage over many pairs ------------
 // Device-side description of one pair of a batch.  *_off is the index of the
@@ -184,6 +187,7 @@ struct BatchPair {
     const uint8_t* right;
     int H, W, C, D, radius, ld, mode;
     float neg_ks, neg_kr, tau;
+    long long wait_cycles;   // > 0: the limit of one wait in the aggregation
     CostScratch sc;
     float* cost;
     int32_t* disp_int;

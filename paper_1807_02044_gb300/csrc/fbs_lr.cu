@@ -151,13 +151,13 @@ extern "C" fbs_status fbs_compute_disparity_lr(fbs_ctx* ctx, const uint8_t* left
     {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_f32(cost_l, ld, left, H, W, C, D, radius, sigma_s, sigma_r, nullptr, dl,
-                                      disp_subpix, ctx->derr, true, st);
+                                      disp_subpix, ctx->wait_cycles, ctx->derr, true, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "left aggregation launch");
     if (want_right) {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_f32(cost_r, ld, right, H, W, C, D, radius, sigma_s, sigma_r, nullptr, dr,
-                                      disp_subpix_right, ctx->derr, true, st);
+                                      disp_subpix_right, ctx->wait_cycles, ctx->derr, true, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "right aggregation launch");
     }
     if (lrc) {

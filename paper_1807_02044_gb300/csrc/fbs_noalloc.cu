@@ -73,7 +73,7 @@ extern "C" fbs_status fbs_compute_disparity_noalloc(fbs_ctx* ctx, const uint8_t*
     {
         LaunchScope ls(ctx, FBS_KERNEL_AGG_F32, st);
         e = fbs::launch_aggregate_f32(cost, ld, left, H, W, C, D, radius, sigma_s, sigma_r, nullptr, disp_int,
-                                      disp_subpix, ctx->derr, true, st);
+                                      disp_subpix, ctx->wait_cycles, ctx->derr, true, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "aggregation launch");
     return FBS_OK;

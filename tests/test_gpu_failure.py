@@ -103,6 +103,66 @@ def test_convolution_wait_runs_out_and_stores_nothing(fbs):
         fbs.fbs_sync(ctx.ctx)
 
 
+@pytest.mark.parametrize("form", ["path", "lr", "unaligned", "batch0", "batch3", "batch4", "band"])
+def test_fp32_aggregation_wait_runs_out_and_stores_nothing(fbs, form):
+    """A limit of a clock cycle is over before a copied cost row can have landed:
+    the CTAs of an SM ask for 128 KB of rows at once, and with radius 0 they have
+    a few hundred cycles of work before they wait for them; the 4-byte copies
+    take longer to issue, and there (radius 1) the first warps that are done with
+    a slot wait for the others before they refill it.
+    A tile whose wait ran out lets its copies land and stores nothing, so it
+    still holds the maps of the first call on the same inputs, and every other
+    tile computes them again: the outputs stay bit for bit what they were,
+    while fbs_sync reports FBS_ERR_TIMEOUT; with the default limit the context
+    computes other inputs like a fresh one.  Forms: TMA rows, both views, 4-byte
+    copies (D = 255), the persistent (0, 3) and a branched (4) batch plan, bands."""
+    H, W, D, r = 240, 640, 256, int(form == "unaligned")
+    (dl, dr), (el, er) = _pair(3, H, W), _pair(4, H, W)
+    cost = torch.rand((2, H, W, 255), device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    centre, conf = torch.full((H, W), 6.0, device="cuda"), (torch.arange(W, device="cuda") < W // 2).float().repeat(H, 1)
+    torch.cuda.synchronize()
+
+    def outputs():
+        return [torch.full((H, W), -7, dtype=t, device="cuda") for t in (torch.int32, torch.float32) * 2]
+
+    def call(ctx, left, right, out):
+        st = torch.cuda.current_stream()
+        pair = dict(left=left, right=right, H=H, W=W, C=3, D=D, radius=r, sigma_s=2.0, sigma_r=12.0, tau=0.0,
+                    disp_int=out[0], disp_subpix=out[1])
+        if form == "path":
+            fbs.fbs_compute_disparity(ctx.ctx, left, right, H, W, 3, D, r, 2.0, 12.0, 0.0, out[0], out[1], st)
+        elif form == "lr":
+            fbs.fbs_compute_disparity_lr(ctx.ctx, left, right, H, W, 3, D, r, 2.0, 12.0, 0.0, *out, False, st)
+        elif form == "unaligned":
+            c = cost[0 if left is dl else 1]
+            fbs.fbs_aggregate(ctx.ctx, c, left, H, W, 3, 255, r, 2.0, 12.0, None, out[0], out[1], st)
+        elif form == "band":
+            fbs.fbs_compute_disparity_banded(ctx.ctx, pair, centre, conf, 3, 0.5, st)
+        else:
+            pairs = [pair, dict(pair, radius=1, disp_int=out[2], disp_subpix=out[3])]
+            fbs.fbs_batch_set_plan(ctx.ctx, pairs, int(form[5:]))
+            fbs.fbs_compute_disparity_batched(ctx.ctx, pairs, st)
+        torch.cuda.synchronize()
+        return [o.clone() for o in out]
+
+    with fbs.Context(0) as ref:
+        want = call(ref, el, er, outputs())
+        fbs.fbs_sync(ref.ctx)
+    with fbs.Context(0) as ctx:
+        out = outputs()
+        first = call(ctx, dl, dr, out)
+        fbs.fbs_sync(ctx.ctx)
+        fbs.fbs_set_wait_limit(ctx.ctx, 1e-9)
+        late = call(ctx, dl, dr, out)
+        with pytest.raises(fbs.FBSError) as ei:
+            fbs.fbs_sync(ctx.ctx)
+        assert ei.value.status == fbs.FBS_ERR_TIMEOUT and "code 31" in fbs.fbs_last_error(ctx.ctx)
+        assert all(torch.equal(a, b) for a, b in zip(first, late))
+        fbs.fbs_set_wait_limit(ctx.ctx, 0.0)
+        assert all(torch.equal(a, b) for a, b in zip(want, call(ctx, el, er, outputs())))
+        fbs.fbs_sync(ctx.ctx)
+
+
 @pytest.mark.parametrize("prec", ["f32", "bf16"])
 def test_injected_launch_failure_is_reported_and_clears(fbs, prec):
     """An injected launch error surfaces as FBS_ERR_CUDA (an allocation error
