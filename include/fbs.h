@@ -63,7 +63,8 @@ typedef struct {
     int fused;                  /* reserved, 0 */
     size_t workspace_cap;       /* bytes of scratch the context may hold; 0 = unlimited */
     const char *autotune_cache_path; /* batched form: file of "shape plan" lines the
-                                        autotuner appends to and reads back; may be NULL */
+                                        autotuner appends to and reads back (those of
+                                        this build and SM count); may be NULL */
 } fbs_options;
 
 /* Fill *opt with the defaults: NCC, F32, unfused, no cap, no autotune cache file. */

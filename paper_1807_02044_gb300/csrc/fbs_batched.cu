@@ -79,15 +79,30 @@ std::string batch_signature(fbs_ctx* ctx, int n, const fbs_pair* pairs)
     return os.str();
 }
 
+// In the file a signature is preceded by what a choice holds for besides the
+// shape: the generation of the kernels and plans (kTuneGeneration, to be raised
+// with either) and the device's SM count.  Other entries, those without a prefix
+// among them, are passed over and their shapes tuned again.
+constexpr int kTuneGeneration = 2;
+
+std::string tuned_prefix(const fbs_ctx* ctx)
+{
+    return "g" + std::to_string(kTuneGeneration) + "sm" + std::to_string(ctx->num_sms) + ":";
+}
+
 void load_tuned(fbs_ctx* ctx)
 {
     ctx->btuned_loaded = true;
     if (!ctx->opt.autotune_cache_path) return;
     std::ifstream f(ctx->opt.autotune_cache_path);
-    std::string sig;
+    const std::string prefix = tuned_prefix(ctx);
+    std::string entry;
     int plan;
-    while (f >> sig >> plan)
+    while (f >> entry >> plan) {
+        if (entry.compare(0, prefix.size(), prefix) != 0) continue;
+        const std::string sig = entry.substr(prefix.size());
         if (plan >= 0 && plan < (sig[0] == 't' ? kTcPlans : kPlans)) ctx->btuned[sig] = plan;
+    }
 }
 
 void store_tuned(fbs_ctx* ctx, const std::string& sig, int plan)
@@ -96,7 +111,7 @@ void store_tuned(fbs_ctx* ctx, const std::string& sig, int plan)
     // a leading newline keeps the entry on a line of its own even after a
     // truncated last line (blank lines are skipped by load_tuned)
     std::ofstream f(ctx->opt.autotune_cache_path, std::ios::app);
-    if (f) f << "\n" << sig << " " << plan << "\n";
+    if (f) f << "\n" << tuned_prefix(ctx) << sig << " " << plan << "\n";
 }
 
 // Device buffers that graphs capture by address: grown only here, and every

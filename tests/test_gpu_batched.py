@@ -288,3 +288,28 @@ def test_batch_follows_changed_parameters_on_the_same_buffers(fbs, prec, mode):
                 for i, (q, (di, ds)) in enumerate(zip(pairs, ref)):
                     assert torch.equal(q["disp_int"], di), (plan, change, i)
                     assert torch.equal(q["disp_subpix"], ds), (plan, change, i)
+
+
+@pytest.mark.parametrize("prec", ["f32", "bf16"])
+def test_autotune_entries_of_other_builds_or_devices_are_tuned_again(fbs, tmp_path, prec):
+    """A stored plan holds for the kernels and the SM count it was timed with: entries without a generation, of
+    another one or of another SM count are passed over, and the call tunes the shape and stores its own."""
+    p = fbs.FBS_PREC_F32 if prec == "f32" else fbs.FBS_PREC_BF16
+    pairs = _batch(9, n=3)
+    sig = ("" if prec == "f32" else "tb") + "m0;" + "".join(
+        f"{q['H']}x{q['W']}x{q['C']}x{q['D']}r{q['radius']};" for q in pairs)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    path = tmp_path / "tune.txt"
+    path.write_text(f"{sig} 3\ng1sm{sms}:{sig} 3\ng2sm{sms + 1}:{sig} 3\n")
+    with fbs.Context(0, prec=p, autotune_cache_path=str(path)) as ctx:
+        assert fbs.fbs_batch_plan(ctx.ctx, pairs) == -1
+        fbs.fbs_compute_disparity_batched(ctx.ctx, pairs, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        plan = fbs.fbs_batch_plan(ctx.ctx, pairs)
+    assert plan >= 0
+    last = path.read_text().splitlines()[-1].split()
+    assert last[0].endswith(":" + sig) and int(last[1]) == plan
+    own = last[0]
+    path.write_text(f"{own} {(plan + 1) % 4}\n")       # this build's own entry is taken
+    with fbs.Context(0, prec=p, autotune_cache_path=str(path)) as ctx:
+        assert fbs.fbs_batch_plan(ctx.ctx, pairs) == (plan + 1) % 4
