@@ -187,17 +187,47 @@ __device__ __forceinline__ void tc_row_pairs(uint8_t* arow, const uint8_t* grow,
 // two neighbours for Eq. (10).
 //
 // Of every 16 values only the smallest is compared with the best so far; where
-// it is smaller, the 16 are searched for its first place and its neighbours: two
-// instructions per value, and four more in a search, instead of always six.  With a
-// single accumulator (D > 240) the next tile waits for them (1920 x 1080, D = 256,
-// radius 9 1282 -> 1210 us; 1280 x 720, D = 192, radius 2 152 -> 130 us).  Where the
-// winners of a warp's 32 pixels have nothing in common (two unrelated noise images)
-// nearly every 16 are searched: 1313 and 162 us.  Only noting the 16 and searching
-// them at the end, from tensor memory, is 1182 us at best and 1419 us there.
+// it is smaller, its first place among the 16 and its neighbours are found by
+// halving (tc_first_of): two instructions per value, and two more in a search.
+// With a single accumulator (D > 240) the next tile waits for them.  Always the
+// first of running comparisons, six per value -> a search of four per value more,
+// by comparing each with the smallest -> now: where the winners of a warp's 32
+// pixels have nothing in common (two unrelated noise images, nearly every 16 are
+// searched) fbs_aggregate of 1280 x 720, radius 2, D = 192 323 -> 337 -> 313 us,
+// radius 0, D = 256 411 -> 431 -> 406 us; on a scene the whole call at 1920 x 1080,
+// radius 9, D = 256 1489 -> 1475 us by the last step.
 struct TcWta {
     int bidx;
     float best, a_prev, a_next;
 };
+
+// The first of 16 values w, disparities cb .., that equals their smallest (low;
+// low_a: of the first eight) becomes the best, its neighbours a_prev and a_next
+// (last: the value before w[0]; a_next stays after w[15], the caller sets it).
+// Half of the values, then half of those, by selects.
+__device__ __forceinline__ void tc_first_of(const float (&w)[16], float low, float low_a, float last, int cb, TcWta& r)
+{
+    const bool up8 = low_a != low;
+    float u[8], t[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) u[i] = up8 ? w[8 + i] : w[i];
+    float prev = up8 ? w[7] : last, next = up8 ? r.a_next : w[8];
+    const bool up4 = fminf(fminf(u[0], u[1]), fminf(u[2], u[3])) != low;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = up4 ? u[4 + i] : u[i];
+    prev = up4 ? u[3] : prev;
+    next = up4 ? next : u[4];
+    const bool up2 = fminf(t[0], t[1]) != low;
+    const float s0 = up2 ? t[2] : t[0], s1 = up2 ? t[3] : t[1];
+    prev = up2 ? t[1] : prev;
+    next = up2 ? next : t[2];
+    const bool up1 = s0 != low;
+    r.best = low;
+    r.bidx = cb + (up8 ? 8 : 0) + (up4 ? 4 : 0) + (up2 ? 2 : 0) + (up1 ? 1 : 0);
+    r.a_prev = up1 ? s0 : prev;
+    r.a_next = up1 ? next : s1;
+}
+
 __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N, int D, float* arow)
 {
     float dv[16];
@@ -231,23 +261,16 @@ __device__ __forceinline__ TcWta tc_wta(uint32_t tbase, uint32_t den_col, int N,
                 for (int i = 0; i < 16; ++i)
                     if (cb + i >= D) w[i] = finf;
             }
-            float low = w[15];
+            float low_a = w[7], low_b = w[15];
 #pragma unroll
-            for (int i = 0; i < 14; i += 2) low = fminf(fminf(w[i], w[i + 1]), low);
-            low = fminf(low, w[14]);
-            if (r.bidx == cb - 1) r.a_next = w[0];   // the best was the last of the 16 before
-            if (low < r.best) {
-                r.best = low;
-                r.bidx = cb + 15;
-                r.a_prev = w[14];
-#pragma unroll
-                for (int i = 14; i >= 0; --i) {
-                    const bool eq = w[i] == low;
-                    r.bidx = eq ? cb + i : r.bidx;
-                    r.a_prev = eq ? (i > 0 ? w[i - 1] : last) : r.a_prev;
-                    r.a_next = eq ? w[i + 1] : r.a_next;
-                }
+            for (int i = 0; i < 6; i += 2) {
+                low_a = fminf(fminf(w[i], w[i + 1]), low_a);
+                low_b = fminf(fminf(w[8 + i], w[9 + i]), low_b);
             }
+            low_a = fminf(low_a, w[6]);
+            const float low = fminf(low_a, fminf(low_b, w[14]));
+            if (r.bidx == cb - 1) r.a_next = w[0];   // the best was the last of the 16 before
+            if (low < r.best) tc_first_of(v[hc], low, low_a, last, cb, r);
             last = w[15];
         }
     }

@@ -128,6 +128,37 @@ def test_tc_winner_takes_the_first_of_equal_costs(fbs, prec, D):
     np.testing.assert_array_equal(ds.cpu().numpy(), ref)
 
 
+@pytest.mark.parametrize("D", [16, 23, 40, 256])
+def test_tc_winner_at_every_place(fbs, D):
+    """With radius 0 the aggregated value is the cost itself (16ths up to 8, exact in 16 bits).  Pixel x of a row has
+    its smallest cost at d = x: alone; with an equal one next to it; with one further on; after costs that fall to
+    it from place to place; among far larger ones.  Winner and parabola (Eq. (10)) as in FP32."""
+    rng = np.random.default_rng(D)
+    A = (rng.integers(32, 129, (5, D, D)) / 16).astype(np.float32)
+    x = np.arange(D)
+    for d in range(D):
+        A[3, d, :d + 1] = 1.0 + np.minimum(7.0, (d - x[:d + 1]) / 16)
+        A[4, d, rng.random(D) < 0.5] = 512.0
+        if d + 1 < D:
+            A[1, d, d + 1] = 1.0
+            A[2, d, rng.integers(d + 1, D)] = 1.0
+    A[:, x, x] = 1.0
+    assert np.array_equal(A.argmin(2), np.broadcast_to(x, (5, D)))
+    cost, guide = torch.from_numpy(A).cuda(), torch.zeros((5, D, 3), dtype=torch.uint8, device="cuda")
+    with fbs.Context(0, prec=fbs.FBS_PREC_F16) as ctx:
+        _, di, ds = ctx.aggregate(cost, guide, 0, 1.0, 10.0)
+        torch.cuda.synchronize()
+        fbs.fbs_sync(ctx.ctx)
+    assert np.array_equal(di.cpu().numpy(), np.broadcast_to(x, (5, D)))
+    i = x[1:-1]
+    a, b, c = A[:, i, i - 1], A[:, i, i], A[:, i, i + 1]
+    den = np.float32(2) * a + np.float32(2) * c - np.float32(4) * b
+    sub = i + np.where(den > 0, (a - c) / np.where(den > 0, den, np.float32(1)), np.float32(0))
+    got = ds.cpu().numpy()
+    assert np.array_equal(got[:, [0, -1]], np.broadcast_to(x[[0, -1]], (5, 2)).astype(np.float32))
+    np.testing.assert_allclose(got[:, 1:-1], sub.astype(np.float32), rtol=0, atol=2.0 ** -22 * D)
+
+
 @pytest.mark.parametrize("prec", ["bf16", "f16"])
 def test_tc_full_size_bench_workload_bad_pixels(fbs, oracle_mod, prec):
     """640x480 RGB, D=64, radius 7 (the benchmark workload): aggregated costs
