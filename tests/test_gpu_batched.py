@@ -313,3 +313,22 @@ def test_autotune_entries_of_other_builds_or_devices_are_tuned_again(fbs, tmp_pa
     path.write_text(f"{own} {(plan + 1) % 4}\n")       # this build's own entry is taken
     with fbs.Context(0, prec=p, autotune_cache_path=str(path)) as ctx:
         assert fbs.fbs_batch_plan(ctx.ctx, pairs) == (plan + 1) % 4
+
+
+def test_fp32_batch_of_the_smallest_and_the_widest_window(fbs):
+    """Radius 0 and 31 in one batch: the persistent plans size one CTA for the widest window and walk tiles of both."""
+    pairs = _batch(61, n=6)
+    for i, q in enumerate(pairs):
+        q.update(radius=(0, 31, 17)[i % 3], sigma_s=9.0)
+    with fbs.Context(0) as ctx:
+        ref = _per_pair(ctx, pairs)
+        for plan in range(7):
+            for q in pairs:
+                q["disp_int"].fill_(-1)
+                q["disp_subpix"].fill_(-1.0)
+            fbs.fbs_batch_set_plan(ctx.ctx, pairs, plan)
+            fbs.fbs_compute_disparity_batched(ctx.ctx, pairs, torch.cuda.current_stream())
+            torch.cuda.synchronize()
+            fbs.fbs_sync(ctx.ctx)
+            for i, (q, (di, ds)) in enumerate(zip(pairs, ref)):
+                assert torch.equal(q["disp_int"], di) and torch.equal(q["disp_subpix"], ds), (plan, i)

@@ -332,6 +332,41 @@ def test_aggregate_chunk_and_window_edges(ctx, oracle_mod, D, radius, H, W):
     check_disparities(di, ds, ref, ref_di, ref_ds, 2.0, err)
 
 
+@pytest.mark.parametrize("D", [15, 16, 17, 32, 36, 63, 64, 65, 68])
+@pytest.mark.parametrize("radius,H,W", [(16, 9, 70), (19, 41, 39), (24, 30, 45), (31, 40, 66)])
+def test_aggregate_wide_windows(ctx, oracle_mod, D, radius, H, W):
+    """Ring, box width, guide window and weight buffers grow with the radius, up to the largest (31)."""
+    test_aggregate_chunk_and_window_edges(ctx, oracle_mod, D, radius, H, W)
+
+
+@pytest.mark.parametrize("offset", [1, 2])
+@pytest.mark.parametrize("D,radius", [(64, 3), (20, 17)])
+def test_volumes_that_start_off_16_bytes(fbs, ctx, oracle_mod, D, radius, offset):
+    """A volume of D % 4 == 0 that starts 4 or 8 bytes past a 16-byte boundary: copied 4 bytes at a time by the
+    aggregation and stored 1 or 2 floats at a time by the cost kernel, with the results of an aligned one."""
+    H, W = 11, 70
+    rng = np.random.default_rng(D + offset)
+    L = rng.integers(0, 256, (H, W, 3)).astype(np.uint8)
+    R = np.clip(np.roll(L, -4, axis=1).astype(np.int32) + rng.integers(-30, 31, L.shape), 0, 255).astype(np.uint8)
+    dl, dr = _dev(L), _dev(R)
+    cost = ctx.cost_volume(dl, dr, D)
+    agg, di, ds = ctx.aggregate(cost, dl, radius, 5.0, 30.0)
+    n = H * W * D
+    room = torch.full((2, n + 8), -3.0, device="cuda")
+    out = [room[k, offset:offset + n].view(H, W, D) for k in range(2)]
+    mi, ms = torch.empty_like(di), torch.empty_like(ds)
+    st = torch.cuda.current_stream()
+    fbs.fbs_cost_volume(ctx.ctx, dl, dr, H, W, 3, D, 0.0, out[0], st)
+    fbs.fbs_aggregate(ctx.ctx, out[0], dl, H, W, 3, D, radius, 5.0, 30.0, out[1], mi, ms, st)
+    torch.cuda.synchronize()
+    fbs.fbs_sync(ctx.ctx)
+    for got, want in zip(out + [mi, ms], [cost, agg, di, ds]):
+        assert torch.equal(got, want)
+    assert (room[:, :offset] == -3.0).all() and (room[:, offset + n:] == -3.0).all()
+    ref = oracle_mod.aggregate(oracle_mod.cost_volume(L, R, D, 0, 0.0), L, radius, 5.0, 30.0)
+    check_agg(agg.cpu().numpy(), ref, 2.0)
+
+
 @pytest.mark.parametrize("D,radius", [(12, 2), (40, 5), (70, 3)])
 def test_aggregate_keeps_infinities_and_nans_to_their_windows(ctx, oracle_mod, D, radius):
     """An infinite or NaN cost reaches exactly the sums whose window holds it, and neither wins the WTA."""
