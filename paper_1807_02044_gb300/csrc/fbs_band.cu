@@ -443,7 +443,7 @@ struct NetScratch {
 size_t net_scratch_bytes(int H, int W, int D, bool training, bool full_res)
 {
     const size_t Hq = (H + 3) / 4, Wq = (W + 3) / 4, P = Hq * Wq, Dq = (D + 3) / 4;
-    size_t n = al256(2 * P * 4) + 2 * al256(P * Dq * 4) + al256(P * 4) + al256(P * 24) + al256(P * 16) + 5 * al256(P * 64) + al256(P * 8);
+    size_t n = al256(2 * P * 4) + al256(P * Dq * 4) + al256(P * 4) + al256(P * 24) + al256(P * 16) + 5 * al256(P * 64) + al256(P * 8);
     if (training)
         n += 5 * al256(P * 64) + al256(P * 16) + al256(wgrad_partial_floats((int)Hq, (int)Wq) * 4) +
              al256((size_t)loss_blocks((int)P) * 4);
@@ -467,7 +467,6 @@ NetScratch carve_net(void* base, int H, int W, int D, bool training, bool full_r
     NetScratch s{};
     s.gq = (int32_t*)take(2 * P * 4);
     s.kh = (float*)take(P * Dq * 4);
-    take(P * Dq * 4);   // unused: the same calls fit under a workspace_cap as when the costs were stored too
     s.estar = (int32_t*)take(P * 4);
     s.featf = (float*)take(P * 24);
     s.x0 = (__nv_bfloat16*)take(P * 16);

@@ -566,3 +566,23 @@ def test_feature_points_match_the_oracle(fbs, oracle_mod, H, W, D, shift, th):
     assert ok.mean() >= 0.9
     assert np.array_equal(k.cpu().numpy()[ok], rk[ok])
     assert np.array_equal(c.cpu().numpy()[ok], rc[ok])
+
+
+def test_network_scratch_holds_the_row_sums_once(fbs):
+    """256 quarter pixels and Dq = 256: row sums of 256 KB and 95 KB of everything else fit under a workspace cap of
+    400 KB, and give what a context without a cap gives."""
+    H = W = 64
+    L, R = _rand_pair(5, H, W)
+    dl, dr = _dev(L), _dev(R)
+
+    def forward(cap):
+        out = [torch.empty(s, device="cuda") for s in ((H // 4, W // 4, 2), (H, W), (H, W))]
+        with fbs.Context(0, workspace_cap=cap) as ctx:
+            fbs.fbs_band_net_load(ctx.ctx, fbs.default_band_net_path())
+            fbs.fbs_band_net_forward(ctx.ctx, dl, dr, H, W, 3, 1024, *out)
+            torch.cuda.synchronize()
+            fbs.fbs_sync(ctx.ctx)
+        return out
+
+    for a, b in zip(forward(400 * 1024), forward(0)):
+        assert torch.equal(a, b)
