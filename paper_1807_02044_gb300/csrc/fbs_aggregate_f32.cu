@@ -120,7 +120,7 @@ __host__ __device__ inline int guide_words(int rho) { return (kTY + 2 * rho) * (
 // spatial terms, the guide window, then the cost rows [S][NC][DC] and the warps'
 // weights [4][4][WS]; the stage [4][32][DC + 4] of the epilogue lies over these.
 constexpr int kMaxSlots = 4;
-constexpr int kHeaderBytes = 80;   // full[4], done[4] (8 bytes each), abort flag
+constexpr int kHeaderBytes = 88;   // RingState
 __host__ __device__ inline size_t front_bytes(int rho)
 {
     return (kHeaderBytes + 4 * (size_t)spatial_floats(rho) + 4 * (size_t)guide_words(rho) + 127) & ~(size_t)127;
@@ -144,13 +144,69 @@ __host__ __device__ inline size_t smem_bytes(int rho, int dc, int slots)
 // Every wait is bounded.  When one runs out the error word is set, the warps walk
 // the rows that are left without waiting or copying, and the CTA lets the copies
 // in flight land (drain) and leaves its tile without storing anything.
-struct Ring {
-    uint32_t full, done;      // shared addresses, 8 bytes per slot
-    volatile uint32_t* abort;
+struct RingState {
+    uint64_t full[kMaxSlots], done[kMaxSlots];
+    uint32_t abort;           // a wait ran out
     int* err;
     long long limit;          // SM clock cycles that a wait may take
+};
+static_assert(sizeof(RingState) == kHeaderBytes, "at the start of shared memory");
+
+// A bounded wait for the phase of the given parity: by tries that sleep, or, for
+// limits shorter than a sleep, by polling.  One block, because it is inlined at
+// every wait and the small frames pay for the kernel's size.
+template <bool POLLS>
+__device__ __forceinline__ bool wait_within(uint32_t bar, uint32_t par, uint32_t limit_addr)
+{
+    uint32_t ok;
+    if (POLLS)
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t.reg .b64 t, u, lim;\n\t"
+            "ld.shared.b64 lim, [%3];\n\t"
+            "mov.u64 t, %%clock64;\n"
+            "POLL:\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "@p bra DONE;\n\t"
+            "mov.u64 u, %%clock64;\n\t"
+            "sub.s64 u, u, t;\n\t"
+            "setp.le.s64 q, u, lim;\n\t"
+            "@q bra POLL;\n"
+            "DONE:\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(par), "r"(limit_addr)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t.reg .b64 t, u, lim;\n\t"
+            "ld.shared.b64 lim, [%3];\n\t"
+            "mov.u64 t, %%clock64;\n"
+            "TRY:\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %4;\n\t"
+            "@p bra DONE;\n\t"
+            "mov.u64 u, %%clock64;\n\t"
+            "sub.s64 u, u, t;\n\t"
+            "setp.le.s64 q, u, lim;\n\t"
+            "@q bra TRY;\n"
+            "DONE:\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(par), "r"(limit_addr), "n"(tc::kSuspendNs)
+            : "memory");
+    return ok != 0;
+}
+
+template <bool POLLS>
+struct Ring {
+    RingState* st;
+    uint32_t full, done;      // shared addresses, 8 bytes per slot
     int S, slot;
     uint32_t parity;
+    // by every thread, before a barrier of the CTA
+    __device__ __forceinline__ void set_limit(long long limit)
+    {
+        if (threadIdx.x == 0) st->limit = limit;
+    }
     __device__ __forceinline__ void next()
     {
         if (++slot == S) {
@@ -158,19 +214,20 @@ struct Ring {
             parity ^= 1u;
         }
     }
+    __device__ __forceinline__ bool aborted() const { return *(volatile uint32_t*)&st->abort != 0; }
     // False when the phase is not complete and nothing is waited for any more.
     __device__ __forceinline__ bool wait(uint32_t bar, uint32_t par) const
     {
-        if (limit >= tc::kShortWait && tc::mbar_try_wait(bar, par)) return true;
-        if (*abort != 0) return false;
-        if (tc::mbar_wait_for(bar, par, limit)) return true;
-        *abort = 1u;
-        atomicCAS(err, 0, 31);
+        if (!POLLS && tc::mbar_try_wait(bar, par)) return true;
+        if (aborted()) return false;
+        if (wait_within<POLLS>(bar, par, tc::smem_u32(&st->limit))) return true;
+        *(volatile uint32_t*)&st->abort = 1u;
+        atomicCAS(st->err, 0, 31);
         return false;
     }
-    // After a wait ran out, between barriers of the CTA: the copies in flight (those
-    // of a slot's last box; the ones before it were waited for) have landed, or had
-    // about 2 s more.
+    // After a wait ran out and a barrier of the CTA: the copies in flight (those of a
+    // slot's last box; the ones before it were waited for) have landed, or had about
+    // 2 s more.
     template <Copy COPY>
     __device__ __forceinline__ void drain() const
     {
@@ -198,17 +255,17 @@ struct Volume {
 // slot; zeros outside the image and for disparities >= D.  kTma: one warp, which
 // notes the phase (parity) that the box completes; otherwise all of them, a thread
 // its share.
-template <int DC, Copy COPY>
-__device__ __forceinline__ void load_cost_row(const Ring& ring, int slot, uint32_t parity, uint32_t rows_a, const Volume& v,
+template <int DC, Copy COPY, bool POLLS>
+__device__ __forceinline__ void load_cost_row(const Ring<POLLS>& ring, int slot, uint32_t parity, uint32_t rows_a, const Volume& v,
                                               int r, int xlo, int NC, int dc0)
 {
     const uint32_t dst = rows_a + slot * (uint32_t)(NC * DC * 4), bar = ring.full + 8 * slot;
     if constexpr (COPY == kTma) {
         if ((threadIdx.x & 31) == 0) {
-            asm volatile("st.shared.u32 [%0], %1;" ::"r"(ring.done + 8 * slot + 4), "r"(2u + parity) : "memory");
             tc::fence_proxy_async();   // the slot was read, and may hold staged sums, through the generic proxy
             tc::mbar_expect_tx(bar, 4u * DC * (uint32_t)NC);
             tma_load_3d(dst, v.map, dc0, xlo, r, bar);
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(ring.done + 8 * slot + 4), "r"(2u + parity) : "memory");
         }
     } else {
         constexpr int E = COPY / 4;                     // floats per copy
@@ -472,10 +529,9 @@ __device__ __forceinline__ void wta_chunk(Tile& t, const float* st, int dc0, int
 }
 
 // Disparities dc0 .. dc0 + 8 KD - 1 of a tile (columns of DC staged disparities).
-// Starts and ends with every warp at the same point (a __syncthreads).  False (in
-// every thread) when a wait ran out: no copy is in flight and the ring is done with.
-template <int KD, int DC, Copy COPY, int ROWS>
-__device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_out, int dc0)
+// Starts and ends with every warp at the same point (a __syncthreads).
+template <int KD, int DC, Copy COPY, int ROWS, bool POLLS>
+__device__ __forceinline__ void aggregate_chunk(Tile& t, Ring<POLLS>& ring, float* agg_out, int dc0)
 {
     constexpr int NDC = 8 * KD;       // disparities of this chunk
     constexpr int PW = 32 / ROWS;     // pixels of a warp along x
@@ -492,16 +548,16 @@ __device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_
     // rows some pixel of the warp needs (none when no pixel has its band in this chunk)
     const bool on = t.whi >= dc0 && t.wlo < dc0 + NDC;
     const int w_lo = on ? t.wy - rho : t.H, w_hi = min(t.H - 1, t.wy + ROWS - 1) + rho;
-    // a chunk that no warp needs is passed over
-    if (!__syncthreads_or(on)) return true;
+    // a chunk that no warp needs is passed over, and every one after a wait that ran out
+    if (!__syncthreads_or(on && !ring.aborted())) return;
     auto load_row = [&](int r, int slot, uint32_t parity) {
         load_cost_row<DC, COPY>(ring, slot, parity, rows_a, t.vol, r, xlo, NC, dc0);
     };
     // the first S rows
     for (int i = COPY == kTma ? warp : 0; i < ring.S && t.r_lo + i <= t.r_hi; i += COPY == kTma ? kWarps : 1) {
         const int slot = ring.slot + i;
-        if (slot < ring.S) load_row(t.r_lo + i, slot, ring.parity);
-        else load_row(t.r_lo + i, slot - ring.S, ring.parity ^ 1u);
+        const bool wraps = slot >= ring.S;
+        load_row(t.r_lo + i, wraps ? slot - ring.S : slot, ring.parity ^ (wraps ? 1u : 0u));
     }
 
     // accumulating role: lane bits 0, 2, 3 = disparity group k, bits 1, 4 = pixel group
@@ -555,18 +611,17 @@ __device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_
             if (lane == 0) done = count_done(ring.done + 8 * ring.slot);
             done = __shfl_sync(0xffffffffu, done, 0);
             // the last warp to finish the row refills its slot
-            if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && *ring.abort == 0)
+            if ((done & (kWarps - 1)) == kWarps - 1 && r + ring.S <= t.r_hi && !ring.aborted())
                 load_row(r + ring.S, ring.slot, ring.parity ^ 1u);
         } else {
             if (lane == 0) tc::mbar_arrive(ring.done + 8 * ring.slot);
         }
         ring.next();
     }
-    // every row consumed: the stage may overwrite the rows and weights
-    if (__syncthreads_or(*ring.abort != 0)) {
-        ring.drain<COPY>();
-        return false;
-    }
+    __syncthreads();   // every row consumed: the stage may overwrite the rows and weights
+    // disparities to store and to search: none after a wait that ran out (no wait
+    // follows the barrier, so every thread reads the same)
+    const int nd = ring.aborted() ? 0 : min(NDC, t.d_end - dc0);
 
     // normalise and stage [pixel of the warp][d]
     float* const stage = t.rows + warp * 32 * SP;
@@ -592,7 +647,6 @@ __device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_
         }
     }
     __syncwarp();
-    const int nd = min(NDC, t.d_end - dc0);
     if (agg_out != nullptr) {
         for (int row = 0; row < ROWS && t.wy + row < t.H; ++row) {
             const int npx = min(PW, t.W - t.x0 - wx);
@@ -609,29 +663,28 @@ __device__ __forceinline__ bool aggregate_chunk(Tile& t, Ring& ring, float* agg_
     wta_chunk(t, stage + lane * SP, dc0, max(0, t.blo - dc0), min(nd, t.bhi + 1 - dc0));
     tc::fence_proxy_async();   // the next chunk's bulk copies overwrite the stage
     __syncthreads();
-    return true;
 }
 
 // The ring's barriers and counters, set up once per CTA (ends with a __syncthreads).
-template <Copy COPY>
-__device__ __forceinline__ Ring make_ring(void* smem, int slots, long long limit, int* err)
+template <Copy COPY, bool POLLS>
+__device__ __forceinline__ Ring<POLLS> make_ring(void* smem, int slots, long long limit, int* err)
 {
-    Ring ring;
-    ring.full = tc::smem_u32(smem);
-    ring.done = ring.full + 8 * kMaxSlots;
-    ring.abort = (volatile uint32_t*)((uint8_t*)smem + 16 * kMaxSlots);
-    ring.err = err;
-    ring.limit = limit;
+    Ring<POLLS> ring;
+    ring.st = (RingState*)smem;
+    ring.full = tc::smem_u32(ring.st->full);
+    ring.done = tc::smem_u32(ring.st->done);
     ring.S = slots;
     ring.slot = 0;
     ring.parity = 0;
+    ring.set_limit(limit);
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxSlots; ++s) {
             tc::mbar_init(ring.full + 8 * s, COPY == kTma ? 1 : kThreads);
-            if (COPY == kTma) ((uint64_t*)smem)[kMaxSlots + s] = 0;
+            if (COPY == kTma) ring.st->done[s] = 0;
             else tc::mbar_init(ring.done + 8 * s, kWarps);
         }
-        *ring.abort = 0;
+        ring.st->abort = 0;
+        ring.st->err = err;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -644,12 +697,12 @@ __device__ __forceinline__ Ring make_ring(void* smem, int slots, long long limit
 // each pixel to its own band [lo, hi], a sub-range of [d_begin, d_end);
 // without it every pixel uses [0, D-1].  d_begin must be a multiple of 4.
 // False (in every thread) when a wait ran out: nothing was stored.
-template <Copy COPY, int ROWS>
+template <Copy COPY, int ROWS, bool POLLS>
 __device__ __forceinline__ bool aggregate_tile(const float* __restrict__ cost, const CUtensorMap* map, int ld,
                                                const uint8_t* __restrict__ guide, int H, int W, int C, int D,
                                                int rho, float neg_ks, float neg_kr, float* __restrict__ agg_out,
                                                int32_t* __restrict__ disp_int, float* __restrict__ disp_sub, int x0,
-                                               int y0, void* smem, Ring& ring, int d_begin, int d_end,
+                                               int y0, void* smem, Ring<POLLS>& ring, int d_begin, int d_end,
                                                const uint32_t* __restrict__ band)
 {
     constexpr int PW = 32 / ROWS;
@@ -715,16 +768,18 @@ __device__ __forceinline__ bool aggregate_tile(const float* __restrict__ cost, c
 
     for (int dc0 = d_begin; dc0 < d_end; dc0 += 64) {
         const int left = d_end - dc0;
-        bool ok;
         if (D > 32) {
-            if (left > 32) ok = aggregate_chunk<8, 64, COPY, ROWS>(t, ring, agg_out, dc0);
-            else ok = aggregate_chunk<4, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+            if (left > 32) aggregate_chunk<8, 64, COPY, ROWS>(t, ring, agg_out, dc0);
+            else aggregate_chunk<4, 64, COPY, ROWS>(t, ring, agg_out, dc0);
         } else if (D > 16) {
-            ok = aggregate_chunk<4, 32, COPY, ROWS>(t, ring, agg_out, dc0);
+            aggregate_chunk<4, 32, COPY, ROWS>(t, ring, agg_out, dc0);
         } else {
-            ok = aggregate_chunk<2, 16, COPY, ROWS>(t, ring, agg_out, dc0);
+            aggregate_chunk<2, 16, COPY, ROWS>(t, ring, agg_out, dc0);
         }
-        if (!ok) return false;
+    }
+    if (ring.aborted()) {
+        ring.template drain<COPY>();
+        return false;
     }
 
     if (valid) {
@@ -743,7 +798,7 @@ __device__ __forceinline__ bool aggregate_tile(const float* __restrict__ cost, c
 
 constexpr int kCtasPerSm = 4;
 
-template <Copy COPY>
+template <Copy COPY, bool POLLS>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 aggregate_f32_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
                      const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
@@ -751,7 +806,7 @@ aggregate_f32_kernel(const __grid_constant__ CUtensorMap map, const float* __res
                      int slots, long long wait_cycles, int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<COPY>(smem_f4, slots, wait_cycles, err);
+    Ring<POLLS> ring = make_ring<COPY, POLLS>(smem_f4, slots, wait_cycles, err);
     aggregate_tile<COPY, 2>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
                             blockIdx.x * kTX, blockIdx.y * kTY, smem_f4, ring, 0, D, nullptr);
 }
@@ -759,6 +814,7 @@ aggregate_f32_kernel(const __grid_constant__ CUtensorMap map, const float* __res
 // Band form: tile t aggregates its range tile_range[t] and each pixel takes
 // its winner inside its own band.  A warp owns 8 x 4 pixels here (bands come in
 // 4 x 4 blocks, and a warp computes the chunks that any of its pixels needs).
+template <bool POLLS>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __restrict__ cost, int ld,
                       const uint8_t* __restrict__ guide, int H, int W, int C, int D, int rho, float neg_ks, float neg_kr,
@@ -767,7 +823,7 @@ aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __re
                       int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<kTma>(smem_f4, slots, wait_cycles, err);
+    Ring<POLLS> ring = make_ring<kTma, POLLS>(smem_f4, slots, wait_cycles, err);
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the ranges and bands come from earlier kernels
     const int2 r = tile_range[(size_t)blockIdx.y * gridDim.x + blockIdx.x];
     aggregate_tile<kTma, 4>(cost, &map, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, nullptr, disp_int, disp_sub,
@@ -777,12 +833,13 @@ aggregate_band_kernel(const __grid_constant__ CUtensorMap map, const float* __re
 // Persistent form over a batch: CTAs claim (pair, tile) items from a counter;
 // pairs[p].agg_off is the first item of pair p, items of a pair are its tiles
 // in row-major order.  No CTA waits on another.
+template <bool POLLS>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, int nitems, int* __restrict__ counter,
                              int slots, int* __restrict__ err)
 {
     extern __shared__ __align__(128) float4 smem_f4[];
-    Ring ring = make_ring<kAsync16>(smem_f4, slots, 0, err);
+    Ring<POLLS> ring = make_ring<kAsync16, POLLS>(smem_f4, slots, 0, err);
     __shared__ int item_s;
     for (;;) {
         if (threadIdx.x == 0) item_s = atomicAdd(counter, 1);
@@ -794,7 +851,7 @@ aggregate_f32_batched_kernel(const BatchPair* __restrict__ pairs, int npairs, in
         const BatchPair& bp = pairs[pi];
         const int t = item - bp.agg_off;
         const int ntx = (bp.W + kTX - 1) / kTX;
-        ring.limit = bp.wait_cycles;
+        ring.set_limit(bp.wait_cycles);
         if (!aggregate_tile<kAsync16, 2>(bp.cost, nullptr, bp.ld, bp.left, bp.H, bp.W, bp.C, bp.D, bp.radius, bp.neg_ks,
                                          bp.neg_kr, nullptr, bp.disp_int, bp.disp_sub, (t % ntx) * kTX, (t / ntx) * kTY,
                                          smem_f4, ring, 0, bp.D, nullptr))
@@ -831,21 +888,21 @@ bool encode_volume(CUtensorMap* map, const float* cost, int ld, int H, int W, in
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <Copy COPY>
+template <Copy COPY, bool POLLS>
 cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
                         int D, int rho, float neg_ks, float neg_kr, float* agg_out, int32_t* disp_int, float* disp_sub,
                         long long wait_cycles, int* err, bool after_cost, cudaStream_t stream)
 {
     const int slots = ring_slots(rho, column_size(D));
     const size_t smem = smem_bytes(rho, column_size(D), slots);
-    cudaError_t e = fbs::raise_smem_limit(aggregate_f32_kernel<COPY>, (int)smem);
+    cudaError_t e = fbs::raise_smem_limit(aggregate_f32_kernel<COPY, POLLS>, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
     if (after_cost)
-        return fbs::launch_after(aggregate_f32_kernel<COPY>, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D,
+        return fbs::launch_after(aggregate_f32_kernel<COPY, POLLS>, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D,
                                  rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, wait_cycles, err);
     fbs::note_launch();
-    aggregate_f32_kernel<COPY><<<grid, kThreads, smem, stream>>>(
+    aggregate_f32_kernel<COPY, POLLS><<<grid, kThreads, smem, stream>>>(
         map, cost, ld, guide, H, W, C, D, rho, neg_ks, neg_kr, agg_out, disp_int, disp_sub, slots, wait_cycles, err);
     return cudaGetLastError();
 }
@@ -853,22 +910,24 @@ cudaError_t launch_copy(const CUtensorMap& map, const float* cost, int ld, const
 }  // namespace
 
 long long wait_limit(long long wait_cycles) { return wait_cycles > 0 ? wait_cycles : tc::kWaitCycles; }
+bool wait_polls(long long wait_cycles) { return wait_limit(wait_cycles) < tc::kShortWait; }
 
 int agg_f32_tiles(int H, int W) { return ((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY); }
 
-cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out, int* slots_out)
+cudaError_t prepare_aggregate_f32_batched(int max_radius, bool polls, size_t* smem_out, int* slots_out)
 {
     *slots_out = ring_slots(max_radius, 64);
     const size_t smem = smem_bytes(max_radius, 64, *slots_out);
     *smem_out = smem;
-    return fbs::raise_smem_limit(aggregate_f32_batched_kernel, (int)smem);
+    return fbs::raise_smem_limit(polls ? aggregate_f32_batched_kernel<true> : aggregate_f32_batched_kernel<false>, (int)smem);
 }
 
 cudaError_t launch_aggregate_f32_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
-                                         size_t smem, int slots, int* err, cudaStream_t stream)
+                                         size_t smem, int slots, bool polls, int* err, cudaStream_t stream)
 {
     fbs::note_launch();
-    aggregate_f32_batched_kernel<<<grid, kThreads, smem, stream>>>(pairs, npairs, nitems, counter, slots, err);
+    auto kernel = polls ? aggregate_f32_batched_kernel<true> : aggregate_f32_batched_kernel<false>;
+    kernel<<<grid, kThreads, smem, stream>>>(pairs, npairs, nitems, counter, slots, err);
     return cudaGetLastError();
 }
 
@@ -884,11 +943,12 @@ cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guid
     const size_t smem = smem_bytes(radius, column_size(D), slots);
     CUtensorMap map;
     if (!encode_volume(&map, cost, ld, H, W, D, radius)) return cudaErrorInvalidValue;   // the context's own volume
-    cudaError_t e = fbs::raise_smem_limit(aggregate_band_kernel, (int)smem);
+    auto kernel = wait_polls(wait_cycles) ? aggregate_band_kernel<true> : aggregate_band_kernel<false>;
+    cudaError_t e = fbs::raise_smem_limit(kernel, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY);
-    return fbs::launch_after(aggregate_band_kernel, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D, radius,
-                             neg_ks, neg_kr, tile_range, band, disp_int, disp_sub, slots, wait_limit(wait_cycles), err);
+    return fbs::launch_after(kernel, grid, kThreads, smem, stream, map, cost, ld, guide, H, W, C, D, radius, neg_ks,
+                             neg_kr, tile_range, band, disp_int, disp_sub, slots, wait_limit(wait_cycles), err);
 }
 
 cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide, int H, int W, int C,
@@ -901,11 +961,11 @@ cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide
     const float neg_ks = (float)(-log2e / ((double)sigma_s * sigma_s));
     const float neg_kr = (float)(-log2e / ((double)sigma_r * sigma_r));
     CUtensorMap map{};
-    if (encode_volume(&map, cost, ld, H, W, D, radius))
-        return launch_copy<kTma>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                 wait_limit(wait_cycles), err, after_cost, stream);
-    return launch_copy<kAsync4>(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
-                                wait_limit(wait_cycles), err, after_cost, stream);
+    const bool tma = encode_volume(&map, cost, ld, H, W, D, radius), polls = wait_polls(wait_cycles);
+    auto launch = tma ? (polls ? launch_copy<kTma, true> : launch_copy<kTma, false>)
+                      : (polls ? launch_copy<kAsync4, true> : launch_copy<kAsync4, false>);
+    return launch(map, cost, ld, guide, H, W, C, D, radius, neg_ks, neg_kr, agg_out, disp_int, disp_sub,
+                  wait_limit(wait_cycles), err, after_cost, stream);
 }
 
 }  // namespace fbs

@@ -225,7 +225,8 @@ fbs_status build_graph(fbs_ctx* ctx, const Layout& L, int n, int plan, int slot,
 {
     size_t agg_smem = 0;
     int agg_slots = 0;
-    cudaError_t e = fbs::prepare_aggregate_f32_batched(L.max_radius, &agg_smem, &agg_slots);
+    const bool polls = fbs::wait_polls(ctx->wait_cycles);
+    cudaError_t e = fbs::prepare_aggregate_f32_batched(L.max_radius, polls, &agg_smem, &agg_slots);
     if (e == cudaSuccess) e = fbs::prepare_cost_batched();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batched kernel attributes");
     const int agg_per_sm = 2 * ((plan & 1) + 1);
@@ -241,7 +242,7 @@ fbs_status build_graph(fbs_ctx* ctx, const Layout& L, int n, int plan, int slot,
     if (e == cudaSuccess) e = fbs::launch_cost_batched(ctx->bpairs, n, L.items[1], ctx->bcounters + 1, g_cost, cs);
     if (e == cudaSuccess)
         e = fbs::launch_aggregate_f32_batched(ctx->bpairs, n, L.items[2], ctx->bcounters + 2, g_agg, agg_smem,
-                                              agg_slots, ctx->derr, cs);
+                                              agg_slots, polls, ctx->derr, cs);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     if (e == cudaSuccess) e = e2;
@@ -254,7 +255,9 @@ fbs_status build_graph(fbs_ctx* ctx, const Layout& L, int n, int plan, int slot,
 fbs_status get_graph(fbs_ctx* ctx, const std::string& sig, const Layout& L, int n, int plan, int slot,
                      cudaGraphExec_t* out)
 {
-    const std::string key = sig + "|p" + std::to_string(plan) + "|s" + std::to_string(slot);
+    // the wait limit is read from the table, but a short one takes other kernels
+    const std::string key = sig + "|p" + std::to_string(plan) + "|s" + std::to_string(slot) +
+                            (fbs::wait_polls(ctx->wait_cycles) ? "|polls" : "");
     auto it = ctx->bgraphs.find(key);
     if (it != ctx->bgraphs.end()) {
         *out = it->second.exec;

@@ -109,8 +109,10 @@ cudaError_t launch_aggregate_f32(const float* cost, int ld, const uint8_t* guide
                                  int C, int D, int radius, float sigma_s, float sigma_r,
                                  float* agg_out, int32_t* disp_int, float* disp_sub, long long wait_cycles,
                                  int* err, bool after_cost, cudaStream_t stream);
-// The limit in SM clock cycles that wait_cycles stands for.
+// The limit in SM clock cycles that wait_cycles stands for, and whether it is so
+// short that the FP32 aggregation has to poll (other instances of its kernels).
 long long wait_limit(long long wait_cycles);
+bool wait_polls(long long wait_cycles);
 
 // ---- steps 2-4 on the tensor cores (BF16 / FP16 operands, FP32 accumulate) ---
 // cost: 16-bit x-blocked volume (see launch_cost_build_xblock16), 16-byte
@@ -187,7 +189,7 @@ struct BatchPair {
     const uint8_t* right;
     int H, W, C, D, radius, ld, mode;
     float neg_ks, neg_kr, tau;
-    long long wait_cycles;   // > 0: the limit of one wait in the aggregation
+    long long wait_cycles;   // wait_limit(): of one wait in the aggregation
     CostScratch sc;
     float* cost;
     int32_t* disp_int;
@@ -214,9 +216,9 @@ cudaError_t launch_stats_batched(const BatchPair* pairs, int npairs, int nitems,
                                  cudaStream_t stream);
 cudaError_t launch_cost_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
                                 cudaStream_t stream);
-cudaError_t prepare_aggregate_f32_batched(int max_radius, size_t* smem_out, int* slots_out);
+cudaError_t prepare_aggregate_f32_batched(int max_radius, bool polls, size_t* smem_out, int* slots_out);
 cudaError_t launch_aggregate_f32_batched(const BatchPair* pairs, int npairs, int nitems, int* counter, int grid,
-                                         size_t smem, int slots, int* err, cudaStream_t stream);
+                                         size_t smem, int slots, bool polls, int* err, cudaStream_t stream);
 
 // ---- context helpers for entry points defined outside fbs_api.cu -------------
 // Host-side checks of fbs_compute_disparity's arguments (sets the message).
