@@ -88,7 +88,7 @@ fbs_status run_path(fbs_ctx* ctx, const uint8_t* left, const uint8_t* right, int
     cudaError_t e;
     {
         LaunchScope ls(ctx, FBS_KERNEL_COST, st);
-        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost, radius, st);
+        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost, radius, ctx->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cost build launch");
     {
@@ -408,7 +408,7 @@ fbs_status fbs_cost_volume(fbs_ctx* ctx, const uint8_t* left, const uint8_t* rig
     cudaError_t e;
     {
         LaunchScope ls(ctx, FBS_KERNEL_COST, st);
-        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, D, ctx->opt.cost, tau, cost_out, 0, st);
+        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, D, ctx->opt.cost, tau, cost_out, 0, ctx->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cost build launch");
     return FBS_OK;

@@ -665,7 +665,8 @@ fbs_status run_banded(fbs_ctx* ctx, const fbs_pair* p, const float* centre, cons
     if (e != cudaSuccess) return cuda_fail(ctx, e, "band planning launch");
     {
         LaunchScope ls(ctx, FBS_KERNEL_COST, st);
-        e = fbs::launch_cost_band(sc, p->left, p->right, H, W, p->C, D, ld, p->radius, s.tile_range, cost, st);
+        e = fbs::launch_cost_band(sc, p->left, p->right, H, W, p->C, D, ld, p->radius, s.tile_range, cost, ctx->num_sms,
+                                  st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "band cost launch");
     {

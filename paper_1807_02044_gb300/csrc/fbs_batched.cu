@@ -378,7 +378,8 @@ fbs_status build_branch_graph(fbs_ctx* ctx, int n, const fbs_pair* pairs, int nb
             const fbs::CostScratch sc = fbs::carve_cost_scratch(base, q.H, q.W);
             const int ld = fbs::padded_ld(q.D);
             float* cost = (float*)(base + stats);
-            e = fbs::launch_cost_build(sc, q.left, q.right, q.H, q.W, q.C, q.D, ld, mode, q.tau, cost, q.radius, s);
+            e = fbs::launch_cost_build(sc, q.left, q.right, q.H, q.W, q.C, q.D, ld, mode, q.tau, cost, q.radius,
+                                       ctx->num_sms, s);
             g->kernels[FBS_KERNEL_COST] += fbs::launch_count() - k0;
             k0 = fbs::launch_count();
             if (e == cudaSuccess)

@@ -293,7 +293,6 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
             const float4* slw = sl + rp * kCostLeft + skew4(xl);
             const float4* grw = gr + rp * kCostRight + skew4(base);
             const float4* srw = sr + rp * kCostRight + skew4(base);
-            constexpr int ST = MIRROR ? 1 : -1;     // columns the window moves per disparity
             constexpr int IN = MIRROR ? 5 : 0;      // where the new column comes in
 
             auto put = [&](int s, const float (&c)[4][2][2]) {   // c[pixel][row][s even, odd]
@@ -398,7 +397,6 @@ __device__ __forceinline__ void cost_tile(const CostArgs& a, int x0, int y0, int
                     if (s & 1) put(s, c);
                 }
             }
-            (void)ST;
             __syncthreads();
             // a warp writes one row: up to 128 contiguous bytes per pixel
             if (y0 + warp < H) {
@@ -995,15 +993,22 @@ cudaError_t launch_cost_vw(const CostArgs& a, cudaStream_t stream)
 // When may the aggregation's CTAs start: with the cost kernel's (they set up
 // while it runs), or as its CTAs end?  An early CTA takes any place that is
 // free, so where the aggregation does not fill the chip (four CTAs per SM) some
-// SMs get several and others none.  Early for a grid that fills it or for tiles
-// of so little work that the set-up is what counts: 160x120, D = 16, rho = 4 26
-// against 28 us late; late otherwise: 82x196, D = 198, rho = 15 356 against 488 us
-// early, 160x120, D = 64, rho = 7 42 against 50 us, 200x200, D = 64, rho = 3 33
-// against 35 us.
-bool agg_early(int H, int W, int D, int radius)
+// SMs get several and others none.  Early for a grid that fills it, for one so
+// small that every CTA of both kernels finds an SM of its own, and for tiles of so
+// little work that the set-up is what counts (work: window rows x window columns
+// of 8 pixels x disparities staged).  Measured, early and late, at 12 to 640 tiles,
+// D = 8 .. 200, radius 0 .. 15, calls in a row: up to 45 tiles early is 0 - 16%
+// faster, most of all at little work (40x24, D = 64, radius 3 20.6 and 22.6 us); at
+// 150 to 350 tiles late wins from about 6400 on (160x120, D = 128, radius 15 by 40%;
+// 160x120, D = 16, radius 4 takes 20.7 us early, 22.6 late); at 480 tiles late is
+// 8% faster at most; from 600 on early is never more than 2% behind.  Over all of
+// these the rule is 0.2% above the better of the two on average, always early 3.7%.
+bool agg_early(int H, int W, int D, int radius, int num_sms)
 {
     const long long tiles = (long long)((W + kAggTileX - 1) / kAggTileX) * ((H + kAggTileY - 1) / kAggTileY);
-    return tiles >= 4 * 152 || (kAggTileY + 2 * radius) * (8 + 2 * radius) * (long long)D < 100 * 64;
+    const long long staged = D <= 16 ? 16 : (D + 31) / 32 * 32;
+    return tiles >= 4LL * num_sms || 2 * tiles <= num_sms ||
+           (kAggTileY + 2 * radius) * (8 + 2 * radius) * staged < 100 * 64;
 }
 
 // One view of the FP32 volume (mode 0: after the statistics).
@@ -1093,35 +1098,36 @@ CostScratch carve_cost_scratch(void* base, int H, int W)
 }
 
 cudaError_t launch_cost_build(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                              int C, int D, int ld, int mode, float tau, float* cost, int agg_radius,
+                              int C, int D, int ld, int mode, float tau, float* cost, int agg_radius, int num_sms,
                               cudaStream_t stream)
 {
     cudaError_t e = mode == 0 ? launch_stats(sc, left, right, H, W, C, stream) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost, agg_early(H, W, D, agg_radius)}, mode, false,
-                            stream);
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost, agg_early(H, W, D, agg_radius, num_sms)},
+                            mode, false, stream);
 }
 
 cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                             int C, int D, int ld, int radius, const int2* tile_range, float* cost, cudaStream_t stream)
+                             int C, int D, int ld, int radius, const int2* tile_range, float* cost, int num_sms, cudaStream_t stream)
 {
     cudaError_t e = launch_stats(sc, left, right, H, W, C, stream);
     if (e == cudaSuccess) e = fbs::raise_smem_limit(cost_band_kernel, (int)kCostSmem);
     if (e != cudaSuccess) return e;
     const int ntx = (W + kAggTileX - 1) / kAggTileX, nty = (H + kAggTileY - 1) / kAggTileY;
     return fbs::launch_after(cost_band_kernel, dim3((W + kCostPx - 1) / kCostPx, (H + kCostRows - 1) / kCostRows), kCostThreads,
-                             kCostSmem, stream, CostArgs{sc, left, right, H, W, C, D, ld, 0.f, cost, agg_early(H, W, D, radius)}, radius, tile_range, ntx,
-                             nty);
+                             kCostSmem, stream,
+                             CostArgs{sc, left, right, H, W, C, D, ld, 0.f, cost, agg_early(H, W, D, radius, num_sms)}, radius,
+                             tile_range, ntx, nty);
 }
 
 cudaError_t launch_cost_build_lr(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                                  int C, int D, int ld, int mode, float tau, float* cost, float* cost_r, int agg_radius,
-                                 cudaStream_t stream)
+                                 int num_sms, cudaStream_t stream)
 {
-    cudaError_t e = launch_cost_build(sc, left, right, H, W, C, D, ld, mode, tau, cost, agg_radius, stream);
+    cudaError_t e = launch_cost_build(sc, left, right, H, W, C, D, ld, mode, tau, cost, agg_radius, num_sms, stream);
     if (e != cudaSuccess) return e;
-    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost_r, agg_early(H, W, D, agg_radius)}, mode, true,
-                            stream);
+    return launch_cost_view(CostArgs{sc, left, right, H, W, C, D, ld, tau, cost_r, agg_early(H, W, D, agg_radius, num_sms)},
+                            mode, true, stream);
 }
 
 cudaError_t launch_cost_build_xblock16(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H,

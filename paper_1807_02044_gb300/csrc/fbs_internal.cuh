@@ -70,17 +70,17 @@ __host__ __device__ inline int rgbx_pitch(int W) { return (W + 1) & ~1; }
 
 // cost[(y*W + x)*ld + d] for d < D; entries D <= d < ld are written as 0.
 // agg_radius: the window radius of the aggregation that follows (0 if none does);
-// it decides when that kernel's CTAs may start, not the results.
+// with num_sms it decides when that kernel's CTAs may start, not the results.
 cudaError_t launch_cost_build(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                               int C, int D, int ld, int mode, float tau, float* cost, int agg_radius,
-                              cudaStream_t stream);
+                              int num_sms, cudaStream_t stream);
 
 // Both views (Sec. II-A, Sec. III): cost as launch_cost_build, and cost_r
 // [H][W][ld] the right volume, cost_r(x, y, d) = cost(x + d, y, d), the maximum
 // cost where x + d >= W.
 cudaError_t launch_cost_build_lr(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
                                  int C, int D, int ld, int mode, float tau, float* cost, float* cost_r, int agg_radius,
-                                 cudaStream_t stream);
+                                 int num_sms, cudaStream_t stream);
 
 // 16-bit x-blocked volume cost[((y*ceil(W/8) + x/8)*Dp + d)*8 + x%8] with
 // Dp = tc_block_rows(D) = round_up(D,16) + 16 rows per block: d < D the cost,
@@ -173,7 +173,7 @@ cudaError_t launch_xblock16_pad_rows(int H, int W, int D, bool bf16, void* out, 
 cudaError_t launch_band_tiles(const float* centre, const float* conf, int H, int W, int D, int half_band,
                               float theta, uint32_t* band, int2* tile_range, cudaStream_t stream);
 cudaError_t launch_cost_band(const CostScratch& sc, const uint8_t* left, const uint8_t* right, int H, int W,
-                             int C, int D, int ld, int radius, const int2* tile_range, float* cost,
+                             int C, int D, int ld, int radius, const int2* tile_range, float* cost, int num_sms,
                              cudaStream_t stream);
 cudaError_t launch_aggregate_band(const float* cost, int ld, const uint8_t* guide, int H, int W, int C, int D,
                                   int radius, float sigma_s, float sigma_r, const int2* tile_range,

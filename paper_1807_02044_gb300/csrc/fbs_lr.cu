@@ -145,7 +145,8 @@ extern "C" fbs_status fbs_compute_disparity_lr(fbs_ctx* ctx, const uint8_t* left
     cudaError_t e;
     {
         LaunchScope ls(ctx, FBS_KERNEL_COST, st);
-        e = fbs::launch_cost_build_lr(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost_l, cost_r, radius, st);
+        e = fbs::launch_cost_build_lr(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost_l, cost_r, radius,
+                                      ctx->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cost build (both views) launch");
     {

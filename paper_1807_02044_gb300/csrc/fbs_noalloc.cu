@@ -67,7 +67,7 @@ extern "C" fbs_status fbs_compute_disparity_noalloc(fbs_ctx* ctx, const uint8_t*
     float* cost = (float*)((uint8_t*)scratch + stats);
     {
         LaunchScope ls(ctx, FBS_KERNEL_COST, st);
-        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost, radius, st);
+        e = fbs::launch_cost_build(sc, left, right, H, W, C, D, ld, ctx->opt.cost, tau, cost, radius, ctx->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cost build launch");
     {
