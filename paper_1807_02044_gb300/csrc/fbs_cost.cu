@@ -668,7 +668,8 @@ cost_xb_tad_kernel(const uint8_t* __restrict__ L, const uint8_t* __restrict__ R,
 }
 
 // ---- NCC, 16-bit x-blocked volume ----------------------------------------------
-// A CTA covers 64 pixels x 4 rows and every disparity.  All of Eq. (1) runs in
+// A CTA covers 64 pixels x 4 rows and every disparity (ncc_groups_per_cta: fewer on
+// small frames).  All of Eq. (1) runs in
 // FP32 on exact integers (grey_shift), and 9 P' - S_l' S_r' comes out of one FMA
 // rounded once -- the integer converted to float.  A thread computes two output
 // rows at once (block_sums: 4 FMAs for a column's two sums), and everything
@@ -701,22 +702,37 @@ constexpr int kNccWarps = 4;
 constexpr int kNccRows = 4;      // two pairs
 
 __host__ __device__ inline int ncc_groups(int D) { return (D + 15) / 16; }          // of 16 disparities
-__host__ __device__ inline int ncc_right_cols(int D) { return 16 * ncc_groups(D) + kNccPx + 1; }
+__host__ __device__ inline int ncc_right_cols(int groups) { return 16 * groups + kNccPx + 1; }
 // float4 entries of the four staged arrays, per pair of rows
 __host__ __device__ inline int ncc_left_len() { return skew4(kNccPx + 2); }
-__host__ __device__ inline int ncc_right_len(int D) { return skew4(ncc_right_cols(D)) + 1; }
+__host__ __device__ inline int ncc_right_len(int groups) { return skew4(ncc_right_cols(groups)) + 1; }
 // Store buffer of a warp: two pairs of rows, each [d / 8][block][row][8 d x 8
 // pixels] (128-byte lines, TMA's 128-byte swizzle) of 16 disparities and 8 blocks.
 constexpr int kNccPairBytes = 2 * 8 * 2 * 128, kNccWarpBytes = 2 * kNccPairBytes;
-__host__ __device__ inline size_t ncc_smem_bytes(int D)
+__host__ __device__ inline size_t ncc_smem_bytes(int groups)
 {
-    return 1024 + (size_t)kNccWarps * kNccWarpBytes + (size_t)2 * 16 * 2 * (ncc_left_len() + ncc_right_len(D));
+    return 1024 + (size_t)kNccWarps * kNccWarpBytes + (size_t)2 * 16 * 2 * (ncc_left_len() + ncc_right_len(groups));
+}
+// Groups per CTA, of the ng groups of costs and one more (the rows after them): all,
+// or where the tiles leave SMs without a CTA, a share of them (whole rounds of the
+// warps) such that no SM gets two, if that saves two rounds (each CTA stages the
+// grey rows of its own range; one round saved was 300x60, D = 128, radius 0 14.7 ->
+// 15.5 us).  On the smallest frames one CTA for all of D was slower than the
+// integer form: BF16 path, integer form -> undivided -> now: 80x60, D = 208, radius
+// 5 16.5 -> 20.6 -> 14.5 us; 40x24, D = 256, radius 0 14.5 -> 18.5 -> 12.3 us; 300x60,
+// D = 256, radius 5 22.7 -> 24.7 -> 22.6 us.
+inline int ncc_groups_per_cta(int D, int tiles, int num_sms)
+{
+    const int all = ncc_groups(D) + 1, rounds = (all + kNccWarps - 1) / kNccWarps;
+    const int share = num_sms / tiles < 1 ? 1 : num_sms / tiles;
+    const int own = (rounds + share - 1) / share;
+    return (rounds - own < 2 ? rounds : own) * kNccWarps;
 }
 
 template <bool BF16>
 __global__ void __launch_bounds__(32 * kNccWarps, 4)
 cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* __restrict__ L,
-                   const uint8_t* __restrict__ R, int H, int W, int C, int D, uint2* __restrict__ rgbx)
+                   const uint8_t* __restrict__ R, int H, int W, int C, int D, int per_cta, uint2* __restrict__ rgbx)
 {
     extern __shared__ uint8_t sm_ncc[];
     // let a programmatically launched successor (the tensor-core aggregation)
@@ -726,9 +742,12 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
     constexpr int ROWS = kNccRows, PAIRS = ROWS / 2, nthr = 32 * kNccWarps;
     const int tid = threadIdx.x, lane = tid & 31;
     const int x0 = blockIdx.x * kNccPx, y0 = blockIdx.y * ROWS;
-    const int ng = ncc_groups(D), nr = ncc_right_cols(D);
-    const int rb = x0 - 16 * ng;             // image column of right column 0
-    const int LL = ncc_left_len(), RL = ncc_right_len(D);
+    const int ng = ncc_groups(D);
+    // this CTA's groups g0 .. g1-1, of which those before gc have costs
+    const int g0 = blockIdx.z * per_cta, g1 = min(g0 + per_cta, ng + 1), gc = min(g1, ng);
+    const int nr = ncc_right_cols(gc - g0);
+    const int rb = x0 - 16 * gc;             // image column of right column 0
+    const int LL = ncc_left_len(), RL = ncc_right_len(gc - g0);
     uint8_t* const buffers = sm_ncc + ((1024u - (tc::smem_u32(sm_ncc) & 1023u)) & 1023u);
     float4* const gl = (float4*)(buffers + kNccWarps * kNccWarpBytes);   // [PAIRS][LL]: columns x0 - 1 ..
     float4* const sl = gl + PAIRS * LL;      // [PAIRS][LL]: centres x0 ..
@@ -756,7 +775,7 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
 #pragma unroll
         for (int k = 0; k < PAIRS; ++k)
             dst[k * (left ? LL : RL)] = make_float4(g[2 * k], g[2 * k + 1], g[2 * k + 2], g[2 * k + 3]);
-        if (left && c >= 1 && c <= kNccPx && xs < W) {
+        if (left && c >= 1 && c <= kNccPx && xs < W && g0 == 0) {
             uint2* o = rgbx + (size_t)y0 * rgbx_pitch(W) + xs;
 #pragma unroll
             for (int j = 1; j <= ROWS; ++j)
@@ -806,7 +825,7 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
     };
 
     const int rp = lane >> 4;
-    for (int grp = tid >> 5; grp <= ng; grp += kNccWarps) {
+    for (int grp = g0 + (tid >> 5); grp < g1; grp += kNccWarps) {
         // the warp's previous stores have read its buffer
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncwarp();
@@ -855,7 +874,7 @@ cost_xb_ncc_kernel(const __grid_constant__ CUtensorMap out_map, const uint8_t* _
 
         const int d0 = 16 * grp;
         // right column of (x, d), window offset k: x - d + k - rb = base + (i + k - s)
-        const int base = xl + 16 * ng - d0;
+        const int base = xl + 16 * gc - d0;
         const float4* grw = gr + rp * RL + skew4(base);
         const float4* srw = sr + rp * RL + skew4(base);
         auto at = [](int m) { return m + (m >> 2); };   // offset of column base + m (base is a multiple of 4)
@@ -936,12 +955,18 @@ cudaError_t launch_cost_xb_ncc(const CostScratch& sc, const uint8_t* left, const
             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    const size_t smem = ncc_smem_bytes(D);
-    cudaError_t e = fbs::raise_smem_limit(cost_xb_ncc_kernel<BF16>, (int)smem);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kNccPx - 1) / kNccPx, (H + kNccRows - 1) / kNccRows);
+    const int ng = ncc_groups(D), per_cta = ncc_groups_per_cta(D, (int)(grid.x * grid.y), sms);
+    grid.z = (ng + per_cta) / per_cta;   // ng + 1 groups
+    const size_t smem = ncc_smem_bytes(per_cta < ng ? per_cta : ng);
+    e = fbs::raise_smem_limit(cost_xb_ncc_kernel<BF16>, (int)smem);
+    if (e != cudaSuccess) return e;
     fbs::note_launch();
-    cost_xb_ncc_kernel<BF16><<<grid, 32 * kNccWarps, smem, stream>>>(map, left, right, H, W, C, D, sc.rgbx);
+    cost_xb_ncc_kernel<BF16><<<grid, 32 * kNccWarps, smem, stream>>>(map, left, right, H, W, C, D, per_cta, sc.rgbx);
     return cudaGetLastError();
 }
 

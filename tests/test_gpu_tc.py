@@ -288,3 +288,12 @@ def test_radius_zero_maps_are_those_of_the_rounded_fp32_costs(fbs, prec, H, W, C
     sub = best + np.where(ok, (a - c) / np.where(ok, den, np.float32(1)), np.float32(0)).astype(np.float32)
     assert np.array_equal(di.cpu().numpy(), best)
     np.testing.assert_allclose(ds.cpu().numpy(), sub, rtol=0, atol=2.0 ** -22 * max(1, D))
+
+
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("H,W,C,D", [(24, 40, 3, 49), (24, 40, 1, 128), (40, 200, 3, 256), (60, 300, 3, 241),
+                                     (61, 310, 1, 256), (120, 300, 3, 256)])
+def test_cost_groups_divided_over_ctas(fbs, prec, H, W, C, D):
+    """Frames whose tiles leave SMs without a CTA share out the groups of 16 disparities (one round of the warps and
+    more, one CTA with the rows after the costs only), larger ones do not."""
+    test_radius_zero_maps_are_those_of_the_rounded_fp32_costs(fbs, prec, H, W, C, D)
