@@ -152,8 +152,8 @@ fbs_status fbs_compute_disparity_host(fbs_ctx *ctx, const uint8_t *left, const u
  *     lrc != 0 every left pixel whose disparity d fails Eq. (9) -- u - d < 0 or
  *     the right disparity at (u - d, v) differs from d -- is set to -1 in both.
  *   disp_int_right / disp_subpix_right (each nullable): the right map.
- * FP32 context: each matching cost is computed once and stored in the left
- * volume at (u, v, d) and in the right volume at (u - d, v, d); scratch: two
+ * FP32 context: two cost kernels write the left volume and the right one,
+ * whose entry (u - d, v, d) is the left one's (u, v, d) bit for bit; scratch: two
  * cost volumes (2 * H*W*round_up(D,4)*4 bytes) and two integer maps.
  * BF16 / FP16 context: the tensor-core path of fbs_compute_disparity for the
  * left view, and for the right view the same path on the horizontally
@@ -236,9 +236,10 @@ fbs_status fbs_compute_disparity_batched(fbs_ctx *ctx, int n, const fbs_pair *pa
 /* The plan the autotuner chose for this batch shape, or -1 if none yet.
  * FP32 (0..6): plans 0..3 persistent, plan = 2 * order + (aggregation CTAs
  * per SM / 2 - 1), order 0 = largest pair first, 1 = as given; plans 4..6
- * branched with {1, 2, 4}[plan - 4] branches.  BF16 / FP16 (0..5): plan = 2 * b + s,
- * graph branches {1, 2, 4}[b], window rows per tensor-core pipeline stage
- * s = 0: the kernel's maximum, s = 1: at most 3. */
+ * branched with {1, 2, 4}[plan - 4] branches.  BF16 / FP16 (0..6): plans 0..5
+ * = 2 * b + s, graph branches {1, 2, 4}[b], window rows per tensor-core pipeline
+ * stage s = 0: the kernel's maximum, s = 1: at most 3; plan 6 the persistent
+ * aggregations. */
 fbs_status fbs_batch_plan(fbs_ctx *ctx, int n, const fbs_pair *pairs, int *plan);
 
 /* Pin the plan of this batch shape in ctx (numbered as above), skipping the

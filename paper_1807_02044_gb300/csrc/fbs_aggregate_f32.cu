@@ -46,10 +46,15 @@
 //
 // Measured on GB300 (CUDA events), before -> now; before: 4 pixels x 8 disparities
 // per thread, scalar FMAs, 256-thread CTAs in step through a cp.async ring:
-//   640x480,  D = 64,  rho = 7:    425 -> 232 us (38.1 TFLOP/s)
-//   640x480,  D = 64,  rho = 2:    125 ->  62 us
-//   767x575,  D = 93,  rho = 11:  2263 -> 1184 us
-//   1280x960, D = 128, rho = 15: 10390 -> 6896 us (43.8 TFLOP/s)
+//   640x480,  D = 64,  rho = 7:    427 ->  232 us (38.1 TFLOP/s)
+//   640x480,  D = 64,  rho = 2:    132 ->   62 us
+//   767x575,  D = 96,  rho = 11:  2261 -> 1131 us
+//   1280x960, D = 128, rho = 15: 10383 -> 6550 us (46.2 TFLOP/s)
+// and where the wide windows leave fewer warps per SM (12 at rho = 13 .. 19, 8 at 20
+// .. 24, 4 at 31, for 16, 16 and 8 before):
+//   640x480,  D = 64,  rho = 20:  2173 -> 1572 us (42.1 TFLOP/s)
+//   640x480,  D = 64,  rho = 24:  2983 -> 2178 us (43.4 TFLOP/s)
+//   640x480,  D = 64,  rho = 31:  6079 -> 4860 us (32.1 TFLOP/s)
 #include "fbs_internal.cuh"
 #include "packed_f32.cuh"
 #include "tc_aggregate.cuh"
@@ -78,7 +83,7 @@ __host__ __device__ inline int column_size(int D) { return D > 32 ? 64 : D > 16 
 // How a cost row is copied to shared memory: one TMA box (volumes that are 16-byte
 // aligned with ld % 4 == 0), or cp.async of so many bytes by every thread: 16
 // (the same volumes, where no tensor map is at hand) or 4 (any volume: 640x480,
-// D = 63, rho = 7: 318 us against 236 us at D = 64 by TMA; 470 us before).
+// D = 63, rho = 7: 328 us against 232 us at D = 64 by TMA; 474 us before).
 enum Copy { kTma = 0, kAsync16 = 16, kAsync4 = 4 };
 
 template <int BYTES>

@@ -215,7 +215,7 @@ __device__ __forceinline__ float warp_min(float v)
 // column, lanes over e: the twelve row sums that their windows cover are read
 // once each, and the eight pixels' features are finished together, one lane
 // each.  Bound by issue.  The division by the tap count is a multiplication by
-// its reciprocal and one residual step (Markstein's theorem; checked for every
+// its reciprocal and one residual step (Markstein's theorem; tested on the CPU for every
 // significand and all tap counts to be the correctly rounded quotient).  A
 // kernel that stored the means and one thread per pixel that read them twice
 // took 23.5 + 35 us at 320 x 160, Dq = 64; now 14.6 (alone, cold caches).

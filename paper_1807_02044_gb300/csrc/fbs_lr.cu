@@ -1,6 +1,6 @@
 // Both disparity maps and the left-right consistency check (Sec. II-A,
-// Sec. III, Eq. (9)).  FP32: each matching cost is computed once and stored in
-// the left volume at (u, v, d) and in the right volume at (u - d, v, d); each
+// Sec. III, Eq. (9)).  FP32: two cost kernels write the left volume and the right
+// one, whose entry (u - d, v, d) is the left one's (u, v, d) bit for bit; each
 // volume is aggregated with its own image as guide (Sec. II-B), WTA and
 // Eq. (10) give both maps.  BF16 / FP16: the tensor-core path runs on the pair
 // and on its mirrored, swapped copy (whose left view is the mirrored right
